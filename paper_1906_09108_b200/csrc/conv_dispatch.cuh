@@ -33,7 +33,7 @@ struct TensorMapCache {
 
 inline bool tc_eligible(const ConvGeom& g) {
   return g.R == 3 && g.S == 3 && g.stride == 1 && g.pad == 1 && g.P == g.H && g.Q == g.W &&
-         tc::conv_tc_supported(g.N, g.H, g.W, g.Ci, g.Co);
+         tc::conv_tc_supported(g.N, g.H, g.W, g.Ci, g.Co, (size_t)g.N * g.P * g.Q);
 }
 
 // Runs D = conv3x3(act, wgt) on the tensor cores.  `Ck`/`Cn` are the GEMM-K and GEMM-N channel
@@ -94,8 +94,8 @@ inline bool halo_s2_shape(const ConvGeom& g) {
 inline bool halo_s2_fprop_eligible(const ConvGeom& g) { return halo_s2_shape(g) && halo::fwd_supported(g.N, g.H, g.W, g.Ci, g.Co); }
 inline bool halo_s2_dgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && halo::fwd_supported(g.N, g.H, g.W, g.Co, g.Ci); }
 // the same for layers too wide for the halo kernel: the per-tap kernel at full resolution
-inline bool tc_s2_fprop_eligible(const ConvGeom& g) { return halo_s2_shape(g) && tc::conv_tc_supported(g.N, g.H, g.W, g.Ci, g.Co); }
-inline bool tc_s2_dgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && tc::conv_tc_supported(g.N, g.H, g.W, g.Co, g.Ci); }
+inline bool tc_s2_fprop_eligible(const ConvGeom& g) { return halo_s2_shape(g) && tc::conv_tc_supported(g.N, g.H, g.W, g.Ci, g.Co, (size_t)g.N * g.P * g.Q); }
+inline bool tc_s2_dgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && tc::conv_tc_supported(g.N, g.H, g.W, g.Co, g.Ci, (size_t)g.N * g.P * g.Q); }
 inline bool halo_s2_wgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && halo::wgrad_supported(g.N, g.H, g.W, g.Ci, g.Co); }
 // 1x1 convolutions without padding (projection shortcuts), stride 1 or 2: one "tap" of the per-tap kernel on the output
 // grid; a stride-2 forward reads the even pixels of x as a strided tensor, a stride-2 data gradient writes dx at the
@@ -104,8 +104,8 @@ inline bool tc_1x1_shape(const ConvGeom& g) {
   return g.R == 1 && g.S == 1 && g.pad == 0 && (g.stride == 1 || (g.stride == 2 && g.H % 2 == 0 && g.W % 2 == 0)) &&
          g.P == g.H / g.stride && g.Q == g.W / g.stride;
 }
-inline bool tc_1x1_fprop_eligible(const ConvGeom& g) { return tc_1x1_shape(g) && tc::conv_tc_supported(g.N, g.P, g.Q, g.Ci, g.Co); }
-inline bool tc_1x1_dgrad_eligible(const ConvGeom& g) { return tc_1x1_shape(g) && tc::conv_tc_supported(g.N, g.P, g.Q, g.Co, g.Ci); }
+inline bool tc_1x1_fprop_eligible(const ConvGeom& g) { return tc_1x1_shape(g) && tc::conv_tc_supported(g.N, g.P, g.Q, g.Ci, g.Co, (size_t)g.N * g.P * g.Q); }
+inline bool tc_1x1_dgrad_eligible(const ConvGeom& g) { return tc_1x1_shape(g) && tc::conv_tc_supported(g.N, g.P, g.Q, g.Co, g.Ci, (size_t)g.N * g.P * g.Q); }
 // wide layers: the exact-tile weight-gradient kernel (stride 2 with dy spread onto the input grid; 1x1 filters on the output grid)
 // (layers under 128 channels stay with the halo-tile kernel where it covers them)
 inline bool wide_wgrad_eligible(const ConvGeom& g) {
@@ -220,7 +220,7 @@ inline cudaError_t run_wgrad_wide(cudaStream_t st, TensorMapCache* cache, int N,
   const wide::WideParams p = wide::wide_params(N, H, W, Ci, Co, cached_sm_count(cache), R);
   const CUtensorMap *mx, *my;
   cudaError_t e = cached_slab_map(cache, x, N, H, W, Ci, p.xw, p.S, &mx, x_sub);
-  if (e == cudaSuccess) e = cached_slab_map(cache, dy, N, H, W, Co, p.W, p.S, &my);
+  if (e == cudaSuccess) e = cached_slab_map(cache, dy, N, H, W, Co, p.Wk, p.S, &my);
   if (e == cudaSuccess) e = wide::wide_set_attrs();
   if (e != cudaSuccess) return e;
   const dim3 grid(p.co_blocks * p.ci_chunks * p.rdim, p.splits);
@@ -228,7 +228,7 @@ inline cudaError_t run_wgrad_wide(cudaStream_t st, TensorMapCache* cache, int N,
   else wide::wgrad_wide_kernel<1><<<grid, wide::kWideThreads, wide::wide_smem_bytes(p), st>>>(*mx, *my, p, scratch, err_dev);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const size_t n4 = (size_t)Co * R * R * Ci / 4;                 // Ci is a multiple of 16
+  const size_t n4 = (size_t)Co * R * R * Ci / 4;                 // Ci is a multiple of 8
   // the sum's launch overlaps the tail of the kernel above; it waits for that kernel before it reads
   return launch_chained(wide::wgrad_wide_sum_kernel, dim3((unsigned)((n4 + 255) / 256)), dim3(256), 0, st,
                         reinterpret_cast<const float4*>(scratch), reinterpret_cast<float4*>(dw), n4, p.splits);

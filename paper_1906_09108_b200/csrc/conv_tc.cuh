@@ -3,7 +3,10 @@
 // accumulators in tensor memory, epilogue through tcgen05.ld.
 //
 //   D[m][n] = sum_{tap, c} A_tap[m][c] * B_tap[n][c]
-//     m   = 128 consecutive output pixels: whole image rows (or whole images) of an NHWC tensor
+//     m   = up to 128 output pixels: whole image rows, or whole images, of an NHWC tensor.  Any image width up to
+//           128 tiles this way: an image is cut into the fewest equal row groups that fit 128 rows of the
+//           accumulator (24x24: five groups of 5 rows, 90 % of the rows used; 12x12: two of 6, 56 %; 6x6: three
+//           images, 84 %); accumulator rows beyond the tile are computed from stale operands and never stored
 //     A   = the input shifted by the tap offset; the TMA box starts at (w-1+s, h-1+r) and the
 //           hardware zero-fills what falls outside the image, which is the padding
 //     B   = weights [N][9*C]: forward [c_out][r][s][c_in]; data gradient: the flipped and
@@ -35,13 +38,14 @@ struct ConvTcParams {
   int W, H, N;              // image width, height, batch
   int rows_per_tile;        // image rows per tile when a tile stays inside one image, else H
   int imgs_per_tile;        // images per tile (1 unless 128 pixels span whole images)
+  int tiles_per_img;        // row groups of an image (1 when a tile spans whole images)
   int Ci, Co;               // GEMM-K channels per tap, GEMM-N total
   int kc;                   // channel chunk per stage: 16, 32 or 64
   int n_tile;               // GEMM-N per tile (multiple of 16, <= 256)
   int m_tiles, n_tiles;
   int stages;
-  uint32_t a_bytes, b_bytes, stage_bytes;   // b_bytes is padded to 1 KiB; b_tx_bytes is what TMA moves
-  uint32_t b_tx_bytes;
+  uint32_t a_bytes, b_bytes, stage_bytes;   // b_bytes is padded to 1 KiB; a_tx_bytes, b_tx_bytes is what TMA moves
+  uint32_t a_tx_bytes, b_tx_bytes;
   uint32_t tmem_cols;       // allocated columns (power of two >= 2*n_tile)
   int mpair;                // 128-row tiles a CTA works on at once with one weight tile: 1 (two accumulator sets, the
                             // epilogue of a tile overlaps the next tile's instructions) or 2 (one set of two accumulators:
@@ -266,12 +270,8 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         const int halves = (mg * p.mpair + 1 < p.m_tiles) ? p.mpair : 1;
         for (int hf = 0; hf < halves; ++hf) {
           const int mt = mg * p.mpair + hf;
-          if (p.imgs_per_tile == 1) {
-            const int tiles_per_img = p.H / p.rows_per_tile;
-            n0[hf] = mt / tiles_per_img; h0[hf] = (mt - n0[hf] * tiles_per_img) * p.rows_per_tile;
-          } else {
-            n0[hf] = mt * p.imgs_per_tile; h0[hf] = 0;
-          }
+          const int grp = mt / p.tiles_per_img;
+          n0[hf] = grp * p.imgs_per_tile; h0[hf] = (mt - grp * p.tiles_per_img) * p.rows_per_tile;
         }
         for (int ki = 0; ki < k_iters; ++ki, ++it) {
           const int s = it % p.stages;
@@ -282,7 +282,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
           const int dw = p.taps == 1 ? 0 : sx - 1, dh = p.taps == 1 ? 0 : r - 1;
           uint8_t* a_dst = smem + (size_t)s * p.stage_bytes;
           uint8_t* b_dst = a_dst + (size_t)p.mpair * p.a_bytes;
-          mbar_expect_tx(&full[s], (uint32_t)halves * p.a_bytes + p.b_tx_bytes);
+          mbar_expect_tx(&full[s], (uint32_t)halves * p.a_tx_bytes + p.b_tx_bytes);
           for (int hf = 0; hf < halves; ++hf)
             tma_load_4d(a_dst + (size_t)hf * p.a_bytes, &map_a, &full[s], cc * p.kc, dw, h0[hf] + dh, n0[hf]);
           tma_load_2d(b_dst, &map_b, &full[s], tap * p.Ci + cc * p.kc, nt * p.n_tile);
@@ -304,7 +304,8 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         b_desc[i] = smem_desc_kmajor(a_addr + (uint32_t)p.mpair * p.a_bytes, row_bytes);
       }
       const uint64_t half_off = (uint64_t)p.a_bytes >> 4;
-      const int ksub = p.kc / 16;
+      // K steps of a chunk; the last chunk of a channel count that is no multiple of the chunk has fewer
+      const int ksub_full = p.kc / 16, ksub_last = (p.Ci - (chunks - 1) * p.kc + 15) / 16;
       int s = 0;
       uint32_t ph = 0;                                         // it % stages and that stage's phase, kept incrementally
       for (int tile = blockIdx.x; tile < total_tiles && !*abort_flag; tile += gridDim.x, ++tcount) {
@@ -316,7 +317,10 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         const int mg = tile / p.n_tiles;
         const int halves = (mg * p.mpair + 1 < p.m_tiles) ? p.mpair : 1;
         bool ok = true;
+        int cc = 0;
         for (int ki = 0; ki < k_iters; ++ki, ++it) {
+          int ksub = ksub_full;
+          if (++cc == chunks) { cc = 0; ksub = ksub_last; }
           if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const uint64_t a0 = a_desc[s], b0 = b_desc[s];
@@ -344,6 +348,10 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     (void)ew;
     uint32_t tcount = 0;
     const int nsets = p.mpair == 1 ? 2 : 1;
+    // this thread's accumulator row as a pixel of the tile: image, row, column
+    const int acc_row = lane_grp * 32 + lane;
+    const int img_px = p.rows_per_tile * p.W;
+    const int di = acc_row / img_px, dh = (acc_row - di * img_px) / p.W, dw = acc_row - di * img_px - dh * p.W;
     for (int tile = blockIdx.x; tile < total_tiles && !*abort_flag; tile += gridDim.x, ++tcount) {
       const int mg = tile / p.n_tiles, nt = tile - mg * p.n_tiles;
       const int acc = (int)(tcount % nsets);
@@ -353,31 +361,31 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       const int halves = (mg * p.mpair + 1 < p.m_tiles) ? p.mpair : 1;
       for (int hf = 0; hf < halves; ++hf) {
       const int mt = mg * p.mpair + hf;
-      const size_t row = (size_t)mt * kTileM + lane_grp * 32 + lane;
-      size_t base = row * p.Co + (size_t)nt * p.n_tile;
-      bool keep = true;
+      const int grp = mt / p.tiles_per_img;
+      const int n = grp * p.imgs_per_tile + di, h = (mt - grp * p.tiles_per_img) * p.rows_per_tile + dh, w = dw;
+      bool keep = di < p.imgs_per_tile && n < p.N && h < p.H;
+      size_t base = ((size_t)n * p.H + h) * p.W + w;
       if (p.sub == 2) {
-        const size_t hw = (size_t)p.H * p.W, n = row / hw, rem = row - n * hw;
-        const int h = (int)(rem / p.W), w = (int)(rem - (size_t)h * p.W);
-        keep = ((h | w) & 1) == 0;
-        base = (((n * (p.H >> 1) + (h >> 1)) * (p.W >> 1)) + (w >> 1)) * p.Co + (size_t)nt * p.n_tile;
+        keep = keep && ((h | w) & 1) == 0;
+        base = ((size_t)n * (p.H >> 1) + (h >> 1)) * (p.W >> 1) + (w >> 1);
       } else if (p.sub == 3) {
-        const size_t hw = (size_t)p.H * p.W, n = row / hw, rem = row - n * hw;
-        const int h = (int)(rem / p.W), w = (int)(rem - (size_t)h * p.W);
-        base = (((n * (2 * p.H) + 2 * h) * (2 * p.W)) + 2 * w) * p.Co + (size_t)nt * p.n_tile;
+        base = ((size_t)n * (2 * p.H) + 2 * h) * (2 * p.W) + 2 * w;
       }
+      base = base * p.Co + (size_t)nt * p.n_tile;
+      const int cols = p.Co - nt * p.n_tile < p.n_tile ? p.Co - nt * p.n_tile : p.n_tile;   // a multiple of 8
       const uint32_t taddr = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(acc + hf) * p.n_tile;
-      for (int c0 = 0; c0 < p.n_tile; c0 += 16) {
+      for (int c0 = 0; c0 < cols; c0 += 16) {
         uint32_t v[16];
         tmem_ld16(taddr + c0, v);
         tmem_ld_wait();
         if (!keep && !stat_partial) continue;
+        const bool both = c0 + 8 < cols;              // false: only the first eight columns are channels of the output
         float f[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
         if (res && keep) {
           uint4 r0 = *reinterpret_cast<const uint4*>(res + base + c0);
-          uint4 r1 = *reinterpret_cast<const uint4*>(res + base + c0 + 8);
+          uint4 r1 = both ? *reinterpret_cast<const uint4*>(res + base + c0 + 8) : make_uint4(0, 0, 0, 0);
           const __nv_bfloat16* rb0 = reinterpret_cast<const __nv_bfloat16*>(&r0);
           const __nv_bfloat16* rb1 = reinterpret_cast<const __nv_bfloat16*>(&r1);
           float g[16];
@@ -385,7 +393,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
           for (int i = 0; i < 8; ++i) { g[i] = __bfloat162float(rb0[i]); g[8 + i] = __bfloat162float(rb1[i]); }
           if (res_mask) {
             uint4 m0 = *reinterpret_cast<const uint4*>(res_mask + base + c0);
-            uint4 m1 = *reinterpret_cast<const uint4*>(res_mask + base + c0 + 8);
+            uint4 m1 = both ? *reinterpret_cast<const uint4*>(res_mask + base + c0 + 8) : make_uint4(0, 0, 0, 0);
             const __nv_bfloat16* mb0 = reinterpret_cast<const __nv_bfloat16*>(&m0);
             const __nv_bfloat16* mb1 = reinterpret_cast<const __nv_bfloat16*>(&m1);
 #pragma unroll
@@ -407,7 +415,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         }
         if (keep) {
           *reinterpret_cast<uint4*>(out + base + c0) = o0;
-          *reinterpret_cast<uint4*>(out + base + c0 + 8) = o1;
+          if (both) *reinterpret_cast<uint4*>(out + base + c0 + 8) = o1;
         } else {
           o0 = o1 = make_uint4(0, 0, 0, 0);
         }
@@ -603,17 +611,19 @@ conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
           base = (((size_t)n * (p.H >> 1) + (h >> 1)) * (p.W >> 1) + (w >> 1)) * p.Co + (size_t)nt * p.n_tile;
         }
         const uint32_t taddr = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + slot * (uint32_t)p.n_tile;
-        for (int c0 = 0; c0 < p.n_tile; c0 += 16) {
+        const int cols = p.Co - nt * p.n_tile < p.n_tile ? p.Co - nt * p.n_tile : p.n_tile;
+        for (int c0 = 0; c0 < cols; c0 += 16) {
           uint32_t v[16];
           tmem_ld16(taddr + c0, v);
           tmem_ld_wait();
           if (!keep && !stat_partial) continue;
+          const bool both = c0 + 8 < cols;
           float f[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e) f[e] = __uint_as_float(v[e]);
           if (res && keep) {
             uint4 r0 = *reinterpret_cast<const uint4*>(res + base + c0);
-            uint4 r1 = *reinterpret_cast<const uint4*>(res + base + c0 + 8);
+            uint4 r1 = both ? *reinterpret_cast<const uint4*>(res + base + c0 + 8) : make_uint4(0, 0, 0, 0);
             const __nv_bfloat16* rb0 = reinterpret_cast<const __nv_bfloat16*>(&r0);
             const __nv_bfloat16* rb1 = reinterpret_cast<const __nv_bfloat16*>(&r1);
             float gq[16];
@@ -621,7 +631,7 @@ conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             for (int e = 0; e < 8; ++e) { gq[e] = __bfloat162float(rb0[e]); gq[8 + e] = __bfloat162float(rb1[e]); }
             if (res_mask) {
               uint4 m0 = *reinterpret_cast<const uint4*>(res_mask + base + c0);
-              uint4 m1 = *reinterpret_cast<const uint4*>(res_mask + base + c0 + 8);
+              uint4 m1 = both ? *reinterpret_cast<const uint4*>(res_mask + base + c0 + 8) : make_uint4(0, 0, 0, 0);
               const __nv_bfloat16* mb0 = reinterpret_cast<const __nv_bfloat16*>(&m0);
               const __nv_bfloat16* mb1 = reinterpret_cast<const __nv_bfloat16*>(&m1);
 #pragma unroll
@@ -643,7 +653,7 @@ conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
           }
           if (keep) {
             *reinterpret_cast<uint4*>(out + base + c0) = o0;
-            *reinterpret_cast<uint4*>(out + base + c0 + 8) = o1;
+            if (both) *reinterpret_cast<uint4*>(out + base + c0 + 8) = o1;
           } else {
             o0 = o1 = make_uint4(0, 0, 0, 0);
           }
@@ -700,32 +710,40 @@ inline CUtensorMapSwizzle swizzle_for(int row_bytes) {
   return row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
 }
 
-// Can this convolution run on the tensor-core kernel?  (3x3, stride 1, pad 1, channel counts
-// that are multiples of 16, image rows that tile 128 pixels exactly.)
-inline bool conv_tc_supported(int N, int H, int W, int Ci, int Co) {
-  if (Ci % 16 || Co % 16 || Ci < 16 || Co < 16) return false;
-  if (kTileM % W) return false;
-  const int rows = kTileM / W;
-  if (rows <= H) { if (H % rows) return false; }
-  else { if (rows % H || N % (rows / H)) return false; }
-  if (W > 256 || H > 256) return false;
-  return true;
+// Can this convolution run on the tensor-core kernel?  (3x3, stride 1, pad 1, or 1x1, on an H x W grid of `pixels`
+// stored outputs in all; channel counts that are multiples of 8 -- a pixel is then a whole number of 16-byte TMA units --
+// and image rows of at most 128 pixels.)  Channel counts that fill no K step of 16 are left to the CUDA cores where the
+// output is one accumulator tile or less: such a launch is latency, and the tensor cores' set-up is the longer one.
+inline bool conv_tc_supported(int N, int H, int W, int Ci, int Co, size_t pixels) {
+  if (Ci % 8 || Co % 8 || Ci < 8 || Co < 8 || N < 1) return false;
+  if ((Ci % 16 || Co % 16) && pixels <= (size_t)kTileM) return false;
+  return W >= 1 && H >= 1 && W <= kTileM && H <= 256;
 }
 
 inline ConvTcParams conv_tc_params(int N, int H, int W, int Ci, int Co, int taps = 9) {
   ConvTcParams p{};
   p.W = W; p.H = H; p.N = N; p.Ci = Ci; p.Co = Co; p.sub = 1; p.taps = taps; p.act_sub = 1;
   const int rows = kTileM / W;
-  if (rows <= H) { p.rows_per_tile = rows; p.imgs_per_tile = 1; }
-  else { p.rows_per_tile = H; p.imgs_per_tile = rows / H; }
+  if (rows < H) {
+    p.tiles_per_img = (H + rows - 1) / rows;
+    p.rows_per_tile = (H + p.tiles_per_img - 1) / p.tiles_per_img; p.imgs_per_tile = 1;
+  } else {
+    p.tiles_per_img = 1;
+    p.rows_per_tile = H; p.imgs_per_tile = rows / H;
+  }
   // Channel chunk of a pipeline stage = one swizzle span.  Operand tiles arrive from L2 row by row, and a 128-byte
-  // row costs the same as a 64-byte one, so wide layers whose channel count is not a multiple of 64 (160) still
-  // take 64-channel chunks: the last chunk's surplus channels lie outside the activation tensor, are filled with
-  // zeros by the hardware, and so cancel whatever weights they meet.
-  p.kc = (Ci % 64 == 0 || Ci >= 128) ? 64 : (Ci % 32 == 0 ? 32 : 16);
-  int nt = Co;
-  if (nt > 256) { nt = 256; while (Co % nt || nt % 16) nt -= 16; }
-  p.m_tiles = (int)((size_t)N * H * W / kTileM);
+  // row costs the same as a 64-byte one, so layers of more than 32 channels take 64-channel chunks whether or not
+  // their count is a multiple of 64: the last chunk's surplus channels lie outside the activation tensor, are filled
+  // with zeros by the hardware, and so cancel whatever weights they meet.
+  p.kc = Ci > 32 ? 64 : (Ci > 16 ? 32 : 16);
+  // Columns per tile: all of them up to 256, else equal multiples of 16 (columns past the last channel are zeros).
+  int nt = (Co + 15) / 16 * 16;
+  if (nt > 256) {                      // the fewest tiles, or one more where that leaves fewer surplus columns
+    const int k = (nt + 255) / 256;
+    const int a = ((nt + k - 1) / k + 15) / 16 * 16, b = ((nt + k) / (k + 1) + 15) / 16 * 16;
+    nt = (k + 1) * b < k * a ? b : a;
+  }
+  p.m_tiles = ((N + p.imgs_per_tile - 1) / p.imgs_per_tile) * p.tiles_per_img;
   // 16x16-pixel patches with their halo wherever the image allows it and the chunks are full swizzle spans
   p.patch = (taps == 9 && H % kPatch == 0 && W % kPatch == 0 && p.kc == 64) ? 1 : 0;
   // The kernel is bound by the rate at which operand tiles arrive from L2, so a weight tile is shared by two
@@ -733,13 +751,14 @@ inline ConvTcParams conv_tc_params(int N, int H, int W, int Ci, int Co, int taps
   // most SMs idle: then single 128-row tiles and narrower column tiles, down to 64, until there are about 96.
   p.mpair = p.m_tiles >= 2 ? 2 : 1;
   if (!p.patch) {
-    auto tiles = [&]() { return ((p.m_tiles + p.mpair - 1) / p.mpair) * (Co / nt); };
+    auto tiles = [&]() { return ((p.m_tiles + p.mpair - 1) / p.mpair) * ((Co + nt - 1) / nt); };
     if (tiles() < 96) p.mpair = 1;
     while (tiles() < 96 && nt % 32 == 0 && nt / 2 >= 64 && Co % (nt / 2) == 0) nt /= 2;
   }
   p.n_tile = nt;
-  p.n_tiles = Co / nt;
+  p.n_tiles = (Co + nt - 1) / nt;
   p.a_bytes = (uint32_t)kTileM * p.kc * 2;
+  p.a_tx_bytes = (uint32_t)(p.W * p.rows_per_tile * p.imgs_per_tile) * p.kc * 2;
   p.b_tx_bytes = (uint32_t)nt * p.kc * 2;
   p.b_bytes = (p.b_tx_bytes + 1023u) & ~1023u;
   p.stage_bytes = (uint32_t)p.mpair * p.a_bytes + p.b_bytes;

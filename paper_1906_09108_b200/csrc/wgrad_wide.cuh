@@ -7,13 +7,15 @@
 // Pixels are the reduction dimension, so both operands are read MN-major (channels contiguous).  A CTA
 // owns one output tile -- 128 output channels x one filter row r x its taps s x up to 160 input
 // channels: one fp32 accumulator of 128 x nci per tap in tensor memory (<= 480 of its 512 columns) -- and a
-// share of the pixels, which it walks in SLABS of 64 pixels (S = 64/W image rows of one image):
-//   dY slab: [S*W pixels][128 co]     as two 64-channel sub-tiles, one 128-byte swizzle span per pixel
-//   X  slab: 3x3: [S*(W+2) pixels][nci ci], rows h0+r-1 .. h0+r-2+S with the border columns -1 and W (out-of-
-//            bounds rows and columns are the hardware's zero fill = the padding); 1x1: [S*W pixels][nci ci];
+// share of the pixels, which it walks in SLABS of up to 64 pixels: S = 64/Wk image rows of one image, each Wk
+// pixels wide, where Wk is W rounded up to 8 (W <= 8) or to a multiple of 16.  The pixels past the image's edge are
+// the hardware's zero fill in the dY slab, so they add nothing (24x24, 12x12, 6x6 maps: 75 % of the slab counts).
+//   dY slab: [S*Wk pixels][128 co]    as two 64-channel sub-tiles, one 128-byte swizzle span per pixel
+//   X  slab: 3x3: [S*(Wk+2) pixels][nci ci], rows h0+r-1 .. h0+r-2+S with the border columns -1 and W (out-of-
+//            bounds rows and columns are the hardware's zero fill = the padding); 1x1: [S*Wk pixels][nci ci];
 //            64-channel sub-tiles either way
-// One instruction takes 16 pixels: 16 consecutive pixels of an image row (W >= 16) or two rows of 8
-// (W = 8: the second 8-pixel group of the X slab lies one slab row further on, which is the descriptor's
+// One instruction takes 16 pixels: 16 consecutive pixels of a slab row (Wk >= 16) or two rows of 8
+// (Wk = 8: the second 8-pixel group of the X slab lies one slab row further on, which is the descriptor's
 // stride between 8-row groups).  For tap s the X operand simply starts s pixels later, so the dY block
 // is read once for three instructions and no multiplication is spent on border pixels.
 // The CTAs that share an output tile write their partial sums to scratch; a second kernel adds them in
@@ -35,16 +37,19 @@ constexpr int kCoBlock = 128;
 constexpr size_t kWideSmemBudget = 200 * 1024;
 
 struct WideParams {
-  int N, H, W, Wp;
+  int N, H, W;
+  int Wk;                   // pixels per slab row: W rounded up to 8 or to a multiple of 16
+  int ksteps;               // 16-pixel reduction steps per slab
   int Ci, Co;
   int nci;                  // input channels per CTA = N of the instruction (multiple of 16, <= 160)
   int ci_chunks, co_blocks;
   int xsub;                 // 64-channel sub-tiles of the X slab: ceil(nci / 64)
   int taps;                 // 3: one filter row of a 3x3 filter (pad 1); 1: a 1x1 filter (no padding)
   int rdim;                 // filter rows: 3 or 1 (the CTAs of blockIdx.x % rdim share everything but r)
-  int xw;                   // pixels per image row of the X slab: W + 2 with the border columns, W without
+  int xw;                   // pixels per image row of the X slab: Wk + 2 with the border columns, Wk without
   int S;                    // image rows per slab
-  int slabs;                // N * H / S
+  int slabs_per_img;        // ceil(H / S)
+  int slabs;                // N * slabs_per_img
   int splits;               // CTAs per output tile
   int stages;
   uint32_t y_sub_bytes, x_sub_bytes;      // one 64-channel sub-tile of each slab (multiples of 1 KiB)
@@ -85,7 +90,7 @@ wgrad_wide_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   const int pair = (int)blockIdx.x / p.rdim;
   const int chunk = pair % p.ci_chunks, cob = pair / p.ci_chunks;
   const int ci0 = chunk * p.nci, co0 = cob * kCoBlock;
-  const int slabs_per_img = p.H / p.S;
+  const int slabs_per_img = p.slabs_per_img;
 
   if (threadIdx.x == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_x)) : "memory");
@@ -132,7 +137,7 @@ wgrad_wide_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       uint64_t b_off[ksteps];
       for (int ks = 0; ks < ksteps; ++ks) {
         const int pix = ks * 16;                                 // first pixel of the step inside the dY slab
-        const int row = pix / p.W, col = pix - row * p.W;        // W = 8: row is even and the step takes rows row, row+1
+        const int row = pix / p.Wk, col = pix - row * p.Wk;      // Wk = 8: row is even and the step takes rows row, row+1
         b_off[ks] = (uint64_t)((row * p.xw + col) * 8);          // one pixel = 128 bytes = 8 units
       }
       const uint32_t d1 = tmem_base + (uint32_t)p.nci, d2 = tmem_base + 2u * (uint32_t)p.nci;
@@ -146,6 +151,7 @@ wgrad_wide_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         const uint64_t a0 = a_first + (uint64_t)s * stage_units, b0 = b_first + (uint64_t)s * stage_units;
 #pragma unroll
         for (int ks = 0; ks < ksteps; ++ks) {
+          if (ks >= p.ksteps) break;
           const uint64_t a = a0 + (uint64_t)(ks * 128), b = b0 + b_off[ks];      // 16 pixels = 2048 bytes = 128 units
           const uint32_t acc = (it | (uint32_t)ks) != 0;
           tc_mma_bf16(tmem_base, a, b, idesc, acc);
@@ -238,33 +244,37 @@ __global__ void __launch_bounds__(256) wgrad_wide_sum_kernel(const float4* __res
 }
 
 // ----------------------------------------------------------------- host side ---
+// Input channels per CTA: equal multiples of 16 of at most 160 (three accumulators of 160 columns fill tensor memory);
+// columns past the last channel are zeros and are not written out.
 inline int wide_nci(int Ci) {
   if (Ci % 160 == 0) return 160;
   if (Ci % 128 == 0) return 128;
-  if (Ci <= 160) return Ci;
-  return 0;
+  const int k = (Ci + 159) / 160;
+  return ((Ci + k - 1) / k + 15) / 16 * 16;
 }
 
 // R = 3: x and dy are [N][H][W][.]; R = 1: dy is [N][H][W][Co] and x the tensor of the same pixels (for stride 2, the
 // even pixels of the layer input, see make_slab_map).
 inline WideParams wide_params(int N, int H, int W, int Ci, int Co, int sm_count, int R = 3) {
   WideParams p{};
-  p.N = N; p.H = H; p.W = W; p.Wp = W + 2; p.Ci = Ci; p.Co = Co;
-  p.taps = R; p.rdim = R; p.xw = R == 3 ? W + 2 : W;
+  p.N = N; p.H = H; p.W = W; p.Ci = Ci; p.Co = Co;
   p.nci = wide_nci(Ci);
-  if (p.nci == 0 || W < 8 || kSlabPixels % W) { p.stages = 0; return p; }
-  p.S = kSlabPixels / W;
-  if (H % p.S) { p.stages = 0; return p; }
-  p.ci_chunks = Ci / p.nci;
+  if (W < 1 || W > kSlabPixels) { p.stages = 0; return p; }
+  p.Wk = W <= 8 ? 8 : (W + 15) / 16 * 16;
+  p.taps = R; p.rdim = R; p.xw = R == 3 ? p.Wk + 2 : p.Wk;
+  p.S = kSlabPixels / p.Wk;
+  p.ksteps = p.S * p.Wk / 16;
+  p.ci_chunks = (Ci + p.nci - 1) / p.nci;
   p.co_blocks = (Co + kCoBlock - 1) / kCoBlock;
   p.xsub = (p.nci + 63) / 64;
-  p.slabs = N * (H / p.S);
+  p.slabs_per_img = (H + p.S - 1) / p.S;
+  p.slabs = N * p.slabs_per_img;
   p.y_sub_bytes = kSlabPixels * 128;
   p.x_sub_bytes = halo::round_up_u32((uint32_t)(p.S * p.xw) * 128u, 1024);
   p.y_bytes = 2 * p.y_sub_bytes;
   p.x_bytes = (uint32_t)p.xsub * p.x_sub_bytes;
-  p.tx_bytes = 2 * p.y_sub_bytes + (uint32_t)p.xsub * (uint32_t)(p.S * p.xw) * 128u;
-  p.sbo_x = W == 8 ? (uint32_t)p.xw * 128u : 1024u;
+  p.tx_bytes = (2u * (uint32_t)(p.S * p.Wk) + (uint32_t)p.xsub * (uint32_t)(p.S * p.xw)) * 128u;
+  p.sbo_x = p.Wk == 8 ? (uint32_t)p.xw * 128u : 1024u;
   int stages = (int)((kWideSmemBudget - 2048) / (p.y_bytes + p.x_bytes));
   if (stages > 6) stages = 6;
   p.stages = stages;
@@ -283,11 +293,11 @@ inline WideParams wide_params(int N, int H, int W, int Ci, int Co, int sm_count,
 inline size_t wide_smem_bytes(const WideParams& p) {
   return (size_t)p.stages * ((size_t)p.y_bytes + p.x_bytes) + (size_t)(2 * p.stages + 1) * 8 + 16 + 1024;
 }
-// 64 channels and more on both sides (a 64-channel sub-tile is one swizzle span).  Narrow 3x3 layers that the
-// halo-tile kernel covers are left to it by the dispatcher: they are bound by memory traffic, where its single
-// pass over whole images wins.
+// Channel counts that are multiples of 8 (a pixel is a whole number of 16-byte TMA units), images up to 64 pixels wide.
+// Narrow 3x3 layers that the halo-tile kernel covers are left to it by the dispatcher: they are bound by memory
+// traffic, where its single pass over whole images wins.
 inline bool wide_supported(int N, int H, int W, int Ci, int Co, int R = 3) {
-  if (Ci < 64 || Co < 64 || Ci % 16 || Co % 16 || N < 1 || H < 1) return false;
+  if (Ci < 8 || Co < 8 || Ci % 8 || Co % 8 || N < 1 || H < 1) return false;
   WideParams p = wide_params(N, H, W, Ci, Co, 148, R);
   return p.stages >= 2 && p.tmem_cols <= 512 && p.co_blocks * p.ci_chunks * p.rdim <= 65535;
 }
