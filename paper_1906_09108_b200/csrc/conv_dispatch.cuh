@@ -6,6 +6,7 @@
 #include <map>
 #include <vector>
 
+#include "conv_direct.cuh"
 #include "conv_simt.cuh"
 #include "conv_tc.cuh"
 #include "conv_halo.cuh"
@@ -245,7 +246,7 @@ inline bool s2_uses_spread_dy(const ConvGeom& g) {
 
 // fp32 scratch elements a weight-gradient call may need (bf16 storage: whichever kernel is chosen).
 inline size_t conv_wgrad_scratch_elems(bool bf16_storage, const ConvGeom& g) {
-  size_t n = wgrad_scratch_elems(g);
+  size_t n = std::max(wgrad_scratch_elems(g), direct::wgrad_direct_scratch_elems(g));
   if (bf16_storage && (halo_wgrad_eligible(g) || halo_s2_wgrad_eligible(g)))
     n = std::max(n, halo::wgrad_scratch_elems(g.N, g.H, g.W, g.Ci, g.Co));
   if (bf16_storage && (wide_wgrad_eligible(g) || wide_s2_wgrad_eligible(g)))
@@ -253,6 +254,29 @@ inline size_t conv_wgrad_scratch_elems(bool bf16_storage, const ConvGeom& g) {
   if (bf16_storage && wide_1x1_wgrad_eligible(g))
     n = std::max(n, wide::wide_scratch_elems(g.N, g.P, g.Q, g.Ci, g.Co, 1));
   return n;
+}
+
+// ---- the CUDA-core kernels, either storage type: register-tiled for 3x3 filters with padding 1 (weight gradient: also
+// 1x1), the general implicit GEMM for the rest ----
+// `red` (nullable) asks for per-channel sums of the output; they are formed where the consumer can add the rows up (at
+// most 128 channels, whole vectors), *nparts = 0 tells the caller they were not.
+template <typename T>
+inline cudaError_t cuda_core_conv(cudaStream_t st, const ConvGeom& g, bool dgrad, const T* act, const T* w, T* out, const T* res,
+                                  const T* mask, const direct::Reduce<T>* red, int* nparts, uint64_t* launches) {
+  if (nparts) *nparts = 0;
+  if (direct::conv_supported(g, dgrad)) {
+    const int cn = dgrad ? g.Ci : g.Co;
+    const bool sums = red && red->mode != 0 && cn % 4 == 0 && 2 * cn <= kEwThreads;
+    return direct::launch_conv<T>(st, g, dgrad, act, w, out, res, mask, sums ? red : nullptr, nparts, launches);
+  }
+  if (dgrad) return launch_conv_simt<T, CONV_DGRAD>(st, g, act, w, out, nullptr, nullptr, res, mask, launches);
+  return launch_conv_simt<T, CONV_FPROP>(st, g, act, w, out, nullptr, nullptr, res, mask, launches);
+}
+template <typename T>
+inline cudaError_t cuda_core_wgrad(cudaStream_t st, const ConvGeom& g, const T* x, const T* dy, float* scratch, float* dw,
+                                   uint64_t* launches) {
+  if (direct::wgrad_direct_supported(g)) return direct::launch_wgrad<T>(st, g, x, dy, scratch, dw, launches);
+  return launch_conv_simt<T, CONV_WGRAD>(st, g, x, dy, (T*)nullptr, scratch, dw, (const T*)nullptr, (const T*)nullptr, launches);
 }
 
 // ---- one convolution operator in bf16 storage: which kernel, in which launch shape ------------------
@@ -321,7 +345,8 @@ inline cudaError_t bf16_conv_fprop(cudaStream_t st, TensorMapCache* cache, const
     }
     return run_conv_tc(st, cache, g.N, g.P, g.Q, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, 1, 1, g.stride);
   }
-  return launch_conv_simt<bf16_t, CONV_FPROP>(st, g, x, w, y, nullptr, nullptr, res, (const bf16_t*)nullptr, launches);
+  const direct::Reduce<bf16_t> r = red ? direct::Reduce<bf16_t>{red->mode, nullptr, nullptr, nullptr, red->partial} : direct::Reduce<bf16_t>{};
+  return cuda_core_conv(st, g, false, x, w, y, res, (const bf16_t*)nullptr, red ? &r : nullptr, nparts, launches);
 }
 
 // dx = conv^T(dy, w) [+ res * [mask > 0]].  `wflip` is the flipped/transposed weight copy (null: CUDA cores);
@@ -358,7 +383,8 @@ inline cudaError_t bf16_conv_dgrad(cudaStream_t st, TensorMapCache* cache, const
     ++*launches;
     return run_conv_tc(st, cache, g.N, g.P, g.Q, g.Co, g.Ci, dy, wflip, dx, res, mask, err_dev, g.stride == 2 ? 3 : 1, 1, 1);
   }
-  return launch_conv_simt<bf16_t, CONV_DGRAD>(st, g, dy, w, dx, nullptr, nullptr, res, mask, launches);
+  const direct::Reduce<bf16_t> r = red ? direct::Reduce<bf16_t>{red->mode, red->mask, red->xprev, red->pstats, red->partial} : direct::Reduce<bf16_t>{};
+  return cuda_core_conv(st, g, true, dy, w, dx, res, mask, red ? &r : nullptr, nparts, launches);
 }
 
 // dw (fp32) from x and dy; `scratch` of conv_wgrad_scratch_elems floats; `side`: bound the pixel split by
@@ -382,9 +408,7 @@ inline cudaError_t bf16_conv_wgrad(cudaStream_t st, TensorMapCache* cache, const
     *launches += 2;
     return run_wgrad_halo(st, cache, g.N, g.H, g.W, g.Ci, g.Co, x, dy, dw, scratch, err_dev, side);
   }
-  if (small_wgrad_eligible(g)) return launch_small_wgrad<bf16_t>(st, g, x, dy, scratch, dw, launches);
-  if (proj_wgrad_eligible(g)) return launch_proj_wgrad<bf16_t>(st, g, x, dy, scratch, dw, launches);
-  return launch_conv_simt<bf16_t, CONV_WGRAD>(st, g, x, dy, (bf16_t*)nullptr, scratch, dw, (const bf16_t*)nullptr, (const bf16_t*)nullptr, launches);
+  return cuda_core_wgrad(st, g, x, dy, scratch, dw, launches);
 }
 
 }  // namespace fdg

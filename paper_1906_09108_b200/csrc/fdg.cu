@@ -35,7 +35,7 @@ namespace fdg {
 typedef __nv_bfloat16 bf16;
 constexpr int kEventRing = 4;
 constexpr size_t kLogIterations = 4096;
-constexpr int kRedPartialCtas = 256;                 // upper bound of the CTAs of one convolution launch
+constexpr int kRedPartialCtas = FDG_CONV_PARTIAL_ROWS;   // upper bound of the CTAs of one convolution launch that leaves sums
 constexpr float kBnMomentum = 0.1f;                  // weight of the newest batch in the running statistics
 
 enum UnitType { U_STEM, U_BASIC, U_PREACT, U_HEAD };
@@ -111,6 +111,7 @@ struct Module {
   // host state
   int64_t updates = 0;
   std::vector<int64_t> slot_version, slot_batch;
+  bool head_stats_ready = false;           // the last block's convolution formed the statistics of the head's batch norm
   int64_t last_out_batch = -1, last_grad_batch = -1;
   int last_out_slot = -1, last_grad_slot = -1;
   cudaStream_t stream = nullptr;
@@ -657,7 +658,8 @@ static int conv_fprop(Launch& L, Module& m, const ConvGeom& g, const T* x, const
     L.note(bf16_conv_fprop(L.st, &L.c->tmaps, g, x, w, y, res, want_stats ? &r : nullptr, &nparts, L.c->tc_error, &L.c->launches,
                            (want_stats && stats) ? &ws : nullptr));
   } else {
-    L.note(launch_conv_simt<T, CONV_FPROP>(L.st, g, x, w, y, nullptr, nullptr, res, (const T*)nullptr, &L.c->launches));
+    const direct::Reduce<T> r{1, nullptr, nullptr, nullptr, m.red_partial};
+    L.note(cuda_core_conv<T>(L.st, g, false, x, w, y, res, nullptr, want_stats ? &r : nullptr, &nparts, &L.c->launches));
   }
   return nparts;
 }
@@ -677,19 +679,19 @@ static int conv_dgrad(Launch& L, Module& m, const ConvGeom& g, const T* dy, cons
     if (next) { r.mode = 2; r.mask = next->mask; r.xprev = next->x; r.pstats = next->stats; r.partial = m.red_partial; }
     L.note(bf16_conv_dgrad(L.st, &L.c->tmaps, g, dy, w, wflip, dy_up, dx, res, mask, next ? &r : nullptr, &nparts, L.c->tc_error, &L.c->launches));
   } else {
-    L.note(launch_conv_simt<T, CONV_DGRAD>(L.st, g, dy, w, dx, nullptr, nullptr, res, mask, &L.c->launches));
+    direct::Reduce<T> r{};
+    if (next) r = direct::Reduce<T>{2, next->mask, next->x, next->stats, m.red_partial};
+    L.note(cuda_core_conv<T>(L.st, g, true, dy, w, dx, res, mask, next ? &r : nullptr, &nparts, &L.c->launches));
   }
   return nparts;
 }
 template <typename T>
 static void conv_wgrad(Launch& L, Module& m, const ConvGeom& g, const T* x, const T* dy, float* dw, const T* dy_up = nullptr) {
   L.begin(KC_CONV_WGRAD, (in_elems(g) + out_elems(g)) * sizeof(T) + w_elems(g) * 4, conv_flops(g));
-  // the tensor-core and small-shape kernels serve bf16 storage only: the fp32 mode keeps one summation
-  // scheme for all its weight gradients
   if constexpr (std::is_same<T, bf16>::value)
     L.note(bf16_conv_wgrad(L.st, &L.c->tmaps, g, x, dy, dy_up, dw, m.wscratch, L.c->tc_error, L.st == m.stream2, &L.c->launches));
   else
-    L.note(launch_conv_simt<T, CONV_WGRAD>(L.st, g, x, dy, (T*)nullptr, m.wscratch, dw, (const T*)nullptr, (const T*)nullptr, &L.c->launches));
+    L.note(cuda_core_wgrad<T>(L.st, g, x, dy, m.wscratch, dw, &L.c->launches));
 }
 
 template <typename T> static const T* flipped_of(const Module& m, int vslot, long long off);
@@ -746,8 +748,10 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
   int x_np = 0;     // -1: the statistics of x (the next pre-activation block's first batch norm) are already in place
   for (size_t ui = 0; ui < m.units.size(); ++ui) {
     const Unit& u = m.units[ui];
-    // the pre-activation block that normalises this unit's output first, if it is in this module
-    const Unit* nxt = (ui + 1 < m.units.size() && m.units[ui + 1].type == U_PREACT) ? &m.units[ui + 1] : nullptr;
+    // the pre-activation block (or the head's batch norm) that normalises this unit's output first, if it is in this module
+    const Unit* nxt = nullptr;
+    if (ui + 1 < m.units.size() && (m.units[ui + 1].type == U_PREACT || (m.units[ui + 1].type == U_HEAD && m.units[ui + 1].bn)))
+      nxt = &m.units[ui + 1];
     const size_t rows_in = (size_t)B * u.H * u.W, rows_out = (size_t)B * u.P * u.Q;
     switch (u.type) {
       case U_STEM: {
@@ -802,7 +806,15 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
         } else {
           x_np = conv_fprop<T>(L, m, g2, S + u.t_c, wt + u.w2, S + u.t_y, x, !eval && nxt, nxt ? F + nxt->st1 : nullptr, nxt ? nxt->r1 : -1);
         }
-        if (x_np > 0) x_np = 0;     // rows for a narrow layer's apply kernel: not used here, the block's input is reduced as before
+        if (x_np > 0) {             // a narrow layer left its rows of sums: the next batch norm's statistics are their totals
+          const RunningStats run{nxt->r1 >= 0 ? m.running + nxt->r1 : nullptr, kBnMomentum,
+                                 rows_out > 1 ? (float)((double)rows_out / (double)(rows_out - 1)) : 1.f};
+          L.begin(KC_BN_STATS, 8.0 * x_np * u.co, 2.0 * x_np * u.co);
+          L.note(launch_chained(stats_finalize_kernel, dim3((unsigned)((u.co + 31) / 32)), dim3(256), 0, L.st, (const float*)m.red_partial,
+                                x_np, u.co, 1.0 / (double)rows_out, eps, F + nxt->st1, run));
+          ++c->launches;
+          x_np = -1;
+        }
         break;
       }
       case U_HEAD:
@@ -810,6 +822,7 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
     }
     if (u.type != U_HEAD) x = S + u.t_y;
   }
+  m.head_stats_ready = x_np < 0;
 }
 
 // Module K, inference: [BN + ReLU,] global average pool, FC, arg-max against the labels.
@@ -846,7 +859,7 @@ static void head_forward_backward(fdg_ctx* c, Module& m, Launch& L, int64_t tau,
   const size_t rows = (size_t)B * HW;
   const T* feat = x;
   if (u.bn) {
-    bn_stats<T>(L, m, x, rows, F, c->arch.bn_eps, Fs + u.st1, u.r1);
+    if (!m.head_stats_ready) bn_stats<T>(L, m, x, rows, F, c->arch.bn_eps, Fs + u.st1, u.r1);
     bn_apply<T>(L, m, x, Fs + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_a, rows, F);
     feat = S + u.t_a;
   }

@@ -1,0 +1,50 @@
+"""The register-tiled CUDA-core convolutions on shapes where their tiling can go wrong -- row segments, row tiles, channel
+chunks and channel blocks that are not full, several images per tile -- in both storage types, against the oracle's
+convolution with the bars of test_gpu_conv_ops.py; and the sums they form for the batch norm that follows."""
+import numpy as np
+import pytest
+import torch
+
+from tests.test_gpu_conv_ops import _run
+
+pytestmark = pytest.mark.gpu
+
+# (N, H, W, Ci, Co, R, stride, pad)
+SHAPES = [(2, 33, 30, 3, 16, 3, 1, 1),       # the stem: three channels; odd height, a last segment of two pixels
+          (3, 7, 7, 20, 36, 3, 1, 1),        # channel counts that fill neither a chunk nor a thread column of 8
+          (2, 9, 64, 4, 68, 3, 1, 1),        # two channel blocks, the widest rows
+          (5, 4, 6, 17, 66, 3, 1, 1),        # odd channel counts
+          (300, 4, 4, 12, 20, 3, 1, 1),      # several images per tile
+          (160, 16, 16, 16, 32, 3, 1, 1),    # 8 channels per thread
+          (2, 64, 64, 4, 4, 3, 2, 1),        # stride 2: rows of a tile bounded by shared memory
+          (3, 14, 14, 36, 40, 3, 2, 1),
+          (2, 10, 12, 40, 72, 1, 1, 0), (3, 12, 10, 36, 68, 1, 2, 0)]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_direct_conv_fp32(shape):
+    _run("fp32", shape, False)
+
+
+@pytest.mark.parametrize("shape", [s for s in SHAPES if s[3] % 8 or s[4] % 8])
+def test_direct_conv_bf16(shape):
+    _run("bf16", shape, False)
+
+
+@pytest.mark.parametrize("shape", [(4, 32, 30, 3, 16), (200, 9, 7, 3, 64), (2, 12, 20, 5, 128)])
+def test_statistics_rows_of_the_stem(shape):
+    """The rows of (sum y, sum y^2) add up to those of the stored output; at most 256 rows."""
+    from paper_1906_09108_b200 import binding as B
+    n, h, w, ci, co = shape
+    ops = B.ConvOps(B.FDG_BF16_TC)
+    s = B.fdg_conv_shape(n, h, w, ci, co, 3, 1, 1)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn((n, h, w, ci), device="cuda", generator=g).to(ops.dtype)
+    wt = torch.randn((co, 3, 3, ci), device="cuda", generator=g).to(ops.dtype)
+    y, rows = ops.forward(s, x, wt, reduce=True)
+    assert 0 < rows.shape[0] <= B.FDG_CONV_PARTIAL_ROWS
+    got = rows.double().sum(0).cpu().numpy()
+    yd = y.double().reshape(-1, co)
+    want = torch.cat([yd.sum(0), (yd * yd).sum(0)]).cpu().numpy()
+    scale = np.concatenate([yd.abs().sum(0).cpu().numpy(), want[co:]])
+    assert np.max(np.abs(got - want) / scale) < 1e-5
