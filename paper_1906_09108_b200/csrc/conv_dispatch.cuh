@@ -10,6 +10,7 @@
 #include "conv_simt.cuh"
 #include "conv_tc.cuh"
 #include "conv_halo.cuh"
+#include "conv_rows.cuh"
 #include "wgrad_wide.cuh"
 #include "elementwise.cuh"
 
@@ -174,6 +175,53 @@ inline cudaError_t run_conv_halo(cudaStream_t st, TensorMapCache* cache, int N, 
   return launch_chained(halo::conv_halo_kernel, grid, halo::kConvThreads, halo::fwd_smem_bytes(p), st, *mx, *mw, p, out, res, res_mask, r, err_dev);
 }
 
+// The same contract for layers of equal width (rows::conv_rows_kernel).  `res_bits`: the residual's gate as bits (or null:
+// `res_mask`, or none).
+inline bool rows_eligible(const ConvGeom& g) { return halo_shape(g) && rows::rows_supported(g.N, g.H, g.W, g.Ci, g.Co); }
+inline cudaError_t cached_group_map(TensorMapCache* cache, const void* t, int N, int H, int W, int C, int box_g, int box_h,
+                                    const CUtensorMap** out) {
+  TensorMapCache::Key k;
+  std::memset(&k, 0, sizeof(k));
+  k.ptr = t; k.d[0] = 6; k.d[1] = N; k.d[2] = H; k.d[3] = W; k.d[4] = C; k.d[5] = box_g; k.d[6] = box_h;
+  auto it = cache->maps.find(k);
+  if (it == cache->maps.end()) {
+    CUtensorMap m;
+    cudaError_t e = rows::make_group_map(t, N, H, W, C, box_g, box_h, &m);
+    if (e != cudaSuccess) return e;
+    it = cache->maps.insert({k, m}).first;
+  }
+  *out = &it->second;
+  return cudaSuccess;
+}
+inline cudaError_t run_conv_rows(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int C, const bf16_t* act,
+                                 const bf16_t* wgt, bf16_t* out, const bf16_t* res, const bf16_t* res_mask,
+                                 const unsigned char* res_bits, int* err_dev, const halo::EpiReduce* red, int* ctas_out) {
+  int sms = cached_sm_count(cache) / (cache->share > 0 ? cache->share : 1);
+  if (sms < 16) sms = 16;
+  // the fewest CTAs that keep the number of images of the busiest one at ceil(N / sms)
+  const int per_cta = (N + sms - 1) / sms, grid = (N + per_cta - 1) / per_cta;
+  rows::EpiParams e{};
+  const int mode = red ? red->mode : 0;
+  e.res_gate = rows::Gate{res_bits, res_bits ? nullptr : res_mask};
+  if (red) {
+    e.gate = rows::Gate{red->mask_bits, red->mask_bits ? nullptr : red->mask};
+    e.pstats = red->pstats; e.partial = red->partial;
+  }
+  const int n_ops = (res ? 1 : 0) + (mode == 2 ? 1 : 0);
+  const rows::RowsParams p = rows::rows_params(N, H, W, C, per_cta, n_ops);
+  const CUtensorMap *ma, *mw, *mo, *mr, *mx;
+  cudaError_t er = cached_group_map(cache, act, N, H, W, C, rows::kTileGroups * p.cb + 2, H + 2, &ma);
+  if (er == cudaSuccess) er = cached_weight_map(cache, wgt, C, C, &mw);
+  if (er == cudaSuccess) er = cached_group_map(cache, out, N, H, W, C, rows::kTileGroups, rows::kTileRows, &mo);
+  mr = mx = mo;
+  if (er == cudaSuccess && res) er = cached_group_map(cache, res, N, H, W, C, rows::kTileGroups, rows::kTileRows, &mr);
+  if (er == cudaSuccess && mode == 2) er = cached_group_map(cache, red->xprev, N, H, W, C, rows::kTileGroups, rows::kTileRows, &mx);
+  if (er == cudaSuccess) er = rows::set_attrs();
+  if (er != cudaSuccess) return er;
+  if (ctas_out) *ctas_out = grid;
+  return launch_chained(rows::kernel_of(C, mode, res != nullptr), grid, rows::kThreads, rows::rows_smem_bytes(p), st, *ma, *mw, *mo, *mr, *mx, p, e, err_dev);
+}
+
 // dw[Co][3][3][Ci] (fp32) from x [N][H][W][Ci] and dy [N][H][W][Co]; `scratch` holds the per-CTA partials
 // (halo::wgrad_scratch_elems floats).  Two launches: the tensor-core kernel and the fixed-order sum.
 inline cudaError_t run_wgrad_halo(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int Ci, int Co,
@@ -237,7 +285,7 @@ inline cudaError_t run_wgrad_wide(cudaStream_t st, TensorMapCache* cache, int N,
 
 // Does the data gradient of this convolution read the flipped/transposed weight copy?
 inline bool dgrad_uses_flipped(const ConvGeom& g) {
-  return halo_dgrad_eligible(g) || halo_s2_dgrad_eligible(g) || tc_eligible(g) || tc_s2_dgrad_eligible(g) || tc_1x1_dgrad_eligible(g);
+  return rows_eligible(g) || halo_dgrad_eligible(g) || halo_s2_dgrad_eligible(g) || tc_eligible(g) || tc_s2_dgrad_eligible(g) || tc_1x1_dgrad_eligible(g);
 }
 // Do the stride-2 gradients of this convolution run on the tensor cores, given a spread-out copy of dy?
 inline bool s2_uses_spread_dy(const ConvGeom& g) {
@@ -318,6 +366,14 @@ inline cudaError_t bf16_conv_fprop(cudaStream_t st, TensorMapCache* cache, const
                                    const bf16_t* w, bf16_t* y, const bf16_t* res, const halo::EpiReduce* red, int* nparts,
                                    int* err_dev, uint64_t* launches, const WideStats* ws = nullptr) {
   if (nparts) *nparts = 0;
+  if (rows_eligible(g)) {
+    ++*launches;
+    const bool fuse = red && red->mode == 1;
+    int ctas = 0;
+    const cudaError_t e = run_conv_rows(st, cache, g.N, g.H, g.W, g.Ci, x, w, y, res, nullptr, nullptr, err_dev, fuse ? red : nullptr, &ctas);
+    if (fuse && nparts) *nparts = ctas;
+    return e;
+  }
   const bool s1 = halo_fprop_eligible(g), s2 = !s1 && halo_s2_fprop_eligible(g);
   if (s1 || s2) {
     ++*launches;
@@ -355,8 +411,16 @@ inline cudaError_t bf16_conv_fprop(cudaStream_t st, TensorMapCache* cache, const
 inline cudaError_t bf16_conv_dgrad(cudaStream_t st, TensorMapCache* cache, const ConvGeom& g, const bf16_t* dy,
                                    const bf16_t* w, const bf16_t* wflip, const bf16_t* dy_up, bf16_t* dx, const bf16_t* res,
                                    const bf16_t* mask, const halo::EpiReduce* red, int* nparts, int* err_dev,
-                                   uint64_t* launches) {
+                                   uint64_t* launches, const unsigned char* mask_bits = nullptr) {
   if (nparts) *nparts = 0;
+  if (wflip && rows_eligible(g)) {
+    ++*launches;
+    const bool fuse = red && red->mode == 2;
+    int ctas = 0;
+    const cudaError_t e = run_conv_rows(st, cache, g.N, g.H, g.W, g.Ci, dy, wflip, dx, res, mask, mask_bits, err_dev, fuse ? red : nullptr, &ctas);
+    if (fuse && nparts) *nparts = ctas;
+    return e;
+  }
   const bool h1 = wflip && halo_dgrad_eligible(g), h2 = !h1 && wflip && dy_up && halo_s2_dgrad_eligible(g);
   if (h1 || h2) {
     ++*launches;

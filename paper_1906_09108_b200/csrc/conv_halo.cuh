@@ -91,6 +91,7 @@ struct EpiReduce {
   const __nv_bfloat16* xprev;
   const float* pstats;        // mode 2: mean[Cn], invstd[Cn] of xprev's batch norm
   float* partial;             // [gridDim.x][2*Cn]
+  const unsigned char* mask_bits;   // mode 2: the gate as one bit per element where there is such a copy (conv_rows.cuh)
 };
 // Threads of conv_halo_kernel: TMA warp, two MMA warps, kEpiGroups groups of four epilogue warps.
 // The groups take the (128-row tile, 16-column chunk) items in turn: an item's epilogue is a chain

@@ -355,13 +355,15 @@ template <typename T, int VEC> __device__ __forceinline__ void raw_to_f(const Ra
   }
 }
 
+// `bits` (nullable; bf16 vectors only): one bit per element, set where y > 0 -- byte i holds those of vector i.  They are
+// the ReLU gates of the backward pass at a sixteenth of the tensor's size.
 template <typename T, int VEC, bool RES_BN>
 __global__ void __launch_bounds__(kEwThreads, 3)
 bn_apply_kernel(const T* __restrict__ x, const float* __restrict__ stats,
                 const float* __restrict__ gamma, const float* __restrict__ beta,
                 const T* __restrict__ res, const float* __restrict__ res_stats,
                 const float* __restrict__ res_gamma, const float* __restrict__ res_beta,
-                int relu, T* __restrict__ y, size_t nvec, int C, PartialSums ps) {
+                int relu, T* __restrict__ y, unsigned char* __restrict__ bits, size_t nvec, int C, PartialSums ps) {
   __shared__ float s_stats[2 * 128];
   grid_dependency_wait();
   grid_dependency_release();
@@ -391,6 +393,15 @@ bn_apply_kernel(const T* __restrict__ x, const float* __restrict__ stats,
       o[j] = relu ? fmaxf(t, 0.f) : t;
     }
     store_vec<T, VEC>(y + i * VEC, o);
+    if constexpr (VEC == 8) {
+      if (bits) {
+        // the gate is taken on the value as stored: a positive value below half the smallest bf16 number rounds to zero
+        unsigned int m = 0;
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) m |= (to_f(from_f<T>(o[j])) > 0.f ? 1u : 0u) << j;
+        bits[i] = (unsigned char)m;
+      }
+    }
   };
   size_t i = gtid;
   for (; i + (kEwUnroll - 1) * stride < nvec; i += kEwUnroll * stride) {
@@ -412,30 +423,39 @@ bn_apply_kernel(const T* __restrict__ x, const float* __restrict__ stats,
 }
 
 // ------------------------------------------------- batch norm, backward -----
+// The ReLU gate of a backward pass: none (both null), the tensor itself (open where > 0), or its bits (bn_apply_kernel).
+template <typename T> struct GateOf {
+  const T* tensor;
+  const unsigned char* bits;
+};
 // dz = dy * [mask > 0];  s0 = sum dz, s1 = sum dz*xhat (xhat from x, stats),
 // s2 = sum dz*xhat2 (second normalised tensor sharing dz: the projection shortcut).
 // The sums are the parameter gradients: dbeta = s0, dgamma = s1 (dgamma2 = s2, dbeta2 = s0).
 template <typename T, int VEC, int NS>
 __global__ void __launch_bounds__(kRedThreads)
-bn_bwd_reduce_kernel(const T* __restrict__ dy, const T* __restrict__ mask, const T* __restrict__ x,
+bn_bwd_reduce_kernel(const T* __restrict__ dy, const GateOf<T> gate, const T* __restrict__ x,
                      const float* __restrict__ stats, const T* __restrict__ x2, const float* __restrict__ stats2,
                      RedGeom g, float* __restrict__ sums, float* __restrict__ dgamma, float* __restrict__ dbeta,
                      float* __restrict__ dgamma2, float* __restrict__ dbeta2, float* __restrict__ partial,
                      unsigned int* __restrict__ counter) {
   const int C = g.ld;
+  const bool by_bits = VEC == 8 && gate.bits != nullptr;
+  const T* mask = by_bits ? nullptr : gate.tensor;
   channel_reduce<NS, VEC>(
       g, partial, counter,
       [&](int row, int c0, float (&s)[NS][VEC]) {
         const size_t off = (size_t)row * C + c0;
         float d[VEC], m[VEC], v[VEC], v2[VEC];
         load_vec<T, VEC>(dy + off, d);
-        if (mask) load_vec<T, VEC>(mask + off, m);
+        unsigned int open = 0xffu;
+        if (by_bits) open = gate.bits[off / VEC];
+        else if (mask) load_vec<T, VEC>(mask + off, m);
         load_vec<T, VEC>(x + off, v);
         if (NS == 3) load_vec<T, VEC>(x2 + off, v2);
 #pragma unroll
         for (int i = 0; i < VEC; ++i) {
           const int c = c0 + i;
-          float dz = (mask && !(m[i] > 0.f)) ? 0.f : d[i];
+          float dz = ((mask && !(m[i] > 0.f)) || (VEC == 8 && !(open >> i & 1u))) ? 0.f : d[i];
           s[0][i] += dz;
           s[1][i] += dz * ((v[i] - stats[c]) * stats[C + c]);
           if (NS == 3) s[2][i] += dz * ((v2[i] - stats2[c]) * stats2[C + c]);
@@ -458,7 +478,7 @@ bn_bwd_reduce_kernel(const T* __restrict__ dy, const T* __restrict__ mask, const
 // normalised tensor (dx2, TWO).  Per-thread channel constants and loads in flight as in bn_apply_kernel.
 template <typename T, int VEC, bool TWO>
 __global__ void __launch_bounds__(kEwThreads, 3)
-bn_bwd_apply_kernel(const T* __restrict__ dy, const T* __restrict__ mask, const T* __restrict__ x,
+bn_bwd_apply_kernel(const T* __restrict__ dy, const GateOf<T> gate, const T* __restrict__ x,
                     const float* __restrict__ stats, const float* __restrict__ gamma,
                     const float* __restrict__ sums, const T* __restrict__ x2,
                     const float* __restrict__ stats2, const float* __restrict__ gamma2,
@@ -479,7 +499,9 @@ bn_bwd_apply_kernel(const T* __restrict__ dy, const T* __restrict__ mask, const 
     s0[j] = sums[c0 + j] * inv_m; s1[j] = sums[C + c0 + j] * inv_m;
     if constexpr (TWO) { mean2[j] = stats2[c0 + j]; inv2[j] = stats2[C + c0 + j]; gi2[j] = gamma2[c0 + j] * inv2[j]; s2[j] = sums[2 * C + c0 + j] * inv_m; }
   }
-  auto one = [&](size_t i, const RawVec<T, VEC>& dv, const RawVec<T, VEC>& mv, const RawVec<T, VEC>& xv) {
+  const bool by_bits = VEC == 8 && gate.bits != nullptr;
+  const T* mask = by_bits ? nullptr : gate.tensor;
+  auto one = [&](size_t i, const RawVec<T, VEC>& dv, const RawVec<T, VEC>& mv, unsigned int open, const RawVec<T, VEC>& xv) {
     float d[VEC], m[VEC], v[VEC], v2[VEC], r[VEC], o[VEC], o2[VEC];
     raw_to_f<T, VEC>(dv, d);
     if (mask) raw_to_f<T, VEC>(mv, m);
@@ -488,7 +510,7 @@ bn_bwd_apply_kernel(const T* __restrict__ dy, const T* __restrict__ mask, const 
     if (res) load_vec<T, VEC>(res + i * VEC, r);
 #pragma unroll
     for (int j = 0; j < VEC; ++j) {
-      const float dz = (mask && !(m[j] > 0.f)) ? 0.f : d[j];
+      const float dz = ((mask && !(m[j] > 0.f)) || (VEC == 8 && !(open >> j & 1u))) ? 0.f : d[j];
       const float xh = (v[j] - mean[j]) * inv[j];
       const float t = gi[j] * (dz - s0[j] - xh * s1[j]);
       o[j] = res ? t + r[j] : t;
@@ -504,19 +526,21 @@ bn_bwd_apply_kernel(const T* __restrict__ dy, const T* __restrict__ mask, const 
   size_t i = gtid;
   for (; i + (U - 1) * stride < nvec; i += U * stride) {
     RawVec<T, VEC> dv[U], mv[U], xv[U];
+    unsigned int open[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       dv[u] = load_raw<T, VEC>(dy + (i + u * stride) * VEC);
       mv[u] = mask ? load_raw<T, VEC>(mask + (i + u * stride) * VEC) : dv[u];
+      open[u] = by_bits ? gate.bits[i + u * stride] : 0xffu;
       xv[u] = load_raw<T, VEC>(x + (i + u * stride) * VEC);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) one(i + u * stride, dv[u], mv[u], xv[u]);
+    for (int u = 0; u < U; ++u) one(i + u * stride, dv[u], mv[u], open[u], xv[u]);
   }
   for (; i < nvec; i += stride) {
     RawVec<T, VEC> dv = load_raw<T, VEC>(dy + i * VEC), mv = dv, xv = load_raw<T, VEC>(x + i * VEC);
     if (mask) mv = load_raw<T, VEC>(mask + i * VEC);
-    one(i, dv, mv, xv);
+    one(i, dv, mv, by_bits ? gate.bits[i] : 0xffu, xv);
   }
 }
 
@@ -961,7 +985,7 @@ template <typename T>
 inline cudaError_t launch_bn_apply(cudaStream_t st, const T* x, float* stats, const float* gamma, const float* beta,
                                    const T* res, const float* res_stats, const float* res_gamma, const float* res_beta,
                                    bool relu, T* y, size_t rows, int C, float eps, const float* partial, int nparts,
-                                   int block_cap, float* running = nullptr, float momentum = 0.f) {
+                                   int block_cap, float* running = nullptr, float momentum = 0.f, unsigned char* bits = nullptr) {
   constexpr int V = full_vec<T>();
   const size_t n = rows * C;
   PartialSums ps{};
@@ -973,18 +997,18 @@ inline cudaError_t launch_bn_apply(cudaStream_t st, const T* x, float* stats, co
   }
   if (C % V == 0) {
     const int blocks = ew_grid_for_channels(n / V, C / V, ps.partial ? block_cap : 0);
-    if (res_stats) return launch_chained(bn_apply_kernel<T, V, true>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, n / V, C, ps);
-    return launch_chained(bn_apply_kernel<T, V, false>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, n / V, C, ps);
+    if (res_stats) return launch_chained(bn_apply_kernel<T, V, true>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, bits, n / V, C, ps);
+    return launch_chained(bn_apply_kernel<T, V, false>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, bits, n / V, C, ps);
   }
   const int blocks = ew_grid_for_channels(n, C, 0);
-  if (res_stats) return launch_chained(bn_apply_kernel<T, 1, true>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, n, C, ps);
-  return launch_chained(bn_apply_kernel<T, 1, false>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, n, C, ps);
+  if (res_stats) return launch_chained(bn_apply_kernel<T, 1, true>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, (unsigned char*)nullptr, n, C, ps);
+  return launch_chained(bn_apply_kernel<T, 1, false>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, (unsigned char*)nullptr, n, C, ps);
 }
 
 // First half of the batch-norm backward: the per-channel sums of dz = dy*[mask>0] (and dz*xhat, dz*xhat2),
 // which are also the parameter gradients; totals to `sums` [3*C].
 template <typename T>
-inline cudaError_t launch_bn_bwd_reduce(cudaStream_t st, const T* dy, const T* mask, const T* x, const float* stats,
+inline cudaError_t launch_bn_bwd_reduce(cudaStream_t st, const T* dy, const GateOf<T> gate, const T* x, const float* stats,
                                         const T* x2, const float* stats2, size_t rows, int C, float* sums,
                                         float* dgamma, float* dbeta, float* dgamma2, float* dbeta2, float* scratch,
                                         unsigned int* counter) {
@@ -994,7 +1018,7 @@ inline cudaError_t launch_bn_bwd_reduce(cudaStream_t st, const T* dy, const T* m
   RedGeom g = red_geom((int)rows, C, vec ? V : 1);
   const size_t smem = (size_t)(g.rp > 2 ? g.rp : 2) * ns * g.C * 4;
 #define FDG_RED(VV, NS) bn_bwd_reduce_kernel<T, VV, NS><<<dim3(g.blocks, g.slabs), kRedThreads, smem, st>>>( \
-      dy, mask, x, stats, x2, stats2, g, sums, dgamma, dbeta, dgamma2, dbeta2, scratch, counter)
+      dy, gate, x, stats, x2, stats2, g, sums, dgamma, dbeta, dgamma2, dbeta2, scratch, counter)
   if (vec) { if (two) FDG_RED(V, 3); else FDG_RED(V, 2); }
   else     { if (two) FDG_RED(1, 3); else FDG_RED(1, 2); }
 #undef FDG_RED
@@ -1005,7 +1029,7 @@ inline cudaError_t launch_bn_bwd_reduce(cudaStream_t st, const T* dy, const T* m
 // The sums come from `sums`, or, when `partial` != null, from `nparts` rows of per-CTA sums (sum dz, sum dz*xhat)
 // left by the data-gradient kernel that produced dy (block 0 then also writes dbeta / dgamma).
 template <typename T>
-inline cudaError_t launch_bn_bwd_apply(cudaStream_t st, const T* dy, const T* mask, const T* x, const float* stats,
+inline cudaError_t launch_bn_bwd_apply(cudaStream_t st, const T* dy, const GateOf<T> gate, const T* x, const float* stats,
                                        const float* gamma, const float* sums, const T* x2, const float* stats2,
                                        const float* gamma2, const T* res, T* dx, T* dx2, size_t rows, int C,
                                        const float* partial, int nparts, float* dgamma, float* dbeta, int block_cap) {
@@ -1019,12 +1043,12 @@ inline cudaError_t launch_bn_bwd_apply(cudaStream_t st, const T* dy, const T* ma
   }
   if (C % V == 0) {
     const int blocks = ew_grid_for_channels(n / V, C / V, ps.partial ? block_cap : 0);
-    if (dx2) return launch_chained(bn_bwd_apply_kernel<T, V, true>, blocks, kEwThreads, 0, st, dy, mask, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n / V, C, inv_m, ps);
-    return launch_chained(bn_bwd_apply_kernel<T, V, false>, blocks, kEwThreads, 0, st, dy, mask, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n / V, C, inv_m, ps);
+    if (dx2) return launch_chained(bn_bwd_apply_kernel<T, V, true>, blocks, kEwThreads, 0, st, dy, gate, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n / V, C, inv_m, ps);
+    return launch_chained(bn_bwd_apply_kernel<T, V, false>, blocks, kEwThreads, 0, st, dy, gate, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n / V, C, inv_m, ps);
   }
   const int blocks = ew_grid_for_channels(n, C, 0);
-  if (dx2) return launch_chained(bn_bwd_apply_kernel<T, 1, true>, blocks, kEwThreads, 0, st, dy, mask, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n, C, inv_m, ps);
-  return launch_chained(bn_bwd_apply_kernel<T, 1, false>, blocks, kEwThreads, 0, st, dy, mask, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n, C, inv_m, ps);
+  if (dx2) return launch_chained(bn_bwd_apply_kernel<T, 1, true>, blocks, kEwThreads, 0, st, dy, gate, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n, C, inv_m, ps);
+  return launch_chained(bn_bwd_apply_kernel<T, 1, false>, blocks, kEwThreads, 0, st, dy, gate, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n, C, inv_m, ps);
 }
 
 template <typename T>

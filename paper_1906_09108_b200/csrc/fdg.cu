@@ -63,6 +63,8 @@ struct Unit {
   size_t w1, g1, b1, w2, g2, b2, ws, gs, bs;
   // offsets (elements of T) of saved tensors inside an activation-FIFO slot; y is the unit output
   size_t t_a, t_b, t_c, t_y, t_s;
+  // offsets of the ReLU gates of t_a / t_b / t_c / t_y as bits (bf16 mode; elements of T, one bit per element of the tensor)
+  size_t q_a, q_b, q_c, q_y;
   // offsets (floats) of saved statistics inside the slot's fp32 region
   size_t st1, st2, sts;
   // offsets of the flipped copies of w1 / w2 (and of the transposed 1x1 shortcut filter) inside a wflip16 slot, or -1
@@ -382,6 +384,7 @@ static void plan_modules(fdg_ctx* c) {
     m.in_elems = B * m.in_h * m.in_w * m.in_c;
     size_t te = 0, tf = 0, maxa = m.in_elems, scr = 0, wscr = 0;
     auto tens = [&](size_t e) { size_t o = te; te += align_up(e, 128); maxa = std::max(maxa, e); return o; };
+    auto bits = [&](size_t e) { size_t o = te; if (c->bf16_mode) te += align_up(e / 16 + 8, 128); return o; };
     auto stat = [&](int ch) { size_t o = tf; tf += align_up((size_t)2 * ch, 64); return o; };
     auto red_scratch = [&](size_t rows, int ch) { scr = std::max(scr, (size_t)kRedMaxBlocks * kRedMaxSums * ch); (void)rows; };
     auto wg_scratch = [&](int n, int h, int w, int cin, int p, int q, int cout, int r, int stride, int pad) {
@@ -395,10 +398,12 @@ static void plan_modules(fdg_ctx* c) {
         case U_STEM:
           if (u.bn) { u.t_a = tens(out_e); u.st1 = stat(u.co); red_scratch(B * u.P * u.Q, u.co); }
           u.t_y = tens(out_e);
+          if (u.bn) u.q_y = bits(out_e);
           wg_scratch(a.batch, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, 1, 1);
           break;
         case U_BASIC:
           u.t_a = tens(out_e); u.t_b = tens(out_e); u.t_c = tens(out_e); u.t_y = tens(out_e);
+          u.q_b = bits(out_e); u.q_y = bits(out_e);
           u.st1 = stat(u.co); u.st2 = stat(u.co);
           if (u.proj) { u.t_s = tens(out_e); u.sts = stat(u.co); }
           red_scratch(B * u.P * u.Q, u.co);
@@ -408,6 +413,7 @@ static void plan_modules(fdg_ctx* c) {
           break;
         case U_PREACT:
           u.t_a = tens(in_e); u.t_b = tens(out_e); u.t_c = tens(out_e); u.t_y = tens(out_e);
+          u.q_a = bits(in_e); u.q_c = bits(out_e);
           u.st1 = stat(u.ci); u.st2 = stat(u.co);
           red_scratch(B * u.H * u.W, std::max(u.ci, u.co));
           wg_scratch(a.batch, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, u.stride, 1);
@@ -415,7 +421,7 @@ static void plan_modules(fdg_ctx* c) {
           if (u.proj) wg_scratch(a.batch, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
           break;
         case U_HEAD:
-          if (u.bn) { u.t_a = tens(in_e); u.st1 = stat(u.ci); red_scratch(B * u.H * u.W, u.ci); }
+          if (u.bn) { u.t_a = tens(in_e); u.q_a = bits(in_e); u.st1 = stat(u.ci); red_scratch(B * u.H * u.W, u.ci); }
           break;
       }
     }
@@ -587,33 +593,33 @@ static void bn_stats(Launch& L, Module& m, const T* x, size_t rows, int C, float
 template <typename T>
 static void bn_apply(Launch& L, Module& m, const T* x, float* stats, const float* gamma, const float* beta, const T* res,
                      const float* res_stats, const float* res_gamma, const float* res_beta, bool relu, T* y,
-                     size_t rows, int C, int nparts = 0, long long run = -1) {
+                     size_t rows, int C, int nparts = 0, long long run = -1, unsigned char* bits = nullptr) {
   if (nparts < 0) nparts = 0;               // the statistics were finalised behind the convolution
   const size_t n = rows * C;
   L.begin(KC_BN_APPLY, (double)n * sizeof(T) * (res ? 3 : 2), 6.0 * n);
   L.note(launch_bn_apply<T>(L.st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, relu, y, rows, C,
                             L.c->arch.bn_eps, nparts > 0 ? m.red_partial : nullptr, nparts, L.c->ew_block_cap,
-                            (nparts > 0 && run >= 0) ? m.running + run : nullptr, kBnMomentum));
+                            (nparts > 0 && run >= 0) ? m.running + run : nullptr, kBnMomentum, bits));
   ++L.c->launches;
 }
 
 // Backward of y = BN(x) (and optionally y2 = BN2(x2) sharing the same upstream gradient):
 // dz = dy*[mask>0]; parameter gradients into dgamma/dbeta; dx (+res) and dx2.
 template <typename T>
-static void bn_backward(Launch& L, Module& m, const T* dy, const T* mask, const T* x, const float* stats,
+static void bn_backward(Launch& L, Module& m, const T* dy, const GateOf<T> mask, const T* x, const float* stats,
                         const float* gamma, float* dgamma, float* dbeta, const T* x2, const float* stats2,
                         const float* gamma2, float* dgamma2, float* dbeta2, const T* res, T* dx, T* dx2,
                         size_t rows, int C, int nparts = 0) {
   const bool two = x2 != nullptr;
   const bool sums_ready = nparts > 0;    // the kernel that produced dy left nparts rows of partial sums in m.red_partial
   if (!sums_ready) {
-    L.begin(KC_BN_BWD_REDUCE, (double)rows * C * sizeof(T) * (2 + (mask ? 1 : 0) + (two ? 1 : 0)), 8.0 * rows * C);
+    L.begin(KC_BN_BWD_REDUCE, (double)rows * C * sizeof(T) * (2 + (mask.bits ? 0.0625 : mask.tensor ? 1 : 0) + (two ? 1 : 0)), 8.0 * rows * C);
     L.note(launch_bn_bwd_reduce<T>(L.st, dy, mask, x, stats, x2, stats2, rows, C, m.bnsums, dgamma, dbeta, dgamma2, dbeta2,
                                    m.scratch, m.counter));
     ++L.c->launches;
   }
   const size_t n = rows * C;
-  L.begin(KC_BN_BWD_APPLY, (double)n * sizeof(T) * (3 + (mask ? 1 : 0) + (two ? 2 : 0) + (res ? 1 : 0)), 10.0 * n);
+  L.begin(KC_BN_BWD_APPLY, (double)n * sizeof(T) * (3 + (mask.bits ? 0.0625 : mask.tensor ? 1 : 0) + (two ? 2 : 0) + (res ? 1 : 0)), 10.0 * n);
   L.note(launch_bn_bwd_apply<T>(L.st, dy, mask, x, stats, gamma, m.bnsums, x2, stats2, gamma2, res, dx, dx2, rows, C,
                                 sums_ready ? m.red_partial : nullptr, nparts, dgamma, dbeta, L.c->ew_block_cap));
   ++L.c->launches;
@@ -667,21 +673,21 @@ static int conv_fprop(Launch& L, Module& m, const ConvGeom& g, const T* x, const
 // The batch-norm backward that will consume dx as its upstream gradient: dz = dx * [mask > 0],
 // xhat from (x, stats).  When the data-gradient kernel can, it forms that backward's two sums
 // per CTA in its epilogue and conv_dgrad returns the number of partial rows left in m.red_partial.
-template <typename T> struct NextBnBwd { const T* mask; const T* x; const float* stats; };
+template <typename T> struct NextBnBwd { GateOf<T> mask; const T* x; const float* stats; };
 
 template <typename T>
 static int conv_dgrad(Launch& L, Module& m, const ConvGeom& g, const T* dy, const T* w, const T* wflip, T* dx,
-                       const T* res, const T* mask, const NextBnBwd<T>* next = nullptr, const T* dy_up = nullptr) {
-  L.begin(KC_CONV_DGRAD, (out_elems(g) + w_elems(g) + in_elems(g) * (1 + (res ? 1 : 0) + (mask ? 1 : 0) + (next ? 2 : 0))) * sizeof(T), conv_flops(g));
+                       const T* res, const GateOf<T> mask, const NextBnBwd<T>* next = nullptr, const T* dy_up = nullptr) {
+  L.begin(KC_CONV_DGRAD, (out_elems(g) + w_elems(g) + in_elems(g) * (1 + (res ? 1 : 0) + (mask.tensor ? 1 : 0) + (next ? 2 : 0))) * sizeof(T), conv_flops(g));
   int nparts = 0;
   if constexpr (std::is_same<T, bf16>::value) {
     halo::EpiReduce r{};
-    if (next) { r.mode = 2; r.mask = next->mask; r.xprev = next->x; r.pstats = next->stats; r.partial = m.red_partial; }
-    L.note(bf16_conv_dgrad(L.st, &L.c->tmaps, g, dy, w, wflip, dy_up, dx, res, mask, next ? &r : nullptr, &nparts, L.c->tc_error, &L.c->launches));
+    if (next) { r.mode = 2; r.mask = next->mask.tensor; r.mask_bits = next->mask.bits; r.xprev = next->x; r.pstats = next->stats; r.partial = m.red_partial; }
+    L.note(bf16_conv_dgrad(L.st, &L.c->tmaps, g, dy, w, wflip, dy_up, dx, res, mask.tensor, next ? &r : nullptr, &nparts, L.c->tc_error, &L.c->launches, mask.bits));
   } else {
     direct::Reduce<T> r{};
-    if (next) r = direct::Reduce<T>{2, next->mask, next->x, next->stats, m.red_partial};
-    L.note(cuda_core_conv<T>(L.st, g, true, dy, w, dx, res, mask, next ? &r : nullptr, &nparts, &L.c->launches));
+    if (next) r = direct::Reduce<T>{2, next->mask.tensor, next->x, next->stats, m.red_partial};
+    L.note(cuda_core_conv<T>(L.st, g, true, dy, w, dx, res, mask.tensor, next ? &r : nullptr, &nparts, &L.c->launches));
   }
   return nparts;
 }
@@ -741,6 +747,7 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
   float* F = slot_F(m, slot);
   const T* x = module_input<T>(c, m, tau, eval);
   T* tmp = reinterpret_cast<T*>(m.temps[2]);
+  auto gate_bits = [&](size_t q) { return (sizeof(T) == 2 && !eval) ? reinterpret_cast<unsigned char*>(S + q) : nullptr; };
   // statistics of a convolution output y that left `np` rows of partial sums (0: reduce y now)
   auto stats_of = [&](int np, const T* y, size_t rows, int C, float* stats, long long run) {
     if (!eval && np == 0) bn_stats<T>(L, m, y, rows, C, eps, stats, run);
@@ -759,7 +766,7 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
         if (u.bn) {
           const int np = conv_fprop<T>(L, m, g, x, wt + u.w1, S + u.t_a, nullptr, !eval, F + u.st1, u.r1);
           stats_of(np, S + u.t_a, rows_out, u.co, F + u.st1, u.r1);
-          bn_apply<T>(L, m, S + u.t_a, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_y, rows_out, u.co, np, u.r1);
+          bn_apply<T>(L, m, S + u.t_a, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_y, rows_out, u.co, np, u.r1, gate_bits(u.q_y));
         } else {
           conv_fprop<T>(L, m, g, x, wt + u.w1, S + u.t_y, nullptr);
         }
@@ -770,7 +777,7 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
         ConvGeom g2 = geom(B, u.P, u.Q, u.co, u.P, u.Q, u.co, 3, 1, 1);
         const int np1 = conv_fprop<T>(L, m, g1, x, wt + u.w1, S + u.t_a, nullptr, !eval, F + u.st1, u.r1);   // c1
         stats_of(np1, S + u.t_a, rows_out, u.co, F + u.st1, u.r1);
-        bn_apply<T>(L, m, S + u.t_a, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_b, rows_out, u.co, np1, u.r1);  // a1
+        bn_apply<T>(L, m, S + u.t_a, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_b, rows_out, u.co, np1, u.r1, gate_bits(u.q_b));  // a1
         if (u.proj) {          // shortcut first: its statistics must not disturb the partial sums conv2 leaves for BN2
           ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
           const int nps = conv_fprop<T>(L, m, gs, x, wt + u.ws, S + u.t_s, nullptr, !eval, F + u.sts, u.rs);   // cs
@@ -779,14 +786,14 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
         const int np2 = conv_fprop<T>(L, m, g2, S + u.t_b, wt + u.w2, S + u.t_c, nullptr, !eval, F + u.st2, u.r2);   // c2
         stats_of(np2, S + u.t_c, rows_out, u.co, F + u.st2, u.r2);
         if (u.proj) {
-          bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, S + u.t_s, F + u.sts, wf + u.gs, wf + u.bs, true, S + u.t_y, rows_out, u.co, np2, u.r2);
+          bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, S + u.t_s, F + u.sts, wf + u.gs, wf + u.bs, true, S + u.t_y, rows_out, u.co, np2, u.r2, gate_bits(u.q_y));
         } else if (u.zpad) {   // the shortcut is x at every stride-th pixel between zero channels: built in a temporary
           L.begin(KC_BN_APPLY, (double)rows_out * (u.ci + u.co) * sizeof(T), 0.0);
           pad_shortcut_kernel<T><<<ew_blocks(rows_out * u.co), 256, 0, L.st>>>(x, tmp, rows_out, u.P, u.Q, u.H, u.W, u.ci, u.co, u.stride);
           L.check();
-          bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, tmp, nullptr, nullptr, nullptr, true, S + u.t_y, rows_out, u.co, np2, u.r2);
+          bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, tmp, nullptr, nullptr, nullptr, true, S + u.t_y, rows_out, u.co, np2, u.r2, gate_bits(u.q_y));
         } else {
-          bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, x, nullptr, nullptr, nullptr, true, S + u.t_y, rows_out, u.co, np2, u.r2);
+          bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, x, nullptr, nullptr, nullptr, true, S + u.t_y, rows_out, u.co, np2, u.r2, gate_bits(u.q_y));
         }
         break;
       }
@@ -795,10 +802,10 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
         ConvGeom g2 = geom(B, u.P, u.Q, u.co, u.P, u.Q, u.co, 3, 1, 1);
         stats_of(x_np, x, rows_in, u.ci, F + u.st1, u.r1);
         x_np = 0;
-        bn_apply<T>(L, m, x, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_a, rows_in, u.ci);   // o
+        bn_apply<T>(L, m, x, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_a, rows_in, u.ci, 0, -1, gate_bits(u.q_a));   // o
         const int np = conv_fprop<T>(L, m, g1, S + u.t_a, wt + u.w1, S + u.t_b, nullptr, !eval, F + u.st2, u.r2);   // c1
         stats_of(np, S + u.t_b, rows_out, u.co, F + u.st2, u.r2);
-        bn_apply<T>(L, m, S + u.t_b, F + u.st2, wf + u.g2, wf + u.b2, nullptr, nullptr, nullptr, nullptr, true, S + u.t_c, rows_out, u.co, np, u.r2); // a2
+        bn_apply<T>(L, m, S + u.t_b, F + u.st2, wf + u.g2, wf + u.b2, nullptr, nullptr, nullptr, nullptr, true, S + u.t_c, rows_out, u.co, np, u.r2, gate_bits(u.q_c)); // a2
         if (u.proj) {
           ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
           conv_fprop<T>(L, m, gs, S + u.t_a, wt + u.ws, tmp, nullptr);
@@ -860,7 +867,7 @@ static void head_forward_backward(fdg_ctx* c, Module& m, Launch& L, int64_t tau,
   const T* feat = x;
   if (u.bn) {
     if (!m.head_stats_ready) bn_stats<T>(L, m, x, rows, F, c->arch.bn_eps, Fs + u.st1, u.r1);
-    bn_apply<T>(L, m, x, Fs + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_a, rows, F);
+    bn_apply<T>(L, m, x, Fs + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_a, rows, F, 0, -1, sizeof(T) == 2 ? reinterpret_cast<unsigned char*>(S + u.q_a) : nullptr);
     feat = S + u.t_a;
   }
   const int32_t* labels = c->labels + (size_t)(tau % c->label_ring) * B;
@@ -874,7 +881,7 @@ static void head_forward_backward(fdg_ctx* c, Module& m, Launch& L, int64_t tau,
                         m.grad + u.w1, m.grad + u.w2, m.loss, c->flags, true, false));
   ++c->launches;
   if (u.bn)
-    bn_backward<T>(L, m, dfeat, feat, x, Fs + u.st1, wf + u.g1, m.grad + u.g1, m.grad + u.b1, nullptr, nullptr, nullptr,
+    bn_backward<T>(L, m, dfeat, GateOf<T>{feat, sizeof(T) == 2 ? reinterpret_cast<const unsigned char*>(S + u.q_a) : nullptr}, x, Fs + u.st1, wf + u.g1, m.grad + u.g1, m.grad + u.b1, nullptr, nullptr, nullptr,
                    nullptr, nullptr, nullptr, gout, nullptr, rows, F);
 }
 
@@ -898,6 +905,8 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
   T* T2 = reinterpret_cast<T*>(m.temps[3]);
   T* T3 = reinterpret_cast<T*>(m.temps[4]);
   T* T4 = reinterpret_cast<T*>(m.temps[5]);
+  auto gate = [&](size_t t, size_t q) { return GateOf<T>{S + t, sizeof(T) == 2 ? reinterpret_cast<const unsigned char*>(S + q) : nullptr}; };
+  const GateOf<T> open{};
   bool buf_read[4] = {false, false, false, false};
   bool side_used = false;
   auto fork = [&]() {
@@ -934,8 +943,8 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
     const NextBnBwd<T>* next = nullptr;
     if (i > 0) {
       const Unit& pu = m.units[i - 1];
-      if (pu.type == U_BASIC && !pu.proj) { nb = {S + pu.t_y, S + pu.t_c, F + pu.st2}; next = &nb; }
-      if (pu.type == U_STEM && pu.bn) { nb = {S + pu.t_y, S + pu.t_a, F + pu.st1}; next = &nb; }
+      if (pu.type == U_BASIC && !pu.proj) { nb = {gate(pu.t_y, pu.q_y), S + pu.t_c, F + pu.st2}; next = &nb; }
+      if (pu.type == U_STEM && pu.bn) { nb = {gate(pu.t_y, pu.q_y), S + pu.t_a, F + pu.st1}; next = &nb; }
     }
     int out_sum_parts = 0;
     switch (u.type) {
@@ -945,7 +954,7 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
         keep(i, 0, dy);
         if (u.bn) {
           wait_buf(0);
-          bn_backward<T>(L, m, dy, S + u.t_y, S + u.t_a, F + u.st1, wf + u.g1, m.grad + u.g1, m.grad + u.b1, nullptr,
+          bn_backward<T>(L, m, dy, gate(u.t_y, u.q_y), S + u.t_a, F + u.st1, wf + u.g1, m.grad + u.g1, m.grad + u.b1, nullptr,
                          nullptr, nullptr, nullptr, nullptr, nullptr, T1, nullptr, rows_out, u.co, dy_sum_parts);
           dc = T1;
           keep(i, 3, T1);
@@ -962,10 +971,10 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
         wait_buf(0);
         if (u.proj) {
           wait_buf(2);
-          bn_backward<T>(L, m, dy, S + u.t_y, S + u.t_c, F + u.st2, wf + u.g2, m.grad + u.g2, m.grad + u.b2, S + u.t_s,
+          bn_backward<T>(L, m, dy, gate(u.t_y, u.q_y), S + u.t_c, F + u.st2, wf + u.g2, m.grad + u.g2, m.grad + u.b2, S + u.t_s,
                          F + u.sts, wf + u.gs, m.grad + u.gs, m.grad + u.bs, nullptr, T1, T2, rows_out, u.co);
         } else {
-          bn_backward<T>(L, m, dy, S + u.t_y, S + u.t_c, F + u.st2, wf + u.g2, m.grad + u.g2, m.grad + u.b2, nullptr,
+          bn_backward<T>(L, m, dy, gate(u.t_y, u.q_y), S + u.t_c, F + u.st2, wf + u.g2, m.grad + u.g2, m.grad + u.b2, nullptr,
                          nullptr, nullptr, nullptr, nullptr, nullptr, T1, nullptr, rows_out, u.co, dy_sum_parts);
         }
         keep(i, 1, T1);
@@ -973,11 +982,11 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
         fork();
         conv_wgrad<T>(LS, m, g2, S + u.t_b, T1, m.grad + u.w2);                                          // side
         side_done(0);
-        const NextBnBwd<T> bn1{S + u.t_b, S + u.t_a, F + u.st1};
-        const int bn1_parts = conv_dgrad<T>(L, m, g2, T1, wt + u.w2, flipped_of<T>(m, vslot, u.f2), T3, nullptr, nullptr, &bn1);   // da1
+        const NextBnBwd<T> bn1{gate(u.t_b, u.q_b), S + u.t_a, F + u.st1};
+        const int bn1_parts = conv_dgrad<T>(L, m, g2, T1, wt + u.w2, flipped_of<T>(m, vslot, u.f2), T3, nullptr, open, &bn1);   // da1
         keep(i, 2, T3);
         wait_buf(1);
-        bn_backward<T>(L, m, T3, S + u.t_b, S + u.t_a, F + u.st1, wf + u.g1, m.grad + u.g1, m.grad + u.b1, nullptr,
+        bn_backward<T>(L, m, T3, gate(u.t_b, u.q_b), S + u.t_a, F + u.st1, wf + u.g1, m.grad + u.g1, m.grad + u.b1, nullptr,
                        nullptr, nullptr, nullptr, nullptr, nullptr, T4, nullptr, rows_out, u.co, bn1_parts);      // dc1
         keep(i, 3, T4);
         const T* up = nullptr;
@@ -992,17 +1001,17 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
           conv_wgrad<T>(LS, m, gs, x, T2, m.grad + u.ws);                                                // side
           side_done(2);
           if (need_dx) {
-            conv_dgrad<T>(L, m, gs, T2, wt + u.ws, flipped_of<T>(m, vslot, u.fs), T3, nullptr, nullptr);
-            out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, nullptr, next, up);
+            conv_dgrad<T>(L, m, gs, T2, wt + u.ws, flipped_of<T>(m, vslot, u.fs), T3, nullptr, open);
+            out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, open, next, up);
           }
         } else if (need_dx && u.zpad) {
           // the shortcut's share: the gated upstream gradient's middle channels, put back at every stride-th pixel
           L.begin(KC_BN_BWD_APPLY, (double)(rows_out * u.co * 2 + rows_in * u.ci) * sizeof(T), 0.0);
           pad_shortcut_bwd_kernel<T><<<ew_blocks(rows_in * u.ci), 256, 0, L.st>>>(dy, S + u.t_y, T3, rows_in, u.P, u.Q, u.H, u.W, u.ci, u.co, u.stride);
           L.check();
-          out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, nullptr, next, up);
+          out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, open, next, up);
         } else if (need_dx) {
-          out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, dy, S + u.t_y, next);
+          out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, dy, gate(u.t_y, u.q_y), next);
         }
         if (need_dx) keep(i, 4, gout);
         break;
@@ -1012,9 +1021,9 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
         ConvGeom g2 = geom(B, u.P, u.Q, u.co, u.P, u.Q, u.co, 3, 1, 1);
         keep(i, 0, dy);
         conv_wgrad<T>(L, m, g2, S + u.t_c, dy, m.grad + u.w2);
-        conv_dgrad<T>(L, m, g2, dy, wt + u.w2, flipped_of<T>(m, vslot, u.f2), T1, nullptr, nullptr);   // da2
+        conv_dgrad<T>(L, m, g2, dy, wt + u.w2, flipped_of<T>(m, vslot, u.f2), T1, nullptr, open);   // da2
         keep(i, 1, T1);
-        bn_backward<T>(L, m, T1, S + u.t_c, S + u.t_b, F + u.st2, wf + u.g2, m.grad + u.g2, m.grad + u.b2, nullptr,
+        bn_backward<T>(L, m, T1, gate(u.t_c, u.q_c), S + u.t_b, F + u.st2, wf + u.g2, m.grad + u.g2, m.grad + u.b2, nullptr,
                        nullptr, nullptr, nullptr, nullptr, nullptr, T2, nullptr, rows_out, u.co);      // dc1
         keep(i, 2, T2);
         const T* up = u.stride == 2 ? upsample_dy<T>(L, m, g1, T2) : nullptr;
@@ -1022,14 +1031,14 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
         if (u.proj) {
           ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
           conv_wgrad<T>(L, m, gs, S + u.t_a, dy, m.grad + u.ws);
-          conv_dgrad<T>(L, m, gs, dy, wt + u.ws, flipped_of<T>(m, vslot, u.fs), T3, nullptr, nullptr);
+          conv_dgrad<T>(L, m, gs, dy, wt + u.ws, flipped_of<T>(m, vslot, u.fs), T3, nullptr, open);
           keep(i, 5, T3);
-          conv_dgrad<T>(L, m, g1, T2, wt + u.w1, flipped_of<T>(m, vslot, u.f1), T1, T3, nullptr, nullptr, up);   // do
+          conv_dgrad<T>(L, m, g1, T2, wt + u.w1, flipped_of<T>(m, vslot, u.f1), T1, T3, open, nullptr, up);   // do
         } else {
-          conv_dgrad<T>(L, m, g1, T2, wt + u.w1, flipped_of<T>(m, vslot, u.f1), T1, nullptr, nullptr);
+          conv_dgrad<T>(L, m, g1, T2, wt + u.w1, flipped_of<T>(m, vslot, u.f1), T1, nullptr, open);
         }
         keep(i, 3, T1);
-        bn_backward<T>(L, m, T1, S + u.t_a, x, F + u.st1, wf + u.g1, m.grad + u.g1, m.grad + u.b1, nullptr, nullptr,
+        bn_backward<T>(L, m, T1, gate(u.t_a, u.q_a), x, F + u.st1, wf + u.g1, m.grad + u.g1, m.grad + u.b1, nullptr, nullptr,
                        nullptr, nullptr, nullptr, u.proj ? nullptr : dy, gout, nullptr, rows_in, u.ci);
         keep(i, 4, gout);
         break;
@@ -1273,6 +1282,7 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
   }
   // shared-memory limits of the tensor-core kernels, raised here so that a kernel's first launch may be a recorded one
   if (e == cudaSuccess && c->bf16_mode) e = halo::set_smem_attrs();
+  if (e == cudaSuccess && c->bf16_mode) e = rows::set_attrs();
   if (e == cudaSuccess && c->bf16_mode) e = tc::conv_tc_set_attrs();
   c->own_streams = streams == nullptr;
   for (int k = 0; k < c->K && e == cudaSuccess; ++k) {
