@@ -358,8 +358,7 @@ inline cudaError_t finish_wide_stats(cudaStream_t st, const ConvGeom& g, const W
   const RunningStats run{ws->running, ws->momentum, ws->rows > 1 ? (float)((double)ws->rows / (double)(ws->rows - 1)) : 1.f};
   ++*launches;
   if (nparts) *nparts = -1;
-  return launch_chained(stats_finalize_kernel, dim3((unsigned)((g.Co + 31) / 32)), dim3(256), 0, st, (const float*)ws->partial, ctas,
-                        g.Co, 1.0 / (double)ws->rows, ws->eps, ws->stats, run);
+  return launch_stats_finalize(st, ws->partial, ctas, ws->rows, g.Co, ws->eps, ws->stats, run);
 }
 
 inline cudaError_t bf16_conv_fprop(cudaStream_t st, TensorMapCache* cache, const ConvGeom& g, const bf16_t* x,

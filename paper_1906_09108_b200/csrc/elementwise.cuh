@@ -93,185 +93,213 @@ __device__ __forceinline__ void update_running(const RunningStats& r, int C, int
   r.running[C + c] = (1.f - r.momentum) * r.running[C + c] + r.momentum * (biased_var * r.unbias);
 }
 
-constexpr int kRedThreads = 256;      // threads per block of the channel-reduction kernels
-// Blocks of a channel reduction along the rows.  The last block of a channel slab to finish adds that slab's
-// partial sums, a serial tail that grows with the block count and with the slab's width; wide tensors are
-// therefore cut into slabs of kRedSlab channels (grid.y), each with its own tail on its own SM.
+// ------------------------------------------------- channel reductions ------
+// Sums over the rows of a [rows][C] tensor, per channel, in two launches: bn_sums_kernel leaves one row of NS * C sums per
+// block, sums_finalize_kernel (or the apply kernel that consumes them, up to 128 channels) adds the rows in a fixed order.
+// The first streams the operands: a block owns a contiguous range of rows, thread (r, cv) walks rows r, r + rp, ... of
+// channel vector cv with kRedUnroll of them in flight, whole rows of the tensor at a time (a slab of 32 channels per block,
+// with the block that finished last adding up, read 64-byte pieces and ended in a serial tail: 0.29 of the copy rate on a
+// 42 MB tensor).
+constexpr int kRedThreads = 512;
 constexpr int kRedMaxBlocks = 148;
 constexpr int kRedMaxSums = 3;
-constexpr int kRedSlab = 32;
-constexpr int kRedMaxSlabs = 64;      // ticket words available
+constexpr int kRedUnroll = 4;
+constexpr int kRedMaxVecs = 256;      // channel vectors of a row that a block addresses
 
 // Per-channel statistics record written by the forward and read by the backward.
 // stats[0..C) = mean, stats[C..2C) = 1/sqrt(var+eps).
 
-// Geometry shared by the channel-reduction kernels: a block owns a contiguous range
-// of rows; thread (r, cv) walks rows r, r+RP, ... of channel vector cv.
-// C: channels of one slab (what a block reduces); ld: channels of a row of the tensor; the slab of block
-// (x, y) starts at channel y * C.
 struct RedGeom {
-  int rows, C, cv, rp, blocks, rows_per_block, ld, slabs;
+  int rows, C, cv, rp, blocks, rows_per_block;
 };
-inline RedGeom red_geom(int rows, int C, int vec) {
+// `elem_bytes`: of the tensor.  bf16: every thread of the block, at least one full batch of rows each.  fp32 (the exact mode,
+// a few layers of a network): half the threads and as few as two rows each, i.e. shorter chains of fp32 additions.
+inline RedGeom red_geom(int rows, int C, int vec, size_t elem_bytes) {
   RedGeom g;
-  g.ld = C;
-  g.slabs = 1;
-  if (C > 2 * kRedSlab && C % kRedSlab == 0 && kRedSlab % vec == 0 && C / kRedSlab <= kRedMaxSlabs) { g.slabs = C / kRedSlab; C = kRedSlab; }
   g.rows = rows; g.C = C; g.cv = C / vec;
-  g.rp = kRedThreads / g.cv; if (g.rp < 1) g.rp = 1;
-  int want = (rows + g.rp * 4 - 1) / (g.rp * 4);           // >= 4 passes per block
+  g.rp = (elem_bytes == 4 ? kRedThreads / 2 : kRedThreads) / g.cv; if (g.rp < 1) g.rp = 1;
+  const int least = g.rp * (elem_bytes == 4 ? 2 : kRedUnroll);
+  const int want = (rows + least - 1) / least;
   g.blocks = want < 1 ? 1 : (want > kRedMaxBlocks ? kRedMaxBlocks : want);
   g.rows_per_block = (rows + g.blocks - 1) / g.blocks;
   return g;
 }
 
-// Block-level part: NS sums per channel -> partial[block][NS][C]; the last block to
-// finish adds the partials in block order (fp64) and calls `fin(c, sums[NS])`.
-// The dynamic shared memory of the reduction kernels, reused as doubles for the final totals
-// (NS*C doubles <= rp*NS*C floats whenever rp >= 2; the launchers reserve at least that).
-__device__ __forceinline__ double* red_smem_d() {
-  extern __shared__ double red_smem_as_double[];
-  return red_smem_as_double;
+// 16 raw bytes (or one element when VEC == 1) of T, converted to floats only when used, so that
+// several loads can be in flight without holding their float images in registers.
+template <typename T, int VEC> struct RawVec { uint4 q; };
+template <typename T> struct RawVec<T, 1> { T q; };
+template <typename T, int VEC> __device__ __forceinline__ RawVec<T, VEC> load_raw(const T* __restrict__ p) {
+  RawVec<T, VEC> r;
+  if constexpr (VEC == 1) r.q = p[0]; else r.q = *reinterpret_cast<const uint4*>(p);
+  return r;
+}
+template <typename T, int VEC> __device__ __forceinline__ void raw_to_f(const RawVec<T, VEC>& r, float (&out)[VEC]) {
+  if constexpr (VEC == 1) {
+    out[0] = to_f(r.q);
+  } else {
+    const T* e = reinterpret_cast<const T*>(&r.q);
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) out[i] = to_f(e[i]);
+  }
 }
 
-template <int NS, int VEC, typename Acc, typename Fin>
-__device__ __forceinline__ void channel_reduce(const RedGeom g, float* __restrict__ partial,
-                                               unsigned int* __restrict__ counter, Acc acc, Fin fin_fn) {
-  extern __shared__ float red_smem[];                        // [rp][NS][C]
-  __shared__ bool is_last;
-  const int tid = threadIdx.x;
+// The ReLU gate of a backward pass: none (both null), the tensor itself (open where > 0), or its bits (bn_apply_kernel).
+template <typename T> struct GateOf {
+  const T* tensor;
+  const unsigned char* bits;
+};
+
+// The gate of vector `vec` (VEC elements from element vec * VEC on) as bits.
+template <typename T, int VEC> __device__ __forceinline__ unsigned int gate_bits_of(const GateOf<T>& g, size_t vec) {
+  if (VEC == 8 && g.bits) return g.bits[vec];
+  if (!g.tensor) return 0xffu;
+  float m[VEC];
+  raw_to_f<T, VEC>(load_raw<T, VEC>(g.tensor + vec * VEC), m);
+  unsigned int b = 0;
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) b |= (m[i] > 0.f ? 1u : 0u) << i;
+  return b;
+}
+
+// KIND 1: sum x, sum x^2.  KIND 2: with dz = dy * [gate], sum dz, sum dz * xhat (xhat from x, stats).  KIND 3: also
+// sum dz * xhat2 of a second normalised tensor sharing dz (the projection shortcut).
+// partial[block][NS][C], NS = 2, 2, 3.
+template <typename T, int VEC, int KIND>
+__global__ void __launch_bounds__(kRedThreads, 1)
+bn_sums_kernel(const T* __restrict__ dy, const GateOf<T> gate, const T* __restrict__ x, const float* __restrict__ stats,
+               const T* __restrict__ x2, const float* __restrict__ stats2, RedGeom g, float* __restrict__ partial) {
+  constexpr int NS = KIND == 3 ? 3 : 2;
+  __shared__ float red[kRedThreads * VEC];                   // [rp][C] of one sum
+  const int tid = threadIdx.x, C = g.C;
   const int cvi = tid % g.cv, r = tid / g.cv;
-  const int C = g.C;
-  const int c_off = blockIdx.y * C;                          // first channel of this block's slab
-  partial += (size_t)blockIdx.y * gridDim.x * NS * C;         // this slab's partial sums
-  counter += blockIdx.y;
+  const bool active = r < g.rp;
+  constexpr int U = KIND == 3 ? kRedUnroll / 2 : kRedUnroll;   // vectors in flight: what the registers hold
+  grid_dependency_wait();
+  float mean[KIND >= 2 ? VEC : 1], inv[KIND >= 2 ? VEC : 1], mean2[KIND == 3 ? VEC : 1], inv2[KIND == 3 ? VEC : 1];
+  if constexpr (KIND >= 2) {
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) {
+      const int c = active ? cvi * VEC + i : 0;
+      mean[i] = stats[c]; inv[i] = stats[C + c];
+      if constexpr (KIND == 3) { mean2[i] = stats2[c]; inv2[i] = stats2[C + c]; }
+    }
+  }
   float sums[NS][VEC];
 #pragma unroll
   for (int s = 0; s < NS; ++s)
 #pragma unroll
     for (int i = 0; i < VEC; ++i) sums[s][i] = 0.f;
-  const int row0 = blockIdx.x * g.rows_per_block;
-  const int row1 = min(row0 + g.rows_per_block, g.rows);
-  if (r < g.rp) {
-#pragma unroll 4
-    for (int row = row0 + r; row < row1; row += g.rp) acc(row, c_off + cvi * VEC, sums);
-  }
-  if (r < g.rp) {
+  struct Item { RawVec<T, VEC> d, v, v2; unsigned int open; };
+  auto fetch = [&](size_t row, Item& it) {
+    const size_t off = row * C + (size_t)cvi * VEC;
+    it.v = load_raw<T, VEC>(x + off);
+    if constexpr (KIND >= 2) {
+      it.d = load_raw<T, VEC>(dy + off);
+      it.open = gate_bits_of<T, VEC>(gate, off / VEC);
+      if constexpr (KIND == 3) it.v2 = load_raw<T, VEC>(x2 + off);
+    }
+  };
+  auto add = [&](const Item& it) {
+    float v[VEC];
+    raw_to_f<T, VEC>(it.v, v);
+    if constexpr (KIND == 1) {
 #pragma unroll
-    for (int s = 0; s < NS; ++s)
+      for (int i = 0; i < VEC; ++i) { sums[0][i] += v[i]; sums[1][i] += v[i] * v[i]; }
+    } else {
+      float d[VEC], w[VEC];
+      raw_to_f<T, VEC>(it.d, d);
+      if constexpr (KIND == 3) raw_to_f<T, VEC>(it.v2, w);
 #pragma unroll
-      for (int i = 0; i < VEC; ++i) red_smem[(r * NS + s) * C + cvi * VEC + i] = sums[s][i];
-  }
-  __syncthreads();
-  for (int j = tid; j < NS * C; j += blockDim.x) {
-    float a = 0.f;
-    for (int rr = 0; rr < g.rp; ++rr) a += red_smem[rr * NS * C + j];
-    partial[(size_t)blockIdx.x * NS * C + j] = a;
-  }
-  // Release: the block's partial sums were written by all of its threads, the ticket is taken by one.
-  // The fence that makes them visible before the ticket has to be executed by the ticket's thread
-  // AFTER the barrier that orders it behind the other threads' writes: a fence each writer executes
-  // before the barrier orders only that writer's own later accesses, and the ticket could then reach
-  // L2 ahead of another warp's partial sums (seen on some GPUs as a last block adding stale rows).
-  __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    is_last = (atomicInc(counter, gridDim.x - 1) == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();                                           // acquire: before the other blocks' partial sums are read
-  // NS*C (sum, channel) pairs; kRedThreads / pairs threads share a pair, each taking every
-  // nseg-th block with 8 loads in flight; the segment sums are then added in segment order.
-  __shared__ double fin[kRedThreads];
-  const int pairs = NS * C;
-  for (int p0 = 0; p0 < pairs; p0 += kRedThreads) {
-    const int np = min(pairs - p0, kRedThreads);
-    const int nseg = kRedThreads / np;
-    const int t = tid % np, seg = tid / np;
-    double a = 0.0;
-    if (seg < nseg)
-      for (unsigned b0 = seg; b0 < gridDim.x; b0 += 8 * nseg) {
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const unsigned b = b0 + u * nseg;
-          v[u] = b < gridDim.x ? __ldcg(&partial[(size_t)b * pairs + p0 + t]) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) a += (double)v[u];
+      for (int i = 0; i < VEC; ++i) {
+        const float dz = (it.open >> i & 1u) ? d[i] : 0.f;
+        sums[0][i] += dz;
+        sums[1][i] += dz * ((v[i] - mean[i]) * inv[i]);
+        if constexpr (KIND == 3) sums[2][i] += dz * ((w[i] - mean2[i]) * inv2[i]);
       }
-    fin[tid] = a;
+    }
+  };
+  if (active) {
+    const int row0 = blockIdx.x * g.rows_per_block, row1 = min(row0 + g.rows_per_block, g.rows);
+    int row = row0 + r;
+    for (; row + (U - 1) * g.rp < row1; row += U * g.rp) {
+      Item it[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) fetch((size_t)row + u * g.rp, it[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) add(it[u]);
+    }
+    for (; row < row1; row += g.rp) { Item it; fetch(row, it); add(it); }
+  }
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
     __syncthreads();
-    if (tid < np) {
-      double tot = 0.0;
-      for (int q = 0; q < nseg; ++q) tot += fin[q * np + tid];
-      red_smem_d()[p0 + tid] = tot;
+    if (active) {
+#pragma unroll
+      for (int i = 0; i < VEC; ++i) red[r * C + cvi * VEC + i] = sums[s][i];
     }
     __syncthreads();
-  }
-  for (int c = tid; c < C; c += blockDim.x) {
-    double tot[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) tot[s] = red_smem_d()[s * C + c];
-    fin_fn(c_off + c, tot);
+    for (int c = tid; c < C; c += kRedThreads) {
+      double a = 0.0;
+      for (int rr = 0; rr < g.rp; ++rr) a += (double)red[rr * C + c];
+      partial[(size_t)blockIdx.x * NS * C + s * C + c] = (float)a;
+    }
   }
 }
 
-// ------------------------------------------------- batch norm, forward ------
-// mean and 1/sqrt(var+eps) of each channel over all rows (biased variance).
-template <typename T, int VEC>
-__global__ void __launch_bounds__(kRedThreads)
-bn_stats_kernel(const T* __restrict__ x, RedGeom g, float eps, float* __restrict__ stats,
-                float* __restrict__ partial, unsigned int* __restrict__ counter, RunningStats run) {
-  const int C = g.ld;
-  const double inv_m = 1.0 / (double)g.rows;
-  channel_reduce<2, VEC>(
-      g, partial, counter,
-      [&](int row, int c0, float (&s)[2][VEC]) {
-        float v[VEC];
-        load_vec<T, VEC>(x + (size_t)row * C + c0, v);
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) { s[0][i] += v[i]; s[1][i] += v[i] * v[i]; }
-      },
-      [&](int c, double (&tot)[2]) {
-        double mean = tot[0] * inv_m;
-        double var = tot[1] * inv_m - mean * mean;
-        if (var < 0.0) var = 0.0;
-        stats[c] = (float)mean;
-        stats[C + c] = (float)(1.0 / sqrt(var + (double)eps));
-        if (run.running) update_running(run, C, c, (float)mean, (float)var);
-      });
-}
-
-// Statistics from the rows of partial sums a wide convolution's epilogue left: partial[nparts][2][C] (sum, sum of
-// squares per CTA) -> stats[0..C) = mean, stats[C..2C) = 1/sqrt(var + eps), and the running statistics.  A block
-// takes 32 channels; its 8 warps take every 8th row, their sums are added in warp order (fp64).
-__global__ void __launch_bounds__(256) stats_finalize_kernel(const float* __restrict__ partial, int nparts, int C, double inv_count,
-                                                             float eps, float* __restrict__ stats, RunningStats run) {
-  grid_dependency_wait();                   // launched ahead of the end of the convolution that writes `partial`
-  __shared__ double fin[2][8][32];
-  const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+// The totals of `nparts` rows partial[nparts][NS][C] and what they are for:
+//   KIND 1  statistics: stats[0..C) = mean, stats[C..2C) = 1/sqrt(var + eps), and the running statistics;
+//   KIND 2  out = the sums, o1 = dbeta, o2 = dgamma;   KIND 3  also o3 = dbeta2, o4 = dgamma2.
+// A block takes 32 channels; its 32 warps take every 32nd row (a few loads each, all in flight), then warp w combines
+// channel w: the order is fixed.  fp64 from here on.
+template <int KIND>
+__global__ void __launch_bounds__(1024) sums_finalize_kernel(const float* __restrict__ partial, int nparts, int C, double inv_count,
+                                                             float eps, float* __restrict__ out, RunningStats run,
+                                                             float* __restrict__ o1, float* __restrict__ o2,
+                                                             float* __restrict__ o3, float* __restrict__ o4) {
+  constexpr int NS = KIND == 3 ? 3 : 2;
+  __shared__ double fin[NS][32][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
-  double s = 0.0, ss = 0.0;
-  if (c < C)
-    for (int r = seg; r < nparts; r += 8) {
-      s += (double)partial[(size_t)r * 2 * C + c];
-      ss += (double)partial[(size_t)r * 2 * C + C + c];
-    }
-  fin[0][seg][lane] = s; fin[1][seg][lane] = ss;
-  __syncthreads();
-  if (seg == 0 && c < C) {
-    double a = 0.0, b = 0.0;
+  grid_dependency_wait();                   // launched ahead of the end of the kernel that writes `partial`
+  double t[NS];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) { a += fin[0][q][lane]; b += fin[1][q][lane]; }
-    const double mean = a * inv_count;
-    double var = b * inv_count - mean * mean;
-    if (var < 0.0) var = 0.0;
-    stats[c] = (float)mean;
-    stats[C + c] = (float)(1.0 / sqrt(var + (double)eps));
-    if (run.running) update_running(run, C, c, (float)mean, (float)var);
+  for (int s = 0; s < NS; ++s) t[s] = 0.0;
+  if (c < C)
+#pragma unroll 8
+    for (int r = warp; r < nparts; r += 32) {
+#pragma unroll
+      for (int s = 0; s < NS; ++s) t[s] += (double)partial[((size_t)r * NS + s) * C + c];
+    }
+#pragma unroll
+  for (int s = 0; s < NS; ++s) fin[s][warp][lane] = t[s];
+  __syncthreads();
+  const int cc = blockIdx.x * 32 + warp;
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    t[s] = fin[s][lane][warp];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t[s] += __shfl_xor_sync(0xffffffffu, t[s], o);
   }
+  if (lane != 0 || cc >= C) return;
+  if constexpr (KIND == 1) {
+    const double mean = t[0] * inv_count;
+    double var = t[1] * inv_count - mean * mean;
+    if (var < 0.0) var = 0.0;
+    out[cc] = (float)mean;
+    out[C + cc] = (float)(1.0 / sqrt(var + (double)eps));
+    if (run.running) update_running(run, C, cc, (float)mean, (float)var);
+  } else {
+    out[cc] = (float)t[0]; out[C + cc] = (float)t[1];
+    o1[cc] = (float)t[0]; o2[cc] = (float)t[1];
+    if constexpr (KIND == 3) { out[2 * C + cc] = (float)t[2]; o3[cc] = (float)t[0]; o4[cc] = (float)t[2]; }
+  }
+}
+inline cudaError_t launch_stats_finalize(cudaStream_t st, const float* partial, int nparts, size_t rows, int C, float eps,
+                                         float* stats, const RunningStats& run) {
+  float* none = nullptr;
+  return launch_chained(sums_finalize_kernel<1>, dim3((unsigned)((C + 31) / 32)), dim3(1024), 0, st, partial, nparts, C,
+                        1.0 / (double)rows, eps, stats, run, none, none, none, none);
 }
 
 // Per-CTA partial sums left by a convolution epilogue, partial[nparts][2*C], to be added up by
@@ -291,15 +319,27 @@ struct PartialSums {
 };
 constexpr int kEwThreads = 256;
 
-// Fills out2c[2*C] (shared memory) from the partials; requires blockDim.x == kEwThreads and 2*C <= kEwThreads.
-__device__ __forceinline__ void finalize_partials(const PartialSums ps, int C, float* out2c) {
+// The first eight rows of a thread's share, requested ahead of everything else an apply kernel loads.
+__device__ __forceinline__ void fetch_partials(const PartialSums& ps, int C, float (&v)[8]) {
+  const int pairs = 2 * C, nseg = kEwThreads / pairs, t = threadIdx.x % pairs, seg = threadIdx.x / pairs;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int b = seg + u * nseg;
+    v[u] = (seg < nseg && b < ps.nparts) ? __ldcg(&ps.partial[(size_t)b * pairs + t]) : 0.f;
+  }
+}
+// Fills out2c[2*C] (shared memory) from the partials; requires blockDim.x == kEwThreads and 2*C <= kEwThreads.  `v` as
+// fetched above.
+__device__ __forceinline__ void finalize_partials(const PartialSums& ps, int C, const float (&first)[8], float* out2c) {
   __shared__ double fin[kEwThreads];
   const int tid = threadIdx.x, pairs = 2 * C;
   const int nseg = kEwThreads / pairs;
   const int t = tid % pairs, seg = tid / pairs;
   double a = 0.0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) a += (double)first[u];
   if (seg < nseg)
-    for (int b0 = seg; b0 < ps.nparts; b0 += 8 * nseg) {
+    for (int b0 = seg + 8 * nseg; b0 < ps.nparts; b0 += 8 * nseg) {
       float v[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -330,217 +370,210 @@ __device__ __forceinline__ void finalize_partials(const PartialSums ps, int C, f
   __syncthreads();
 }
 
-// y = [relu]( gamma*(x-mean)*invstd + beta + residual ), residual = none | r | BN_r(r).
-// The statistics come from `stats`, or are first formed from `ps.partial` (and saved to stats).
-// The launcher makes the grid's thread count a multiple of the channel vectors per row, so a thread
-// meets the same VEC channels in every iteration: their constants live in registers, and the loop
-// keeps kEwUnroll independent 16-byte loads per operand in flight.
-constexpr int kEwUnroll = 4;
-// 16 raw bytes (or one element when VEC == 1) of T, converted to floats only when used, so that
-// several loads can be in flight without holding their float images in registers.
-template <typename T, int VEC> struct RawVec { uint4 q; };
-template <typename T> struct RawVec<T, 1> { T q; };
-template <typename T, int VEC> __device__ __forceinline__ RawVec<T, VEC> load_raw(const T* __restrict__ p) {
-  RawVec<T, VEC> r;
-  if constexpr (VEC == 1) r.q = p[0]; else r.q = *reinterpret_cast<const uint4*>(p);
-  return r;
-}
-template <typename T, int VEC> __device__ __forceinline__ void raw_to_f(const RawVec<T, VEC>& r, float (&out)[VEC]) {
-  if constexpr (VEC == 1) {
-    out[0] = to_f(r.q);
-  } else {
-    const T* e = reinterpret_cast<const T*>(&r.q);
+// N consecutive floats, by 16-byte loads where `vec` says the pointer allows it.
+template <int N> __device__ __forceinline__ void load_consts(const float* p, bool vec, float (&v)[N]) {
+  if constexpr (N % 4 == 0) {
+    if (vec) {
 #pragma unroll
-    for (int i = 0; i < VEC; ++i) out[i] = to_f(e[i]);
+      for (int j = 0; j < N; j += 4) {
+        const float4 q = *reinterpret_cast<const float4*>(p + j);
+        v[j] = q.x; v[j + 1] = q.y; v[j + 2] = q.z; v[j + 3] = q.w;
+      }
+      return;
+    }
   }
+#pragma unroll
+  for (int j = 0; j < N; ++j) v[j] = p[j];
 }
 
+// ------------------------------------------------- batch norm, forward ------
+// y = [relu]( gamma*(x-mean)*invstd + beta + residual ), residual = none (RES 0) | r (1) | BN_r(r) (2).
+// The statistics come from `stats`, or are first formed from `ps.partial` (and saved to stats).
+// The launcher makes the grid's thread count a multiple of the channel vectors per row, so a thread
+// meets the same VEC channels in every iteration: their constants (mean, gamma * invstd, beta; the fp32 mode, whose results
+// are compared at 1e-4 through many layers, keeps gamma and invstd apart) live in registers.  A
+// thread's first batch of U vectors is requested right behind the partial sums, whose addition then hides its latency.
 // `bits` (nullable; bf16 vectors only): one bit per element, set where y > 0 -- byte i holds those of vector i.  They are
 // the ReLU gates of the backward pass at a sixteenth of the tensor's size.
-template <typename T, int VEC, bool RES_BN>
-__global__ void __launch_bounds__(kEwThreads, 3)
+constexpr int kEwUnroll = 4;
+template <typename T, int VEC, int RES>
+__global__ void __launch_bounds__(kEwThreads, RES == 2 ? 2 : 3)
 bn_apply_kernel(const T* __restrict__ x, const float* __restrict__ stats,
                 const float* __restrict__ gamma, const float* __restrict__ beta,
                 const T* __restrict__ res, const float* __restrict__ res_stats,
                 const float* __restrict__ res_gamma, const float* __restrict__ res_beta,
-                int relu, T* __restrict__ y, unsigned char* __restrict__ bits, size_t nvec, int C, PartialSums ps) {
-  __shared__ float s_stats[2 * 128];
-  grid_dependency_wait();
-  grid_dependency_release();
-  const float* st = stats;
-  if (ps.partial) { finalize_partials(ps, C, s_stats); st = s_stats; }
+                int relu, int vec_consts, T* __restrict__ y, unsigned char* __restrict__ bits, size_t nvec, int C, PartialSums ps) {
+  constexpr int U = RES == 2 ? 2 : kEwUnroll;
+  __shared__ __align__(16) float s_stats[2 * 128];
   const int cv = C / VEC;
   const size_t gtid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
   const int c0 = (int)(gtid % cv) * VEC;
-  float mean[VEC], inv[VEC], ga[VEC], be[VEC], rmean[RES_BN ? VEC : 1], rinv[RES_BN ? VEC : 1], rga[RES_BN ? VEC : 1], rbe[RES_BN ? VEC : 1];
+  grid_dependency_wait();
+  grid_dependency_release();
+  float first[8];
+  if (ps.partial) fetch_partials(ps, C, first);
+  RawVec<T, VEC> xv[U], rv[RES ? U : 1];
+  auto fetch = [&](size_t i) {
 #pragma unroll
-  for (int j = 0; j < VEC; ++j) {
-    mean[j] = st[c0 + j]; inv[j] = st[C + c0 + j]; ga[j] = gamma[c0 + j]; be[j] = beta[c0 + j];
-    if constexpr (RES_BN) { rmean[j] = res_stats[c0 + j]; rinv[j] = res_stats[C + c0 + j]; rga[j] = res_gamma[c0 + j]; rbe[j] = res_beta[c0 + j]; }
-  }
-  auto one = [&](size_t i, const RawVec<T, VEC>& xv, const RawVec<T, VEC>& rv) {
-    float v[VEC], r[VEC], o[VEC];
-    raw_to_f<T, VEC>(xv, v);
-    if (res) raw_to_f<T, VEC>(rv, r);
+    for (int u = 0; u < U; ++u) xv[u] = load_raw<T, VEC>(x + (i + u * stride) * VEC);
+    if constexpr (RES != 0) {
 #pragma unroll
-    for (int j = 0; j < VEC; ++j) {
-      float t = ga[j] * ((v[j] - mean[j]) * inv[j]) + be[j];
-      if (res) {
-        float rr = r[j];
-        if constexpr (RES_BN) rr = rga[j] * ((rr - rmean[j]) * rinv[j]) + rbe[j];
-        t += rr;
-      }
-      o[j] = relu ? fmaxf(t, 0.f) : t;
-    }
-    store_vec<T, VEC>(y + i * VEC, o);
-    if constexpr (VEC == 8) {
-      if (bits) {
-        // the gate is taken on the value as stored: a positive value below half the smallest bf16 number rounds to zero
-        unsigned int m = 0;
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) m |= (to_f(from_f<T>(o[j])) > 0.f ? 1u : 0u) << j;
-        bits[i] = (unsigned char)m;
-      }
+      for (int u = 0; u < U; ++u) rv[u] = load_raw<T, VEC>(res + (i + u * stride) * VEC);
     }
   };
   size_t i = gtid;
-  for (; i + (kEwUnroll - 1) * stride < nvec; i += kEwUnroll * stride) {
-    RawVec<T, VEC> xv[kEwUnroll], rv[kEwUnroll];
+  bool full = i + (U - 1) * stride < nvec;
+  if (full) fetch(i);
+  constexpr bool EXACT = sizeof(T) == 4;
+  float mean[VEC], ga[VEC], be[VEC], rmean[RES == 2 ? VEC : 1], rga[RES == 2 ? VEC : 1], rbe[RES == 2 ? VEC : 1];
+  float inv[VEC], rinv[RES == 2 ? VEC : 1];
+  const bool vc = vec_consts != 0;
+  load_consts<VEC>(gamma + c0, vc, ga);
+  load_consts<VEC>(beta + c0, vc, be);
+  if constexpr (RES == 2) {
+    load_consts<VEC>(res_gamma + c0, vc, rga);
+    load_consts<VEC>(res_beta + c0, vc, rbe);
+    load_consts<VEC>(res_stats + c0, vc, rmean);
+    load_consts<VEC>(res_stats + C + c0, vc, rinv);
 #pragma unroll
-    for (int u = 0; u < kEwUnroll; ++u) xv[u] = load_raw<T, VEC>(x + (i + u * stride) * VEC);
-    if (res) {
+    for (int j = 0; j < VEC; ++j) if (!EXACT) rga[j] *= rinv[j];
+  }
+  const float* st = stats;
+  if (ps.partial) { finalize_partials(ps, C, first, s_stats); st = s_stats; }
+  load_consts<VEC>(st + c0, vc, mean);
+  load_consts<VEC>(st + C + c0, vc, inv);
 #pragma unroll
-      for (int u = 0; u < kEwUnroll; ++u) rv[u] = load_raw<T, VEC>(res + (i + u * stride) * VEC);
+  for (int j = 0; j < VEC; ++j) if (!EXACT) ga[j] *= inv[j];
+  auto one = [&](size_t at, const RawVec<T, VEC>& xq, const RawVec<T, VEC>& rq) {
+    float v[VEC], r[VEC], o[VEC];
+    raw_to_f<T, VEC>(xq, v);
+    if constexpr (RES != 0) raw_to_f<T, VEC>(rq, r);
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) {
+      float t = EXACT ? ga[j] * ((v[j] - mean[j]) * inv[j]) + be[j] : fmaf(v[j] - mean[j], ga[j], be[j]);
+      if constexpr (RES == 1) t += r[j];
+      if constexpr (RES == 2) t += EXACT ? rga[j] * ((r[j] - rmean[j]) * rinv[j]) + rbe[j] : fmaf(r[j] - rmean[j], rga[j], rbe[j]);
+      o[j] = relu ? fmaxf(t, 0.f) : t;
     }
+    if constexpr (VEC == 8) {
+      // the gate is taken on the value as stored (a positive value below half the smallest bf16 number rounds to zero):
+      // a stored bf16 is positive where its sign is clear and it is not zero
+      uint32_t w[4];
+      unsigned int m = 0;
 #pragma unroll
-    for (int u = 0; u < kEwUnroll; ++u) one(i + u * stride, xv[u], rv[u]);
+      for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 q = __floats2bfloat162_rn(o[2 * j], o[2 * j + 1]);
+        w[j] = *reinterpret_cast<const uint32_t*>(&q);
+      }
+      *reinterpret_cast<uint4*>(y + at * VEC) = make_uint4(w[0], w[1], w[2], w[3]);
+      if (bits) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          m |= ((int)(w[j] << 16) > 0 ? 1u : 0u) << (2 * j);
+          m |= ((int)(w[j] & 0xffff0000u) > 0 ? 1u : 0u) << (2 * j + 1);
+        }
+        bits[at] = (unsigned char)m;
+      }
+    } else {
+      store_vec<T, VEC>(y + at * VEC, o);
+    }
+  };
+  while (full) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) one(i + u * stride, xv[u], rv[RES ? u : 0]);
+    i += U * stride;
+    full = i + (U - 1) * stride < nvec;
+    if (full) fetch(i);
   }
   for (; i < nvec; i += stride) {
-    RawVec<T, VEC> xv = load_raw<T, VEC>(x + i * VEC), rv = xv;
-    if (res) rv = load_raw<T, VEC>(res + i * VEC);
-    one(i, xv, rv);
+    const RawVec<T, VEC> xq = load_raw<T, VEC>(x + i * VEC);
+    RawVec<T, VEC> rq = xq;
+    if constexpr (RES != 0) rq = load_raw<T, VEC>(res + i * VEC);
+    one(i, xq, rq);
   }
 }
 
 // ------------------------------------------------- batch norm, backward -----
-// The ReLU gate of a backward pass: none (both null), the tensor itself (open where > 0), or its bits (bn_apply_kernel).
-template <typename T> struct GateOf {
-  const T* tensor;
-  const unsigned char* bits;
-};
-// dz = dy * [mask > 0];  s0 = sum dz, s1 = sum dz*xhat (xhat from x, stats),
-// s2 = sum dz*xhat2 (second normalised tensor sharing dz: the projection shortcut).
-// The sums are the parameter gradients: dbeta = s0, dgamma = s1 (dgamma2 = s2, dbeta2 = s0).
-template <typename T, int VEC, int NS>
-__global__ void __launch_bounds__(kRedThreads)
-bn_bwd_reduce_kernel(const T* __restrict__ dy, const GateOf<T> gate, const T* __restrict__ x,
-                     const float* __restrict__ stats, const T* __restrict__ x2, const float* __restrict__ stats2,
-                     RedGeom g, float* __restrict__ sums, float* __restrict__ dgamma, float* __restrict__ dbeta,
-                     float* __restrict__ dgamma2, float* __restrict__ dbeta2, float* __restrict__ partial,
-                     unsigned int* __restrict__ counter) {
-  const int C = g.ld;
-  const bool by_bits = VEC == 8 && gate.bits != nullptr;
-  const T* mask = by_bits ? nullptr : gate.tensor;
-  channel_reduce<NS, VEC>(
-      g, partial, counter,
-      [&](int row, int c0, float (&s)[NS][VEC]) {
-        const size_t off = (size_t)row * C + c0;
-        float d[VEC], m[VEC], v[VEC], v2[VEC];
-        load_vec<T, VEC>(dy + off, d);
-        unsigned int open = 0xffu;
-        if (by_bits) open = gate.bits[off / VEC];
-        else if (mask) load_vec<T, VEC>(mask + off, m);
-        load_vec<T, VEC>(x + off, v);
-        if (NS == 3) load_vec<T, VEC>(x2 + off, v2);
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) {
-          const int c = c0 + i;
-          float dz = ((mask && !(m[i] > 0.f)) || (VEC == 8 && !(open >> i & 1u))) ? 0.f : d[i];
-          s[0][i] += dz;
-          s[1][i] += dz * ((v[i] - stats[c]) * stats[C + c]);
-          if (NS == 3) s[2][i] += dz * ((v2[i] - stats2[c]) * stats2[C + c]);
-        }
-      },
-      [&](int c, double (&tot)[NS]) {
-        sums[c] = (float)tot[0];
-        sums[C + c] = (float)tot[1];
-        dbeta[c] = (float)tot[0];
-        dgamma[c] = (float)tot[1];
-        if (NS == 3) {
-          sums[2 * C + c] = (float)tot[2];
-          dbeta2[c] = (float)tot[0];
-          dgamma2[c] = (float)tot[2];
-        }
-      });
-}
-
-// dx = gamma*invstd*(dz - s0/M - xhat*s1/M) [+ res];  optionally the same for the second
-// normalised tensor (dx2, TWO).  Per-thread channel constants and loads in flight as in bn_apply_kernel.
+// dx = gamma*invstd*(dz - s0/M - xhat*s1/M) [+ res] with dz = dy * [gate];  optionally the same for the second
+// normalised tensor (dx2, TWO).  Written as  gi*dz - (x - mean)*k1 - k0  with gi = gamma*invstd, k1 = gi*invstd*s1/M,
+// k0 = gi*s0/M: four constants per channel in registers (the fp32 mode keeps the first form).  First batch of loads ahead of the sums' addition as above.
 template <typename T, int VEC, bool TWO>
-__global__ void __launch_bounds__(kEwThreads, 3)
+__global__ void __launch_bounds__(kEwThreads, TWO ? 2 : 3)
 bn_bwd_apply_kernel(const T* __restrict__ dy, const GateOf<T> gate, const T* __restrict__ x,
                     const float* __restrict__ stats, const float* __restrict__ gamma,
                     const float* __restrict__ sums, const T* __restrict__ x2,
                     const float* __restrict__ stats2, const float* __restrict__ gamma2,
-                    const T* __restrict__ res, T* __restrict__ dx, T* __restrict__ dx2,
+                    const T* __restrict__ res, int vec_consts, T* __restrict__ dx, T* __restrict__ dx2,
                     size_t nvec, int C, float inv_m, PartialSums ps) {
-  __shared__ float s_sums[2 * 128];
-  grid_dependency_wait();
-  grid_dependency_release();
-  if (ps.partial) { finalize_partials(ps, C, s_sums); sums = s_sums; }
+  constexpr int U = 2;
+  __shared__ __align__(16) float s_sums[2 * 128];
   const int cv = C / VEC;
   const size_t gtid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
   const int c0 = (int)(gtid % cv) * VEC;
-  constexpr int V2 = TWO ? VEC : 1;
-  float mean[VEC], inv[VEC], gi[VEC], s0[VEC], s1[VEC], mean2[V2], inv2[V2], gi2[V2], s2[V2];
-#pragma unroll
-  for (int j = 0; j < VEC; ++j) {
-    mean[j] = stats[c0 + j]; inv[j] = stats[C + c0 + j]; gi[j] = gamma[c0 + j] * inv[j];
-    s0[j] = sums[c0 + j] * inv_m; s1[j] = sums[C + c0 + j] * inv_m;
-    if constexpr (TWO) { mean2[j] = stats2[c0 + j]; inv2[j] = stats2[C + c0 + j]; gi2[j] = gamma2[c0 + j] * inv2[j]; s2[j] = sums[2 * C + c0 + j] * inv_m; }
-  }
-  const bool by_bits = VEC == 8 && gate.bits != nullptr;
-  const T* mask = by_bits ? nullptr : gate.tensor;
-  auto one = [&](size_t i, const RawVec<T, VEC>& dv, const RawVec<T, VEC>& mv, unsigned int open, const RawVec<T, VEC>& xv) {
-    float d[VEC], m[VEC], v[VEC], v2[VEC], r[VEC], o[VEC], o2[VEC];
-    raw_to_f<T, VEC>(dv, d);
-    if (mask) raw_to_f<T, VEC>(mv, m);
-    raw_to_f<T, VEC>(xv, v);
-    if constexpr (TWO) load_vec<T, VEC>(x2 + i * VEC, v2);
-    if (res) load_vec<T, VEC>(res + i * VEC, r);
-#pragma unroll
-    for (int j = 0; j < VEC; ++j) {
-      const float dz = ((mask && !(m[j] > 0.f)) || (VEC == 8 && !(open >> j & 1u))) ? 0.f : d[j];
-      const float xh = (v[j] - mean[j]) * inv[j];
-      const float t = gi[j] * (dz - s0[j] - xh * s1[j]);
-      o[j] = res ? t + r[j] : t;
-      if constexpr (TWO) {
-        const float xh2 = (v2[j] - mean2[j]) * inv2[j];
-        o2[j] = gi2[j] * (dz - s0[j] - xh2 * s2[j]);
-      }
-    }
-    store_vec<T, VEC>(dx + i * VEC, o);
-    if constexpr (TWO) store_vec<T, VEC>(dx2 + i * VEC, o2);
-  };
-  constexpr int U = 2;
-  size_t i = gtid;
-  for (; i + (U - 1) * stride < nvec; i += U * stride) {
-    RawVec<T, VEC> dv[U], mv[U], xv[U];
-    unsigned int open[U];
+  grid_dependency_wait();
+  grid_dependency_release();
+  float first[8];
+  if (ps.partial) fetch_partials(ps, C, first);
+  RawVec<T, VEC> dv[U], xv[U];
+  unsigned int open[U];
+  auto fetch = [&](size_t i) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       dv[u] = load_raw<T, VEC>(dy + (i + u * stride) * VEC);
-      mv[u] = mask ? load_raw<T, VEC>(mask + (i + u * stride) * VEC) : dv[u];
-      open[u] = by_bits ? gate.bits[i + u * stride] : 0xffu;
       xv[u] = load_raw<T, VEC>(x + (i + u * stride) * VEC);
+      open[u] = gate_bits_of<T, VEC>(gate, i + u * stride);
     }
+  };
+  size_t i = gtid;
+  bool full = i + (U - 1) * stride < nvec;
+  if (full) fetch(i);
+  const bool vc = vec_consts != 0;
+  constexpr bool EXACT = sizeof(T) == 4;
+  float mean[VEC], gi[VEC], k0[VEC], k1[VEC], mean2[TWO ? VEC : 1], gi2[TWO ? VEC : 1], k02[TWO ? VEC : 1], k12[TWO ? VEC : 1];
+  float inv[VEC], inv2[TWO ? VEC : 1];
+  auto consts = [&](const float* stv, const float* gav, const float* s0p, const float* s1p, float (&mu)[VEC], float (&iv)[VEC],
+                    float (&g)[VEC], float (&a0)[VEC], float (&a1)[VEC]) {
+    load_consts<VEC>(stv + c0, vc, mu);
+    load_consts<VEC>(stv + C + c0, vc, iv);
+    load_consts<VEC>(gav + c0, vc, g);
+    load_consts<VEC>(s0p + c0, vc, a0);
+    load_consts<VEC>(s1p + c0, vc, a1);
 #pragma unroll
-    for (int u = 0; u < U; ++u) one(i + u * stride, dv[u], mv[u], open[u], xv[u]);
+    for (int j = 0; j < VEC; ++j) {
+      g[j] *= iv[j];
+      a0[j] *= inv_m; a1[j] *= inv_m;
+      if (!EXACT) { a0[j] *= g[j]; a1[j] *= g[j] * iv[j]; }
+    }
+  };
+  if (ps.partial) { finalize_partials(ps, C, first, s_sums); sums = s_sums; }
+  consts(stats, gamma, sums, sums + C, mean, inv, gi, k0, k1);
+  if constexpr (TWO) consts(stats2, gamma2, sums, sums + 2 * C, mean2, inv2, gi2, k02, k12);
+  auto one = [&](size_t at, const RawVec<T, VEC>& dq, unsigned int op, const RawVec<T, VEC>& xq) {
+    float d[VEC], v[VEC], v2[VEC], r[VEC], o[VEC], o2[VEC];
+    raw_to_f<T, VEC>(dq, d);
+    raw_to_f<T, VEC>(xq, v);
+    if constexpr (TWO) load_vec<T, VEC>(x2 + at * VEC, v2);
+    if (res) load_vec<T, VEC>(res + at * VEC, r);
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) {
+      const float dz = (op >> j & 1u) ? d[j] : 0.f;
+      const float t = EXACT ? gi[j] * (dz - k0[j] - (v[j] - mean[j]) * inv[j] * k1[j]) : fmaf(gi[j], dz, fmaf(mean[j] - v[j], k1[j], -k0[j]));
+      o[j] = res ? t + r[j] : t;
+      if constexpr (TWO) o2[j] = EXACT ? gi2[j] * (dz - k02[j] - (v2[j] - mean2[j]) * inv2[j] * k12[j]) : fmaf(gi2[j], dz, fmaf(mean2[j] - v2[j], k12[j], -k02[j]));
+    }
+    store_vec<T, VEC>(dx + at * VEC, o);
+    if constexpr (TWO) store_vec<T, VEC>(dx2 + at * VEC, o2);
+  };
+  while (full) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) one(i + u * stride, dv[u], open[u], xv[u]);
+    i += U * stride;
+    full = i + (U - 1) * stride < nvec;
+    if (full) fetch(i);
   }
   for (; i < nvec; i += stride) {
-    RawVec<T, VEC> dv = load_raw<T, VEC>(dy + i * VEC), mv = dv, xv = load_raw<T, VEC>(x + i * VEC);
-    if (mask) mv = load_raw<T, VEC>(mask + i * VEC);
-    one(i, dv, mv, by_bits ? gate.bits[i] : 0xffu, xv);
+    const RawVec<T, VEC> dq = load_raw<T, VEC>(dy + i * VEC), xq = load_raw<T, VEC>(x + i * VEC);
+    one(i, dq, gate_bits_of<T, VEC>(gate, i), xq);
   }
 }
 
@@ -945,24 +978,24 @@ inline int ew_blocks(size_t nvec) {
 }
 template <typename T> constexpr int full_vec() { return 16 / sizeof(T); }
 
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 // Floats of scratch a channel reduction over C channels may write (per-block partial sums).
 inline size_t red_scratch_floats(int C) { return (size_t)kRedMaxBlocks * kRedMaxSums * C; }
 
-// stats[0..C) = mean, stats[C..2C) = 1/sqrt(var + eps) of x [rows][C]; `counter` is a zeroed ticket word
-// (the kernel leaves it zero again).
+// stats[0..C) = mean, stats[C..2C) = 1/sqrt(var + eps) of x [rows][C].
 template <typename T>
 inline cudaError_t launch_bn_stats(cudaStream_t st, const T* x, size_t rows, int C, float eps, float* stats,
-                                   float* scratch, unsigned int* counter, float* running = nullptr, float momentum = 0.f) {
+                                   float* scratch, float* running = nullptr, float momentum = 0.f) {
   constexpr int V = full_vec<T>();
   const RunningStats run{running, momentum, rows > 1 ? (float)((double)rows / (double)(rows - 1)) : 1.f};
-  if (C % V == 0) {
-    RedGeom g = red_geom((int)rows, C, V);
-    bn_stats_kernel<T, V><<<dim3(g.blocks, g.slabs), kRedThreads, (size_t)(g.rp > 2 ? g.rp : 2) * 2 * g.C * 4, st>>>(x, g, eps, stats, scratch, counter, run);
-  } else {
-    RedGeom g = red_geom((int)rows, C, 1);
-    bn_stats_kernel<T, 1><<<dim3(g.blocks, g.slabs), kRedThreads, (size_t)(g.rp > 2 ? g.rp : 2) * 2 * g.C * 4, st>>>(x, g, eps, stats, scratch, counter, run);
-  }
-  return cudaGetLastError();
+  const RedGeom g = red_geom((int)rows, C, C % V == 0 ? V : 1, sizeof(T));
+  const T* no = nullptr;
+  const float* nof = nullptr;
+  const cudaError_t e = C % V == 0
+      ? launch_chained(bn_sums_kernel<T, V, 1>, g.blocks, kRedThreads, 0, st, no, GateOf<T>{}, x, nof, no, nof, g, scratch)
+      : launch_chained(bn_sums_kernel<T, 1, 1>, g.blocks, kRedThreads, 0, st, no, GateOf<T>{}, x, nof, no, nof, g, scratch);
+  return e != cudaSuccess ? e : launch_stats_finalize(st, scratch, g.blocks, rows, C, eps, stats, run);
 }
 
 // Grid of the batch-norm apply kernels: what `nvec` vectors need, bounded by `cap` (0 = none), and such that
@@ -995,34 +1028,40 @@ inline cudaError_t launch_bn_apply(cudaStream_t st, const T* x, float* stats, co
     ps.save0 = stats; ps.save1 = stats + C;
     ps.run = RunningStats{running, momentum, rows > 1 ? (float)((double)rows / (double)(rows - 1)) : 1.f};
   }
-  if (C % V == 0) {
-    const int blocks = ew_grid_for_channels(n / V, C / V, ps.partial ? block_cap : 0);
-    if (res_stats) return launch_chained(bn_apply_kernel<T, V, true>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, bits, n / V, C, ps);
-    return launch_chained(bn_apply_kernel<T, V, false>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, bits, n / V, C, ps);
-  }
-  const int blocks = ew_grid_for_channels(n, C, 0);
-  if (res_stats) return launch_chained(bn_apply_kernel<T, 1, true>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, (unsigned char*)nullptr, n, C, ps);
-  return launch_chained(bn_apply_kernel<T, 1, false>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, res_gamma, res_beta, (int)relu, y, (unsigned char*)nullptr, n, C, ps);
+  const int vc = aligned16(gamma) && aligned16(beta) && aligned16(stats) && aligned16(res_stats) && aligned16(res_gamma) &&
+                 aligned16(res_beta) && C % 4 == 0;
+  const bool vec = C % V == 0;
+  const int blocks = ew_grid_for_channels(vec ? n / V : n, vec ? C / V : C, (vec && ps.partial) ? block_cap : 0);
+#define FDG_APPLY(VV, R) launch_chained(bn_apply_kernel<T, VV, R>, blocks, kEwThreads, 0, st, x, stats, gamma, beta, res, res_stats, \
+      res_gamma, res_beta, (int)relu, vc, y, VV == 8 ? bits : (unsigned char*)nullptr, n / VV, C, ps)
+  if (vec) return res_stats ? FDG_APPLY(V, 2) : (res ? FDG_APPLY(V, 1) : FDG_APPLY(V, 0));
+  return res_stats ? FDG_APPLY(1, 2) : (res ? FDG_APPLY(1, 1) : FDG_APPLY(1, 0));
+#undef FDG_APPLY
 }
 
-// First half of the batch-norm backward: the per-channel sums of dz = dy*[mask>0] (and dz*xhat, dz*xhat2),
-// which are also the parameter gradients; totals to `sums` [3*C].
+// First half of the batch-norm backward: the per-channel sums of dz = dy*[gate] (and dz*xhat, dz*xhat2), which are also
+// the parameter gradients.  Leaves the rows of partial sums in `scratch`; with *rows_left given and two sums of up to 128
+// channels that is all (the apply kernel adds the rows), otherwise the totals go to `sums` [3*C] and the gradients.
 template <typename T>
 inline cudaError_t launch_bn_bwd_reduce(cudaStream_t st, const T* dy, const GateOf<T> gate, const T* x, const float* stats,
                                         const T* x2, const float* stats2, size_t rows, int C, float* sums,
                                         float* dgamma, float* dbeta, float* dgamma2, float* dbeta2, float* scratch,
-                                        unsigned int* counter) {
+                                        int* rows_left, uint64_t* launches) {
   constexpr int V = full_vec<T>();
   const bool two = x2 != nullptr, vec = C % V == 0;
-  const int ns = two ? 3 : 2;
-  RedGeom g = red_geom((int)rows, C, vec ? V : 1);
-  const size_t smem = (size_t)(g.rp > 2 ? g.rp : 2) * ns * g.C * 4;
-#define FDG_RED(VV, NS) bn_bwd_reduce_kernel<T, VV, NS><<<dim3(g.blocks, g.slabs), kRedThreads, smem, st>>>( \
-      dy, gate, x, stats, x2, stats2, g, sums, dgamma, dbeta, dgamma2, dbeta2, scratch, counter)
-  if (vec) { if (two) FDG_RED(V, 3); else FDG_RED(V, 2); }
-  else     { if (two) FDG_RED(1, 3); else FDG_RED(1, 2); }
+  const RedGeom g = red_geom((int)rows, C, vec ? V : 1, sizeof(T));
+#define FDG_RED(VV, K) launch_chained(bn_sums_kernel<T, VV, K>, g.blocks, kRedThreads, 0, st, dy, gate, x, stats, x2, stats2, g, scratch)
+  cudaError_t e = vec ? (two ? FDG_RED(V, 3) : FDG_RED(V, 2)) : (two ? FDG_RED(1, 3) : FDG_RED(1, 2));
 #undef FDG_RED
-  return cudaGetLastError();
+  ++*launches;
+  if (rows_left) *rows_left = 0;
+  if (e != cudaSuccess) return e;
+  if (rows_left && !two && 2 * C <= kEwThreads) { *rows_left = g.blocks; return cudaSuccess; }
+  ++*launches;
+  const dim3 grid((unsigned)((C + 31) / 32));
+  const RunningStats none{};
+  return two ? launch_chained(sums_finalize_kernel<3>, grid, dim3(1024), 0, st, (const float*)scratch, g.blocks, C, 0.0, 0.f, sums, none, dbeta, dgamma, dbeta2, dgamma2)
+             : launch_chained(sums_finalize_kernel<2>, grid, dim3(1024), 0, st, (const float*)scratch, g.blocks, C, 0.0, 0.f, sums, none, dbeta, dgamma, (float*)nullptr, (float*)nullptr);
 }
 
 // Second half: dx = gamma*invstd*(dz - s0/M - xhat*s1/M) [+ res] (and dx2 for the second normalised tensor).
@@ -1041,14 +1080,14 @@ inline cudaError_t launch_bn_bwd_apply(cudaStream_t st, const T* dy, const GateO
     if (2 * C > kEwThreads) return cudaErrorInvalidValue;
     ps.partial = partial; ps.nparts = nparts; ps.kind = 2; ps.save0 = dbeta; ps.save1 = dgamma;
   }
-  if (C % V == 0) {
-    const int blocks = ew_grid_for_channels(n / V, C / V, ps.partial ? block_cap : 0);
-    if (dx2) return launch_chained(bn_bwd_apply_kernel<T, V, true>, blocks, kEwThreads, 0, st, dy, gate, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n / V, C, inv_m, ps);
-    return launch_chained(bn_bwd_apply_kernel<T, V, false>, blocks, kEwThreads, 0, st, dy, gate, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n / V, C, inv_m, ps);
-  }
-  const int blocks = ew_grid_for_channels(n, C, 0);
-  if (dx2) return launch_chained(bn_bwd_apply_kernel<T, 1, true>, blocks, kEwThreads, 0, st, dy, gate, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n, C, inv_m, ps);
-  return launch_chained(bn_bwd_apply_kernel<T, 1, false>, blocks, kEwThreads, 0, st, dy, gate, x, stats, gamma, sums, x2, stats2, gamma2, res, dx, dx2, n, C, inv_m, ps);
+  const int vc = aligned16(stats) && aligned16(gamma) && aligned16(sums) && aligned16(stats2) && aligned16(gamma2) && C % 4 == 0;
+  const bool vec = C % V == 0;
+  const int blocks = ew_grid_for_channels(vec ? n / V : n, vec ? C / V : C, (vec && ps.partial) ? block_cap : 0);
+#define FDG_BAPPLY(VV, TWO) launch_chained(bn_bwd_apply_kernel<T, VV, TWO>, blocks, kEwThreads, 0, st, dy, gate, x, stats, gamma, sums, x2, \
+      stats2, gamma2, res, vc, dx, dx2, n / VV, C, inv_m, ps)
+  if (vec) return dx2 ? FDG_BAPPLY(V, true) : FDG_BAPPLY(V, false);
+  return dx2 ? FDG_BAPPLY(1, true) : FDG_BAPPLY(1, false);
+#undef FDG_BAPPLY
 }
 
 template <typename T>

@@ -103,12 +103,10 @@ struct Module {
   float *scratch = nullptr, *bnsums = nullptr;
   float* wscratch = nullptr;               // partial sums of the weight-gradient kernels (they run on the side stream)
   size_t wscratch_floats = 0;
-  unsigned int* counter = nullptr;
   char* up = nullptr;                      // dy of a stride-2 convolution spread onto the input's pixel grid
   size_t up_elems = 0;
   float* red_partial = nullptr;            // per-CTA partial sums of the reductions fused into convolution epilogues
   size_t red_partial_floats = 0;
-  unsigned int* red_counter = nullptr;
   float *pooled = nullptr, *dlogits = nullptr, *loss_n = nullptr, *loss = nullptr;   // head
   // host state
   int64_t updates = 0;
@@ -279,7 +277,7 @@ static fdg_status validate(const fdg_arch* a, const fdg_config* c, std::string* 
   int chans[5] = {a->stem_width, a->widths[0], a->widths[0], a->widths[0], a->widths[0]};
   for (int i = 0; i < a->n_stages; ++i) chans[1 + i] = a->widths[i];
   for (int ch : chans) {
-    if ((ch % vec != 0 && ch > kRedThreads) || ch / vec > kRedThreads) { *why = "channel count not addressable by the reduction kernels"; return FDG_ERR_UNSUPPORTED; }
+    if ((ch % vec != 0 && ch > kRedMaxVecs) || ch / vec > kRedMaxVecs) { *why = "channel count not addressable by the reduction kernels"; return FDG_ERR_UNSUPPORTED; }
     if (c->precision == FDG_BF16_TC && ch % 8 != 0) { *why = "bf16 mode needs channel counts that are multiples of 8"; return FDG_ERR_UNSUPPORTED; }
   }
   if ((size_t)a->batch * a->in_h * a->in_w * (size_t)std::max({chans[0], chans[1], chans[2], chans[3], chans[4]}) > (size_t)1 << 31) {
@@ -524,7 +522,6 @@ static size_t carve(fdg_ctx* c, char* base) {
     int maxc = 1;
     for (const Unit& u : m.units) maxc = std::max(maxc, std::max(u.ci, u.co));
     m.bnsums = cv.take<float>((size_t)kRedMaxSums * maxc * 4);
-    m.counter = cv.take<unsigned int>(256);
     m.up = m.up_elems ? cv.take<char>(align_up(m.up_elems, 128) * es) : nullptr;
     {
       int widest = 64;                        // rows of 2 * C floats: narrow layers up to 64 channels, wide ones up to 640
@@ -532,7 +529,6 @@ static size_t carve(fdg_ctx* c, char* base) {
       m.red_partial_floats = (size_t)kRedPartialCtas * 2 * widest;
       m.red_partial = cv.take<float>(m.red_partial_floats * 4);
     }
-    m.red_counter = cv.take<unsigned int>(256);
     if (m.k == c->K) {
       const Unit& h = m.units.back();
       m.pooled = cv.take<float>((size_t)c->arch.batch * h.ci * 4);
@@ -584,8 +580,8 @@ struct Launch {
 template <typename T>
 static void bn_stats(Launch& L, Module& m, const T* x, size_t rows, int C, float eps, float* stats, long long run) {
   L.begin(KC_BN_STATS, (double)rows * C * sizeof(T), 3.0 * rows * C);
-  L.note(launch_bn_stats<T>(L.st, x, rows, C, eps, stats, m.scratch, m.counter, run >= 0 ? m.running + run : nullptr, kBnMomentum));
-  ++L.c->launches;
+  L.note(launch_bn_stats<T>(L.st, x, rows, C, eps, stats, m.scratch, run >= 0 ? m.running + run : nullptr, kBnMomentum));
+  L.c->launches += 2;
 }
 
 // `nparts` > 0: the statistics are not in `stats` yet; the convolution that produced x left nparts
@@ -611,17 +607,17 @@ static void bn_backward(Launch& L, Module& m, const T* dy, const GateOf<T> mask,
                         const float* gamma2, float* dgamma2, float* dbeta2, const T* res, T* dx, T* dx2,
                         size_t rows, int C, int nparts = 0) {
   const bool two = x2 != nullptr;
-  const bool sums_ready = nparts > 0;    // the kernel that produced dy left nparts rows of partial sums in m.red_partial
-  if (!sums_ready) {
+  const float* rows_of_sums = m.red_partial;  // nparts > 0: the kernel that produced dy left its rows of partial sums there
+  if (nparts <= 0) {
     L.begin(KC_BN_BWD_REDUCE, (double)rows * C * sizeof(T) * (2 + (mask.bits ? 0.0625 : mask.tensor ? 1 : 0) + (two ? 1 : 0)), 8.0 * rows * C);
     L.note(launch_bn_bwd_reduce<T>(L.st, dy, mask, x, stats, x2, stats2, rows, C, m.bnsums, dgamma, dbeta, dgamma2, dbeta2,
-                                   m.scratch, m.counter));
-    ++L.c->launches;
+                                   m.scratch, &nparts, &L.c->launches));
+    rows_of_sums = m.scratch;
   }
   const size_t n = rows * C;
   L.begin(KC_BN_BWD_APPLY, (double)n * sizeof(T) * (3 + (mask.bits ? 0.0625 : mask.tensor ? 1 : 0) + (two ? 2 : 0) + (res ? 1 : 0)), 10.0 * n);
   L.note(launch_bn_bwd_apply<T>(L.st, dy, mask, x, stats, gamma, m.bnsums, x2, stats2, gamma2, res, dx, dx2, rows, C,
-                                sums_ready ? m.red_partial : nullptr, nparts, dgamma, dbeta, L.c->ew_block_cap));
+                                nparts > 0 ? rows_of_sums : nullptr, nparts, dgamma, dbeta, L.c->ew_block_cap));
   ++L.c->launches;
 }
 
@@ -817,8 +813,7 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
           const RunningStats run{nxt->r1 >= 0 ? m.running + nxt->r1 : nullptr, kBnMomentum,
                                  rows_out > 1 ? (float)((double)rows_out / (double)(rows_out - 1)) : 1.f};
           L.begin(KC_BN_STATS, 8.0 * x_np * u.co, 2.0 * x_np * u.co);
-          L.note(launch_chained(stats_finalize_kernel, dim3((unsigned)((u.co + 31) / 32)), dim3(256), 0, L.st, (const float*)m.red_partial,
-                                x_np, u.co, 1.0 / (double)rows_out, eps, F + nxt->st1, run));
+          L.note(launch_stats_finalize(L.st, m.red_partial, x_np, rows_out, u.co, eps, F + nxt->st1, run));
           ++c->launches;
           x_np = -1;
         }
