@@ -239,11 +239,9 @@ inline cudaError_t run_wgrad_halo(cudaStream_t st, TensorMapCache* cache, int N,
   if (e != cudaSuccess) return e;
   const size_t n = (size_t)Co * 9 * Ci;
   if (n >= ((size_t)1 << 17) && ctas <= 8)        // large filters, few partials: four outputs per thread, partials in turn
-    wide::wgrad_wide_sum_kernel<<<(unsigned)((n / 4 + 255) / 256), 256, 0, st>>>(reinterpret_cast<const float4*>(scratch),
-                                                                               reinterpret_cast<float4*>(dw), n / 4, ctas);
-  else
-    halo::wgrad_halo_reduce_kernel<<<(int)((n + 31) / 32), 256, 0, st>>>(scratch, dw, n, ctas);
-  return cudaGetLastError();
+    return launch_chained(wide::wgrad_wide_sum_kernel, dim3((unsigned)((n / 4 + 255) / 256)), dim3(256), 0, st,
+                          reinterpret_cast<const float4*>(scratch), reinterpret_cast<float4*>(dw), n / 4, ctas);
+  return launch_chained(halo::wgrad_halo_reduce_kernel, dim3((unsigned)((n + 31) / 32)), dim3(256), 0, st, (const float*)scratch, dw, n, ctas);
 }
 
 // The same contract for wide layers and 1x1 filters (wide::wgrad_wide_kernel; scratch of wide::wide_scratch_elems

@@ -744,9 +744,12 @@ __global__ void __launch_bounds__(256) wgrad_halo_reduce_kernel(const float* __r
   __shared__ float part[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const size_t i = (size_t)blockIdx.x * 32 + lane;
+  grid_dependency_wait();                 // launched ahead of the end of the kernel that writes `partial`
   float a = 0.f;
-  if (i < n)
+  if (i < n) {
+#pragma unroll 4
     for (int z = warp; z < ctas; z += 8) a += partial[(size_t)z * n + i];
+  }
   part[warp][lane] = a;
   __syncthreads();
   if (warp == 0 && i < n) {

@@ -1307,7 +1307,10 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
   // 8 tiles per CTA: the four chains' convolutions then fit the SMs together and a CTA's start-up is paid once
   // per four tiles).
   c->tmaps.share = c->cfg.serial ? 1 : c->K;
-  c->tmaps.wgrad_side_cap = 16;
+  // A weight gradient on a side stream takes as many CTAs as give each four images (measured with the present data
+  // gradients: 16 / 24 / 32 / 48 CTAs at batch 128: K = 2 1228 / 1148 / 1091 / 1085 us per ResNet-56 iteration, K = 4
+  // 1580 / 1505 / 1484 / 1498 us per ResNet-110 iteration; at batch 64 16 CTAs are the best by 1 %).
+  c->tmaps.wgrad_side_cap = std::max(16, (c->arch.batch + 3) / 4);
   // Blocks of a batch-norm apply kernel that first re-adds a convolution's partial sums: 4 per SM shared
   // between the module streams, not fewer than 222 (measured: 222 blocks at K = 4 against 74 / 111 / 148 / 185 /
   // 259 / 296; K = 2 is flat between 222 and 592).
