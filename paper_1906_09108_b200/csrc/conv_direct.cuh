@@ -77,7 +77,8 @@ template <typename T> struct Reduce {
 template <typename T, int VEC, int STRIDE, int NC, bool FLIP>
 __global__ void __launch_bounds__(kThreads, 2)
 direct_conv_kernel(ConvParams p, const T* __restrict__ act, const T* __restrict__ wgt, T* __restrict__ out,
-                   const T* __restrict__ res, const T* __restrict__ res_mask, Reduce<T> red) {
+                   const T* __restrict__ res, const T* __restrict__ res_mask, Reduce<T> red, EpiAffine aff) {
+  grid_dependency_wait();
   extern __shared__ __align__(16) float dc_smem[];
   float* sa = dc_smem;                                       // [kKc][plane]
   float* sw = dc_smem + kKc * p.plane;                       // [kKc][9][cb]
@@ -253,6 +254,15 @@ direct_conv_kernel(ConvParams p, const T* __restrict__ act, const T* __restrict_
           if (j >= live) break;
           float v[4] = {acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]};
           const bool vec = p.vec != 0;
+          if (aff.stats) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              if (j + e >= live) break;
+              const int c = c0 + j + e;
+              const float x = to_f(from_f<T>(v[e])) - aff.stats[c], g = aff.gamma[c], iv = aff.stats[p.Cn + c];
+              v[e] = sizeof(T) == 4 ? g * (x * iv) + aff.beta[c] : fmaf(x, g * iv, aff.beta[c]);
+            }
+          }
           if (res) {
             float rv[4], mv[4] = {1.f, 1.f, 1.f, 1.f};
             if (vec) load4<T, 4>(res + base + j, 4, rv); else load4<T, 1>(res + base + j, live - j, rv);
@@ -262,7 +272,7 @@ direct_conv_kernel(ConvParams p, const T* __restrict__ act, const T* __restrict_
           }
           T o[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) o[e] = from_f<T>(v[e]);
+          for (int e = 0; e < 4; ++e) o[e] = from_f<T>(aff.relu ? fmaxf(v[e], 0.f) : v[e]);
           if (vec) {
             if constexpr (sizeof(T) == 4) *reinterpret_cast<float4*>(out + base + j) = *reinterpret_cast<const float4*>(o);
             else *reinterpret_cast<uint2*>(out + base + j) = *reinterpret_cast<const uint2*>(o);
@@ -366,7 +376,7 @@ constexpr size_t kConvSmemMax = 160 * 1024;
 
 template <typename T, int VEC, int STRIDE, int NC, bool FLIP>
 inline cudaError_t conv_launch_one(cudaStream_t st, const ConvParams& p, int grid, const T* act, const T* wgt, T* out,
-                                   const T* res, const T* mask, const Reduce<T>& red) {
+                                   const T* res, const T* mask, const Reduce<T>& red, const EpiAffine& aff) {
   auto kernel = direct_conv_kernel<T, VEC, STRIDE, NC, FLIP>;
   static bool set = false;                                   // raised once; a launch may be a recorded one
   if (!set) {
@@ -374,15 +384,15 @@ inline cudaError_t conv_launch_one(cudaStream_t st, const ConvParams& p, int gri
     if (e != cudaSuccess) return e;
     set = true;
   }
-  kernel<<<dim3(grid, (p.Cn + p.cb - 1) / p.cb), kThreads, conv_smem_bytes(p), st>>>(p, act, wgt, out, res, mask, red);
-  return cudaGetLastError();
+  return launch_chained(kernel, dim3(grid, (p.Cn + p.cb - 1) / p.cb), dim3(kThreads), conv_smem_bytes(p), st, p, act, wgt, out, res, mask, red, aff);
 }
 
 // y = conv3x3(x, w) [+ res], or (dgrad) dx = conv^T(dy, w) [+ res * [mask > 0]].  `red` (nullable) asks for the rows of
 // sums described at Reduce, *nparts receives their number.
 template <typename T>
 inline cudaError_t launch_conv(cudaStream_t st, const ConvGeom& g, bool dgrad, const T* act, const T* wgt, T* out, const T* res,
-                               const T* mask, const Reduce<T>* red, int* nparts, uint64_t* launches) {
+                               const T* mask, const Reduce<T>* red, int* nparts, uint64_t* launches,
+                               const EpiAffine* affine = nullptr) {
   // With 8 channels per thread 8 shared-memory loads serve 96 multiply-adds, with 4 channels 5 serve 48; 4 where 8 would
   // leave an SM fewer than four warps.  (Packed two-wide multiply-adds were tried: the moves that form their operand
   // pairs go through the same pipe, no gain.)
@@ -400,9 +410,10 @@ inline cudaError_t launch_conv(cudaStream_t st, const ConvGeom& g, bool dgrad, c
   const bool vec = p.Ck % 4 == 0 && (reinterpret_cast<uintptr_t>(act) & 15) == 0;
   Reduce<T> r{};
   if (red) r = *red;
+  const EpiAffine a = affine ? *affine : EpiAffine{};
   if (nparts) *nparts = red ? grid : 0;
   ++*launches;
-#define FDG_DC(V, S, C, F) return conv_launch_one<T, V, S, C, F>(st, p, grid, act, wgt, out, res, mask, r)
+#define FDG_DC(V, S, C, F) return conv_launch_one<T, V, S, C, F>(st, p, grid, act, wgt, out, res, mask, r, a)
   if (dgrad) {
     if (vec) { if (wide) FDG_DC(4, 1, 8, true); FDG_DC(4, 1, 4, true); }
     if (wide) FDG_DC(1, 1, 8, true);
@@ -434,6 +445,7 @@ struct WgradParams {
 template <typename T, int VECX, int VECY, int R, int STRIDE>
 __global__ void __launch_bounds__(kThreads)
 direct_wgrad_kernel(WgradParams p, const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ partial) {
+  grid_dependency_wait();
   constexpr int PAD = R == 3 ? 1 : 0;
   extern __shared__ __align__(16) float dw_smem[];
   float* sx = dw_smem;                                       // [rows_x][W + 2 * PAD][cib], rows padded to xrow
@@ -628,8 +640,7 @@ inline cudaError_t wgrad_launch_one(cudaStream_t st, const WgradParams& p, const
     set = true;
   }
   const int pairs = p.ci_blocks * ((p.Co + p.cob - 1) / p.cob);
-  kernel<<<dim3(p.splits, pairs), p.threads, wgrad_smem_bytes(p, R), st>>>(p, x, dy, dst);
-  return cudaGetLastError();
+  return launch_chained(kernel, dim3(p.splits, pairs), dim3(p.threads), wgrad_smem_bytes(p, R), st, p, x, dy, dst);
 }
 
 // dw [Co][R][R][Ci] (fp32) from x and dy; `scratch` of wgrad_direct_scratch_elems floats.

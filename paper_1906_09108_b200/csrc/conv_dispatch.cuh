@@ -43,7 +43,7 @@ inline bool tc_eligible(const ConvGeom& g) {
 inline cudaError_t run_conv_tc(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int Ck, int Cn,
                                const bf16_t* act, const bf16_t* wgt, bf16_t* out, const bf16_t* res,
                                const bf16_t* res_mask, int* err_dev, int sub = 1, int taps = 9, int act_sub = 1,
-                               float* stat_partial = nullptr, int* ctas_out = nullptr) {
+                               float* stat_partial = nullptr, int* ctas_out = nullptr, const EpiAffine* affine = nullptr) {
   if (cache->sm_count == 0) {
     int dev = 0;
     cudaGetDevice(&dev);
@@ -64,7 +64,7 @@ inline cudaError_t run_conv_tc(cudaStream_t st, TensorMapCache* cache, int N, in
     ia = cache->maps.insert({ka, ma}).first;
     ib = cache->maps.insert({kb, mb}).first;
   }
-  return tc::conv_tc_launch(st, p, ia->second, ib->second, out, res, res_mask, err_dev, cache->sm_count, stat_partial, ctas_out);
+  return tc::conv_tc_launch(st, p, ia->second, ib->second, out, res, res_mask, err_dev, cache->sm_count, stat_partial, ctas_out, affine);
 }
 
 
@@ -195,13 +195,15 @@ inline cudaError_t cached_group_map(TensorMapCache* cache, const void* t, int N,
 }
 inline cudaError_t run_conv_rows(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int C, const bf16_t* act,
                                  const bf16_t* wgt, bf16_t* out, const bf16_t* res, const bf16_t* res_mask,
-                                 const unsigned char* res_bits, int* err_dev, const halo::EpiReduce* red, int* ctas_out) {
+                                 const unsigned char* res_bits, int* err_dev, const halo::EpiReduce* red, int* ctas_out,
+                                 const EpiAffine* affine = nullptr) {
   int sms = cached_sm_count(cache) / (cache->share > 0 ? cache->share : 1);
   if (sms < 16) sms = 16;
   // the fewest CTAs that keep the number of images of the busiest one at ceil(N / sms)
   const int per_cta = (N + sms - 1) / sms, grid = (N + per_cta - 1) / per_cta;
   rows::EpiParams e{};
-  const int mode = red ? red->mode : 0;
+  const int mode = affine ? 3 : (red ? red->mode : 0);
+  if (affine) e.affine = *affine;
   e.res_gate = rows::Gate{res_bits, res_bits ? nullptr : res_mask};
   if (red) {
     e.gate = rows::Gate{red->mask_bits, red->mask_bits ? nullptr : red->mask};
@@ -234,8 +236,8 @@ inline cudaError_t run_wgrad_halo(cudaStream_t st, TensorMapCache* cache, int N,
   if (e == cudaSuccess) e = halo::set_smem_attrs();
   if (e != cudaSuccess) return e;
   const int ctas = halo::wgrad_ctas(p, side ? cache->wgrad_side_cap : 0);
-  halo::wgrad_halo_kernel<<<dim3(ctas, halo::wgrad_pairs(p)), halo::kFwdThreads, halo::wgrad_smem_bytes(p), st>>>(*mx, *my, p, scratch, err_dev);
-  e = cudaGetLastError();
+  e = launch_chained(halo::wgrad_halo_kernel, dim3(ctas, halo::wgrad_pairs(p)), dim3(halo::kFwdThreads), halo::wgrad_smem_bytes(p), st,
+                     *mx, *my, p, scratch, err_dev);
   if (e != cudaSuccess) return e;
   const size_t n = (size_t)Co * 9 * Ci;
   if (n >= ((size_t)1 << 17) && ctas <= 8)        // large filters, few partials: four outputs per thread, partials in turn
@@ -271,9 +273,8 @@ inline cudaError_t run_wgrad_wide(cudaStream_t st, TensorMapCache* cache, int N,
   if (e == cudaSuccess) e = wide::wide_set_attrs();
   if (e != cudaSuccess) return e;
   const dim3 grid(p.co_blocks * p.ci_chunks * p.rdim, p.splits);
-  if (R == 3) wide::wgrad_wide_kernel<3><<<grid, wide::kWideThreads, wide::wide_smem_bytes(p), st>>>(*mx, *my, p, scratch, err_dev);
-  else wide::wgrad_wide_kernel<1><<<grid, wide::kWideThreads, wide::wide_smem_bytes(p), st>>>(*mx, *my, p, scratch, err_dev);
-  e = cudaGetLastError();
+  auto kernel = R == 3 ? wide::wgrad_wide_kernel<3> : wide::wgrad_wide_kernel<1>;
+  e = launch_chained(kernel, grid, dim3(wide::kWideThreads), wide::wide_smem_bytes(p), st, *mx, *my, p, scratch, err_dev);
   if (e != cudaSuccess) return e;
   const size_t n4 = (size_t)Co * R * R * Ci / 4;                 // Ci is a multiple of 8
   // the sum's launch overlaps the tail of the kernel above; it waits for that kernel before it reads
@@ -308,12 +309,13 @@ inline size_t conv_wgrad_scratch_elems(bool bf16_storage, const ConvGeom& g) {
 // most 128 channels, whole vectors), *nparts = 0 tells the caller they were not.
 template <typename T>
 inline cudaError_t cuda_core_conv(cudaStream_t st, const ConvGeom& g, bool dgrad, const T* act, const T* w, T* out, const T* res,
-                                  const T* mask, const direct::Reduce<T>* red, int* nparts, uint64_t* launches) {
+                                  const T* mask, const direct::Reduce<T>* red, int* nparts, uint64_t* launches,
+                                  const EpiAffine* affine = nullptr) {
   if (nparts) *nparts = 0;
   if (direct::conv_supported(g, dgrad)) {
     const int cn = dgrad ? g.Ci : g.Co;
     const bool sums = red && red->mode != 0 && cn % 4 == 0 && 2 * cn <= kEwThreads;
-    return direct::launch_conv<T>(st, g, dgrad, act, w, out, res, mask, sums ? red : nullptr, nparts, launches);
+    return direct::launch_conv<T>(st, g, dgrad, act, w, out, res, mask, sums ? red : nullptr, nparts, launches, affine);
   }
   if (dgrad) return launch_conv_simt<T, CONV_DGRAD>(st, g, act, w, out, nullptr, nullptr, res, mask, launches);
   return launch_conv_simt<T, CONV_FPROP>(st, g, act, w, out, nullptr, nullptr, res, mask, launches);
@@ -331,9 +333,8 @@ inline cudaError_t cuda_core_wgrad(cudaStream_t st, const ConvGeom& g, const T* 
 // dy [N][P][Q][Co] of a stride-2 convolution spread onto the even pixels of a zero [N][H][W][Co] tensor `up`.
 inline cudaError_t bf16_spread_dy(cudaStream_t st, const ConvGeom& g, const bf16_t* dy, bf16_t* up, uint64_t* launches) {
   const size_t nvec = (size_t)g.N * g.H * g.W * g.Co / 8;
-  upsample2_kernel<bf16_t, 8><<<ew_blocks(nvec), 256, 0, st>>>(dy, up, nvec, g.P, g.Q, g.Co);
   ++*launches;
-  return cudaGetLastError();
+  return launch_chained(upsample2_kernel<bf16_t, 8>, ew_blocks(nvec), 256, 0, st, dy, up, nvec, g.P, g.Q, g.Co);
 }
 
 // y = conv(x, w) [+ res].  `red` (mode 1) asks for the per-CTA sums of y and y^2; *nparts receives the number
@@ -359,15 +360,22 @@ inline cudaError_t finish_wide_stats(cudaStream_t st, const ConvGeom& g, const W
   return launch_stats_finalize(st, ws->partial, ctas, ws->rows, g.Co, ws->eps, ws->stats, run);
 }
 
+// Can the kernel this forward convolution takes apply a batch norm in its epilogue (`affine`)?
+inline bool bf16_fprop_affine_ok(const ConvGeom& g) {
+  if (rows_eligible(g)) return true;
+  if (halo_fprop_eligible(g) || halo_s2_fprop_eligible(g)) return false;
+  if (tc_eligible(g) || tc_s2_fprop_eligible(g) || tc_1x1_fprop_eligible(g)) return 3 * g.Co <= tc::kStatFloats;
+  return direct::conv_supported(g, false);
+}
 inline cudaError_t bf16_conv_fprop(cudaStream_t st, TensorMapCache* cache, const ConvGeom& g, const bf16_t* x,
                                    const bf16_t* w, bf16_t* y, const bf16_t* res, const halo::EpiReduce* red, int* nparts,
-                                   int* err_dev, uint64_t* launches, const WideStats* ws = nullptr) {
+                                   int* err_dev, uint64_t* launches, const WideStats* ws = nullptr, const EpiAffine* affine = nullptr) {
   if (nparts) *nparts = 0;
   if (rows_eligible(g)) {
     ++*launches;
     const bool fuse = red && red->mode == 1;
     int ctas = 0;
-    const cudaError_t e = run_conv_rows(st, cache, g.N, g.H, g.W, g.Ci, x, w, y, res, nullptr, nullptr, err_dev, fuse ? red : nullptr, &ctas);
+    const cudaError_t e = run_conv_rows(st, cache, g.N, g.H, g.W, g.Ci, x, w, y, res, nullptr, nullptr, err_dev, fuse ? red : nullptr, &ctas, affine);
     if (fuse && nparts) *nparts = ctas;
     return e;
   }
@@ -387,7 +395,7 @@ inline cudaError_t bf16_conv_fprop(cudaStream_t st, TensorMapCache* cache, const
       const cudaError_t e = run_conv_tc(st, cache, g.N, g.H, g.W, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, g.stride, 9, 1, ws->partial, &ctas);
       return e != cudaSuccess ? e : finish_wide_stats(st, g, ws, ctas, nparts, launches);
     }
-    return run_conv_tc(st, cache, g.N, g.H, g.W, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, g.stride);
+    return run_conv_tc(st, cache, g.N, g.H, g.W, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, g.stride, 9, 1, nullptr, nullptr, affine);
   }
   if (tc_1x1_fprop_eligible(g)) {
     ++*launches;
@@ -396,10 +404,10 @@ inline cudaError_t bf16_conv_fprop(cudaStream_t st, TensorMapCache* cache, const
       const cudaError_t e = run_conv_tc(st, cache, g.N, g.P, g.Q, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, 1, 1, g.stride, ws->partial, &ctas);
       return e != cudaSuccess ? e : finish_wide_stats(st, g, ws, ctas, nparts, launches);
     }
-    return run_conv_tc(st, cache, g.N, g.P, g.Q, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, 1, 1, g.stride);
+    return run_conv_tc(st, cache, g.N, g.P, g.Q, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, 1, 1, g.stride, nullptr, nullptr, affine);
   }
   const direct::Reduce<bf16_t> r = red ? direct::Reduce<bf16_t>{red->mode, nullptr, nullptr, nullptr, red->partial} : direct::Reduce<bf16_t>{};
-  return cuda_core_conv(st, g, false, x, w, y, res, (const bf16_t*)nullptr, red ? &r : nullptr, nparts, launches);
+  return cuda_core_conv(st, g, false, x, w, y, res, (const bf16_t*)nullptr, red ? &r : nullptr, nparts, launches, affine);
 }
 
 // dx = conv^T(dy, w) [+ res * [mask > 0]].  `wflip` is the flipped/transposed weight copy (null: CUDA cores);

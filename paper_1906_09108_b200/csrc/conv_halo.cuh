@@ -619,6 +619,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     mbar_init(done, kMmaWarps);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    grid_dependency_wait();               // this thread alone reads what earlier kernels wrote (by TMA)
     // the producer's first pair of tiles, requested during set-up (they do not touch the slack cleared below)
     mbar_expect_tx(&full[0], p.x_tx_bytes + p.y_tx_bytes);
     tma_load_4d(smem, &map_x, &full[0], chunk_a * p.kcx, -1, -1, (int)blockIdx.x * p.G);
@@ -691,6 +692,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     // items are dealt to the groups in turn.
     const int lane_grp = warp & 3;
     const int group = (warp - kFirstEpiWarp) >> 2;
+    grid_dependency_wait();               // the partial sums of the launch before may still be being added up
     if (mbar_wait(done, 0, abort_flag)) {
       tc_fence_after();
       const int row = lane_grp * 32 + lane;

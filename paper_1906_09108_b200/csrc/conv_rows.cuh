@@ -56,8 +56,10 @@ struct Gate {
   const unsigned char* bits;
   const __nv_bfloat16* tensor;
 };
-// Sums an epilogue forms (template parameter MODE): 0 none, 1 sum v, sum v^2, 2 sum dz, sum dz * xhat with dz = v * [gate].
+// What an epilogue does besides (template parameter MODE): 0 nothing; sums: 1 sum v, sum v^2, 2 sum dz, sum dz * xhat with
+// dz = v * [gate]; 3 the batch norm that follows, with given statistics (inference), before the residual.
 struct EpiParams {
+  EpiAffine affine;           // MODE 3
   Gate res_gate;              // residual counts where the gate is set (both null: everywhere)
   Gate gate;                  // MODE 2
   const float* pstats;        // MODE 2: mean[C], invstd[C]
@@ -184,7 +186,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tile_done + p.op_stages);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* sums = reinterpret_cast<float*>(tmem_slot + 4);        // [kEpiWarps][32]
-  float* mean = sums + kEpiWarps * 32;                          // [C], invstd [C]
+  float* mean = sums + kEpiWarps * 32;                          // [3][C]: mean, invstd (MODE 2); mean, gamma * invstd, beta
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int step = (int)gridDim.x;
@@ -299,13 +301,20 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     const int dr = row >> 3, dg = row & 7;
     const uint32_t o0 = ((col >> 3) ^ dg) << 4, o1 = (((col >> 3) + 1) ^ dg) << 4;   // its two 16-byte pieces of a swizzled line
     const uint32_t taddr = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)col;
-    if (MODE == 2) {
-      for (int i = threadIdx.x - 32 * kFirstEpi; i < 2 * C; i += 32 * kEpiWarps) mean[i] = e.pstats[i];
+    if (MODE >= 2) {
+      if (MODE == 2) {
+        for (int i = threadIdx.x - 32 * kFirstEpi; i < 2 * C; i += 32 * kEpiWarps) mean[i] = e.pstats[i];
+      } else {                                     // mean, gamma * invstd, beta
+        for (int i = threadIdx.x - 32 * kFirstEpi; i < C; i += 32 * kEpiWarps) {
+          mean[i] = e.affine.stats[i]; mean[C + i] = e.affine.gamma[i] * e.affine.stats[C + i]; mean[2 * C + i] = e.affine.beta[i];
+        }
+      }
       asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
     }
-    float run[MODE ? 32 : 1];
+    constexpr bool kSums = MODE == 1 || MODE == 2;
+    float run[kSums ? 32 : 1];
 #pragma unroll
-    for (int i = 0; i < (MODE ? 32 : 1); ++i) run[i] = 0.f;
+    for (int i = 0; i < (kSums ? 32 : 1); ++i) run[i] = 0.f;
     Walk wk((int)blockIdx.x);
     for (int t = 0; t < tiles; ++t, wk.next(p, step)) {
       const int h = wk.rbk * kTileRows + dr, g = wk.cbk * kTileGroups + dg;
@@ -339,6 +348,12 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[wk.slot]);                 // the values are in registers
+      if (MODE == 3) {                             // on the value as it would have been stored: bn_apply_kernel's result
+        const float* mu = mean + c0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          v[q] = __float_as_uint(fmaf(__bfloat162float(__float2bfloat16_rn(__uint_as_float(v[q]))) - mu[q], mu[C + q], mu[2 * C + q]));
+      }
       if (RES) {
         const uint32_t rw[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
 #pragma unroll
@@ -346,6 +361,10 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
           v[2 * q] = __float_as_uint(__uint_as_float(v[2 * q]) + ((rm & (1u << (2 * q))) ? bf_lo(rw[q]) : 0.f));
           v[2 * q + 1] = __float_as_uint(__uint_as_float(v[2 * q + 1]) + ((rm & (2u << (2 * q))) ? bf_hi(rw[q]) : 0.f));
         }
+      }
+      if (MODE == 3 && e.affine.relu) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = __float_as_uint(fmaxf(__uint_as_float(v[q]), 0.f));
       }
       uint32_t y[8];
 #pragma unroll
@@ -376,7 +395,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         }
       }
     }
-    if constexpr (MODE != 0) {
+    if constexpr (kSums) {
       transpose_reduce32(run, lane);               // lane l: item l of this warp's 32 rows (channel l % 16, sum l / 16)
       sums[(warp - kFirstEpi) * 32 + lane] = run[0];
     }
@@ -401,7 +420,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     tc_fence_after();
     tmem_dealloc(tmem_base, kAccSlots * 64);
   }
-  if (MODE && !*abort_flag) {
+  if ((MODE == 1 || MODE == 2) && !*abort_flag) {
     // this CTA's sums, warps in order: the warps of group q hold the 16 channels from (16 * q) % C
     for (int i = threadIdx.x; i < 2 * C; i += kThreads) {
       const int stat = i / C, c = i - stat * C, item = (c & 15) + 16 * stat;
@@ -421,7 +440,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 // ----------------------------------------------------------------- host side ---
 constexpr size_t kSmemLimit = 226 * 1024;
 inline size_t fixed_smem(int a_stages, int op_stages) {
-  return (size_t)(2 * a_stages + 1 + 2 * kAccSlots + 2 * op_stages) * 8 + 16 + (size_t)kEpiWarps * 32 * 4 + 2 * 64 * 4 + 1024;
+  return (size_t)(2 * a_stages + 1 + 2 * kAccSlots + 2 * op_stages) * 8 + 16 + (size_t)kEpiWarps * 32 * 4 + 3 * 64 * 4 + 1024;
 }
 // `per_cta` images per CTA at most, `n_ops` operand tiles; a_stages = 0 where the shape is not covered.
 inline RowsParams rows_params(int N, int H, int W, int C, int per_cta, int n_ops) {
@@ -480,6 +499,7 @@ inline cudaError_t make_group_map(const void* t, int N, int H, int W, int C, int
 typedef void (*RowsKernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, RowsParams, EpiParams, int*);
 template <int C> inline RowsKernel kernel_of(int mode, bool res) {
   if (mode == 1) return res ? conv_rows_kernel<C, 1, true> : conv_rows_kernel<C, 1, false>;
+  if (mode == 3) return res ? conv_rows_kernel<C, 3, true> : conv_rows_kernel<C, 3, false>;
   if (mode == 2) return res ? conv_rows_kernel<C, 2, true> : conv_rows_kernel<C, 2, false>;
   return res ? conv_rows_kernel<C, 0, true> : conv_rows_kernel<C, 0, false>;
 }
@@ -491,7 +511,7 @@ inline cudaError_t set_attrs() {
   static bool done = false;
   if (done) return cudaSuccess;
   for (int c = 16; c <= 64; c *= 2)
-    for (int mode = 0; mode < 3; ++mode)
+    for (int mode = 0; mode < 4; ++mode)
       for (int res = 0; res < 2; ++res) {
         const cudaError_t e = cudaFuncSetAttribute(kernel_of(c, mode, res != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
         if (e != cudaSuccess) return e;

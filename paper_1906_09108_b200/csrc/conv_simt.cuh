@@ -210,6 +210,7 @@ conv_simt_kernel(ConvGeom g, const T* __restrict__ act,      // FPROP/WGRAD: x ;
 
 // grad[i] = sum_z partial[z][i], z ascending.
 __global__ void wgrad_reduce_kernel(const float* __restrict__ partial, float* __restrict__ grad, size_t n, int splits) {
+  grid_dependency_wait();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     float a = 0.f;
     for (int z = 0; z < splits; ++z) a += partial[(size_t)z * n + i];
@@ -223,6 +224,7 @@ __global__ void wgrad_reduce_kernel(const float* __restrict__ partial, float* __
 __global__ void __launch_bounds__(512) wgrad_reduce_tall_kernel(const float* __restrict__ partial, float* __restrict__ grad,
                                                                 size_t n, int splits) {
   __shared__ float part[16][33];
+  grid_dependency_wait();
   const int col = threadIdx.x & 31, rg = threadIdx.x >> 5;
   const size_t i = (size_t)blockIdx.x * 32 + col;
   float a = 0.f;
@@ -242,12 +244,10 @@ __global__ void __launch_bounds__(512) wgrad_reduce_tall_kernel(const float* __r
 // grad = the sum of `splits` partial rows of n floats, on stream st.
 inline cudaError_t launch_wgrad_reduce(cudaStream_t st, const float* partial, float* grad, size_t n, int splits) {
   if (splits >= 32 && n <= (size_t)1 << 16) {
-    wgrad_reduce_tall_kernel<<<(unsigned)((n + 31) / 32), 512, 0, st>>>(partial, grad, n, splits);
-  } else {
-    int blocks = (int)((n + 255) / 256); if (blocks > 1184) blocks = 1184;
-    wgrad_reduce_kernel<<<blocks, 256, 0, st>>>(partial, grad, n, splits);
+    return launch_chained(wgrad_reduce_tall_kernel, dim3((unsigned)((n + 31) / 32)), dim3(512), 0, st, partial, grad, n, splits);
   }
-  return cudaGetLastError();
+  int blocks = (int)((n + 255) / 256); if (blocks > 1184) blocks = 1184;
+  return launch_chained(wgrad_reduce_kernel, blocks, 256, 0, st, partial, grad, n, splits);
 }
 
 // Number of pixel slices the weight-gradient GEMM is split into, and the slice length.

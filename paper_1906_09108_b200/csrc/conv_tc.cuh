@@ -27,6 +27,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "elementwise.cuh"
+
 namespace fdg {
 namespace tc {
 
@@ -226,12 +228,28 @@ __device__ __forceinline__ void stat_flush(const float* stat_run, float* __restr
   }
 }
 
+// The constants of a batch norm in the epilogue (EpiAffine), in the statistics' area (an inference pass forms none):
+// mean[Co], gamma * invstd [Co], beta[Co].
+__device__ __forceinline__ void affine_load(const EpiAffine& a, float* area, int Co) {
+  for (int c = threadIdx.x; c < Co; c += blockDim.x) {
+    area[c] = a.stats[c]; area[Co + c] = a.gamma[c] * a.stats[Co + c]; area[2 * Co + c] = a.beta[c];
+  }
+}
+// f[0..16) = the batch norm of the accumulator columns c .. c+15, rounded to bf16 first.
+__device__ __forceinline__ void affine_apply(const float* area, int Co, int c, float (&f)[16]) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    if (c + i >= Co) break;
+    f[i] = fmaf(__bfloat162float(__float2bfloat16_rn(f[i])) - area[c + i], area[Co + c + i], area[2 * Co + c + i]);
+  }
+}
+
 // ------------------------------------------------------------------- kernel ----
 // out[m][n] (bf16, row stride Co) = conv + (res ? res[m][n] * [mask ? mask[m][n] > 0 : 1] : 0)
 __global__ void __launch_bounds__(kThreads, 1)
 conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                   ConvTcParams p, __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ res,
-                  const __nv_bfloat16* __restrict__ res_mask, float* __restrict__ stat_partial, int* __restrict__ error_word) {
+                  const __nv_bfloat16* __restrict__ res_mask, float* __restrict__ stat_partial, EpiAffine aff, int* __restrict__ error_word) {
   __shared__ float stat_run[kStatFloats];
   if (stat_partial) for (int i = threadIdx.x; i < kStatFloats; i += blockDim.x) stat_run[i] = 0.f;
   extern __shared__ uint8_t smem_raw[];
@@ -256,6 +274,8 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();                  // from here on the preceding kernel's results may be read
+  if (aff.stats) { affine_load(aff, stat_run, p.Co); __syncthreads(); }
 
   const int chunks = (p.Ci + p.kc - 1) / p.kc;
   const int k_iters = p.taps * chunks;
@@ -383,6 +403,7 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         float f[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
+        if (aff.stats) affine_apply(stat_run, p.Co, nt * p.n_tile + c0, f);
         if (res && keep) {
           uint4 r0 = *reinterpret_cast<const uint4*>(res + base + c0);
           uint4 r1 = both ? *reinterpret_cast<const uint4*>(res + base + c0 + 8) : make_uint4(0, 0, 0, 0);
@@ -404,6 +425,10 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
           }
 #pragma unroll
           for (int i = 0; i < 16; ++i) f[i] += g[i];
+        }
+        if (aff.relu) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) f[i] = fmaxf(f[i], 0.f);
         }
         uint4 o0, o1;
         __nv_bfloat162* ob0 = reinterpret_cast<__nv_bfloat162*>(&o0);
@@ -464,7 +489,7 @@ constexpr int kPatchThreads = 224;       // TMA warp, issuing warp of tile 0, fo
 __global__ void __launch_bounds__(kPatchThreads, 1)
 conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                      ConvTcParams p, __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ res,
-                     const __nv_bfloat16* __restrict__ res_mask, float* __restrict__ stat_partial, int* __restrict__ error_word) {
+                     const __nv_bfloat16* __restrict__ res_mask, float* __restrict__ stat_partial, EpiAffine aff, int* __restrict__ error_word) {
   __shared__ float stat_run[kStatFloats];
   if (stat_partial) for (int i = threadIdx.x; i < kStatFloats; i += blockDim.x) stat_run[i] = 0.f;
   extern __shared__ uint8_t smem_raw[];
@@ -493,6 +518,8 @@ conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();                  // from here on the preceding kernel's results may be read
+  if (aff.stats) { affine_load(aff, stat_run, p.Co); __syncthreads(); }
 
   const int chunks = (p.Ci + p.kc - 1) / p.kc;
   const int pw_cnt = p.W / kPatch, ph_cnt = p.H / kPatch;
@@ -621,6 +648,7 @@ conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
           float f[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e) f[e] = __uint_as_float(v[e]);
+          if (aff.stats) affine_apply(stat_run, p.Co, nt * p.n_tile + c0, f);
           if (res && keep) {
             uint4 r0 = *reinterpret_cast<const uint4*>(res + base + c0);
             uint4 r1 = both ? *reinterpret_cast<const uint4*>(res + base + c0 + 8) : make_uint4(0, 0, 0, 0);
@@ -642,6 +670,10 @@ conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             }
 #pragma unroll
             for (int e = 0; e < 16; ++e) f[e] += gq[e];
+          }
+          if (aff.relu) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) f[e] = fmaxf(f[e], 0.f);
           }
           uint4 o0, o1;
           __nv_bfloat162* ob0 = reinterpret_cast<__nv_bfloat162*>(&o0);
@@ -828,7 +860,8 @@ inline cudaError_t conv_tc_set_attrs() {
 inline cudaError_t conv_tc_launch(cudaStream_t st, const ConvTcParams& p, const CUtensorMap& map_a,
                                   const CUtensorMap& map_b, __nv_bfloat16* out, const __nv_bfloat16* res,
                                   const __nv_bfloat16* res_mask, int* error_word, int sm_count,
-                                  float* stat_partial = nullptr, int* ctas_out = nullptr) {
+                                  float* stat_partial = nullptr, int* ctas_out = nullptr, const EpiAffine* affine = nullptr) {
+  const EpiAffine aff = affine ? *affine : EpiAffine{};
   const size_t smem = conv_tc_smem_bytes(p);
   {
     cudaError_t e = conv_tc_set_attrs();
@@ -838,14 +871,12 @@ inline cudaError_t conv_tc_launch(cudaStream_t st, const ConvTcParams& p, const 
     const int tiles = p.N * (p.H / kPatch) * (p.W / kPatch) * p.n_tiles;
     const int grid = tiles < sm_count ? tiles : sm_count;
     if (ctas_out) *ctas_out = grid;
-    conv3x3_patch_kernel<<<grid, kPatchThreads, smem, st>>>(map_a, map_b, p, out, res, res_mask, stat_partial, error_word);
-    return cudaGetLastError();
+    return launch_chained(conv3x3_patch_kernel, grid, kPatchThreads, smem, st, map_a, map_b, p, out, res, res_mask, stat_partial, aff, error_word);
   }
   const int tiles = ((p.m_tiles + p.mpair - 1) / p.mpair) * p.n_tiles;
   const int grid = tiles < sm_count ? tiles : sm_count;
   if (ctas_out) *ctas_out = grid;
-  conv3x3_tc_kernel<<<grid, kThreads, smem, st>>>(map_a, map_b, p, out, res, res_mask, stat_partial, error_word);
-  return cudaGetLastError();
+  return launch_chained(conv3x3_tc_kernel, grid, kThreads, smem, st, map_a, map_b, p, out, res, res_mask, stat_partial, aff, error_word);
 }
 
 // Probe of the tensor pipe's instruction rate, for the roofline arguments about the kernels above: one thread of one
@@ -978,6 +1009,7 @@ __device__ __forceinline__ void wflip_entry(const __nv_bfloat16* __restrict__ sr
 }
 __global__ void __launch_bounds__(256) wflip_kernel(const __nv_bfloat16* __restrict__ src_base, __nv_bfloat16* __restrict__ dst_base,
                                                     const FlipEntry* __restrict__ table) {
+  grid_dependency_wait();
   __shared__ __align__(16) __nv_bfloat16 tile[64][66];
   wflip_entry(src_base, dst_base, table[blockIdx.y], tile);
 }

@@ -37,6 +37,16 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// A batch norm with given statistics (inference) applied in the epilogue of the convolution that produces its input:
+// the convolution's output is rounded to the storage type first, as if it had been stored, so that the result is that of
+// bn_apply_kernel bit for bit.  stats null: none.
+struct EpiAffine {
+  const float* stats;       // mean[C], invstd[C]
+  const float* gamma;
+  const float* beta;
+  int relu;
+};
+
 // ---------------------------------------------------------------- helpers ---
 template <typename T> struct Vec;   // 16-byte vector of T
 template <> struct Vec<float> {
@@ -581,6 +591,7 @@ bn_bwd_apply_kernel(const T* __restrict__ dy, const GateOf<T> gate, const T* __r
 // out = scale * in  (the gradient-shrinking step, Eq. 15).
 template <typename T, int VEC>
 __global__ void scale_kernel(const T* __restrict__ in, T* __restrict__ out, float scale, size_t nvec) {
+  grid_dependency_wait();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
     float v[VEC];
     load_vec<T, VEC>(in + i * VEC, v);
@@ -606,6 +617,7 @@ __global__ void add_kernel(const T* __restrict__ a, const T* __restrict__ b, T* 
 // up[n][2p][2q][:] = dy[n][p][q][:], zero at the other pixels; dy [N][P][Q][C], up [N][2P][2Q][C], 16-byte vectors.
 template <typename T, int VEC>
 __global__ void upsample2_kernel(const T* __restrict__ dy, T* __restrict__ up, size_t nvec_up, int P, int Q, int C) {
+  grid_dependency_wait();
   const int cv = C / VEC;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nvec_up; i += (size_t)gridDim.x * blockDim.x) {
     const int c = (int)(i % cv);
@@ -625,6 +637,7 @@ __global__ void upsample2_kernel(const T* __restrict__ dy, T* __restrict__ up, s
 template <typename T>
 __global__ void pad_shortcut_kernel(const T* __restrict__ x, T* __restrict__ out, size_t rows_out, int P, int Q, int H, int W,
                                     int Ci, int Co, int stride) {
+  grid_dependency_wait();
   const int lo = (Co - Ci) / 2;
   const size_t n = rows_out * (size_t)Co;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -641,6 +654,7 @@ __global__ void pad_shortcut_kernel(const T* __restrict__ x, T* __restrict__ out
 template <typename T>
 __global__ void pad_shortcut_bwd_kernel(const T* __restrict__ dy, const T* __restrict__ y, T* __restrict__ dx, size_t rows_in,
                                         int P, int Q, int H, int W, int Ci, int Co, int stride) {
+  grid_dependency_wait();
   const int lo = (Co - Ci) / 2;
   const size_t n = rows_in * (size_t)Ci;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -662,6 +676,7 @@ __global__ void pad_shortcut_bwd_kernel(const T* __restrict__ dy, const T* __res
 template <typename T>
 __global__ void ingest_kernel(const float* __restrict__ img, T* __restrict__ out, size_t rows, int c_in, int c_out,
                               const int32_t* __restrict__ labels_in, int32_t* __restrict__ labels_out, int batch) {
+  grid_dependency_wait();
   const size_t n = rows * (size_t)c_out;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const size_t row = i / c_out;
@@ -697,6 +712,7 @@ __global__ void head_fwd_bwd_kernel(const T* __restrict__ x, const float* __rest
                                     const int32_t* __restrict__ labels, int HW, int F, int classes, int batch, int groups,
                                     float* __restrict__ pooled, float* __restrict__ dlogits,
                                     float* __restrict__ loss_n, T* __restrict__ dx, int* __restrict__ bad_label) {
+  grid_dependency_wait();
   constexpr int V = 16 / (int)sizeof(T);
   extern __shared__ __align__(16) float hs[];   // pooled[F] | dpooled[F] | partial[groups][F] | logits[classes]
   float* s_pool = hs;
@@ -820,6 +836,7 @@ __global__ void head_param_grad_kernel(const float* __restrict__ pooled, const f
                                        const float* __restrict__ loss_n, int F, int classes, int batch,
                                        float* __restrict__ dW, float* __restrict__ db, float* __restrict__ loss,
                                        int* __restrict__ nonfinite) {
+  grid_dependency_wait();
   __shared__ float s_part[4][32];
   const int c = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -861,15 +878,13 @@ inline cudaError_t launch_head(cudaStream_t st, const T* x, const float* w, cons
   if (first) {
     int groups = head_groups(F, classes, HW, sizeof(T));
     if ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dx)) & 15) groups = 0;   // vectors need 16-byte alignment
-    head_fwd_bwd_kernel<T><<<batch, kHeadThreads, head_smem_bytes(F, classes, groups), st>>>(
-        x, w, b, labels, HW, F, classes, batch, groups, pooled, dlogits, loss_n, dx, flags + 1);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(head_fwd_bwd_kernel<T>, batch, kHeadThreads, head_smem_bytes(F, classes, groups), st,
+                                         x, w, b, labels, HW, F, classes, batch, groups, pooled, dlogits, loss_n, dx, flags + 1);
     if (e != cudaSuccess) return e;
   }
   if (second) {
-    head_param_grad_kernel<<<dim3(classes, (F + 31) / 32), 128, 0, st>>>(pooled, dlogits, loss_n, F, classes, batch, dW, db,
-                                                                          loss, flags);
-    return cudaGetLastError();
+    return launch_chained(head_param_grad_kernel, dim3(classes, (F + 31) / 32), 128, 0, st, (const float*)pooled,
+                          (const float*)dlogits, (const float*)loss_n, F, classes, batch, dW, db, loss, flags);
   }
   return cudaSuccess;
 }
@@ -883,6 +898,7 @@ inline cudaError_t launch_head(cudaStream_t st, const T* x, const float* w, cons
 __global__ void sgd_kernel(float* __restrict__ theta, float* __restrict__ v, const float* __restrict__ g,
                            float* __restrict__ next32, __nv_bfloat16* __restrict__ next16, size_t n, float lr,
                            const float* __restrict__ lr_dev, float mu, float wd) {
+  grid_dependency_wait();
   if (lr_dev) lr = *lr_dev;
   const size_t n4 = n / 4;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
@@ -929,6 +945,7 @@ __global__ void cast_kernel(const float* __restrict__ in, T* __restrict__ out, s
 struct EvalStatEntry { size_t roff, soff; int C; };
 __global__ void bn_eval_stats_kernel(const float* __restrict__ running, float* __restrict__ out,
                                      const EvalStatEntry* __restrict__ table, float eps) {
+  grid_dependency_wait();
   const EvalStatEntry e = table[blockIdx.x];
   for (int c = threadIdx.x; c < e.C; c += blockDim.x) {
     out[e.soff + c] = running[e.roff + c];
@@ -942,6 +959,7 @@ template <typename T>
 __global__ void head_eval_kernel(const T* __restrict__ x, const float* __restrict__ w, const float* __restrict__ b,
                                  const int32_t* __restrict__ labels, int HW, int F, int classes,
                                  float* __restrict__ logits_out, int* __restrict__ correct) {
+  grid_dependency_wait();
   extern __shared__ float hs[];            // pooled[F] | logits[classes]
   float* s_pool = hs;
   float* s_logit = hs + F;
@@ -1093,24 +1111,21 @@ inline cudaError_t launch_bn_bwd_apply(cudaStream_t st, const T* dy, const GateO
 template <typename T>
 inline cudaError_t launch_scale(cudaStream_t st, const T* in, T* out, float s, size_t n) {
   constexpr int V = full_vec<T>();
-  if (n % V == 0) scale_kernel<T, V><<<ew_blocks(n / V), 256, 0, st>>>(in, out, s, n / V);
-  else scale_kernel<T, 1><<<ew_blocks(n), 256, 0, st>>>(in, out, s, n);
-  return cudaGetLastError();
+  if (n % V == 0) return launch_chained(scale_kernel<T, V>, ew_blocks(n / V), 256, 0, st, in, out, s, n / V);
+  return launch_chained(scale_kernel<T, 1>, ew_blocks(n), 256, 0, st, in, out, s, n);
 }
 
 inline cudaError_t launch_sgd(cudaStream_t st, float* theta, float* v, const float* g, float* next32,
                               __nv_bfloat16* next16, size_t n, float lr, const float* lr_dev, float mu, float wd) {
   size_t b = (n / 4 + 255) / 256;
   const int blocks = (int)(b < 1 ? 1 : (b > 148 * 8 ? 148 * 8 : b));
-  sgd_kernel<<<blocks, 256, 0, st>>>(theta, v, g, next32, next16, n, lr, lr_dev, mu, wd);
-  return cudaGetLastError();
+  return launch_chained(sgd_kernel, blocks, 256, 0, st, theta, v, g, next32, next16, n, lr, lr_dev, mu, wd);
 }
 
 template <typename T>
 inline cudaError_t launch_ingest(cudaStream_t st, const float* img, T* out, size_t rows, int c_in, int c_out,
                                  const int32_t* labels_in, int32_t* labels_out, int batch) {
-  ingest_kernel<T><<<ew_blocks(rows * c_out), 256, 0, st>>>(img, out, rows, c_in, c_out, labels_in, labels_out, batch);
-  return cudaGetLastError();
+  return launch_chained(ingest_kernel<T>, ew_blocks(rows * c_out), 256, 0, st, img, out, rows, c_in, c_out, labels_in, labels_out, batch);
 }
 
 }  // namespace fdg

@@ -649,7 +649,7 @@ template <typename T>
 // a narrow layer), 0 when it formed none, or -1 when the statistics are already in `stats` (a wide layer, whose
 // totals are finalised right behind the convolution; needs `stats`, with `run` the running statistics' offset or -1).
 static int conv_fprop(Launch& L, Module& m, const ConvGeom& g, const T* x, const T* w, T* y, const T* res,
-                      bool want_stats = false, float* stats = nullptr, long long run = -1) {
+                      bool want_stats = false, float* stats = nullptr, long long run = -1, const EpiAffine* affine = nullptr) {
   L.begin(KC_CONV_FPROP, (in_elems(g) + w_elems(g) + out_elems(g) * (res ? 2 : 1)) * sizeof(T), conv_flops(g));
   int nparts = 0;
   if constexpr (std::is_same<T, bf16>::value) {
@@ -658,10 +658,10 @@ static int conv_fprop(Launch& L, Module& m, const ConvGeom& g, const T* x, const
     const WideStats ws{m.red_partial, m.red_partial_floats, stats, (size_t)g.N * g.P * g.Q, L.c->arch.bn_eps,
                        run >= 0 ? m.running + run : nullptr, kBnMomentum};
     L.note(bf16_conv_fprop(L.st, &L.c->tmaps, g, x, w, y, res, want_stats ? &r : nullptr, &nparts, L.c->tc_error, &L.c->launches,
-                           (want_stats && stats) ? &ws : nullptr));
+                           (want_stats && stats) ? &ws : nullptr, affine));
   } else {
     const direct::Reduce<T> r{1, nullptr, nullptr, nullptr, m.red_partial};
-    L.note(cuda_core_conv<T>(L.st, g, false, x, w, y, res, nullptr, want_stats ? &r : nullptr, &nparts, &L.c->launches));
+    L.note(cuda_core_conv<T>(L.st, g, false, x, w, y, res, nullptr, want_stats ? &r : nullptr, &nparts, &L.c->launches, affine));
   }
   return nparts;
 }
@@ -748,6 +748,15 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
   auto stats_of = [&](int np, const T* y, size_t rows, int C, float* stats, long long run) {
     if (!eval && np == 0) bn_stats<T>(L, m, y, rows, C, eps, stats, run);
   };
+  // Inference: a convolution and the batch norm + ReLU (+ residual) behind it as one kernel, where the convolution's kernel
+  // can apply it to the values it would otherwise store; false: the caller launches the two.
+  auto conv_bn_eval = [&](const ConvGeom& g, const T* in, const T* w, const float* st, const float* ga, const float* be, const T* res, T* y) {
+    const bool ok = eval && (std::is_same<T, bf16>::value ? bf16_fprop_affine_ok(g) : direct::conv_supported(g, false));
+    if (!ok) return false;
+    const EpiAffine a{st, ga, be, 1};
+    conv_fprop<T>(L, m, g, in, w, y, res, false, nullptr, -1, &a);
+    return true;
+  };
   int x_np = 0;     // -1: the statistics of x (the next pre-activation block's first batch norm) are already in place
   for (size_t ui = 0; ui < m.units.size(); ++ui) {
     const Unit& u = m.units[ui];
@@ -759,6 +768,7 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
     switch (u.type) {
       case U_STEM: {
         ConvGeom g = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, 1, 1);
+        if (u.bn && conv_bn_eval(g, x, wt + u.w1, F + u.st1, wf + u.g1, wf + u.b1, nullptr, S + u.t_y)) break;
         if (u.bn) {
           const int np = conv_fprop<T>(L, m, g, x, wt + u.w1, S + u.t_a, nullptr, !eval, F + u.st1, u.r1);
           stats_of(np, S + u.t_a, rows_out, u.co, F + u.st1, u.r1);
@@ -771,25 +781,30 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
       case U_BASIC: {
         ConvGeom g1 = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, u.stride, 1);
         ConvGeom g2 = geom(B, u.P, u.Q, u.co, u.P, u.Q, u.co, 3, 1, 1);
-        const int np1 = conv_fprop<T>(L, m, g1, x, wt + u.w1, S + u.t_a, nullptr, !eval, F + u.st1, u.r1);   // c1
-        stats_of(np1, S + u.t_a, rows_out, u.co, F + u.st1, u.r1);
-        bn_apply<T>(L, m, S + u.t_a, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_b, rows_out, u.co, np1, u.r1, gate_bits(u.q_b));  // a1
+        if (!conv_bn_eval(g1, x, wt + u.w1, F + u.st1, wf + u.g1, wf + u.b1, nullptr, S + u.t_b)) {
+          const int np1 = conv_fprop<T>(L, m, g1, x, wt + u.w1, S + u.t_a, nullptr, !eval, F + u.st1, u.r1);   // c1
+          stats_of(np1, S + u.t_a, rows_out, u.co, F + u.st1, u.r1);
+          bn_apply<T>(L, m, S + u.t_a, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_b, rows_out, u.co, np1, u.r1, gate_bits(u.q_b));  // a1
+        }
         if (u.proj) {          // shortcut first: its statistics must not disturb the partial sums conv2 leaves for BN2
           ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
           const int nps = conv_fprop<T>(L, m, gs, x, wt + u.ws, S + u.t_s, nullptr, !eval, F + u.sts, u.rs);   // cs
           stats_of(nps < 0 ? nps : 0, S + u.t_s, rows_out, u.co, F + u.sts, u.rs);
         }
+        const T* shortcut = x;
+        if (u.zpad) {          // the shortcut is x at every stride-th pixel between zero channels: built in a temporary
+          L.begin(KC_BN_APPLY, (double)rows_out * (u.ci + u.co) * sizeof(T), 0.0);
+          L.note(launch_chained(pad_shortcut_kernel<T>, ew_blocks(rows_out * u.co), 256, 0, L.st, x, tmp, rows_out, u.P, u.Q, u.H, u.W, u.ci, u.co, u.stride));
+          ++c->launches;
+          shortcut = tmp;
+        }
+        if (!u.proj && conv_bn_eval(g2, S + u.t_b, wt + u.w2, F + u.st2, wf + u.g2, wf + u.b2, shortcut, S + u.t_y)) break;
         const int np2 = conv_fprop<T>(L, m, g2, S + u.t_b, wt + u.w2, S + u.t_c, nullptr, !eval, F + u.st2, u.r2);   // c2
         stats_of(np2, S + u.t_c, rows_out, u.co, F + u.st2, u.r2);
         if (u.proj) {
           bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, S + u.t_s, F + u.sts, wf + u.gs, wf + u.bs, true, S + u.t_y, rows_out, u.co, np2, u.r2, gate_bits(u.q_y));
-        } else if (u.zpad) {   // the shortcut is x at every stride-th pixel between zero channels: built in a temporary
-          L.begin(KC_BN_APPLY, (double)rows_out * (u.ci + u.co) * sizeof(T), 0.0);
-          pad_shortcut_kernel<T><<<ew_blocks(rows_out * u.co), 256, 0, L.st>>>(x, tmp, rows_out, u.P, u.Q, u.H, u.W, u.ci, u.co, u.stride);
-          L.check();
-          bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, tmp, nullptr, nullptr, nullptr, true, S + u.t_y, rows_out, u.co, np2, u.r2, gate_bits(u.q_y));
         } else {
-          bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, x, nullptr, nullptr, nullptr, true, S + u.t_y, rows_out, u.co, np2, u.r2, gate_bits(u.q_y));
+          bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, shortcut, nullptr, nullptr, nullptr, true, S + u.t_y, rows_out, u.co, np2, u.r2, gate_bits(u.q_y));
         }
         break;
       }
@@ -799,9 +814,11 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
         stats_of(x_np, x, rows_in, u.ci, F + u.st1, u.r1);
         x_np = 0;
         bn_apply<T>(L, m, x, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_a, rows_in, u.ci, 0, -1, gate_bits(u.q_a));   // o
-        const int np = conv_fprop<T>(L, m, g1, S + u.t_a, wt + u.w1, S + u.t_b, nullptr, !eval, F + u.st2, u.r2);   // c1
-        stats_of(np, S + u.t_b, rows_out, u.co, F + u.st2, u.r2);
-        bn_apply<T>(L, m, S + u.t_b, F + u.st2, wf + u.g2, wf + u.b2, nullptr, nullptr, nullptr, nullptr, true, S + u.t_c, rows_out, u.co, np, u.r2, gate_bits(u.q_c)); // a2
+        if (!conv_bn_eval(g1, S + u.t_a, wt + u.w1, F + u.st2, wf + u.g2, wf + u.b2, nullptr, S + u.t_c)) {
+          const int np = conv_fprop<T>(L, m, g1, S + u.t_a, wt + u.w1, S + u.t_b, nullptr, !eval, F + u.st2, u.r2);   // c1
+          stats_of(np, S + u.t_b, rows_out, u.co, F + u.st2, u.r2);
+          bn_apply<T>(L, m, S + u.t_b, F + u.st2, wf + u.g2, wf + u.b2, nullptr, nullptr, nullptr, nullptr, true, S + u.t_c, rows_out, u.co, np, u.r2, gate_bits(u.q_c)); // a2
+        }
         if (u.proj) {
           ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
           conv_fprop<T>(L, m, gs, S + u.t_a, wt + u.ws, tmp, nullptr);
@@ -843,9 +860,9 @@ static void head_eval(fdg_ctx* c, Module& m, Launch& L, int slot, int vslot, con
     feat = S + u.t_a;
   }
   L.begin(KC_HEAD, (double)B * HW * F * sizeof(T), 2.0 * B * F * classes);
-  head_eval_kernel<T><<<B, 128, (size_t)(F + classes) * 4, L.st>>>(feat, wf + u.w1, wf + u.w2, labels_dev, HW, F, classes,
-                                                                  logits_dev, correct_dev);
-  L.check();
+  L.note(launch_chained(head_eval_kernel<T>, B, 128, (size_t)(F + classes) * 4, L.st, feat, wf + u.w1, wf + u.w2, labels_dev, HW, F, classes,
+                        logits_dev, correct_dev));
+  ++c->launches;
 }
 
 // Module K only: classifier, loss and their backward; leaves the gradient of the last block's
@@ -1002,8 +1019,8 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
         } else if (need_dx && u.zpad) {
           // the shortcut's share: the gated upstream gradient's middle channels, put back at every stride-th pixel
           L.begin(KC_BN_BWD_APPLY, (double)(rows_out * u.co * 2 + rows_in * u.ci) * sizeof(T), 0.0);
-          pad_shortcut_bwd_kernel<T><<<ew_blocks(rows_in * u.ci), 256, 0, L.st>>>(dy, S + u.t_y, T3, rows_in, u.P, u.Q, u.H, u.W, u.ci, u.co, u.stride);
-          L.check();
+          L.note(launch_chained(pad_shortcut_bwd_kernel<T>, ew_blocks(rows_in * u.ci), 256, 0, L.st, dy, S + u.t_y, T3, rows_in, u.P, u.Q, u.H, u.W, u.ci, u.co, u.stride));
+          ++c->launches;
           out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, open, next, up);
         } else if (need_dx) {
           out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, dy, gate(u.t_y, u.q_y), next);
@@ -1060,8 +1077,9 @@ static void update_module(fdg_ctx* c, Module& m, Launch& L, int next_vslot) {
   ++c->launches;
   if (m.flip_table_dev) {
     L.begin(KC_SGD, 4.0 * m.flip_elems, 0.0);
-    tc::wflip_kernel<<<dim3(m.flip_blocks, (unsigned)m.flip_table.size()), 256, 0, L.st>>>(next16, m.wflip16 + (size_t)next_vslot * m.flip_elems, m.flip_table_dev);
-    L.check();
+    L.note(launch_chained(tc::wflip_kernel, dim3(m.flip_blocks, (unsigned)m.flip_table.size()), 256, 0, L.st, next16,
+                          m.wflip16 + (size_t)next_vslot * m.flip_elems, m.flip_table_dev));
+    ++c->launches;
   }
 }
 
@@ -1742,8 +1760,8 @@ static cudaError_t eval_all(fdg_ctx* c, cudaStream_t cs, const float* images_dev
   for (Module& m : c->mods) {
     const int vslot = (int)(m.updates % m.Dw);
     if (m.eval_table_dev) {
-      bn_eval_stats_kernel<<<(unsigned)m.eval_table.size(), 128, 0, cs>>>(m.running, slot_F(m, m.D), m.eval_table_dev, c->arch.bn_eps);
-      L.check();
+      L.note(launch_chained(bn_eval_stats_kernel, dim3((unsigned)m.eval_table.size()), dim3(128), 0, cs, m.running, slot_F(m, m.D), m.eval_table_dev, c->arch.bn_eps));
+      ++c->launches;
     }
     forward_module<T>(c, m, L, 0, m.D, vslot, true);
     if (m.k == c->K) head_eval<T>(c, m, L, m.D, vslot, labels_dev, logits_dev, correct_dev);

@@ -105,6 +105,7 @@ wgrad_wide_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();
 
   if (warp == 0) {
     if (lane == 0) {
