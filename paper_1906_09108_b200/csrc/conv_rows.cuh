@@ -185,7 +185,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
   uint64_t* tile_done = op_ready + p.op_stages;    // [op_stages]  output tile written
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tile_done + p.op_stages);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* sums = reinterpret_cast<float*>(tmem_slot + 4);        // [kEpiWarps][32]
+  float* sums = reinterpret_cast<float*>(tmem_slot + 2);        // [kEpiWarps][32]; 16-byte aligned (the barriers are odd in number)
   float* mean = sums + kEpiWarps * 32;                          // [3][C]: mean, invstd (MODE 2); mean, gamma * invstd, beta
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -217,6 +217,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   grid_dependency_wait();                          // from here on the preceding kernel's results may be read
+  if (MODE == 3) grid_dependency_release();        // inference: one stream, nothing else wants the places of the next kernel
 
   if (warp >= kFirstEpi && lane == 0) {
     // The weight blocks, a few by each epilogue warp (one thread takes 150 cycles per request: 36 of them one after the
@@ -351,8 +352,14 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
       if (MODE == 3) {                             // on the value as it would have been stored: bn_apply_kernel's result
         const float* mu = mean + c0;
 #pragma unroll
-        for (int q = 0; q < 16; ++q)
-          v[q] = __float_as_uint(fmaf(__bfloat162float(__float2bfloat16_rn(__uint_as_float(v[q]))) - mu[q], mu[C + q], mu[2 * C + q]));
+        for (int q = 0; q < 16; q += 4) {
+          const float4 m = *reinterpret_cast<const float4*>(mu + q), g = *reinterpret_cast<const float4*>(mu + C + q),
+                       b = *reinterpret_cast<const float4*>(mu + 2 * C + q);
+          v[q] = __float_as_uint(fmaf(__bfloat162float(__float2bfloat16_rn(__uint_as_float(v[q]))) - m.x, g.x, b.x));
+          v[q + 1] = __float_as_uint(fmaf(__bfloat162float(__float2bfloat16_rn(__uint_as_float(v[q + 1]))) - m.y, g.y, b.y));
+          v[q + 2] = __float_as_uint(fmaf(__bfloat162float(__float2bfloat16_rn(__uint_as_float(v[q + 2]))) - m.z, g.z, b.z));
+          v[q + 3] = __float_as_uint(fmaf(__bfloat162float(__float2bfloat16_rn(__uint_as_float(v[q + 3]))) - m.w, g.w, b.w));
+        }
       }
       if (RES) {
         const uint32_t rw[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};

@@ -235,12 +235,18 @@ __device__ __forceinline__ void affine_load(const EpiAffine& a, float* area, int
     area[c] = a.stats[c]; area[Co + c] = a.gamma[c] * a.stats[Co + c]; area[2 * Co + c] = a.beta[c];
   }
 }
-// f[0..16) = the batch norm of the accumulator columns c .. c+15, rounded to bf16 first.
+// f[0..16) = the batch norm of the accumulator columns c .. c+15, rounded to bf16 first (four constants a load: one at a
+// time, the 48 loads a row of 16 took longer than the kernel they replace on the wide layers).
 __device__ __forceinline__ void affine_apply(const float* area, int Co, int c, float (&f)[16]) {
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    if (c + i >= Co) break;
-    f[i] = fmaf(__bfloat162float(__float2bfloat16_rn(f[i])) - area[c + i], area[Co + c + i], area[2 * Co + c + i]);
+  for (int i = 0; i < 16; i += 4) {
+    if (c + i >= Co) break;                // Co is a multiple of 8
+    const float4 m = *reinterpret_cast<const float4*>(area + c + i), g = *reinterpret_cast<const float4*>(area + Co + c + i),
+                 b = *reinterpret_cast<const float4*>(area + 2 * Co + c + i);
+    f[i] = fmaf(__bfloat162float(__float2bfloat16_rn(f[i])) - m.x, g.x, b.x);
+    f[i + 1] = fmaf(__bfloat162float(__float2bfloat16_rn(f[i + 1])) - m.y, g.y, b.y);
+    f[i + 2] = fmaf(__bfloat162float(__float2bfloat16_rn(f[i + 2])) - m.z, g.z, b.z);
+    f[i + 3] = fmaf(__bfloat162float(__float2bfloat16_rn(f[i + 3])) - m.w, g.w, b.w);
   }
 }
 
@@ -250,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                   ConvTcParams p, __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ res,
                   const __nv_bfloat16* __restrict__ res_mask, float* __restrict__ stat_partial, EpiAffine aff, int* __restrict__ error_word) {
-  __shared__ float stat_run[kStatFloats];
+  __shared__ __align__(16) float stat_run[kStatFloats];
   if (stat_partial) for (int i = threadIdx.x; i < kStatFloats; i += blockDim.x) stat_run[i] = 0.f;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -275,7 +281,11 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   grid_dependency_wait();                  // from here on the preceding kernel's results may be read
-  if (aff.stats) { affine_load(aff, stat_run, p.Co); __syncthreads(); }
+  if (aff.stats) {
+    grid_dependency_release();             // an inference pass: one stream, nothing else wants the places of the next kernel
+    affine_load(aff, stat_run, p.Co);
+    __syncthreads();
+  }
 
   const int chunks = (p.Ci + p.kc - 1) / p.kc;
   const int k_iters = p.taps * chunks;
@@ -490,7 +500,7 @@ __global__ void __launch_bounds__(kPatchThreads, 1)
 conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                      ConvTcParams p, __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ res,
                      const __nv_bfloat16* __restrict__ res_mask, float* __restrict__ stat_partial, EpiAffine aff, int* __restrict__ error_word) {
-  __shared__ float stat_run[kStatFloats];
+  __shared__ __align__(16) float stat_run[kStatFloats];
   if (stat_partial) for (int i = threadIdx.x; i < kStatFloats; i += blockDim.x) stat_run[i] = 0.f;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -519,7 +529,11 @@ conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   grid_dependency_wait();                  // from here on the preceding kernel's results may be read
-  if (aff.stats) { affine_load(aff, stat_run, p.Co); __syncthreads(); }
+  if (aff.stats) {
+    grid_dependency_release();             // an inference pass: one stream, nothing else wants the places of the next kernel
+    affine_load(aff, stat_run, p.Co);
+    __syncthreads();
+  }
 
   const int chunks = (p.Ci + p.kc - 1) / p.kc;
   const int pw_cnt = p.W / kPatch, ph_cnt = p.H / kPatch;

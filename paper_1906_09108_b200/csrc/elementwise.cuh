@@ -181,6 +181,7 @@ bn_sums_kernel(const T* __restrict__ dy, const GateOf<T> gate, const T* __restri
                const T* __restrict__ x2, const float* __restrict__ stats2, RedGeom g, float* __restrict__ partial) {
   constexpr int NS = KIND == 3 ? 3 : 2;
   __shared__ float red[kRedThreads * VEC];                   // [rp][C] of one sum
+  __shared__ double part[kRedThreads];                       // [nseg][C]
   const int tid = threadIdx.x, C = g.C;
   const int cvi = tid % g.cv, r = tid / g.cv;
   const bool active = r < g.rp;
@@ -241,6 +242,9 @@ bn_sums_kernel(const T* __restrict__ dy, const GateOf<T> gate, const T* __restri
     }
     for (; row < row1; row += g.rp) { Item it; fetch(row, it); add(it); }
   }
+  // A channel has rp sums: up to 16 threads share them (at 8 channels 512 sums are 32 + 16 fp64 additions in a row; one
+  // thread per channel, 512 in a row, was most of the time of a small tensor's reduction).
+  const int nseg = max(1, min(kRedThreads / C, min(g.rp, 16)));
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     __syncthreads();
@@ -249,9 +253,17 @@ bn_sums_kernel(const T* __restrict__ dy, const GateOf<T> gate, const T* __restri
       for (int i = 0; i < VEC; ++i) red[r * C + cvi * VEC + i] = sums[s][i];
     }
     __syncthreads();
+    for (int i = tid; i < nseg * C; i += kRedThreads) {
+      const int seg = i / C, c = i - seg * C;
+      double a = 0.0;
+      for (int rr = seg; rr < g.rp; rr += nseg) a += (double)red[rr * C + c];
+      if (nseg == 1) partial[(size_t)blockIdx.x * NS * C + s * C + c] = (float)a; else part[i] = a;
+    }
+    if (nseg == 1) continue;
+    __syncthreads();
     for (int c = tid; c < C; c += kRedThreads) {
       double a = 0.0;
-      for (int rr = 0; rr < g.rp; ++rr) a += (double)red[rr * C + c];
+      for (int seg = 0; seg < nseg; ++seg) a += part[seg * C + c];
       partial[(size_t)blockIdx.x * NS * C + s * C + c] = (float)a;
     }
   }

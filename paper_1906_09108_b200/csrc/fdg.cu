@@ -21,6 +21,7 @@
 #include <cstdio>
 #include <climits>
 #include <cstring>
+#include <deque>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -163,7 +164,7 @@ struct fdg_ctx {
   size_t ws_bytes = 0;
   float lr = 0.f;
   uint64_t launches = 0;
-  std::vector<fdg_sched_entry> log;
+  std::deque<fdg_sched_entry> log;   // full, it drops its oldest rows at the front on every iteration
   mutable std::string err;
   fdg_status latched = FDG_OK;
   int device = 0;
