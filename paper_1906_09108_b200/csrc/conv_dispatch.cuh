@@ -49,7 +49,7 @@ inline cudaError_t run_conv_tc(cudaStream_t st, TensorMapCache* cache, int N, in
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&cache->sm_count, cudaDevAttrMultiProcessorCount, dev);
   }
-  tc::ConvTcParams p = tc::conv_tc_params(N, H, W, Ck, Cn, taps);
+  tc::ConvTcParams p = tc::conv_tc_params(N, H, W, Ck, Cn, taps, cache->share);
   p.sub = sub;
   p.act_sub = act_sub;
   TensorMapCache::Key ka, kb;
