@@ -37,7 +37,7 @@ BETA, LR, MOM, WD = 0.2, 0.01, 0.9, 5e-4
 # default, and the only one the bench line's metric is quoted on, is resnet110_k4.
 
 
-def profiled_traffic(summary="conv_halo_kernel_fprop_stage1.md", source="conv_halo.cuh"):
+def profiled_traffic(summary="conv_rows_kernel_fprop_stage1.md", source="conv_rows.cuh"):
     """DRAM bytes per launch of the dominant kernel from its committed ncu summary (the line
     `traffic_bytes_per_launch: N`), or None when the summary is missing or was taken on another version of the
     kernel's source (the line `kernel_source_sha16: H` holds the first 16 hex digits of the source's SHA-256)."""
@@ -586,7 +586,7 @@ def run_gpu(args):
             # far below the machine balance, so HBM is the roofline that bounds it.
             us, nbytes, flops = kernel_bench(B, "fprop", "stage1")
             roof = dict(bound="hbm", achieved=nbytes / us / 1e3, peak=peaks["hbm_gbs"], unit="GB/s",
-                        kernel="conv_halo_kernel, 3x3 stride-1 forward, [128,32,32,16] -> 16 channels",
+                        kernel="conv_rows_kernel, 3x3 stride-1 forward, [128,32,32,16] -> 16 channels",
                         avg_us=us, tflops=flops / us / 1e6,
                         how="64 launches on distinct buffers (pool > 2 x L2) replayed from a CUDA graph, CUDA events "
                             "on the replay stream",

@@ -201,7 +201,7 @@ __device__ __forceinline__ void transpose_reduce32(float (&q)[32], int lane) {
 // Batch-norm statistics of the output, formed in the epilogue (optional): every epilogue warp adds, per 16-channel
 // chunk, the sums of the values it stores and of their squares over its 32 rows into its own array in shared
 // memory; at the end the CTA writes one row stat_partial[blockIdx.x][2][Co] (sum, sum of squares), which
-// stats_finalize_kernel adds over the CTAs in CTA order.  Up to kStatChunks * 16 output channels.
+// sums_finalize_kernel adds over the CTAs in CTA order.  Up to kStatChunks * 16 output channels.
 constexpr int kStatChunks = 40;
 constexpr int kStatFloats = 4 * kStatChunks * 32;
 __device__ __forceinline__ void stat_add(float* stat_run, int ew, int chunk, const uint4& o0, const uint4& o1, int lane) {

@@ -613,19 +613,6 @@ __global__ void scale_kernel(const T* __restrict__ in, T* __restrict__ out, floa
   }
 }
 
-// out = a + b
-template <typename T, int VEC>
-__global__ void add_kernel(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out, size_t nvec) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
-    float x[VEC], y[VEC];
-    load_vec<T, VEC>(a + i * VEC, x);
-    load_vec<T, VEC>(b + i * VEC, y);
-#pragma unroll
-    for (int j = 0; j < VEC; ++j) x[j] += y[j];
-    store_vec<T, VEC>(out + i * VEC, x);
-  }
-}
-
 // up[n][2p][2q][:] = dy[n][p][q][:], zero at the other pixels; dy [N][P][Q][C], up [N][2P][2Q][C], 16-byte vectors.
 template <typename T, int VEC>
 __global__ void upsample2_kernel(const T* __restrict__ dy, T* __restrict__ up, size_t nvec_up, int P, int Q, int C) {
