@@ -432,6 +432,7 @@ inline cudaError_t launch_conv(cudaStream_t st, const ConvGeom& g, bool dgrad, c
 
 // ------------------------------------------------------------- weight gradient --
 constexpr int kWgCi = 32, kWgCo = 32;        // channels of a block at most
+constexpr size_t kWgradSmemMax = 128 * 1024;
 struct WgradParams {
   int N, H, W, Ci, P, Q, Co;
   int cib, cob, ci_blocks;      // channels per block (multiples of 4), blocks along ci
@@ -593,9 +594,12 @@ inline WgradParams wgrad_params(const ConvGeom& g) {
   if (p.rg > 4 && g.P % p.rg) p.rg = 4;
   if (p.rg > g.P) p.rg = g.P;
   if (p.rg < 1) p.rg = 1;
-  p.threads = (p.rg * p.tt + 31) / 32 * 32;
   const int pad = g.R == 3 ? 1 : 0;
   p.xrow = (g.W + 2 * pad) * p.cib + (p.cib <= 16 ? 16 : 0);     // rows of a warp's taps on different banks
+  // A step holds a row of dy (and its rows of x) for every group: wide rows of many channels leave room for fewer groups.
+  // One group always fits: 3 rows of 66 x 32 values of x and one of 64 x 32 of dy are 34 KB.
+  while (p.rg > 1 && (((size_t)(p.rg - 1) * g.stride + g.R) * p.xrow + (size_t)p.rg * g.Q * p.cob) * 4 > kWgradSmemMax) --p.rg;
+  p.threads = (p.rg * p.tt + 31) / 32 * 32;
   // rows per step: whole turns of the row groups, about four rows within 40 KB of shared memory, in equal shares of an
   // image (every step reads two rows of x more than it has rows of dy)
   const int row_floats = p.xrow * g.stride + g.Q * p.cob;
@@ -635,7 +639,7 @@ inline cudaError_t wgrad_launch_one(cudaStream_t st, const WgradParams& p, const
   auto kernel = direct_wgrad_kernel<T, VX, VY, R, STRIDE>;
   static bool set = false;
   if (!set) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgradSmemMax);
     if (e != cudaSuccess) return e;
     set = true;
   }

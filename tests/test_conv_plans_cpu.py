@@ -1,0 +1,51 @@
+"""The CUDA-core convolutions' plans, without a GPU: whatever shape the dispatcher hands them, the launch they plan stays
+within the shared memory that the kernels are given and covers the whole problem.  A small host program made from the
+library's own header walks the shapes."""
+import os
+import subprocess
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1906_09108_b200", "csrc")
+
+PROLOGUE = r"""
+#include <cstdio>
+#include "fdg_ops.h"
+#include "conv_direct.cuh"
+using namespace fdg;
+static int bad = 0;
+static void report(const char* what, const ConvGeom& g, size_t bytes) {
+  if (bad++ < 10) printf("%s N=%d %dx%d %d->%d R=%d stride=%d: %zu\n", what, g.N, g.H, g.W, g.Ci, g.Co, g.R, g.stride, bytes);
+}
+template <typename F> static void shapes(F f) {
+  const int chans[] = {1, 4, 5, 8, 16, 24, 32, 33, 64}, batches[] = {1, 128, 600, 2368};
+  for (int N : batches) for (int R = 1; R <= 3; R += 2) for (int s = 1; s <= 2; ++s)
+    for (int H = 1; H <= 70; H += H < 18 ? 1 : 5) for (int W = 1; W <= 64; W += W < 18 ? 1 : 3)
+      for (int ci : chans) for (int co : chans) {
+        const int P = (H + 2 * (R / 2) - R) / s + 1, Q = (W + 2 * (R / 2) - R) / s + 1;
+        f(ConvGeom{N, H, W, ci, P, Q, co, R, R, s, R / 2});
+      }
+}
+"""
+
+
+def _run(tmp_path, body):
+    src = tmp_path / "plans.cu"
+    src.write_text(PROLOGUE + "int main() {\n" + body + "\n  return bad != 0;\n}\n")
+    exe = str(tmp_path / "plans")
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    subprocess.run([nvcc, "-O2", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-I", CSRC, "-I",
+                    os.path.join(os.path.dirname(os.path.dirname(CSRC)), "include"), "-o", exe, str(src)], check=True,
+                   capture_output=True)
+    res = subprocess.run([exe], capture_output=True, text=True)
+    assert res.returncode == 0, res.stdout
+
+
+def test_weight_gradient_plans_fit_shared_memory(tmp_path):
+    _run(tmp_path, r"""
+  shapes([](const ConvGeom& g) {
+    if (!direct::wgrad_direct_supported(g)) return;
+    const direct::WgradParams p = direct::wgrad_params(g);
+    const size_t bytes = direct::wgrad_smem_bytes(p, g.R);
+    if (bytes > direct::kWgradSmemMax) report("shared memory", g, bytes);
+    if (p.rg < 1 || p.rg * p.tt > p.threads || p.threads > direct::kThreads) report("threads", g, (size_t)p.threads);
+    if (p.TH < 1 || p.TH * p.strips < g.P || p.units != g.N * p.strips || p.splits < 1) report("rows", g, (size_t)p.TH);
+  });""")
