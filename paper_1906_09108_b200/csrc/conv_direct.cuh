@@ -339,6 +339,7 @@ inline bool conv_supported(const ConvGeom& g, bool dgrad) {
   return (dgrad ? g.W : g.Q) <= 64 && g.W <= 64;
 }
 
+constexpr size_t kConvSmemMax = 160 * 1024;
 inline ConvParams conv_params(const ConvGeom& g, bool dgrad, int nc) {
   ConvParams p{};
   const int stride = dgrad ? 1 : g.stride;
@@ -347,7 +348,7 @@ inline ConvParams conv_params(const ConvGeom& g, bool dgrad, int nc) {
   p.P = dgrad ? g.H : g.P; p.Q = dgrad ? g.W : g.Q; p.Cn = dgrad ? g.Ci : g.Co;
   p.up = dgrad ? g.stride : 1;
   p.segs = (p.Q + kPx - 1) / kPx;
-  // output channels of a block: equal shares of at most 64, whole thread columns
+  // output channels of a block: equal shares of at most kMaxCb, whole thread columns
   const int blocks_n = (p.Cn + kMaxCb - 1) / kMaxCb;
   p.cb = ((p.Cn + blocks_n - 1) / blocks_n + nc - 1) / nc * nc;
   p.cgs = p.cb / nc;
@@ -360,9 +361,12 @@ inline ConvParams conv_params(const ConvGeom& g, bool dgrad, int nc) {
   while (rows > 1 && (size_t)kKc * (rows * stride + 2) * p.pitch * 4 > 96 * 1024) rows /= 2;
   if (rows >= p.P) { p.TH = p.P; p.TI = std::max(1, std::min(rows / p.P, p.N / 148)); }
   else { const int t = (p.P + rows - 1) / rows; p.TH = (p.P + t - 1) / t; p.TI = 1; }
+  p.rows_in = (p.TH - 1) * stride + 3;
+  // Every image of a tile has border rows of its own, which the bound above does not count: images of one or two rows
+  // take up to three times the shared memory of their output rows.
+  while (p.TI > 1 && ((size_t)kKc * (p.TI * p.rows_in * p.pitch + 4) + (size_t)kKc * 9 * p.cb) * 4 > kConvSmemMax) --p.TI;
   p.row_tiles = (p.P + p.TH - 1) / p.TH;
   p.tiles = ((p.N + p.TI - 1) / p.TI) * p.row_tiles;
-  p.rows_in = (p.TH - 1) * stride + 3;
   p.plane = p.TI * p.rows_in * p.pitch;
   if (p.plane % 8 == 0) p.plane += 4;                        // 4-channel groups of a warp's stores on different banks
   return p;
@@ -372,7 +376,6 @@ inline size_t conv_smem_bytes(const ConvParams& p) {
   const size_t sums = (size_t)p.TI * p.TH * p.segs * 2 * p.cb;
   return (tiles > sums ? tiles : sums) * 4;
 }
-constexpr size_t kConvSmemMax = 160 * 1024;
 
 template <typename T, int VEC, int STRIDE, int NC, bool FLIP>
 inline cudaError_t conv_launch_one(cudaStream_t st, const ConvParams& p, int grid, const T* act, const T* wgt, T* out,

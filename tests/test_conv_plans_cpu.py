@@ -49,3 +49,20 @@ def test_weight_gradient_plans_fit_shared_memory(tmp_path):
     if (p.rg < 1 || p.rg * p.tt > p.threads || p.threads > direct::kThreads) report("threads", g, (size_t)p.threads);
     if (p.TH < 1 || p.TH * p.strips < g.P || p.units != g.N * p.strips || p.splits < 1) report("rows", g, (size_t)p.TH);
   });""")
+
+
+def test_forward_and_data_gradient_plans_fit_shared_memory(tmp_path):
+    _run(tmp_path, r"""
+  shapes([](const ConvGeom& g) {
+    for (int dgrad = 0; dgrad < 2; ++dgrad) {
+      if (!direct::conv_supported(g, dgrad != 0)) continue;
+      for (int nc = 4; nc <= 8; nc += 4) {
+        const direct::ConvParams p = direct::conv_params(g, dgrad != 0, nc);
+        const size_t bytes = direct::conv_smem_bytes(p);
+        if (bytes > direct::kConvSmemMax) report("shared memory", g, bytes);
+        if (p.TI * p.TH * p.segs * p.cgs > direct::kThreads) report("threads", g, (size_t)(p.TI * p.TH * p.segs * p.cgs));
+        if (p.TI < 1 || p.TH < 1 || p.TH * p.row_tiles < p.P || (long)p.tiles * p.TI < (long)g.N * p.row_tiles) report("tiles", g, (size_t)p.tiles);
+        if ((long)p.TI * p.rows_in * (p.Wi * p.up + 2) * 4 >= 1 << 20) report("items", g, (size_t)p.TI);   // div_small's range
+      }
+    }
+  });""")

@@ -21,7 +21,9 @@ SHAPES = [(2, 33, 30, 3, 16, 3, 1, 1),       # the stem: three channels; odd hei
           (2, 10, 12, 40, 72, 1, 1, 0), (3, 12, 10, 36, 68, 1, 2, 0),
           # weight gradients whose rows leave shared memory for fewer row groups than the block has threads for
           (2, 64, 64, 4, 32, 1, 1, 0), (2, 64, 64, 8, 32, 1, 1, 0), (2, 56, 56, 24, 4, 3, 2, 1), (2, 64, 64, 32, 8, 1, 2, 0),
-          (3, 13, 63, 8, 32, 1, 1, 0)]
+          (3, 13, 63, 8, 32, 1, 1, 0),
+          # images of one row: more of them would fill the block than shared memory holds with their border rows
+          (2368, 1, 64, 4, 4, 3, 1, 1)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
