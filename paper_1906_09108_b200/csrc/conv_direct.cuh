@@ -15,7 +15,8 @@
 // direct_wgrad_kernel.  A block takes 32 x 32 channels at most and a share of the image rows; a thread 4 input x 4
 // output channels of one filter row's three taps: walking along a row of pixels, one new vector of x and one of dy
 // serve 48 multiply-adds.  Groups of threads take alternate rows; their sums are added in group order, the blocks'
-// partial sums in block order (launch_wgrad_reduce), so the result does not depend on scheduling.
+// partial sums in block order (launch_wgrad_reduce), so the result does not depend on scheduling.  In bf16 storage (the
+// stem and narrow projections) only a row's products are added in fp32; rows, groups and blocks are added in fp64.
 #pragma once
 #include "conv_simt.cuh"
 
@@ -435,7 +436,7 @@ inline cudaError_t launch_conv(cudaStream_t st, const ConvGeom& g, bool dgrad, c
 
 // ------------------------------------------------------------- weight gradient --
 constexpr int kWgCi = 32, kWgCo = 32;        // channels of a block at most
-constexpr size_t kWgradSmemMax = 128 * 1024;
+constexpr size_t kWgradSmemMax = 176 * 1024;  // what a block may use: one group of 192 threads with fp64 sums takes up to 170 KB
 struct WgradParams {
   int N, H, W, Ci, P, Q, Co;
   int cib, cob, ci_blocks;      // channels per block (multiples of 4), blocks along ci
@@ -446,14 +447,22 @@ struct WgradParams {
   int splits;                   // blocks along the pixels
 };
 
+template <typename T> constexpr bool kByRow = sizeof(T) == 2;         // rows are added in fp64
+
 template <typename T, int VECX, int VECY, int R, int STRIDE>
 __global__ void __launch_bounds__(kThreads)
 direct_wgrad_kernel(WgradParams p, const T* __restrict__ x, const T* __restrict__ dy, float* __restrict__ partial) {
   grid_dependency_wait();
   constexpr int PAD = R == 3 ? 1 : 0;
+  constexpr bool BY_ROW = kByRow<T>;
   extern __shared__ __align__(16) float dw_smem[];
   float* sx = dw_smem;                                       // [rows_x][W + 2 * PAD][cib], rows padded to xrow
   float* sy = dw_smem + p.rows_x * p.xrow;                   // [TH][Q][cob]
+  // By rows: the groups leave their row's products in ex[value][thread] (a value per tap, output and input channel of a
+  // thread), and the block's fp64 totals [value][thread of a group] are divided among all threads: in the registers of the
+  // thread that multiplies they would halve the blocks of an SM (stem of 128 32x32 images: 26.9 us, this way 13.3).
+  float* ex = sy + p.TH * p.Q * p.cob;
+  double* total = reinterpret_cast<double*>(ex + p.rg * p.tt * 16 * R);
   const int tid = threadIdx.x;
   const int ci0 = (blockIdx.y % p.ci_blocks) * p.cib, co0 = (blockIdx.y / p.ci_blocks) * p.cob;
   const int grp = tid / p.tt, t = tid - grp * p.tt;          // row group, thread of the tile
@@ -467,6 +476,7 @@ direct_wgrad_kernel(WgradParams p, const T* __restrict__ x, const T* __restrict_
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[s][i][j] = 0.f;
+  if (BY_ROW && active) for (int v = grp; v < 16 * R; v += p.rg) total[v * p.tt + t] = 0.0;
   const float inv_ct = 1.f / (float)p.ct, inv_ot = 1.f / (float)p.ot, inv_cols = 1.f / (float)cols;
   for (int u = blockIdx.x; u < p.units; u += gridDim.x) {
     const int n = u / p.strips, p0 = (u - n * p.strips) * p.TH;
@@ -512,69 +522,109 @@ direct_wgrad_kernel(WgradParams p, const T* __restrict__ x, const T* __restrict_
           *reinterpret_cast<float4*>(sy + 4 * (i0 + k * p.threads)) = make_float4(q[k][0], q[k][1], q[k][2], q[k][3]);
     }
     __syncthreads();
-    if (active)
-      for (int row = grp; row < rows; row += p.rg) {
-        const float* xp = sx + (row * STRIDE + r) * p.xrow + 4 * c;
-        const float* yp = sy + row * p.Q * p.cob + 4 * o;
-        float4 w0, w1, w2;                                   // x at the taps of this pixel
-        auto xat = [&](int px) { return *reinterpret_cast<const float4*>(xp + px * p.cib); };
-        if constexpr (R == 3) {
-          if constexpr (STRIDE == 1) { w1 = xat(0); w2 = xat(1); } else w2 = xat(0);
-        }
+    auto add_row = [&](int row) {
+      const float* xp = sx + (row * STRIDE + r) * p.xrow + 4 * c;
+      const float* yp = sy + row * p.Q * p.cob + 4 * o;
+      float4 w0, w1, w2;                                     // x at the taps of this pixel
+      auto xat = [&](int px) { return *reinterpret_cast<const float4*>(xp + px * p.cib); };
+      if constexpr (R == 3) {
+        if constexpr (STRIDE == 1) { w1 = xat(0); w2 = xat(1); } else w2 = xat(0);
+      }
 #pragma unroll 4
-        for (int q = 0; q < p.Q; ++q) {
-          const float4 d = *reinterpret_cast<const float4*>(yp + q * p.cob);
-          if constexpr (R == 3) {
-            if constexpr (STRIDE == 1) { w0 = w1; w1 = w2; w2 = xat(q + 2); }
-            else { w0 = w2; w1 = xat(2 * q + 1); w2 = xat(2 * q + 2); }
-          } else {
-            w0 = xat(q * STRIDE);
-          }
-          const float dv[4] = {d.x, d.y, d.z, d.w};
-          const float xv[3][4] = {{w0.x, w0.y, w0.z, w0.w}, {w1.x, w1.y, w1.z, w1.w}, {w2.x, w2.y, w2.z, w2.w}};
+      for (int q = 0; q < p.Q; ++q) {
+        const float4 d = *reinterpret_cast<const float4*>(yp + q * p.cob);
+        if constexpr (R == 3) {
+          if constexpr (STRIDE == 1) { w0 = w1; w1 = w2; w2 = xat(q + 2); }
+          else { w0 = w2; w1 = xat(2 * q + 1); w2 = xat(2 * q + 2); }
+        } else {
+          w0 = xat(q * STRIDE);
+        }
+        const float dv[4] = {d.x, d.y, d.z, d.w};
+        const float xv[3][4] = {{w0.x, w0.y, w0.z, w0.w}, {w1.x, w1.y, w1.z, w1.w}, {w2.x, w2.y, w2.z, w2.w}};
+#pragma unroll
+        for (int s = 0; s < R; ++s)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[s][i][j] = fmaf(dv[i], xv[s][j], acc[s][i][j]);
+      }
+    };
+    if constexpr (!BY_ROW) {
+      if (active)
+        for (int row = grp; row < rows; row += p.rg) add_row(row);
+    } else {
+      for (int row0 = 0; row0 < rows; row0 += p.rg) {
+#pragma unroll
+        for (int s = 0; s < R; ++s)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[s][i][j] = 0.f;
+        if (row0) __syncthreads();                           // the row before has been added (the first: behind the tiles' barriers)
+        if (active && row0 + grp < rows) add_row(row0 + grp);
+        if (active) {
 #pragma unroll
           for (int s = 0; s < R; ++s)
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-              for (int j = 0; j < 4; ++j) acc[s][i][j] = fmaf(dv[i], xv[s][j], acc[s][i][j]);
+              for (int j = 0; j < 4; ++j) ex[((s * 4 + i) * 4 + j) * (p.rg * p.tt) + tid] = acc[s][i][j];
         }
+        __syncthreads();
+        if (active)
+          for (int v = grp; v < 16 * R; v += p.rg) {
+            const float* e = ex + v * p.rg * p.tt + t;
+            double a = total[v * p.tt + t];
+#pragma unroll 4
+            for (int g = 0; g < p.rg; ++g) a += (double)e[g * p.tt];
+            total[v * p.tt + t] = a;
+          }
       }
-  }
-  // the row groups' sums, added in group order through shared memory
-  for (int g = 1; g < p.rg; ++g) {
-    __syncthreads();
-    if (grp == g) {
-#pragma unroll
-      for (int s = 0; s < R; ++s)
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) dw_smem[((s * 4 + i) * 4 + j) * p.tt + t] = acc[s][i][j];
-    }
-    __syncthreads();
-    if (grp == 0) {
-#pragma unroll
-      for (int s = 0; s < R; ++s)
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[s][i][j] += dw_smem[((s * 4 + i) * 4 + j) * p.tt + t];
     }
   }
-  if (grp == 0) {
+  if constexpr (BY_ROW) {
+    if (!active) return;
     float* dst = partial + (size_t)blockIdx.x * p.Co * R * R * p.Ci;
+    for (int v = grp; v < 16 * R; v += p.rg) {
+      const int s = v >> 4, co = co0 + 4 * o + ((v >> 2) & 3), ci = ci0 + 4 * c + (v & 3);
+      if (co < p.Co && ci < p.Ci) dst[(((size_t)co * R + r) * R + s) * p.Ci + ci] = (float)total[v * p.tt + t];
+    }
+  } else {
+    // the row groups' sums, added in group order through shared memory
+    for (int g = 1; g < p.rg; ++g) {
+      __syncthreads();
+      if (grp == g) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int co = co0 + 4 * o + i;
-      if (co >= p.Co) continue;
+        for (int s = 0; s < R; ++s)
 #pragma unroll
-      for (int s = 0; s < R; ++s)
+          for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int ci = ci0 + 4 * c + j;
-          if (ci < p.Ci) dst[(((size_t)co * R + r) * R + s) * p.Ci + ci] = acc[s][i][j];
-        }
+            for (int j = 0; j < 4; ++j) dw_smem[((s * 4 + i) * 4 + j) * p.tt + t] = acc[s][i][j];
+      }
+      __syncthreads();
+      if (grp == 0) {
+#pragma unroll
+        for (int s = 0; s < R; ++s)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[s][i][j] += dw_smem[((s * 4 + i) * 4 + j) * p.tt + t];
+      }
+    }
+    if (grp == 0) {
+      float* dst = partial + (size_t)blockIdx.x * p.Co * R * R * p.Ci;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int co = co0 + 4 * o + i;
+        if (co >= p.Co) continue;
+#pragma unroll
+        for (int s = 0; s < R; ++s)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int ci = ci0 + 4 * c + j;
+            if (ci < p.Ci) dst[(((size_t)co * R + r) * R + s) * p.Ci + ci] = acc[s][i][j];
+          }
+      }
     }
   }
 }
@@ -584,7 +634,14 @@ inline bool wgrad_direct_supported(const ConvGeom& g) {
   else if (g.R != 1 || g.S != 1 || g.pad != 0 || g.stride > 2 || g.W > 64) return false;
   return true;
 }
-inline WgradParams wgrad_params(const ConvGeom& g) {
+// Bytes of shared memory of a block: tiles of `rows` rows of dy; the groups' sums over them (one group's at a time) or, by
+// rows, behind them (all groups', and the totals).
+inline size_t wgrad_smem(const WgradParams& p, int R, int stride, int rows, bool by_row) {
+  const size_t tile = (((size_t)(rows - 1) * stride + R) * p.xrow + (size_t)rows * p.Q * p.cob) * 4;
+  const size_t values = (size_t)p.tt * 16 * R, sums = p.rg > 1 ? values * 4 : 0;
+  return by_row ? tile + values * (4 * p.rg + 8) : (tile > sums ? tile : sums);
+}
+inline WgradParams wgrad_params(const ConvGeom& g, bool by_row) {
   WgradParams p{};
   p.N = g.N; p.H = g.H; p.W = g.W; p.Ci = g.Ci; p.P = g.P; p.Q = g.Q; p.Co = g.Co;
   p.ci_blocks = (g.Ci + kWgCi - 1) / kWgCi;
@@ -600,8 +657,8 @@ inline WgradParams wgrad_params(const ConvGeom& g) {
   const int pad = g.R == 3 ? 1 : 0;
   p.xrow = (g.W + 2 * pad) * p.cib + (p.cib <= 16 ? 16 : 0);     // rows of a warp's taps on different banks
   // A step holds a row of dy (and its rows of x) for every group: wide rows of many channels leave room for fewer groups.
-  // One group always fits: 3 rows of 66 x 32 values of x and one of 64 x 32 of dy are 34 KB.
-  while (p.rg > 1 && (((size_t)(p.rg - 1) * g.stride + g.R) * p.xrow + (size_t)p.rg * g.Q * p.cob) * 4 > kWgradSmemMax) --p.rg;
+  // One group always fits, with the four rows that it may take below.
+  while (p.rg > 1 && wgrad_smem(p, g.R, g.stride, p.rg, by_row) > kWgradSmemMax) --p.rg;
   p.threads = (p.rg * p.tt + 31) / 32 * 32;
   // rows per step: whole turns of the row groups, about four rows within 40 KB of shared memory, in equal shares of an
   // image (every step reads two rows of x more than it has rows of dy)
@@ -629,12 +686,8 @@ inline WgradParams wgrad_params(const ConvGeom& g) {
   p.splits = best;
   return p;
 }
-inline size_t wgrad_direct_scratch_elems(const ConvGeom& g) {
-  return wgrad_direct_supported(g) ? (size_t)wgrad_params(g).splits * g.Co * g.R * g.R * g.Ci : 0;
-}
-inline size_t wgrad_smem_bytes(const WgradParams& p, int R) {
-  const size_t tile = (size_t)p.rows_x * p.xrow + (size_t)p.TH * p.Q * p.cob, sums = p.rg > 1 ? (size_t)p.tt * 16 * R : 0;
-  return (tile > sums ? tile : sums) * 4;
+inline size_t wgrad_direct_scratch_elems(const ConvGeom& g, bool by_row) {
+  return wgrad_direct_supported(g) ? (size_t)wgrad_params(g, by_row).splits * g.Co * g.R * g.R * g.Ci : 0;
 }
 
 template <typename T, int VX, int VY, int R, int STRIDE>
@@ -647,14 +700,14 @@ inline cudaError_t wgrad_launch_one(cudaStream_t st, const WgradParams& p, const
     set = true;
   }
   const int pairs = p.ci_blocks * ((p.Co + p.cob - 1) / p.cob);
-  return launch_chained(kernel, dim3(p.splits, pairs), dim3(p.threads), wgrad_smem_bytes(p, R), st, p, x, dy, dst);
+  return launch_chained(kernel, dim3(p.splits, pairs), dim3(p.threads), wgrad_smem(p, R, STRIDE, p.TH, kByRow<T>), st, p, x, dy, dst);
 }
 
 // dw [Co][R][R][Ci] (fp32) from x and dy; `scratch` of wgrad_direct_scratch_elems floats.
 template <typename T>
 inline cudaError_t launch_wgrad(cudaStream_t st, const ConvGeom& g, const T* x, const T* dy, float* scratch, float* dw,
                                 uint64_t* launches) {
-  const WgradParams p = wgrad_params(g);
+  const WgradParams p = wgrad_params(g, kByRow<T>);
   float* dst = p.splits == 1 ? dw : scratch;
   const bool vx = g.Ci % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
   const bool vy = g.Co % 4 == 0 && (reinterpret_cast<uintptr_t>(dy) & 15) == 0;
@@ -667,7 +720,8 @@ inline cudaError_t launch_wgrad(cudaStream_t st, const ConvGeom& g, const T* x, 
 #undef FDG_DW
   if (e != cudaSuccess || p.splits == 1) return e;
   ++*launches;
-  return launch_wgrad_reduce(st, scratch, dw, (size_t)g.Co * g.R * g.R * g.Ci, p.splits);
+  typedef std::conditional_t<kByRow<T>, double, float> Sum;
+  return launch_wgrad_reduce<Sum>(st, scratch, dw, (size_t)g.Co * g.R * g.R * g.Ci, p.splits);
 }
 
 }  // namespace direct

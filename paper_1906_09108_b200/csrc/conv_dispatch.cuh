@@ -116,7 +116,15 @@ inline bool wide_wgrad_eligible(const ConvGeom& g) {
 inline bool wide_s2_wgrad_eligible(const ConvGeom& g) {
   return halo_s2_shape(g) && wide::wide_supported(g.N, g.H, g.W, g.Ci, g.Co) && ((g.Ci >= 128 && g.Co >= 128) || !halo_s2_wgrad_eligible(g));
 }
-inline bool wide_1x1_wgrad_eligible(const ConvGeom& g) { return tc_1x1_shape(g) && wide::wide_supported(g.N, g.P, g.Q, g.Ci, g.Co, 1); }
+// Projections of fewer than 64 channels on a side stay with direct_wgrad_kernel, which adds their rows in fp64: tensor
+// memory truncates at every instruction, an error that grows with a CTA's pixels, and a narrow projection gives few CTAs.
+// 128 images, error against 64 bits and time, tensor cores / CUDA cores: 16 -> 32 on 32x32, stride 2: 1.0e-6, 15.4 us /
+// 4.2e-8, 10.7 us; 32 -> 64 on 16x16: 2.5e-7, 9.3 us / 3.9e-8, 11.1 us; 16 -> 160 on 32x32: 4.4e-6, 40.6 us / 5.0e-8,
+// 49.5 us; 2048 images of the first: 1.9e-5, 139 us / 4.3e-8, 93 us.  With 64 channels or more on both sides it is arithmetic,
+// where the tensor cores are the faster by 4 to 25 times: 64 -> 128 on 32x32, stride 2: 1.0e-6, 15.7 us / 4.2e-8, 70 us.
+inline bool wide_1x1_wgrad_eligible(const ConvGeom& g) {
+  return tc_1x1_shape(g) && g.Ci >= 64 && g.Co >= 64 && wide::wide_supported(g.N, g.P, g.Q, g.Ci, g.Co, 1);
+}
 
 inline cudaError_t cached_tile_map(TensorMapCache* cache, const void* act, int N, int H, int W, int C, int G,
                                    const CUtensorMap** out, int boxC = 0) {
@@ -295,7 +303,7 @@ inline bool s2_uses_spread_dy(const ConvGeom& g) {
 
 // fp32 scratch elements a weight-gradient call may need (bf16 storage: whichever kernel is chosen).
 inline size_t conv_wgrad_scratch_elems(bool bf16_storage, const ConvGeom& g) {
-  size_t n = std::max(wgrad_scratch_elems(g), direct::wgrad_direct_scratch_elems(g));
+  size_t n = std::max(wgrad_scratch_elems(g), direct::wgrad_direct_scratch_elems(g, bf16_storage));
   if (bf16_storage && (halo_wgrad_eligible(g) || halo_s2_wgrad_eligible(g)))
     n = std::max(n, halo::wgrad_scratch_elems(g.N, g.H, g.W, g.Ci, g.Co));
   if (bf16_storage && (wide_wgrad_eligible(g) || wide_s2_wgrad_eligible(g)))

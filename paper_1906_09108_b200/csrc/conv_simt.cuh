@@ -220,31 +220,34 @@ __global__ void wgrad_reduce_kernel(const float* __restrict__ partial, float* __
 
 // The same sum for many partial rows of a short vector (one row per image): a block takes 32 consecutive outputs,
 // its 16 warps every 16th row (a warp reads 128 contiguous bytes of a row), and the 16 partial sums of an output are
-// added in warp order, so the result does not depend on scheduling.
+// added in warp order, so the result does not depend on scheduling.  Sum = double where the rows themselves hold sums that
+// were formed in fp64 (hundreds of rows added in fp32 would lose what those kept).
+template <typename Sum>
 __global__ void __launch_bounds__(512) wgrad_reduce_tall_kernel(const float* __restrict__ partial, float* __restrict__ grad,
                                                                 size_t n, int splits) {
-  __shared__ float part[16][33];
+  __shared__ Sum part[16][33];
   grid_dependency_wait();
   const int col = threadIdx.x & 31, rg = threadIdx.x >> 5;
   const size_t i = (size_t)blockIdx.x * 32 + col;
-  float a = 0.f;
+  Sum a = 0;
   if (i < n) {
 #pragma unroll 4
-    for (int z = rg; z < splits; z += 16) a += partial[(size_t)z * n + i];
+    for (int z = rg; z < splits; z += 16) a += (Sum)partial[(size_t)z * n + i];
   }
   part[rg][col] = a;
   __syncthreads();
   if (rg == 0 && i < n) {
-    float t = 0.f;
+    Sum t = 0;
 #pragma unroll
     for (int r = 0; r < 16; ++r) t += part[r][col];
-    grad[i] = t;
+    grad[i] = (float)t;
   }
 }
 // grad = the sum of `splits` partial rows of n floats, on stream st.
+template <typename Sum = float>
 inline cudaError_t launch_wgrad_reduce(cudaStream_t st, const float* partial, float* grad, size_t n, int splits) {
   if (splits >= 32 && n <= (size_t)1 << 16) {
-    return launch_chained(wgrad_reduce_tall_kernel, dim3((unsigned)((n + 31) / 32)), dim3(512), 0, st, partial, grad, n, splits);
+    return launch_chained(wgrad_reduce_tall_kernel<Sum>, dim3((unsigned)((n + 31) / 32)), dim3(512), 0, st, partial, grad, n, splits);
   }
   int blocks = (int)((n + 255) / 256); if (blocks > 1184) blocks = 1184;
   return launch_chained(wgrad_reduce_kernel, blocks, 256, 0, st, partial, grad, n, splits);

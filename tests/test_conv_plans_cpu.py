@@ -43,11 +43,14 @@ def test_weight_gradient_plans_fit_shared_memory(tmp_path):
     _run(tmp_path, r"""
   shapes([](const ConvGeom& g) {
     if (!direct::wgrad_direct_supported(g)) return;
-    const direct::WgradParams p = direct::wgrad_params(g);
-    const size_t bytes = direct::wgrad_smem_bytes(p, g.R);
-    if (bytes > direct::kWgradSmemMax) report("shared memory", g, bytes);
-    if (p.rg < 1 || p.rg * p.tt > p.threads || p.threads > direct::kThreads) report("threads", g, (size_t)p.threads);
-    if (p.TH < 1 || p.TH * p.strips < g.P || p.units != g.N * p.strips || p.splits < 1) report("rows", g, (size_t)p.TH);
+    for (int by_row = 0; by_row < 2; ++by_row) {
+      const direct::WgradParams p = direct::wgrad_params(g, by_row != 0);
+      const size_t bytes = direct::wgrad_smem(p, g.R, g.stride, p.TH, by_row != 0);
+      if (bytes > direct::kWgradSmemMax) report("shared memory", g, bytes);
+      if (p.rg < 1 || p.rg * p.tt > p.threads || p.threads > direct::kThreads) report("threads", g, (size_t)p.threads);
+      if (p.rows_x != (p.TH - 1) * g.stride + g.R) report("rows of x", g, (size_t)p.rows_x);
+      if (p.TH < 1 || p.TH * p.strips < g.P || p.units != g.N * p.strips || p.splits < 1) report("rows", g, (size_t)p.TH);
+    }
   });""")
 
 

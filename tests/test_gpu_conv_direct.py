@@ -53,3 +53,24 @@ def test_statistics_rows_of_the_stem(shape):
     want = torch.cat([yd.sum(0), (yd * yd).sum(0)]).cpu().numpy()
     scale = np.concatenate([yd.abs().sum(0).cpu().numpy(), want[co:]])
     assert np.max(np.abs(got - want) / scale) < 1e-5
+
+
+@pytest.mark.parametrize("shape", [(1, 16, 16, 3, 16, 3, 1, 1),       # a row per group of threads: the groups' sums
+                                   (1, 12, 12, 36, 36, 3, 1, 1),      # four rows per group: a thread's own sums
+                                   (1, 16, 16, 16, 24, 1, 2, 0)])     # a projection
+def test_bf16_weight_gradients_add_rows_in_64_bits(shape):
+    """A large row, small ones, and the large one's negative (one block takes the image): the small rows are what is left,
+    to the last bit.  Sums of rows in fp32 lose all of them (2^30 has steps of 128)."""
+    from oracle import layers as L
+    from paper_1906_09108_b200 import binding as B
+    n, h, w, ci, co, r, st, pad = shape
+    ops = B.ConvOps(B.FDG_BF16_TC)
+    s = B.fdg_conv_shape(n, h, w, ci, co, r, st, pad)
+    p, q = ops.out_hw(s)
+    x, dy = np.ones((n, h, w, ci)), np.ones((n, p, q, co))
+    dy[:, 0] = dy[:, -1] = 0
+    dy[:, 0, q // 2], dy[:, -1, q // 2] = 2.0 ** 30, -2.0 ** 30
+    want = L.conv2d_backward(dy, x, np.zeros((co, r, r, ci)), st, pad)[1]
+    got = ops.wgrad(s, torch.from_numpy(x).cuda().to(ops.dtype), torch.from_numpy(dy).cuda().to(ops.dtype)).cpu().numpy()
+    assert np.array_equal(got, want.astype(np.float32))
+    assert np.abs(want).min() < 2.0 ** 10
