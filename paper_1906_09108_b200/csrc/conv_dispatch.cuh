@@ -274,9 +274,7 @@ inline cudaError_t cached_slab_map(TensorMapCache* cache, const void* act, int N
 inline cudaError_t run_wgrad_wide(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int Ci, int Co,
                                   const bf16_t* x, const bf16_t* dy, float* dw, float* scratch, int* err_dev, int R = 3,
                                   int x_sub = 1) {
-  // The module's share of the SMs: a CTA ends with writing up to 245 KB of partial sums, which a finer split multiplies
-  // (ResNet-18, K = 2: 1.68 ms per iteration on all SMs, 1.61 on half, 1.63 on a quarter; WRN-28-10: 6.10, 6.11, 6.54).
-  const wide::WideParams p = wide::wide_params(N, H, W, Ci, Co, cached_sm_count(cache) / (cache->share > 0 ? cache->share : 1), R);
+  const wide::WideParams p = wide::wide_params(N, H, W, Ci, Co, cached_sm_count(cache), R, cache->share);
   const CUtensorMap *mx, *my;
   cudaError_t e = cached_slab_map(cache, x, N, H, W, Ci, p.xw, p.S, &mx, x_sub);
   if (e == cudaSuccess) e = cached_slab_map(cache, dy, N, H, W, Co, p.Wk, p.S, &my);

@@ -1,5 +1,6 @@
-// Weight gradient of 3x3 / stride 1 / pad 1 convolutions of WIDE layers (128 channels and more), and of 1x1
-// convolutions (projection shortcuts, 64 channels and more), on the sm_100a tensor cores, on exact pixel tiles:
+// Weight gradient of the 3x3 / stride 1 / pad 1 convolutions that the halo-tile kernel does not take (128 channels and
+// more, image sizes or channel counts past its tiles), and of 1x1 convolutions (projection shortcuts, 64 channels and
+// more on both sides), on the sm_100a tensor cores, on exact pixel tiles:
 //
 //   dW[co][r][s][ci] = sum over pixels (n,h,w) of dY[n][h][w][co] * X[n][h+r-1][w+s-1][ci]          (3x3)
 //   dW[co][ci]       = sum over pixels (n,h,w) of dY[n][h][w][co] * X[n][h][w][ci]                  (1x1)
@@ -254,9 +255,20 @@ inline int wide_nci(int Ci) {
   return ((Ci + k - 1) / k + 15) / 16 * 16;
 }
 
+// Instructions with pixels in them that a CTA adds into an accumulator, as far as a coarser split goes: see wide_params.
+constexpr int kShareSteps = 256;
 // R = 3: x and dy are [N][H][W][.]; R = 1: dy is [N][H][W][Co] and x the tensor of the same pixels (for stride 2, the
 // even pixels of the layer input, see make_slab_map).
-inline WideParams wide_params(int N, int H, int W, int Ci, int Co, int sm_count, int R = 3) {
+//
+// Blocks along the pixels.  A launch alone takes every SM.  With `share` kernels side by side a split for its share of the
+// SMs does less: a CTA ends with writing up to 245 KB of partial sums, which a finer split multiplies (ms per iteration
+// with every launch on all SMs / this rule: ResNet-18 K = 2 1.68 / 1.63, K = 3 1.66 / 1.59, K = 4 1.65 / 1.53; WRN-16-4 on
+// 24x24 1.032 / 1.023, 0.932 / 0.906, 0.964 / 0.963).  But tensor memory truncates at every instruction, an error that
+// grows with the pixels of an accumulator: 5.9e-6 for 160 channels on 128 32x32 images over the whole GPU, 2.4e-5 on a
+// quarter of it (where WRN-28-10, K = 4, took 5.85 ms instead of 6.00).  So the split gets coarser only as far as an
+// accumulator takes at most kShareSteps instructions: the error that the 64-, 320- and 640-channel layers have over the
+// whole GPU (4.1 to 4.4e-6).
+inline WideParams wide_params(int N, int H, int W, int Ci, int Co, int sm_count, int R = 3, int share = 1) {
   WideParams p{};
   p.N = N; p.H = H; p.W = W; p.Ci = Ci; p.Co = Co;
   p.nci = wide_nci(Ci);
@@ -284,11 +296,9 @@ inline WideParams wide_params(int N, int H, int W, int Ci, int Co, int sm_count,
   p.tmem_cols = cols;
   const int tiles = p.co_blocks * p.ci_chunks * p.rdim;
   const int sms = sm_count > 0 ? sm_count : 148;
-  int splits = sms / tiles;
-  if (splits < 1) splits = 1;
-  if (splits > 32) splits = 32;
-  if (splits > p.slabs) splits = p.slabs;
-  p.splits = splits;
+  auto splits_on = [&](int n) { return std::min(std::max(n / tiles, 1), std::min(32, p.slabs)); };
+  const int slabs_at_most = std::max(kShareSteps / ((std::min(p.S, H) * p.Wk + 15) / 16), 1);    // rows past the image add nothing
+  p.splits = std::max(splits_on(sms / std::max(share, 1)), std::min(splits_on(sms), (p.slabs + slabs_at_most - 1) / slabs_at_most));
   return p;
 }
 inline size_t wide_smem_bytes(const WideParams& p) {

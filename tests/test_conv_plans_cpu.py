@@ -1,6 +1,7 @@
-"""The CUDA-core convolutions' plans, without a GPU: whatever shape the dispatcher hands them, the launch they plan stays
-within the shared memory that the kernels are given and covers the whole problem.  A small host program made from the
-library's own header walks the shapes."""
+"""Launch plans without a GPU: whatever shape the dispatcher hands to the CUDA-core convolutions, the launch they plan stays
+within the shared memory that the kernels are given and covers the whole problem; and the split of the wide weight
+gradients bounds what an accumulator adds up.  A small host program made from the library's own headers walks the
+shapes."""
 import os
 import subprocess
 
@@ -8,8 +9,10 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 PROLOGUE = r"""
 #include <cstdio>
+#include <cuda.h>
 #include "fdg_ops.h"
 #include "conv_direct.cuh"
+#include "wgrad_wide.cuh"
 using namespace fdg;
 static int bad = 0;
 static void report(const char* what, const ConvGeom& g, size_t bytes) {
@@ -69,3 +72,25 @@ def test_forward_and_data_gradient_plans_fit_shared_memory(tmp_path):
       }
     }
   });""")
+
+
+def test_a_share_of_the_gpu_lengthens_no_long_accumulation(tmp_path):
+    """An accumulator's rounding error grows with its instructions: sharing the SMs may bring them up to 256, beyond that
+    the split is the whole GPU's; and never finer than that one, for which the scratch is sized."""
+    _run(tmp_path, r"""
+  const int chans[] = {8, 64, 128, 160, 256, 320, 512, 640};
+  for (int R = 1; R <= 3; R += 2) for (int N : {1, 8, 128, 2048}) for (int H : {4, 6, 8, 13, 16, 24, 32, 64})
+    for (int ci : chans) for (int co : chans) {
+      const ConvGeom g{N, H, H, ci, H, H, co, R, R, 1, R / 2};
+      if (!wide::wide_supported(N, H, H, ci, co, R)) continue;
+      const wide::WideParams whole = wide::wide_params(N, H, H, ci, co, 148, R);
+      for (int share = 1; share <= 16; ++share) {
+        const wide::WideParams p = wide::wide_params(N, H, H, ci, co, 148, R, share);
+        auto steps = [](const wide::WideParams& q) {      // instructions with pixels in them
+          const int rows = q.S < q.H ? q.S : q.H;
+          return (q.slabs + q.splits - 1) / q.splits * ((rows * q.Wk + 15) / 16);
+        };
+        if (p.splits < 1 || p.splits > whole.splits) report("splits", g, (size_t)p.splits);
+        if (steps(p) > 256 && steps(p) > steps(whole)) report("instructions", g, (size_t)steps(p));
+      }
+    }""")
