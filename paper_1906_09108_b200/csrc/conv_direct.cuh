@@ -382,12 +382,9 @@ template <typename T, int VEC, int STRIDE, int NC, bool FLIP>
 inline cudaError_t conv_launch_one(cudaStream_t st, const ConvParams& p, int grid, const T* act, const T* wgt, T* out,
                                    const T* res, const T* mask, const Reduce<T>& red, const EpiAffine& aff) {
   auto kernel = direct_conv_kernel<T, VEC, STRIDE, NC, FLIP>;
-  static bool set = false;                                   // raised once; a launch may be a recorded one
-  if (!set) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kConvSmemMax);
-    if (e != cudaSuccess) return e;
-    set = true;
-  }
+  static OncePerDevice once;
+  const cudaError_t e = once_per_device(&once, [&]() { return set_smem_limit(kernel, kConvSmemMax); });
+  if (e != cudaSuccess) return e;
   return launch_chained(kernel, dim3(grid, (p.Cn + p.cb - 1) / p.cb), dim3(kThreads), conv_smem_bytes(p), st, p, act, wgt, out, res, mask, red, aff);
 }
 
@@ -693,12 +690,9 @@ inline size_t wgrad_direct_scratch_elems(const ConvGeom& g, bool by_row) {
 template <typename T, int VX, int VY, int R, int STRIDE>
 inline cudaError_t wgrad_launch_one(cudaStream_t st, const WgradParams& p, const T* x, const T* dy, float* dst) {
   auto kernel = direct_wgrad_kernel<T, VX, VY, R, STRIDE>;
-  static bool set = false;
-  if (!set) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgradSmemMax);
-    if (e != cudaSuccess) return e;
-    set = true;
-  }
+  static OncePerDevice once;
+  const cudaError_t e = once_per_device(&once, [&]() { return set_smem_limit(kernel, kWgradSmemMax); });
+  if (e != cudaSuccess) return e;
   const int pairs = p.ci_blocks * ((p.Co + p.cob - 1) / p.cob);
   return launch_chained(kernel, dim3(p.splits, pairs), dim3(p.threads), wgrad_smem(p, R, STRIDE, p.TH, kByRow<T>), st, p, x, dy, dst);
 }

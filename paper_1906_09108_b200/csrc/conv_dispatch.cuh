@@ -26,12 +26,21 @@ struct TensorMapCache {
     bool operator<(const Key& o) const { return std::memcmp(this, &o, sizeof(Key)) < 0; }
   };
   std::map<Key, CUtensorMap> maps;
-  int sm_count = 0;
+  int device = 0, sm_count = 0;   // the device the cache is for; 0 SMs: not asked yet (cached_sm_count)
   int share = 1;        // kernels expected to run side by side (one per module stream): a launch takes
                         // about sm_count / share CTAs and walks its tiles with them
   int wgrad_side_cap = 0;   // upper bound of the pixel split of a weight gradient issued beside the stream that
                             // needs its inputs' other consumers (0 = none), see halo::wgrad_ctas
 };
+
+inline int cached_sm_count(TensorMapCache* cache) {
+  if (cache->sm_count == 0) {
+    cudaGetDevice(&cache->device);
+    cudaDeviceGetAttribute(&cache->sm_count, cudaDevAttrMultiProcessorCount, cache->device);
+  }
+  return cache->sm_count;
+}
+inline int cached_device(TensorMapCache* cache) { cached_sm_count(cache); return cache->device; }
 
 inline bool tc_eligible(const ConvGeom& g) {
   return g.R == 3 && g.S == 3 && g.stride == 1 && g.pad == 1 && g.P == g.H && g.Q == g.W &&
@@ -44,11 +53,7 @@ inline cudaError_t run_conv_tc(cudaStream_t st, TensorMapCache* cache, int N, in
                                const bf16_t* act, const bf16_t* wgt, bf16_t* out, const bf16_t* res,
                                const bf16_t* res_mask, int* err_dev, int sub = 1, int taps = 9, int act_sub = 1,
                                float* stat_partial = nullptr, int* ctas_out = nullptr, const EpiAffine* affine = nullptr) {
-  if (cache->sm_count == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&cache->sm_count, cudaDevAttrMultiProcessorCount, dev);
-  }
+  const int sm_count = cached_sm_count(cache);
   tc::ConvTcParams p = tc::conv_tc_params(N, H, W, Ck, Cn, taps, cache->share);
   p.sub = sub;
   p.act_sub = act_sub;
@@ -64,20 +69,13 @@ inline cudaError_t run_conv_tc(cudaStream_t st, TensorMapCache* cache, int N, in
     ia = cache->maps.insert({ka, ma}).first;
     ib = cache->maps.insert({kb, mb}).first;
   }
-  return tc::conv_tc_launch(st, p, ia->second, ib->second, out, res, res_mask, err_dev, cache->sm_count, stat_partial, ctas_out, affine);
+  const cudaError_t e = tc::conv_tc_set_attrs(cached_device(cache));
+  if (e != cudaSuccess) return e;
+  return tc::conv_tc_launch(st, p, ia->second, ib->second, out, res, res_mask, err_dev, sm_count, stat_partial, ctas_out, affine);
 }
 
 
 // ---- halo-tile kernels (16/32/64-channel layers) ------------------------------------------
-inline int cached_sm_count(TensorMapCache* cache) {
-  if (cache->sm_count == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&cache->sm_count, cudaDevAttrMultiProcessorCount, dev);
-  }
-  return cache->sm_count;
-}
-
 inline bool halo_shape(const ConvGeom& g) {
   return g.R == 3 && g.S == 3 && g.stride == 1 && g.pad == 1 && g.P == g.H && g.Q == g.W;
 }
@@ -172,7 +170,7 @@ inline cudaError_t run_conv_halo(cudaStream_t st, TensorMapCache* cache, int N, 
   const CUtensorMap *mx, *mw;
   cudaError_t e = cached_tile_map(cache, act, N, H, W, Ck, p.G, &mx);
   if (e == cudaSuccess) e = cached_weight_map(cache, wgt, Ck, Cn, &mw);
-  if (e == cudaSuccess) e = halo::set_smem_attrs();
+  if (e == cudaSuccess) e = halo::set_smem_attrs(cached_device(cache));
   if (e != cudaSuccess) return e;
   // the fewest CTAs that keep the number of tiles of the busiest one at ceil(tiles / sms)
   const int per_cta = (p.tiles + sms - 1) / sms;
@@ -226,7 +224,7 @@ inline cudaError_t run_conv_rows(cudaStream_t st, TensorMapCache* cache, int N, 
   mr = mx = mo;
   if (er == cudaSuccess && res) er = cached_group_map(cache, res, N, H, W, C, rows::kTileGroups, rows::kTileRows, &mr);
   if (er == cudaSuccess && mode == 2) er = cached_group_map(cache, red->xprev, N, H, W, C, rows::kTileGroups, rows::kTileRows, &mx);
-  if (er == cudaSuccess) er = rows::set_attrs();
+  if (er == cudaSuccess) er = rows::set_attrs(cached_device(cache));
   if (er != cudaSuccess) return er;
   if (ctas_out) *ctas_out = grid;
   return launch_chained(rows::kernel_of(C, mode, res != nullptr), grid, rows::kThreads, rows::rows_smem_bytes(p), st, *ma, *mw, *mo, *mr, *mx, p, e, err_dev);
@@ -241,7 +239,7 @@ inline cudaError_t run_wgrad_halo(cudaStream_t st, TensorMapCache* cache, int N,
   const CUtensorMap *mx, *my;
   cudaError_t e = cached_tile_map(cache, x, N, H, W, Ci, p.G, &mx, p.kcx);
   if (e == cudaSuccess) e = cached_tile_map(cache, dy, N, H, W, Co, p.G, &my, p.kcy);
-  if (e == cudaSuccess) e = halo::set_smem_attrs();
+  if (e == cudaSuccess) e = halo::set_smem_attrs(cached_device(cache));
   if (e != cudaSuccess) return e;
   const int ctas = halo::wgrad_ctas(p, side ? cache->wgrad_side_cap : 0);
   e = launch_chained(halo::wgrad_halo_kernel, dim3(ctas, halo::wgrad_pairs(p)), dim3(halo::kFwdThreads), halo::wgrad_smem_bytes(p), st,
@@ -278,7 +276,7 @@ inline cudaError_t run_wgrad_wide(cudaStream_t st, TensorMapCache* cache, int N,
   const CUtensorMap *mx, *my;
   cudaError_t e = cached_slab_map(cache, x, N, H, W, Ci, p.xw, p.S, &mx, x_sub);
   if (e == cudaSuccess) e = cached_slab_map(cache, dy, N, H, W, Co, p.Wk, p.S, &my);
-  if (e == cudaSuccess) e = wide::wide_set_attrs();
+  if (e == cudaSuccess) e = wide::wide_set_attrs(cached_device(cache));
   if (e != cudaSuccess) return e;
   const dim3 grid(p.co_blocks * p.ci_chunks * p.rdim, p.splits);
   auto kernel = R == 3 ? wide::wgrad_wide_kernel<3> : wide::wgrad_wide_kernel<1>;

@@ -932,13 +932,12 @@ inline cudaError_t make_weight_map(const void* wgt, int Ck, int Cn, CUtensorMap*
   return cudaSuccess;
 }
 
-inline cudaError_t set_smem_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(conv_halo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 8192);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(wgrad_halo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 8192);
-  if (e == cudaSuccess) done = true;
-  return e;
+inline cudaError_t set_smem_attrs(int dev) {
+  static OncePerDevice once;
+  return once.run(dev, []() {
+    const cudaError_t e = set_smem_limit(conv_halo_kernel, kSmemBudget + 8192);
+    return e != cudaSuccess ? e : set_smem_limit(wgrad_halo_kernel, kSmemBudget + 8192);
+  });
 }
 
 }  // namespace halo

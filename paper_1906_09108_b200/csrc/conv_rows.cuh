@@ -514,17 +514,15 @@ inline RowsKernel kernel_of(int C, int mode, bool res) {
   return C == 16 ? kernel_of<16>(mode, res) : (C == 32 ? kernel_of<32>(mode, res) : kernel_of<64>(mode, res));
 }
 
-inline cudaError_t set_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  for (int c = 16; c <= 64; c *= 2)
-    for (int mode = 0; mode < 4; ++mode)
-      for (int res = 0; res < 2; ++res) {
-        const cudaError_t e = cudaFuncSetAttribute(kernel_of(c, mode, res != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-        if (e != cudaSuccess) return e;
-      }
-  done = true;
-  return cudaSuccess;
+inline cudaError_t set_attrs(int dev) {
+  static OncePerDevice once;
+  return once.run(dev, []() {
+    cudaError_t e = cudaSuccess;
+    for (int c = 16; c <= 64; c *= 2)
+      for (int mode = 0; mode < 4; ++mode)
+        for (int res = 0; res < 2 && e == cudaSuccess; ++res) e = set_smem_limit(kernel_of(c, mode, res != 0), kSmemLimit);
+    return e;
+  });
 }
 
 }  // namespace rows

@@ -739,16 +739,14 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 inline EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+  static const EncodeTiledFn fn = []() -> EncodeTiledFn {    // one thread looks it up, the others wait for it
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
+      return reinterpret_cast<EncodeTiledFn>(p);
+    return nullptr;
+  }();
   return fn;
 }
 
@@ -862,15 +860,13 @@ inline cudaError_t conv_tc_make_maps(const ConvTcParams& p, const void* act, con
   return cudaSuccess;
 }
 
-// The kernel's dynamic shared memory exceeds the default limit: raised once (also callable up front, so
-// that the first launch may happen inside a stream capture).
-inline cudaError_t conv_tc_set_attrs() {
-  static bool attr_set = false;
-  if (attr_set) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(conv3x3_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(conv3x3_patch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  if (e == cudaSuccess) attr_set = true;
-  return e;
+// The kernels' dynamic shared memory exceeds the default limit: called before the first launch on device `dev`.
+inline cudaError_t conv_tc_set_attrs(int dev) {
+  static OncePerDevice once;
+  return once.run(dev, []() {
+    const cudaError_t e = set_smem_limit(conv3x3_tc_kernel, 200 * 1024);
+    return e != cudaSuccess ? e : set_smem_limit(conv3x3_patch_kernel, 200 * 1024);
+  });
 }
 
 // `stat_partial` (nullable): room for one row of 2 * Co floats per CTA (at most sm_count rows); *ctas_out = rows written.
@@ -880,10 +876,6 @@ inline cudaError_t conv_tc_launch(cudaStream_t st, const ConvTcParams& p, const 
                                   float* stat_partial = nullptr, int* ctas_out = nullptr, const EpiAffine* affine = nullptr) {
   const EpiAffine aff = affine ? *affine : EpiAffine{};
   const size_t smem = conv_tc_smem_bytes(p);
-  {
-    cudaError_t e = conv_tc_set_attrs();
-    if (e != cudaSuccess) return e;
-  }
   if (p.patch) {
     const int tiles = p.N * (p.H / kPatch) * (p.W / kPatch) * p.n_tiles;
     const int grid = tiles < sm_count ? tiles : sm_count;

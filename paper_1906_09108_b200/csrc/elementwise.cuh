@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "once_per_device.h"
+
 namespace fdg {
 
 // ------------------------------------------------ programmatic dependent launch --
@@ -35,6 +37,19 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Makes a setting of the current device (see OncePerDevice).  Setting a function attribute is no stream operation: a launch
+// may be a recorded one.
+template <typename Work>
+inline cudaError_t once_per_device(OncePerDevice* once, Work work) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e : once->run(dev, work);
+}
+template <typename Kernel>
+inline cudaError_t set_smem_limit(Kernel kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // A batch norm with given statistics (inference) applied in the epilogue of the convolution that produces its input:

@@ -1295,9 +1295,10 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
     }
   }
   // shared-memory limits of the tensor-core kernels, raised here so that a kernel's first launch may be a recorded one
-  if (e == cudaSuccess && c->bf16_mode) e = halo::set_smem_attrs();
-  if (e == cudaSuccess && c->bf16_mode) e = rows::set_attrs();
-  if (e == cudaSuccess && c->bf16_mode) e = tc::conv_tc_set_attrs();
+  if (e == cudaSuccess && c->bf16_mode) e = halo::set_smem_attrs(c->device);
+  if (e == cudaSuccess && c->bf16_mode) e = rows::set_attrs(c->device);
+  if (e == cudaSuccess && c->bf16_mode) e = tc::conv_tc_set_attrs(c->device);
+  if (e == cudaSuccess && c->bf16_mode) e = wide::wide_set_attrs(c->device);
   c->own_streams = streams == nullptr;
   for (int k = 0; k < c->K && e == cudaSuccess; ++k) {
     Module& m = c->mods[k];

@@ -336,13 +336,12 @@ inline cudaError_t make_slab_map(const void* act, int N, int H, int W, int C, in
   return cudaSuccess;
 }
 
-inline cudaError_t wide_set_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(wgrad_wide_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmemBudget + 8192);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(wgrad_wide_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmemBudget + 8192);
-  if (e == cudaSuccess) done = true;
-  return e;
+inline cudaError_t wide_set_attrs(int dev) {
+  static OncePerDevice once;
+  return once.run(dev, []() {
+    const cudaError_t e = set_smem_limit(wgrad_wide_kernel<3>, kWideSmemBudget + 8192);
+    return e != cudaSuccess ? e : set_smem_limit(wgrad_wide_kernel<1>, kWideSmemBudget + 8192);
+  });
 }
 
 }  // namespace wide
