@@ -360,7 +360,7 @@ inline ConvParams conv_params(const ConvGeom& g, bool dgrad, int nc) {
   p.pitch = ((p.segs * kPx - 1) * stride + 3 + 3) / 4 * 4;
   if (p.pitch < p.Wi * p.up + 2) p.pitch = (p.Wi * p.up + 2 + 3) / 4 * 4;
   while (rows > 1 && (size_t)kKc * (rows * stride + 2) * p.pitch * 4 > 96 * 1024) rows /= 2;
-  if (rows >= p.P) { p.TH = p.P; p.TI = std::max(1, std::min(rows / p.P, p.N / 148)); }
+  if (rows >= p.P) { p.TH = p.P; p.TI = std::max(1, std::min(rows / p.P, p.N / kSms)); }
   else { const int t = (p.P + rows - 1) / rows; p.TH = (p.P + t - 1) / t; p.TI = 1; }
   p.rows_in = (p.TH - 1) * stride + 3;
   // Every image of a tile has border rows of its own, which the bound above does not count: images of one or two rows
@@ -395,18 +395,19 @@ inline cudaError_t launch_conv(cudaStream_t st, const ConvGeom& g, bool dgrad, c
                                const T* mask, const Reduce<T>* red, int* nparts, uint64_t* launches,
                                const EpiAffine* affine = nullptr) {
   // With 8 channels per thread 8 shared-memory loads serve 96 multiply-adds, with 4 channels 5 serve 48; 4 where 8 would
-  // leave an SM fewer than four warps.  (Packed two-wide multiply-adds were tried: the moves that form their operand
-  // pairs go through the same pipe, no gain.)
+  // leave an SM fewer than four warps (fp32, 128 images, 8 / 4 channels per thread: 16 channels on 32x32, 14 warps per SM,
+  // 22.3 / 24.9 us; 32 on 16x16, 7 warps, 25.3 / 24.2; 64 on 8x8, 3.5 warps, 46.4 / 30.9).  (Packed two-wide multiply-adds were
+  // tried: the moves that form their operand pairs go through the same pipe, no gain.)
   const long pixels4 = (long)g.N * (dgrad ? g.H : g.P) * (((dgrad ? g.W : g.Q) + kPx - 1) / kPx);
   const int cn = dgrad ? g.Ci : g.Co;
-  const bool wide = cn % 8 == 0 && pixels4 * (cn / 8) >= 148L * 128;
+  const bool wide = cn % 8 == 0 && pixels4 * (cn / 8) >= (long)kSms * 128;
   ConvParams p = conv_params(g, dgrad, wide ? 8 : 4);
   p.wvec = g.Ci % 4 == 0 && (reinterpret_cast<uintptr_t>(wgt) & 15) == 0;   // contiguous along Ci either way
   p.vec = cn % 4 == 0 && ((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(res) | reinterpret_cast<uintptr_t>(mask) |
                            (red ? reinterpret_cast<uintptr_t>(red->mask) | reinterpret_cast<uintptr_t>(red->xprev) : 0)) & 15) == 0;
   if (red && red->mode == 2 && !p.vec) red = nullptr;
   int grid = p.tiles;
-  const int cap = red ? kMaxRows : 4 * 148;
+  const int cap = red ? kMaxRows : 4 * kSms;
   if (grid > cap) { const int per = (grid + cap - 1) / cap; grid = (grid + per - 1) / per; }
   const bool vec = p.Ck % 4 == 0 && (reinterpret_cast<uintptr_t>(act) & 15) == 0;
   Reduce<T> r{};
@@ -665,19 +666,23 @@ inline WgradParams wgrad_params(const ConvGeom& g, bool by_row) {
   p.TH = (g.P + p.strips - 1) / p.strips;
   p.units = g.N * p.strips;
   p.rows_x = (p.TH - 1) * g.stride + g.R;
-  // Blocks along the pixels: the number that leaves the busiest SM the fewest steps (up to two blocks share an SM), as long as the partial sums stay below about twice the operands (they are written and read again).
+  // Blocks along the pixels: the number that leaves the busiest SM the fewest steps (up to two blocks share an SM), as long as
+  // the partial sums stay below about twice the operands (they are written and read again).  A block alone on its SM waits
+  // for its loads: fp32, 16 channels, 128 images of 32x32, 28.7 us on 148 blocks of 7 steps, 22.3 us on 296 of 4, i.e. 1.47
+  // times as long a step; 512 images 107 us (28 steps) and 73.4 us (14), 1.46.  Counted as 1.3: with 1.47 the 64-channel
+  // layers would take 208 blocks instead of 148, 26.9 us instead of 27.0, and 40 % more partial sums.
   const int pairs = p.ci_blocks * co_blocks;
   const size_t outs = (size_t)g.Co * g.R * g.R * g.Ci;
   const size_t operands = (size_t)g.N * ((size_t)g.H * g.W * g.Ci + (size_t)g.P * g.Q * g.Co);
   int most = (int)std::min<size_t>(std::max<size_t>(2 * operands / outs, 1), (size_t)p.units);
-  most = std::min(most, std::max(1, 2 * 148 / pairs));
+  most = std::min(most, std::max(1, 2 * kSms / pairs));
   int best = 1;
   long best_cost = -1;
   for (int sp = 1; sp <= most; ++sp) {
     const int per = (p.units + sp - 1) / sp;
     if ((p.units + per - 1) / per != sp) continue;
-    const int blocks_per_sm = (sp * pairs + 147) / 148;
-    const long cost = (long)per * blocks_per_sm * (blocks_per_sm == 1 ? 13 : 10);    // a block alone on its SM waits for its loads
+    const int blocks_per_sm = (sp * pairs + kSms - 1) / kSms;
+    const long cost = (long)per * blocks_per_sm * (blocks_per_sm == 1 ? 13 : 10);
     if (best_cost < 0 || cost < best_cost) { best = sp; best_cost = cost; }
   }
   p.splits = best;

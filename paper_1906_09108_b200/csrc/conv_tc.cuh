@@ -757,7 +757,9 @@ inline CUtensorMapSwizzle swizzle_for(int row_bytes) {
 // Can this convolution run on the tensor-core kernel?  (3x3, stride 1, pad 1, or 1x1, on an H x W grid of `pixels`
 // stored outputs in all; channel counts that are multiples of 8 -- a pixel is then a whole number of 16-byte TMA units --
 // and image rows of at most 128 pixels.)  Channel counts that fill no K step of 16 are left to the CUDA cores where the
-// output is one accumulator tile or less: such a launch is latency, and the tensor cores' set-up is the longer one.
+// output is one accumulator tile or less.  That is latency: 3x3 on 128 pixels, CUDA cores / tensor cores, 8 -> 8 channels
+// 5.5 / 7.7 us, 8 -> 16 5.8 / 7.9 us forward and 7.1 / 7.9 us backward; but 1x1 8 -> 16 5.7 / 4.1 us, 24 channels 10.8 / 8.2 us,
+// 72 26.3 / 13.0 us: the line is right for 3x3 filters of 8 channels only.
 inline bool conv_tc_supported(int N, int H, int W, int Ci, int Co, size_t pixels) {
   if (Ci % 8 || Co % 8 || Ci < 8 || Co < 8 || N < 1) return false;
   if ((Ci % 16 || Co % 16) && pixels <= (size_t)kTileM) return false;
@@ -794,7 +796,8 @@ inline ConvTcParams conv_tc_params(int N, int H, int W, int Ci, int Co, int taps
   // 128-row tiles -- unless the layer has so few pixels (small images, many channels) that the tiles would leave
   // most SMs idle: then single 128-row tiles and narrower column tiles, down to 64, until there are about 96, or, with
   // `share` kernels running side by side, its share of them: wider tiles read fewer operand bytes in all, and the SMs
-  // left over do the other modules' work (ResNet-18, K = 2: 1.82 -> 1.70 ms per iteration; WRN-16-4 on 24x24: 1.10 -> 1.04).
+  // left over do the other modules' work (ms per iteration, 96 at every K / 96 / K: ResNet-18 K = 2 1.81 / 1.63, K = 3
+  // 1.76 / 1.55, K = 4 1.74 / 1.51; WRN-16-4 on 24x24 1.11 / 1.03, 0.99 / 0.91, 1.06 / 0.96; WRN-28-10 within 1 % at any K).
   p.mpair = p.m_tiles >= 2 ? 2 : 1;
   if (!p.patch) {
     auto tiles = [&]() { return ((p.m_tiles + p.mpair - 1) / p.mpair) * ((Co + nt - 1) / nt); };

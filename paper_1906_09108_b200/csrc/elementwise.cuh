@@ -52,6 +52,10 @@ inline cudaError_t set_smem_limit(Kernel kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// SMs of a B200.  Splits whose rows need scratch are planned for this number, not for the device's own: the size of the
+// workspace is asked for without a device.
+constexpr int kSms = 148;
+
 // A batch norm with given statistics (inference) applied in the epilogue of the convolution that produces its input:
 // the convolution's output is rounded to the storage type first, as if it had been stored, so that the result is that of
 // bn_apply_kernel bit for bit.  stats null: none.
