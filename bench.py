@@ -217,7 +217,7 @@ STEP_VARIANTS = {
     "fprop_stats": "forward + batch-norm statistics of its output (conv1, conv2 of a block)",
     "dgrad_bn": "data gradient + the sums of the batch-norm backward it feeds (conv2's data gradient)",
     "dgrad_res_bn": "data gradient + gated residual + those sums (the block-input gradient of an identity block)",
-    "wgrad_side": "weight gradient with its pixel split capped at 16 CTAs (side stream)",
+    "wgrad_side": "weight gradient with its pixel split as on a side stream of the step: four images per CTA, at least 16 CTAs",
 }
 
 
@@ -246,7 +246,8 @@ def kernel_bench(B, which="fprop", stage="stage1", launches=64, reps=5, use_grap
     extra = None
     extra_tensors = 0
     if variant:
-        ex, keep = ops._extra(s, share=4, wgrad_cta_cap=16 if variant == "wgrad_side" else 0,
+        # the module-step's launch shapes at K = 4; its side-stream weight gradients take four images per CTA, at least 16 CTAs
+        ex, keep = ops._extra(s, share=4, wgrad_cta_cap=max(16, (n + 3) // 4) if variant == "wgrad_side" else 0,
                               reduce={"fprop_stats": 1, "dgrad_bn": 2, "dgrad_res_bn": 2, "wgrad_side": 0}[variant],
                               next_mask=xs[0], next_x=xs[0], next_stats=torch.zeros(2 * c, device="cuda") + 1.0, C_red=c)
         extra = B.C.byref(ex)

@@ -35,8 +35,9 @@ typedef struct {
  *   share          launch shape: the tensor-core kernel takes about (SM count / share) CTAs and walks
  *                  several image tiles per CTA, as it does when `share` modules run side by side
  *                  (0 or 1: one launch may take every SM).
- *   wgrad_cta_cap  fdg_conv_wgrad: upper bound of the pixel split (0 = none); the module-step issues its
- *                  weight gradients with 16 on a side stream.
+ *   wgrad_cta_cap  fdg_conv_wgrad: upper bound of the halo-tile kernel's pixel split (0 = none); on a side stream the
+ *                  module-step gives it max(16, batch / 4).  (fdg_conv_wgrad takes no `share`: the wide
+ *                  kernel's split is the whole GPU's here.)
  *   dy_spread      stride-2 gradients (bf16): scratch of N*H*W*Co bf16 elements.  With it the data and
  *                  weight gradients of a 3x3 stride-2 layer run as the stride-1 tensor-core kernels on dy
  *                  spread onto the even pixels of the input grid (the call fills it); without it they
@@ -116,11 +117,10 @@ fdg_status fdg_conv_wgrad(int precision, const fdg_conv_shape* shape, const void
  * fdg_conv_wgrad on the CUDA-core path, but the partial sums go to a buffer that is part of the
  * library image: FDG_STATIC_SCRATCH_BYTES of device memory on every GPU that loads the library,
  * held until the process exits.  The call itself allocates and frees nothing.
- *   - The call always takes the CUDA-core kernel, whose slice buffer is what
- *     fdg_conv_wgrad_scratch_bytes reports for FDG_FP32_CUDACORE (for bf16 shapes that fdg_conv_wgrad
- *     would run on the tensor cores the bf16 figure is larger and does not apply here).  Shapes whose
- *     slice buffer exceeds FDG_STATIC_SCRATCH_BYTES are refused with FDG_ERR_WORKSPACE_TOO_SMALL and
- *     nothing is launched.
+ *   - The call always takes the general CUDA-core kernel (an implicit GEMM over pixel slices, added in fp32).  Its
+ *     slice buffer is at most what fdg_conv_wgrad_scratch_bytes reports for FDG_FP32_CUDACORE: that figure
+ *     covers the register-tiled kernel, which fdg_conv_wgrad prefers, as well.  Shapes whose slice buffer
+ *     exceeds FDG_STATIC_SCRATCH_BYTES are refused with FDG_ERR_WORKSPACE_TOO_SMALL and nothing is launched.
  *   - The first call on each device looks up the buffer's device address (a host-side query,
  *     made with that device current); make that first call outside any stream capture.
  *   - All calls on a device share the one buffer, and it keeps what the previous call left.

@@ -868,8 +868,7 @@ inline int wgrad_pairs(const WgradParams& p) { return (p.Ci / p.kcx) * (p.Co / p
 // Pixel split: few enough CTAs that their partial sums (Co*9*Ci floats each) stay small next to
 // the operands, enough of them to spread the reduction over the SMs.  `cap` (0 = none) bounds the
 // split further: beside other kernels a weight gradient that is nobody's next input does better on
-// a few SMs for longer than on many at once (measured: 16 CTAs instead of 64-128 take 9 % off an
-// iteration of four concurrent modules).  Scratch is sized for cap = 0.
+// a few SMs for longer than on many at once (fdg_create chooses it, with the measurements).  Scratch is sized for cap = 0.
 inline int wgrad_ctas(const WgradParams& p, int cap = 0) {
   const int pairs = wgrad_pairs(p);
   int want;

@@ -112,7 +112,7 @@ def test_backward_of_every_block_at_full_size():
     """The backward twin of the test above (Eq. 10 with the shrunk gradient of Eq. 15): ResNet-110, K = 4, batch 128,
     one stream per module plus the side stream of the weight gradients, i.e. the kernels and launch shapes the
     benchmark's graphs replay (a convolution on a quarter of the SMs, the weight gradients' pixel split capped at
-    16 CTAs).  A capture keeps every gradient tensor of each module's backward pass at iteration 2K - 1, the first
+    32 CTAs).  A capture keeps every gradient tensor of each module's backward pass at iteration 2K - 1, the first
     one in which all four modules back-propagate.  Every layer of every block is then recomputed by the oracle
     from the library's own inputs to that layer -- the incoming gradient it captured and the activations it saved
     for that batch, so every ReLU gate is the same on both sides -- and compared element by element at 1e-2: the
