@@ -74,3 +74,12 @@ def test_bf16_weight_gradients_add_rows_in_64_bits(shape):
     got = ops.wgrad(s, torch.from_numpy(x).cuda().to(ops.dtype), torch.from_numpy(dy).cuda().to(ops.dtype)).cpu().numpy()
     assert np.array_equal(got, want.astype(np.float32))
     assert np.abs(want).min() < 2.0 ** 10
+
+
+def test_context_of_64x64_images_fp32():
+    """A network whose projection's weight gradient (1x1, 64x64, 8 -> 32 channels) asks for rows of 19 KB: a whole
+    iteration through the context, to the bar of the fp32 mode."""
+    from tests.fdg_pair import run_pair
+    arch = dict(family="resnet6n2", blocks=(1, 1), widths=(32, 32), stem_width=8, in_h=64, in_w=64, in_c=3, num_classes=10, batch=3)
+    res = run_pair(arch, 1, (), 2, lr=0.01, seed=1)
+    assert max(res["grads"], res["params"], res["loss"]) <= 1e-4, res["grads_by_step"]
