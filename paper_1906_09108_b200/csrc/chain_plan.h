@@ -1,0 +1,80 @@
+// Launch shapes of the runs of identity blocks (conv_chain.cuh): host code alone.
+#pragma once
+#include <stddef.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+namespace fdg {
+namespace chain {
+
+constexpr int kEpiWarps = 16, kEpiThreads = 32 * kEpiWarps;
+constexpr int kAccSlots = 8;                     // accumulators of 128 rows x 64 columns: all of tensor memory
+constexpr int kTileRows = 16, kTileGroups = 8;   // a tile: image rows, groups of 64 / C pixels
+constexpr int kMaxCtas = 148;
+enum Pass { TRAIN = 0, INFER = 1, BACKWARD = 2 };
+
+struct Geom {
+  int N, H, W, WG;            // image; groups per row (W / G)
+  int rb, cb, tpi;            // tiles of an image: row blocks, column blocks, rb * cb
+  int images;                 // per CTA at most; images * tpi <= kAccSlots
+  int layers;                 // convolutions of the run (two per block)
+  uint32_t row_bytes;         // shared memory of one image row: (8 * cb + 2) groups
+  uint32_t a_bytes;           // one image, multiple of 1 KiB
+  uint32_t a_tx;              // bytes its load writes
+  uint32_t w_bytes;           // nine taps, multiple of 1 KiB
+  int w_stages;
+};
+
+// A tile: its first element in a tensor of the layers' shape, its place in the operands, how much of it lies inside the image,
+// its image and that image's first tile.
+struct __align__(16) Tile { uint32_t g, s; uint16_t rows, groups, image, first; };
+
+inline uint32_t round_up(uint32_t x, uint32_t a) { return (x + a - 1) / a * a; }
+constexpr size_t kSmemLimit = 226 * 1024;
+// Two CTAs of such launches must never share an SM: both want all of tensor memory, and each may hold it while the other's
+// launch waits for a CTA elsewhere.  Their registers forbid it already (640 threads of 96); their shared memory does too.
+constexpr size_t kSmemLeast = 120 * 1024;
+inline size_t fixed_smem(int C) {
+  return (size_t)kEpiThreads * 8 + (size_t)kEpiWarps * 2 * C * 4 + (size_t)2 * 5 * C * 4 + (3 * kAccSlots + 2) * 8 + 16 + kAccSlots * sizeof(Tile) + 1024;
+}
+// Launch shape: about `sms` CTAs; images = 0 where the shape is not covered.  A CTA holds its images' operands and accumulators.
+inline Geom chain_geom(int N, int H, int W, int C, int layers, int sms, int pass) {
+  Geom p{};
+  const int G = 64 / C;
+  p.N = N; p.H = H; p.W = W; p.WG = W / G; p.layers = layers;
+  p.rb = (H + kTileRows - 1) / kTileRows; p.cb = (p.WG + kTileGroups - 1) / kTileGroups; p.tpi = p.rb * p.cb;
+  p.row_bytes = (uint32_t)(kTileGroups * p.cb + 2) * 128;
+  p.a_bytes = round_up((uint32_t)(p.rb * kTileRows + 2) * p.row_bytes, 1024);
+  p.a_tx = (uint32_t)(H + 2) * p.row_bytes;
+  p.w_bytes = round_up((uint32_t)(9 * C * C * 2), 1024);
+  const size_t left = kSmemLimit - fixed_smem(C) - p.w_bytes;
+  int most = (int)std::min<size_t>(left / p.a_bytes, (size_t)(kAccSlots / p.tpi));
+  const int want = (N + sms - 1) / sms;
+  if (most > want) most = want;
+  p.images = most;
+  if (most < 1) return p;
+  p.w_stages = pass == INFER && (size_t)most * p.a_bytes + 2 * (size_t)p.w_bytes + fixed_smem(C) <= kSmemLimit ? 2 : 1;
+  return p;
+}
+inline int chain_ctas(const Geom& p) { return (p.N + p.images - 1) / p.images; }
+inline size_t chain_smem_bytes(const Geom& p, int C) {
+  return std::max(kSmemLeast, (size_t)p.images * p.a_bytes + (size_t)p.w_stages * p.w_bytes + fixed_smem(C));
+}
+inline bool chain_supported(int N, int H, int W, int C) {
+  if ((C != 16 && C != 32 && C != 64) || N < 1) return false;
+  const int G = 64 / C;
+  if (W % G || H + 2 > 256 || W / G + 2 > 256 || kTileGroups * ((W / G + kTileGroups - 1) / kTileGroups) + 2 > 256) return false;
+  const Geom p = chain_geom(N, H, W, C, 2, kMaxCtas, TRAIN);
+  return p.images >= 1 && p.a_tx < (1u << 20) && chain_ctas(p) <= kMaxCtas;
+}
+
+// Tiles at once: as many as share the CTA's tiles evenly (inference, few tiles: at most 2; the others at least 2).
+inline int chain_streams(const Geom& p, int pass) {
+  const int tiles = p.images * p.tpi;
+  if (pass == INFER) return tiles % 2 == 0 ? 2 : 1;
+  return tiles % 4 == 0 || tiles == 3 || tiles > 6 ? 4 : 2;
+}
+
+}  // namespace chain
+}  // namespace fdg

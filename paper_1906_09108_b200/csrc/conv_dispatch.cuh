@@ -11,6 +11,7 @@
 #include "conv_tc.cuh"
 #include "conv_halo.cuh"
 #include "conv_rows.cuh"
+#include "conv_chain.cuh"
 #include "wgrad_wide.cuh"
 #include "elementwise.cuh"
 
@@ -242,14 +243,48 @@ inline cudaError_t run_wgrad_halo(cudaStream_t st, TensorMapCache* cache, int N,
   if (e == cudaSuccess) e = halo::set_smem_attrs(cached_device(cache));
   if (e != cudaSuccess) return e;
   const int ctas = halo::wgrad_ctas(p, side ? cache->wgrad_side_cap : 0);
-  e = launch_chained(halo::wgrad_halo_kernel, dim3(ctas, halo::wgrad_pairs(p)), dim3(halo::kFwdThreads), halo::wgrad_smem_bytes(p), st,
-                     *mx, *my, p, scratch, err_dev);
+  halo::WgradMaps<1> maps;
+  maps.x[0] = *mx; maps.y[0] = *my;
+  e = launch_chained(halo::wgrad_halo_kernel<1>, dim3(ctas, halo::wgrad_pairs(p)), dim3(halo::kFwdThreads), halo::wgrad_smem_bytes(p), st,
+                     maps, p, scratch, err_dev);
   if (e != cudaSuccess) return e;
   const size_t n = (size_t)Co * 9 * Ci;
   if (n >= ((size_t)1 << 17) && ctas <= 8)        // large filters, few partials: four outputs per thread, partials in turn
     return launch_chained(wide::wgrad_wide_sum_kernel, dim3((unsigned)((n / 4 + 255) / 256)), dim3(256), 0, st,
                           reinterpret_cast<const float4*>(scratch), reinterpret_cast<float4*>(dw), n / 4, ctas);
-  return launch_chained(halo::wgrad_halo_reduce_kernel, dim3((unsigned)((n + 31) / 32)), dim3(256), 0, st, (const float*)scratch, dw, n, ctas);
+  return launch_chained(halo::wgrad_halo_reduce_kernel, dim3((unsigned)((n + 31) / 32)), dim3(256), 0, st, (const float*)scratch, dw, n, ctas, n);
+}
+// The weight gradients of `layers` layers of one shape (c_in = c_out = C) in two launches: x[i], dy[i] -> dw + i * dw_step.
+// `scratch`: wgrad_group_scratch_elems floats.
+inline size_t wgrad_group_scratch_elems(int N, int H, int W, int C, int layers, int cap) {
+  const int group = layers < halo::kWgradLayers ? layers : halo::kWgradLayers;
+  return (size_t)group * halo::wgrad_ctas(halo::wgrad_params(N, H, W, C, C), cap) * C * 9 * C;
+}
+inline cudaError_t run_wgrad_group(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int C, int layers, const bf16_t* const* x,
+                                   const bf16_t* const* dy, float* dw, size_t dw_step, float* scratch, int* err_dev, int cap, uint64_t* launches) {
+  const halo::WgradParams p = halo::wgrad_params(N, H, W, C, C);
+  cudaError_t e = halo::set_smem_attrs(cached_device(cache));
+  const int ctas = halo::wgrad_ctas(p, cap);
+  const size_t n = (size_t)C * 9 * C;
+  for (int l0 = 0; l0 < layers && e == cudaSuccess; l0 += halo::kWgradLayers) {
+    const int nl = std::min(halo::kWgradLayers, layers - l0);
+    halo::WgradMaps<halo::kWgradLayers> maps;
+    for (int i = 0; i < halo::kWgradLayers && e == cudaSuccess; ++i) {
+      const CUtensorMap *mx, *my;
+      const int l = l0 + (i < nl ? i : 0);
+      e = cached_tile_map(cache, x[l], N, H, W, C, p.G, &mx, p.kcx);
+      if (e == cudaSuccess) e = cached_tile_map(cache, dy[l], N, H, W, C, p.G, &my, p.kcy);
+      if (e == cudaSuccess) { maps.x[i] = *mx; maps.y[i] = *my; }
+    }
+    if (e != cudaSuccess) return e;
+    e = launch_chained(halo::wgrad_halo_kernel<halo::kWgradLayers>, dim3(ctas, halo::wgrad_pairs(p), nl), dim3(halo::kFwdThreads),
+                       halo::wgrad_smem_bytes(p), st, maps, p, scratch, err_dev);
+    if (e == cudaSuccess)
+      e = launch_chained(halo::wgrad_halo_reduce_kernel, dim3((unsigned)((n + 31) / 32), nl), dim3(256), 0, st, (const float*)scratch,
+                         dw + (size_t)l0 * dw_step, n, ctas, dw_step);
+    *launches += 2;
+  }
+  return e;
 }
 
 // The same contract for wide layers and 1x1 filters (wide::wgrad_wide_kernel; scratch of wide::wide_scratch_elems

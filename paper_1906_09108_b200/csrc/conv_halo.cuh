@@ -597,9 +597,15 @@ struct WgradParams {
   uint32_t tmem_cols;
 };
 
+// One launch takes up to NL layers of the same shape (blockIdx.z): a layer's split is bounded by what the sums cost, so one
+// layer alone leaves most SMs idle, and every launch costs its start and its end.
+constexpr int kWgradLayers = 32;
+template <int NL> struct WgradMaps { CUtensorMap x[NL], y[NL]; };
+template <int NL>
 __global__ void __launch_bounds__(kFwdThreads, 1)
-wgrad_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_y, WgradParams p,
-                  float* __restrict__ partial, int* __restrict__ error_word) {
+wgrad_halo_kernel(const __grid_constant__ WgradMaps<NL> maps, WgradParams p, float* __restrict__ partial, int* __restrict__ error_word) {
+  const CUtensorMap& map_x = maps.x[NL == 1 ? 0 : blockIdx.z];
+  const CUtensorMap& map_y = maps.y[NL == 1 ? 0 : blockIdx.z];
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t stage_bytes = p.x_bytes + p.y_bytes;
@@ -697,7 +703,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       tc_fence_after();
       const int row = lane_grp * 32 + lane;
       const int sblk = row / p.kcx, ci = chunk_a * p.kcx + (row - sblk * p.kcx);
-      float* dst = partial + (size_t)blockIdx.x * ((size_t)p.Co * 9 * p.Ci);
+      float* dst = partial + ((size_t)blockIdx.z * gridDim.x + blockIdx.x) * ((size_t)p.Co * 9 * p.Ci);
       const int nchunks = ncols >> 4;
       const size_t co_stride = (size_t)9 * p.Ci;
       for (int item = group; item < p.sgroups * nchunks; item += kEpiGroups) {
@@ -741,8 +747,11 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
 }
 
 // dw[i] = sum over the pixel-split CTAs of partial[cta][i], in CTA order.  A block owns 32
-// consecutive outputs; its 8 warps take interleaved CTAs and are added in warp order.
-__global__ void __launch_bounds__(256) wgrad_halo_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, size_t n, int ctas) {
+// consecutive outputs; its 8 warps take interleaved CTAs and are added in warp order.  blockIdx.y: layers, `dw_step` apart.
+__global__ void __launch_bounds__(256) wgrad_halo_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, size_t n, int ctas,
+                                                                size_t dw_step) {
+  partial += (size_t)blockIdx.y * ctas * n;
+  dw += (size_t)blockIdx.y * dw_step;
   __shared__ float part[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const size_t i = (size_t)blockIdx.x * 32 + lane;
@@ -935,7 +944,9 @@ inline cudaError_t set_smem_attrs(int dev) {
   static OncePerDevice once;
   return once.run(dev, []() {
     const cudaError_t e = set_smem_limit(conv_halo_kernel, kSmemBudget + 8192);
-    return e != cudaSuccess ? e : set_smem_limit(wgrad_halo_kernel, kSmemBudget + 8192);
+    if (e != cudaSuccess) return e;
+    const cudaError_t e1 = set_smem_limit(wgrad_halo_kernel<1>, kSmemBudget + 8192);
+    return e1 != cudaSuccess ? e1 : set_smem_limit(wgrad_halo_kernel<kWgradLayers>, kSmemBudget + 8192);
   });
 }
 

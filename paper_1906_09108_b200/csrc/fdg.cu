@@ -75,6 +75,23 @@ struct Unit {
   long long r1 = -1, r2 = -1, rs = -1;
 };
 
+// Consecutive identity blocks that run as one launch per pass (conv_chain.cuh): units first .. last, 2 * (last - first + 1)
+// convolutions of C channels.  Offsets of a unit's tensors, parameters and statistics grow evenly inside a run.
+struct Chain { int first, last, C; size_t dc; };   // dc: where its gradients of convolution outputs start in Module::dc
+// The backward pass takes a run in pieces, from its end: the weight gradients of a piece run beside the next one.  The last
+// piece is short, because nothing runs beside its weight gradients.
+// (ResNet-56 K = 2 / ResNet-110 K = 4 / ResNet-1202 K = 4, ms a logging interval: pieces of 12 and 4 blocks 6.86 / 10.78 / 31.2, 8 and 3
+// 6.95 / 10.73 / 31.2, 5 and 2 7.08 / 10.85 / 31.4, up to 20 in one 7.00 / 11.09 / 30.5.)
+constexpr int kChainBlocks = 12, kLastBlocks = 4;
+inline int chain_piece(int blocks_left) {
+  return blocks_left <= kLastBlocks ? blocks_left : std::min(kChainBlocks, blocks_left - kLastBlocks);
+}
+inline int largest_piece(int blocks) {
+  int most = 0;
+  for (int left = blocks; left > 0; left -= chain_piece(left)) most = std::max(most, chain_piece(left));
+  return most;
+}
+
 struct Module {
   int k;                                   // 1-based
   std::vector<Unit> units;
@@ -108,6 +125,15 @@ struct Module {
   size_t up_elems = 0;
   float* red_partial = nullptr;            // per-CTA partial sums of the reductions fused into convolution epilogues
   size_t red_partial_floats = 0;
+  std::vector<Chain> chains;
+  std::vector<int> chain_of;               // per unit: index into chains, or -1
+  bf16* dc = nullptr;                      // gradients of the chains' convolution outputs
+  size_t dc_elems = 0;
+  float* stem_scratch = nullptr;           // partial sums of the stem's weight gradient, which runs beside the side stream's last ones
+  size_t stem_scratch_floats = 0;
+  float* group_scratch = nullptr;          // partial sums of the grouped weight gradients
+  size_t group_scratch_floats = 0;
+  unsigned long long* exchange = nullptr;  // words of chain::Exchange, the epoch behind them
   float *pooled = nullptr, *dlogits = nullptr, *loss_n = nullptr, *loss = nullptr;   // head
   // host state
   int64_t updates = 0;
@@ -151,7 +177,9 @@ struct fdg_ctx {
   int* flags = nullptr;               // [0] non-finite loss, [1] label out of range, [2] a tensor-core kernel's wait ran out,
                                       // [3] result word of the guard check
   std::vector<size_t> guard_offsets;  // byte offsets of the guard regions behind the workspace buffers
-  unsigned long long* guard_table = nullptr;   // the same on the device
+  unsigned long long* guard_table = nullptr;   // the same on the device: the first `guards_saved` of them ..
+  unsigned long long* guard_table2 = nullptr;  // .. and those of the scratch behind the saved part
+  size_t guards_saved = 0;
   float* staging = nullptr;           // fp32 staging for getters
   float* host_images = nullptr;       // device staging of fdg_step_host
   int32_t* host_labels = nullptr;
@@ -161,7 +189,7 @@ struct fdg_ctx {
   bool has_schedule = false;
   fdg_lr_schedule schedule;
   char* ws_base = nullptr;            // the caller's workspace, as carved
-  size_t ws_bytes = 0;
+  size_t ws_bytes = 0;                // the part of it that a saved state holds; scratch that no call leaves anything in lies behind it
   float lr = 0.f;
   uint64_t launches = 0;
   std::deque<fdg_sched_entry> log;   // full, it drops its oldest rows at the front on every iteration
@@ -231,10 +259,10 @@ __global__ void guard_fill_kernel(char* __restrict__ base, const unsigned long l
   reinterpret_cast<unsigned int*>(base + offsets[blockIdx.x])[threadIdx.x] = kGuardWord;
 }
 // *first_bad = the lowest index of a guard region that no longer holds the pattern (left untouched if all do)
-__global__ void guard_check_kernel(const char* __restrict__ base, const unsigned long long* __restrict__ offsets,
+__global__ void guard_check_kernel(const char* __restrict__ base, const unsigned long long* __restrict__ offsets, int first_index,
                                    int* __restrict__ first_bad) {
   if (reinterpret_cast<const unsigned int*>(base + offsets[blockIdx.x])[threadIdx.x] != kGuardWord)
-    atomicMin(first_bad, (int)blockIdx.x);
+    atomicMin(first_bad, first_index + (int)blockIdx.x);
 }
 
 static int conv_out(int n, int r, int stride, int pad) { return (n + 2 * pad - r) / stride + 1; }
@@ -293,6 +321,39 @@ static void add_param(Module& m, int kind, int unit, int d0, int d1, int d2, int
   *off_out = e.offset;
   m.n_params += e.count;
   m.layout.push_back(e);
+}
+
+// The runs of identity blocks of a module; -1 in chain_of: the unit is issued layer by layer.
+static void plan_chains(const fdg_arch& a, Module& m, bool bf16_mode) {
+  m.chains.clear();
+  m.chain_of.assign(m.units.size(), -1);
+  m.dc_elems = 0;
+  if (!bf16_mode) return;
+  const size_t B = a.batch;
+  for (int i = 0; i < (int)m.units.size(); ++i) {
+    const Unit& u = m.units[i];
+    if (u.type != U_BASIC || u.proj || u.zpad || u.stride != 1 || u.ci != u.co) continue;
+    if (!chain::chain_supported(a.batch, u.P, u.Q, u.co) || !halo::wgrad_supported(a.batch, u.P, u.Q, u.co, u.co)) continue;
+    const size_t E = align_up(B * u.P * u.Q * u.co, 128), cc = (size_t)9 * u.co * u.co;
+    // inside a block everything grows evenly; from block to block too
+    bool even = u.t_b == u.t_a + E && u.t_c == u.t_b + E && u.t_y == u.t_c + E && u.w2 == u.w1 + cc + 2 * u.co && u.g1 == u.w1 + cc &&
+                u.b1 == u.g1 + u.co && u.g2 == u.w2 + cc && u.b2 == u.g2 + u.co && u.r2 == u.r1 + 2 * u.co && u.f1 >= 0 &&
+                (size_t)(u.f2 - u.f1) == align_up(cc, 64) && u.w1 % 8 == 0;
+    if (!even) continue;
+    bool join = false;
+    if (!m.chains.empty() && m.chains.back().last == i - 1) {
+      const Unit& f = m.units[m.chains.back().first];
+      const Unit& v = m.units[i - 1];
+      const size_t n = i - m.chains.back().first;
+      join = v.co == u.co && v.P == u.P && u.t_a == f.t_a + n * (v.q_y + (v.q_y - v.q_b) - v.t_a) && u.q_b - v.q_b == u.t_a - v.t_a &&
+             u.q_y - u.q_b == v.q_y - v.q_b && u.st2 - u.st1 == v.st2 - v.st1 && u.st1 == v.st2 + (v.st2 - v.st1) &&
+             u.w1 == v.w2 + cc + 2 * u.co && u.r1 == v.r2 + 2 * u.co && (size_t)(u.f1 - v.f2) == align_up(cc, 64);
+    }
+    if (join) m.chains.back().last = i;
+    else m.chains.push_back(Chain{i, i, u.co, m.dc_elems});
+    m.chain_of[i] = (int)m.chains.size() - 1;
+    m.dc_elems += 2 * E;
+  }
 }
 
 static long long add_running(Module& m, int C) {
@@ -399,6 +460,7 @@ static void plan_modules(fdg_ctx* c) {
           u.t_y = tens(out_e);
           if (u.bn) u.q_y = bits(out_e);
           wg_scratch(a.batch, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, 1, 1);
+          m.stem_scratch_floats = conv_wgrad_scratch_elems(c->bf16_mode, ConvGeom{a.batch, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, 3, 1, 1});
           break;
         case U_BASIC:
           u.t_a = tens(out_e); u.t_b = tens(out_e); u.t_c = tens(out_e); u.t_y = tens(out_e);
@@ -456,6 +518,12 @@ static void plan_modules(fdg_ctx* c) {
       for (const tc::FlipEntry& fe_ : m.flip_table) largest = std::max(largest, (size_t)fe_.Co * fe_.taps * fe_.Ci);
       m.flip_blocks = (unsigned)std::min<size_t>(std::max<size_t>(largest / 8192, 8), 128);
     }
+    plan_chains(a, m, c->bf16_mode);
+    m.group_scratch_floats = 0;
+    for (const Chain& ch : m.chains) {
+      const Unit& u = m.units[ch.first];
+      m.group_scratch_floats = std::max(m.group_scratch_floats, wgrad_group_scratch_elems(a.batch, u.P, u.Q, ch.C, 2 * largest_piece(ch.last - ch.first + 1), 0));
+    }
     m.slot_elems = te; m.slot_floats = tf; m.max_act = maxa; m.scratch_floats = scr; m.wscratch_floats = wscr;
     for (const Unit& u : m.units) {     // where the inference pass finds each batch norm's statistics
       const int c1 = (u.type == U_PREACT || u.type == U_HEAD) ? u.ci : u.co;
@@ -488,8 +556,9 @@ static void plan_modules(fdg_ctx* c) {
   }
 }
 
-// Assigns every device pointer; with base == nullptr only measures.
-static size_t carve(fdg_ctx* c, char* base) {
+// Assigns every device pointer; with base == nullptr only measures.  Returns the whole size, `*saved` the part that a saved
+// state holds: buffers added behind it leave the states of earlier builds loadable.
+static size_t carve(fdg_ctx* c, char* base, size_t* saved) {
   Carver cv(base);
   c->guard_offsets.clear();
   cv.guards = &c->guard_offsets;
@@ -544,6 +613,17 @@ static size_t carve(fdg_ctx* c, char* base) {
   c->staging_elems = stage;
   c->staging = cv.take<float>(stage * 4);
   c->guard_table = cv.take<unsigned long long>((cv.count + 1) * sizeof(unsigned long long));   // one entry per buffer, itself included
+  c->guards_saved = c->guard_offsets.size();
+  *saved = align_up(cv.off, 256);
+  for (Module& m : c->mods) {
+    if (m.stem_scratch_floats) m.stem_scratch = cv.take<float>(m.stem_scratch_floats * 4);
+    if (m.chains.empty()) continue;
+    m.dc = cv.take<bf16>(m.dc_elems * 2);
+    m.group_scratch = cv.take<float>(m.group_scratch_floats * 4);
+    m.exchange = cv.take<unsigned long long>((chain::kExchangeWords + 32) * 8);
+  }
+  const size_t behind = c->guard_offsets.size() - c->guards_saved;
+  c->guard_table2 = behind ? cv.take<unsigned long long>((behind + 1) * sizeof(unsigned long long)) : nullptr;
   return align_up(cv.off, 256);
 }
 
@@ -689,12 +769,13 @@ static int conv_dgrad(Launch& L, Module& m, const ConvGeom& g, const T* dy, cons
   return nparts;
 }
 template <typename T>
-static void conv_wgrad(Launch& L, Module& m, const ConvGeom& g, const T* x, const T* dy, float* dw, const T* dy_up = nullptr) {
+static void conv_wgrad(Launch& L, Module& m, const ConvGeom& g, const T* x, const T* dy, float* dw, const T* dy_up = nullptr, float* scratch = nullptr) {
+  if (!scratch) scratch = m.wscratch;
   L.begin(KC_CONV_WGRAD, (in_elems(g) + out_elems(g)) * sizeof(T) + w_elems(g) * 4, conv_flops(g));
   if constexpr (std::is_same<T, bf16>::value)
-    L.note(bf16_conv_wgrad(L.st, &L.c->tmaps, g, x, dy, dy_up, dw, m.wscratch, L.c->tc_error, L.st == m.stream2, &L.c->launches));
+    L.note(bf16_conv_wgrad(L.st, &L.c->tmaps, g, x, dy, dy_up, dw, scratch, L.c->tc_error, L.st == m.stream2, &L.c->launches));
   else
-    L.note(cuda_core_wgrad<T>(L.st, g, x, dy, m.wscratch, dw, &L.c->launches));
+    L.note(cuda_core_wgrad<T>(L.st, g, x, dy, scratch, dw, &L.c->launches));
 }
 
 template <typename T> static const T* flipped_of(const Module& m, int vslot, long long off);
@@ -730,6 +811,45 @@ static const T* module_input(fdg_ctx* c, const Module& m, int64_t tau, bool eval
   return slot_T<T>(up, eval ? up.D : (int)(tau % up.D)) + up.units.back().t_y;
 }
 
+// The tensors of a run's blocks from unit `first` on, in FIFO slot `slot` (`w`: forward filters, or the flipped ones).
+static chain::Tensors chain_tensors(const Module& m, const Chain& ch, int first, int slot, int vslot, bool backward) {
+  const Unit& u = m.units[first];
+  const size_t cc = (size_t)9 * ch.C * ch.C;
+  chain::Tensors t{};
+  bf16* S = slot_T<bf16>(m, slot);
+  t.t0 = S + u.t_a; t.t_step = u.t_b - u.t_a;
+  t.b_step = u.q_y + (u.q_y - u.q_b) - u.t_a;
+  t.q0 = reinterpret_cast<unsigned char*>(S + u.q_b); t.q_step = (u.q_y - u.q_b) * 2;
+  t.stats = slot_F(m, slot) + u.st1; t.st_step = u.st2 - u.st1;
+  t.w = backward ? flipped_of<bf16>(m, vslot, u.f1) : weights_of<bf16>(m, vslot) + u.w1;
+  t.w_step = backward ? align_up(cc, 64) : cc + 2 * ch.C;
+  t.gamma = m.wver + (size_t)vslot * align_up(m.n_params, 64) + u.g1;
+  t.p_step = cc + 2 * ch.C;
+  return t;
+}
+// How a run is launched now (images = 0: layer by layer): its CTAs wait for one another, so they must all fit the device.
+static chain::Geom chain_shape(fdg_ctx* c, const Module& m, const Chain& ch, int blocks, int pass) {
+  const Unit& u = m.units[ch.first];
+  const int sms = cached_sm_count(&c->tmaps), share = c->tmaps.share > 0 ? c->tmaps.share : 1;
+  chain::Geom p = chain::chain_geom(c->arch.batch, u.P, u.Q, ch.C, 2 * blocks, std::max(16, sms / share), pass);
+  if (p.images > 0 && chain::chain_ctas(p) > std::min(sms, chain::kMaxCtas)) p.images = 0;
+  return p;
+}
+static void chain_forward(fdg_ctx* c, Module& m, Launch& L, const Chain& ch, const chain::Geom& p, const bf16* x, int slot, int vslot, bool eval) {
+  const Unit& u = m.units[ch.first];
+  const size_t rows = (size_t)p.N * p.H * p.W;
+  chain::Tensors t = chain_tensors(m, ch, ch.first, slot, vslot, false);
+  chain::TrainArgs fa{x, m.running + u.r1, kBnMomentum, rows > 1 ? (float)((double)rows / (double)(rows - 1)) : 1.f, c->arch.bn_eps, 1.0 / (double)rows};
+  if (eval) { t.q0 = nullptr; fa.running = nullptr; }
+  const chain::Exchange ex{m.exchange, reinterpret_cast<unsigned int*>(m.exchange + chain::kExchangeWords)};
+  L.begin(KC_CONV_FPROP, (double)rows * ch.C * 2 * (2 * p.layers + 1), 18.0 * rows * ch.C * ch.C * p.layers);
+  const CUtensorMap* mx;
+  cudaError_t e = cached_group_map(&c->tmaps, x, p.N, p.H, p.W, ch.C, rows::kTileGroups * p.cb + 2, p.H + 2, &mx);
+  if (e == cudaSuccess) e = chain::launch(L.st, ch.C, eval ? chain::INFER : chain::TRAIN, *mx, p, t, fa, chain::BackwardArgs{}, ex, c->tc_error);
+  L.note(e);
+  ++c->launches;
+}
+
 // Forward of the module's units into FIFO slot `slot` with weight version `vslot`.  Training (`eval` false):
 // batch statistics, formed in the convolution epilogues where the kernel can, saved for the backward and
 // folded into the running statistics.  Inference (`eval` true): the statistics of every batch norm were put
@@ -761,6 +881,18 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
   int x_np = 0;     // -1: the statistics of x (the next pre-activation block's first batch norm) are already in place
   for (size_t ui = 0; ui < m.units.size(); ++ui) {
     const Unit& u = m.units[ui];
+    if constexpr (std::is_same<T, bf16>::value) {
+      if (m.chain_of[ui] >= 0) {
+        const Chain& ch = m.chains[m.chain_of[ui]];
+        const chain::Geom p = chain_shape(c, m, ch, ch.last - ch.first + 1, eval ? chain::INFER : chain::TRAIN);
+        if ((int)ui == ch.first && p.images > 0) {
+          chain_forward(c, m, L, ch, p, x, slot, vslot, eval);
+          ui = ch.last;
+          x = S + m.units[ui].t_y;
+          continue;
+        }
+      }
+    }
     // the pre-activation block (or the head's batch norm) that normalises this unit's output first, if it is in this module
     const Unit* nxt = nullptr;
     if (ui + 1 < m.units.size() && (m.units[ui + 1].type == U_PREACT || (m.units[ui + 1].type == U_HEAD && m.units[ui + 1].bn)))
@@ -944,9 +1076,69 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
   int dy_sum_parts = 0;            // > 0: the kernel that produced dy left that many rows of partial sums for the
                                    // first batch-norm backward it meets
   const int nu = (int)m.units.size();
+  // the runs of blocks that go as one launch, and whether unit i belongs to one
+  auto chained = [&](int i) { return std::is_same<T, bf16>::value && m.chain_of[i] >= 0 && chain_shape(c, m, m.chains[m.chain_of[i]], 1, chain::BACKWARD).images > 0; };
   for (int i = nu - 1; i >= 0; --i) {
     const Unit& u = m.units[i];
     if (u.type == U_HEAD) continue;
+    if constexpr (std::is_same<T, bf16>::value) {
+      if (chained(i)) {
+        const Chain& ch = m.chains[m.chain_of[i]];
+        const int blocks = chain_piece(i - ch.first + 1), first = i - blocks + 1;
+        const Unit& f = m.units[first];
+        const chain::Geom p = chain_shape(c, m, ch, blocks, chain::BACKWARD);
+        const size_t rows = (size_t)B * u.P * u.Q, E = align_up(rows * ch.C, 128);
+        chain::BackwardArgs ba{};
+        ba.dy = dy;
+        ba.dx = first == 0 ? gfirst : (dy == G[0] ? G[1] : G[0]);
+        ba.dc = m.dc + ch.dc + (size_t)2 * (first - ch.first) * E; ba.dc_step = E;
+        ba.dgamma = m.grad + f.g1; ba.inv_m = (float)(1.0 / (double)rows);
+        dy_sum_parts = 0;
+        if (first > 0 && !chained(first - 1)) {
+          const Unit& pu = m.units[first - 1];
+          if ((pu.type == U_BASIC && !pu.proj) || (pu.type == U_STEM && pu.bn)) {
+            ba.out_gate = reinterpret_cast<const unsigned char*>(S + pu.q_y);
+            ba.out_x = S + (pu.type == U_STEM ? pu.t_a : pu.t_c);
+            ba.out_stats = F + (pu.type == U_STEM ? pu.st1 : pu.st2);
+            ba.out_partial = m.red_partial;
+            dy_sum_parts = chain::chain_ctas(p);
+          }
+        }
+        auto cap_at = [&](int ui, int which) -> bf16* {
+          for (const CaptureEntry& ce : m.cap_table) if (ce.unit == ui && ce.which == which) return reinterpret_cast<bf16*>(m.cap_buf) + ce.off;
+          return nullptr;
+        };
+        if (m.cap_buf) {
+          ba.keep_a = cap_at(first, 2); ba.keep_x = cap_at(first, 4);
+          ba.keep_step = i > first ? (size_t)(cap_at(first + 1, 2) - ba.keep_a) : 0;
+          keep(i, 0, dy);
+        }
+        const chain::Tensors t = chain_tensors(m, ch, first, slot, vslot, true);
+        const chain::Exchange ex{m.exchange, reinterpret_cast<unsigned int*>(m.exchange + chain::kExchangeWords)};
+        L.begin(KC_CONV_DGRAD, (double)rows * ch.C * 2 * (3 * p.layers + 2), 18.0 * rows * ch.C * ch.C * p.layers);
+        L.note(chain::launch(L.st, ch.C, chain::BACKWARD, CUtensorMap{}, p, t, chain::TrainArgs{}, ba, ex, c->tc_error));
+        ++c->launches;
+        if (m.cap_buf)
+          for (int b = first; b <= i; ++b) {
+            const bf16* d = ba.dc + (size_t)2 * (b - first) * E;
+            keep(b, 3, d); keep(b, 1, d + E);
+            if (b < i) keep(b, 0, cap_at(b + 1, 4));
+          }
+        fork();
+        std::vector<const bf16*> wx(p.layers), wy(p.layers);
+        for (int l = 0; l < p.layers; ++l) {
+          const int b = first + l / 2;
+          wx[l] = (l & 1) ? S + m.units[b].t_b : (b > 0 ? S + m.units[b - 1].t_y : module_input<T>(c, m, tau));
+          wy[l] = ba.dc + (size_t)l * E;
+        }
+        LS.begin(KC_CONV_WGRAD, (double)rows * ch.C * 4 * p.layers, 18.0 * rows * ch.C * ch.C * p.layers);
+        LS.note(run_wgrad_group(LS.st, &c->tmaps, p.N, p.H, p.W, ch.C, p.layers, wx.data(), wy.data(), m.grad + f.w1, t.p_step, m.group_scratch,
+                                c->tc_error, LS.st == m.stream2 ? c->tmaps.wgrad_side_cap : 0, &c->launches));
+        dy = ba.dx;
+        i = first;
+        continue;
+      }
+    }
     const T* x = i > 0 ? S + m.units[i - 1].t_y : module_input<T>(c, m, tau);
     T* gout = (i == 0) ? gfirst : (dy == G[0] ? G[1] : G[0]);
     const size_t rows_in = (size_t)B * u.H * u.W, rows_out = (size_t)B * u.P * u.Q;
@@ -954,7 +1146,7 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
     // data-gradient kernel that writes this unit's input gradient.
     NextBnBwd<T> nb{};
     const NextBnBwd<T>* next = nullptr;
-    if (i > 0) {
+    if (i > 0 && !chained(i - 1)) {
       const Unit& pu = m.units[i - 1];
       if (pu.type == U_BASIC && !pu.proj) { nb = {gate(pu.t_y, pu.q_y), S + pu.t_c, F + pu.st2}; next = &nb; }
       if (pu.type == U_STEM && pu.bn) { nb = {gate(pu.t_y, pu.q_y), S + pu.t_a, F + pu.st1}; next = &nb; }
@@ -972,9 +1164,8 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
           dc = T1;
           keep(i, 3, T1);
         }
-        fork();
-        conv_wgrad<T>(LS, m, g, x, dc, m.grad + u.w1);
-        side_done(0);
+        // nothing follows on this stream: beside the side stream's last weight gradients, with partial sums of its own
+        conv_wgrad<T>(L, m, g, x, dc, m.grad + u.w1, nullptr, m.stem_scratch);
         break;
       }
       case U_BASIC: {
@@ -1252,7 +1443,8 @@ fdg_status fdg_workspace_bytes(const fdg_arch* arch, const fdg_config* cfg, size
   fdg_ctx tmp;
   fdg_status s = make_plan(arch, cfg, &tmp);
   if (s != FDG_OK) return s;
-  *out_bytes = carve(&tmp, nullptr);
+  size_t saved = 0;
+  *out_bytes = carve(&tmp, nullptr, &saved);
   return FDG_OK;
 }
 
@@ -1265,22 +1457,24 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
   if (!c) return FDG_ERR_STATE;
   fdg_status s = make_plan(arch, cfg, c);
   if (s != FDG_OK) { delete c; return s; }
-  const size_t need = carve(c, nullptr);
+  size_t saved = 0;
+  const size_t need = carve(c, nullptr, &saved);
   if (bytes < need) { delete c; return FDG_ERR_WORKSPACE_TOO_SMALL; }
   cudaError_t e = cudaGetDevice(&c->device);
   if (e == cudaSuccess) e = cudaMemset(dev_workspace, 0, need);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) { delete c; return FDG_ERR_CUDA; }
-  carve(c, static_cast<char*>(dev_workspace));
+  carve(c, static_cast<char*>(dev_workspace), &saved);
   c->ws_base = static_cast<char*>(dev_workspace);
-  c->ws_bytes = need;
+  c->ws_bytes = saved;
   {
     std::vector<unsigned long long> table(c->guard_offsets.begin(), c->guard_offsets.end());
-    e = cudaMemcpy(c->guard_table, table.data(), table.size() * sizeof(unsigned long long), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-      guard_fill_kernel<<<(unsigned)table.size(), (unsigned)(kGuardBytes / 4)>>>(c->ws_base, c->guard_table);
-      e = cudaGetLastError();
-    }
+    const size_t n1 = c->guards_saved, n2 = table.size() - n1;
+    e = cudaMemcpy(c->guard_table, table.data(), n1 * sizeof(unsigned long long), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && n2) e = cudaMemcpy(c->guard_table2, table.data() + n1, n2 * sizeof(unsigned long long), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) guard_fill_kernel<<<(unsigned)n1, (unsigned)(kGuardBytes / 4)>>>(c->ws_base, c->guard_table);
+    if (e == cudaSuccess && n2) guard_fill_kernel<<<(unsigned)n2, (unsigned)(kGuardBytes / 4)>>>(c->ws_base, c->guard_table2);
+    if (e == cudaSuccess) e = cudaGetLastError();
   }
   for (Module& m : c->mods) {
     if (m.flip_table_dev && e == cudaSuccess)
@@ -1297,6 +1491,7 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
   // shared-memory limits of the tensor-core kernels, raised here so that a kernel's first launch may be a recorded one
   if (e == cudaSuccess && c->bf16_mode) e = halo::set_smem_attrs(c->device);
   if (e == cudaSuccess && c->bf16_mode) e = rows::set_attrs(c->device);
+  if (e == cudaSuccess && c->bf16_mode) e = chain::set_attrs(c->device);
   if (e == cudaSuccess && c->bf16_mode) e = tc::conv_tc_set_attrs(c->device);
   if (e == cudaSuccess && c->bf16_mode) e = wide::wide_set_attrs(c->device);
   c->own_streams = streams == nullptr;
@@ -1675,8 +1870,10 @@ fdg_status fdg_debug_check_guards(fdg_ctx* c, long long* out_first_bad) {
   const int none = INT_MAX;
   if (e == cudaSuccess) e = cudaMemcpy(c->flags + 3, &none, sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    guard_check_kernel<<<(unsigned)c->guard_offsets.size(), (unsigned)(kGuardBytes / 4)>>>(c->ws_base, c->guard_table, c->flags + 3);
-    ++c->launches;
+    const size_t n1 = c->guards_saved, n2 = c->guard_offsets.size() - n1;
+    guard_check_kernel<<<(unsigned)n1, (unsigned)(kGuardBytes / 4)>>>(c->ws_base, c->guard_table, 0, c->flags + 3);
+    if (n2) guard_check_kernel<<<(unsigned)n2, (unsigned)(kGuardBytes / 4)>>>(c->ws_base, c->guard_table2, (int)n1, c->flags + 3);
+    c->launches += n2 ? 2 : 1;
     e = cudaGetLastError();
   }
   int got = none;

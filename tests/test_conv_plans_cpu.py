@@ -11,6 +11,7 @@ PROLOGUE = r"""
 #include <cstdio>
 #include <cuda.h>
 #include "fdg_ops.h"
+#include "chain_plan.h"
 #include "conv_direct.cuh"
 #include "wgrad_wide.cuh"
 using namespace fdg;
@@ -94,3 +95,25 @@ def test_a_share_of_the_gpu_lengthens_no_long_accumulation(tmp_path):
         if (steps(p) > 256 && steps(p) > steps(whole)) report("instructions", g, (size_t)steps(p));
       }
     }""")
+
+
+def test_runs_of_blocks_fit_an_sm_and_the_device(tmp_path):
+    """Every launch shape of a run holds its images' operands and accumulators, covers the batch with CTAs that can be resident
+    together, and keeps a CTA's tiles below the slots; more than half of an SM's shared memory, so that two never share one."""
+    _run(tmp_path, r"""
+  for (int C = 16; C <= 64; C *= 2) for (int N : {1, 2, 31, 97, 128, 148, 149, 160, 600, 1184}) for (int H = 1; H <= 70; ++H) for (int W = 1; W <= 70; ++W) {
+    const ConvGeom g{N, H, W, C, H, W, C, 3, 3, 1, 1};
+    if (!chain::chain_supported(N, H, W, C)) continue;
+    for (int share = 1; share <= 16; ++share) for (int pass = 0; pass < 3; ++pass) {
+      const chain::Geom p = chain::chain_geom(N, H, W, C, 2, 148 / share < 16 ? 16 : 148 / share, pass);
+      const size_t bytes = chain::chain_smem_bytes(p, C);
+      const int ctas = chain::chain_ctas(p), st = chain::chain_streams(p, pass);
+      if (bytes > chain::kSmemLimit || 2 * bytes <= 228 * 1024) report("shared memory", g, bytes);
+      if (p.images < 1 || p.images * p.tpi > chain::kAccSlots) report("accumulators", g, (size_t)p.images);
+      if (ctas < 1 || ctas > chain::kMaxCtas || ctas > N || (long)ctas * p.images < N) report("CTAs", g, (size_t)ctas);
+      if (p.rb * chain::kTileRows < H || p.cb * chain::kTileGroups * (64 / C) < W || p.WG * (64 / C) != W) report("tiles", g, (size_t)p.tpi);
+      if ((size_t)(p.rb * chain::kTileRows + 2) * p.row_bytes > p.a_bytes || p.a_bytes % 1024 || p.w_bytes % 1024) report("operands", g, p.a_bytes);
+      if ((size_t)p.w_bytes < (size_t)18 * C * C || p.w_stages < 1 || p.w_stages > 2 || (pass != chain::INFER && p.w_stages != 1)) report("weights", g, p.w_bytes);
+      if (pass == chain::INFER ? st > 2 : st < 2) report("streams", g, (size_t)st);
+    }
+  }""")

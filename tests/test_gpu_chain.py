@@ -1,0 +1,128 @@
+"""Runs of identity blocks as one launch per pass, at sizes where their tiles, images per CTA and pieces have edges: every layer
+of the forward and of the backward pass against the oracle's layer functions on the library's own inputs to it (bars: one
+bfloat16 ulp of the largest element is 4e-3), and an inference pass against float64."""
+import numpy as np
+import pytest
+import torch
+import torch.nn.functional as F
+
+import fdg_synth as S
+from oracle import layers as L
+from tests.layerwise import check_backward_layerwise, take, units_of
+
+pytestmark = pytest.mark.gpu
+EPS = 1e-5
+
+# (batch, image side, blocks per stage, K, splits): single images and groups; partly filled tiles (28 = 7 groups, 28 of 32 rows);
+# several column blocks (40) and tiles per image; more images than CTAs (149, 161) and the most that a CTA holds; one-pixel maps;
+# runs of one block, of several pieces in the backward pass
+CASES = [(1, 12, 2, 1, ()), (5, 28, 3, 1, ()), (3, 40, 2, 2, (3,)), (149, 16, 2, 1, ()), (161, 32, 2, 4, (1, 2, 4)), (7, 4, 3, 1, ()),
+         (9, 20, 5, 1, ()), (2, 8, 13, 1, ())]
+
+
+def _context(case, lr=0.0, **kw):
+    from paper_1906_09108_b200 import binding as B
+    batch, hw, n, K, splits = case
+    arch = dict(family="resnet6n2", n_per_stage=n, widths=(16, 32, 64), stem_width=16, in_h=hw, in_w=hw, in_c=3, num_classes=10, batch=batch)
+    g = B.FDG(B.make_arch(**arch), K=K, split_after_block=splits, beta=0.5, precision=B.FDG_BF16_TC, lr=lr, weight_decay=0.0, **kw)
+    params = {}
+    for k in range(1, K + 1):
+        params[k] = S.init_params(0, k, g.param_layout(k), jitter=True)
+        g.set_params(k, params[k])
+    return g, params, arch
+
+
+def _relmax(a, b):
+    return float(np.abs(a - b).max() / max(np.abs(b).max(), 1e-30))
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_backward(case):
+    g, params, arch = _context(case)
+    checked, _ = check_backward_layerwise(g, params, arch, case[3])
+    assert checked == 3 * case[2]
+    assert g.check_guards() == -1
+    g.close()
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+@pytest.mark.parametrize("case", CASES)
+def test_forward(case, graphs):
+    g, params, arch = _context(case, graphs=graphs)
+    b, hw, K = arch["batch"], arch["in_h"], case[3]
+    for t in range(1, 2 * K + 4):
+        g.step(torch.from_numpy(S.images(0, t, b, hw, hw, 3)).cuda(), torch.from_numpy(S.labels(0, t, b, 10)).cuda())
+    g.sync()
+    checked = 0
+    for k in range(1, K + 1):
+        units = units_of(g.param_layout(k))
+        for u in range(1, len(units)):
+            name, ent = units[u]
+            if not name.startswith("block") or len(ent) > 6:
+                continue
+            co = ent[0][1][0]
+            w1, w2 = L.round_bf16(take(params[k], ent[0])), L.round_bf16(take(params[k], ent[3]))
+            bn1, bn2 = [take(params[k], e) for e in ent[1:3]], [take(params[k], e) for e in ent[4:6]]
+            _, x = g.saved_tensor(k, u - 1, 3)
+            side = int(round((x.size / (b * co)) ** 0.5))
+            got = [x] + [g.saved_tensor(k, u, w)[1] for w in range(4)]
+            x, c1, a1, c2, y = (v.reshape(b, side, side, co).astype(np.float64) for v in got)
+            assert _relmax(c1, L.round_bf16(L.conv2d_forward(x, w1, 1, 1))) <= 1e-2, (k, name)
+            assert _relmax(a1, L.round_bf16(L.relu_forward(L.batchnorm_forward(c1, *bn1, EPS)[0]))) <= 1e-2, (k, name)
+            assert _relmax(c2, L.round_bf16(L.conv2d_forward(a1, w2, 1, 1))) <= 1e-2, (k, name)
+            assert _relmax(y, L.round_bf16(L.relu_forward(L.batchnorm_forward(c2, *bn2, EPS)[0] + x))) <= 1e-2, (k, name)
+            checked += 1
+    assert checked > 0 and g.check_guards() == -1
+    g.close()
+
+
+def _eval_reference(g, params, K, x):
+    """float64 with the tensors rounded to bfloat16 that the inference pass keeps between two layers."""
+    def q(v):
+        return v.to(torch.bfloat16).double()
+
+    def conv(v, w, stride, pad):
+        return q(F.conv2d(v, q(torch.from_numpy(w)).permute(0, 3, 1, 2), stride=stride, padding=pad))
+
+    def bn(v, ga, be, mean, var):
+        inv = 1.0 / torch.sqrt(var + EPS)
+        return (v - mean.view(1, -1, 1, 1)) * (torch.from_numpy(ga) * inv).view(1, -1, 1, 1) + torch.from_numpy(be).view(1, -1, 1, 1)
+
+    x = q(x.double().cpu()).permute(0, 3, 1, 2)
+    for k in range(1, K + 1):
+        running, at = torch.from_numpy(np.asarray(g.get_running(k), dtype=np.float64)), 0
+
+        def stats(c):
+            nonlocal at
+            at += 2 * c
+            return running[at - 2 * c:at - c], running[at - c:at]
+        for name, ent in units_of(g.param_layout(k)):
+            p = [take(params[k], e) for e in ent]
+            if name == "stem":
+                x = q(F.relu(bn(conv(x, p[0], 1, 1), p[1], p[2], *stats(p[0].shape[0]))))
+            elif name == "head":
+                return x.mean(dim=(2, 3)) @ torch.from_numpy(p[0].reshape(p[0].shape[0], -1)).T + torch.from_numpy(p[1].reshape(-1))
+            else:
+                proj, co = len(p) > 6, p[0].shape[0]
+                s1, s2 = stats(co), stats(co)
+                a = q(F.relu(bn(conv(x, p[0], 2 if proj else 1, 1), p[1], p[2], *s1)))
+                sc = bn(conv(x, p[6], 2, 0), p[7], p[8], *stats(co)) if proj else x
+                x = q(F.relu(bn(conv(a, p[3], 1, 1), p[4], p[5], *s2) + sc))
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_inference(case):
+    g, params, arch = _context(case)
+    b, hw, K = arch["batch"], arch["in_h"], case[3]
+    for t in range(1, 2 * K + 4):
+        g.step(torch.from_numpy(S.images(0, t, b, hw, hw, 3)).cuda(), torch.from_numpy(S.labels(0, t, b, 10)).cuda())
+    g.sync()
+    x = torch.from_numpy(S.images(0, 99, b, hw, hw, 3)).cuda()
+    logits = torch.empty((b, 10), device="cuda")
+    g.eval(x, torch.zeros(b, dtype=torch.int32, device="cuda"), logits_dev=logits)
+    torch.cuda.synchronize()
+    want = _eval_reference(g, params, K, x).numpy()
+    got = logits.double().cpu().numpy()
+    # half a bfloat16 unit (2^-9) for each tensor rounded differently, 6 n + 2 of them in a row at worst, adding up like noise
+    assert np.linalg.norm(got - want) <= 2.0 ** -9 * (6 * case[2] + 2) ** 0.5 * np.linalg.norm(want)
+    g.close()
