@@ -38,10 +38,11 @@ typedef struct {
  *   wgrad_cta_cap  fdg_conv_wgrad: upper bound of the halo-tile kernel's pixel split (0 = none); on a side stream the
  *                  module-step gives it max(16, batch / 4).  (fdg_conv_wgrad takes no `share`: the wide
  *                  kernel's split is the whole GPU's here.)
- *   dy_spread      stride-2 gradients (bf16): scratch of N*H*W*Co bf16 elements.  With it the data and
- *                  weight gradients of a 3x3 stride-2 layer run as the stride-1 tensor-core kernels on dy
- *                  spread onto the even pixels of the input grid (the call fills it); without it they
- *                  run on the CUDA cores.
+ *   dy_spread      stride-2 weight gradients (bf16): scratch of N*H*W*Co bf16 elements.  With it the weight
+ *                  gradient of a 3x3 stride-2 layer runs as the stride-1 tensor-core kernel on dy spread onto
+ *                  the even pixels of the input grid (the call fills it); without it it runs on the CUDA
+ *                  cores.  The data gradient needs it only to form sums (reduce): without them it runs on
+ *                  the output grid.
  *   reduce         a per-channel reduction formed in the epilogue of the bf16 tensor-core kernels, one row of
  *                  2*C floats per CTA in `partial` (capacity `partial_floats` >= FDG_CONV_PARTIAL_ROWS*2*C);
  *                  `nparts` receives the number of rows, 0 if the shape took a kernel that forms none.  The
@@ -73,7 +74,7 @@ fdg_status fdg_conv_forward(int precision, const fdg_conv_shape* shape, const vo
 
 /* dx = conv^T(dy, w) [+ res * [res_mask > 0]], dx/res/res_mask [N][H][W][Ci], dy [N][P][Q][Co].
  * `w_flipped` (nullable) is the copy made by fdg_conv_flip_weights; with it, bf16 3x3 shapes run on the
- * tensor cores (stride 2: also needs extra->dy_spread) and so do 1x1 shapes without padding (stride 2 without
+ * tensor cores and so do 1x1 shapes without padding (stride 2 without
  * res: dx is cleared, then written at its even pixels); without it every shape runs on the CUDA cores. */
 fdg_status fdg_conv_dgrad(int precision, const fdg_conv_shape* shape, const void* dy, const void* w,
                           const void* w_flipped, void* dx, const void* res, const void* res_mask,

@@ -53,14 +53,14 @@ inline bool tc_eligible(const ConvGeom& g) {
 inline cudaError_t run_conv_tc(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int Ck, int Cn,
                                const bf16_t* act, const bf16_t* wgt, bf16_t* out, const bf16_t* res,
                                const bf16_t* res_mask, int* err_dev, int sub = 1, int taps = 9, int act_sub = 1,
-                               float* stat_partial = nullptr, int* ctas_out = nullptr, const EpiAffine* affine = nullptr) {
+                               float* stat_partial = nullptr, int* ctas_out = nullptr, const EpiAffine* affine = nullptr, int s2 = 0) {
   const int sm_count = cached_sm_count(cache);
-  tc::ConvTcParams p = tc::conv_tc_params(N, H, W, Ck, Cn, taps, cache->share);
+  tc::ConvTcParams p = tc::conv_tc_params(N, H, W, Ck, Cn, taps, cache->share, s2);
   p.sub = sub;
-  p.act_sub = act_sub;
+  if (s2 == 0) p.act_sub = act_sub;
   TensorMapCache::Key ka, kb;
   std::memset(&ka, 0, sizeof(ka)); std::memset(&kb, 0, sizeof(kb));
-  ka.ptr = act; ka.d[0] = 1; ka.d[1] = N; ka.d[2] = H; ka.d[3] = W; ka.d[4] = Ck; ka.d[5] = p.kc; ka.d[6] = p.patch; ka.d[7] = act_sub;
+  ka.ptr = act; ka.d[0] = 1; ka.d[1] = N; ka.d[2] = H; ka.d[3] = W; ka.d[4] = Ck; ka.d[5] = p.kc; ka.d[6] = p.patch; ka.d[7] = p.act_sub;
   kb.ptr = wgt; kb.d[0] = 2; kb.d[1] = Ck; kb.d[2] = Cn; kb.d[3] = p.kc; kb.d[4] = p.n_tile; kb.d[5] = taps;
   auto ia = cache->maps.find(ka), ib = cache->maps.find(kb);
   if (ia == cache->maps.end() || ib == cache->maps.end()) {
@@ -72,7 +72,20 @@ inline cudaError_t run_conv_tc(cudaStream_t st, TensorMapCache* cache, int N, in
   }
   const cudaError_t e = tc::conv_tc_set_attrs(cached_device(cache));
   if (e != cudaSuccess) return e;
-  return tc::conv_tc_launch(st, p, ia->second, ib->second, out, res, res_mask, err_dev, sm_count, stat_partial, ctas_out, affine);
+  tc::ActMaps maps;
+  for (int q = 0; q < 4; ++q) maps.m[q] = ia->second;
+  for (int q = 1; q < 4 && s2 == 1; ++q) {       // the other parities of x [N][2H][2W][Ck]
+    ka.ptr = act + ((size_t)(q >> 1) * 2 * W + (q & 1)) * Ck;
+    auto iq = cache->maps.find(ka);
+    if (iq == cache->maps.end()) {
+      CUtensorMap mq, unused;
+      const cudaError_t eq = tc::conv_tc_make_maps(p, ka.ptr, wgt, &mq, &unused);
+      if (eq != cudaSuccess) return eq;
+      iq = cache->maps.insert({ka, mq}).first;
+    }
+    maps.m[q] = iq->second;
+  }
+  return tc::conv_tc_launch(st, p, maps, ib->second, out, res, res_mask, err_dev, sm_count, stat_partial, ctas_out, affine);
 }
 
 
@@ -85,18 +98,21 @@ inline bool halo_fprop_eligible(const ConvGeom& g) { return halo_shape(g) && hal
 inline bool halo_dgrad_eligible(const ConvGeom& g) { return halo_shape(g) && halo::fwd_supported(g.N, g.H, g.W, g.Co, g.Ci); }
 inline bool halo_wgrad_eligible(const ConvGeom& g) { return halo_shape(g) && halo::wgrad_supported(g.N, g.H, g.W, g.Ci, g.Co); }
 
-// A 3x3 / stride 2 / pad 1 convolution on even image sizes is the stride-1 convolution kept at the
-// even pixels, and its two gradients are the stride-1 ones taken with dy spread onto the even
-// pixels of a zero tensor of the input's size.  Four times the arithmetic, on kernels that are far
-// from arithmetic-bound; the shapes concerned are two layers of a 6n+2 network.
+// A 3x3 / stride 2 / pad 1 convolution on even image sizes runs exactly, on the output grid, forward and data gradient
+// (conv_tc.cuh: ActMaps).  Its weight gradient is the stride-1 one taken with dy spread onto the even pixels of a zero
+// tensor of the input's size: four times the arithmetic.
 inline bool halo_s2_shape(const ConvGeom& g) {
   return g.R == 3 && g.S == 3 && g.stride == 2 && g.pad == 1 && g.H % 2 == 0 && g.W % 2 == 0 && g.P == g.H / 2 && g.Q == g.W / 2;
 }
-inline bool halo_s2_fprop_eligible(const ConvGeom& g) { return halo_s2_shape(g) && halo::fwd_supported(g.N, g.H, g.W, g.Ci, g.Co); }
-inline bool halo_s2_dgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && halo::fwd_supported(g.N, g.H, g.W, g.Co, g.Ci); }
-// the same for layers too wide for the halo kernel: the per-tap kernel at full resolution
-inline bool tc_s2_fprop_eligible(const ConvGeom& g) { return halo_s2_shape(g) && tc::conv_tc_supported(g.N, g.H, g.W, g.Ci, g.Co, (size_t)g.N * g.P * g.Q); }
-inline bool tc_s2_dgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && tc::conv_tc_supported(g.N, g.H, g.W, g.Co, g.Ci, (size_t)g.N * g.P * g.Q); }
+inline bool s2_planned(const ConvGeom& g, int Ck, int Cn) {
+  return (tc::conv_tc_supported(g.N, g.H, g.W, Ck, Cn, (size_t)g.N * g.P * g.Q) || halo::fwd_supported(g.N, g.H, g.W, Ck, Cn)) &&
+         tc::conv_tc_supported(g.N, g.P, g.Q, Ck, Cn, (size_t)g.N * g.P * g.Q);
+}
+// (H and W, not P and Q: images of more than 128 columns stay with the CUDA cores, as their workspaces were planned)
+inline bool tc_s2_fprop_eligible(const ConvGeom& g) { return halo_s2_shape(g) && s2_planned(g, g.Ci, g.Co); }
+inline bool tc_s2_dgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && s2_planned(g, g.Co, g.Ci); }
+// with the sums of the batch-norm backward that dx feeds: those are formed by the halo kernel, at full resolution from a spread-out dy
+inline bool halo_s2_dgrad_sums_eligible(const ConvGeom& g) { return halo_s2_shape(g) && halo::fwd_supported(g.N, g.H, g.W, g.Co, g.Ci) && g.Ci <= 64; }
 inline bool halo_s2_wgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && halo::wgrad_supported(g.N, g.H, g.W, g.Ci, g.Co); }
 // 1x1 convolutions without padding (projection shortcuts), stride 1 or 2: one "tap" of the per-tap kernel on the output
 // grid; a stride-2 forward reads the even pixels of x as a strided tensor, a stride-2 data gradient writes dx at the
@@ -163,11 +179,10 @@ inline bool halo_reduce_ok(int Cn) { return Cn <= 64; }
 inline cudaError_t run_conv_halo(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int Ck, int Cn,
                                  const bf16_t* act, const bf16_t* wgt, bf16_t* out, const bf16_t* res,
                                  const bf16_t* res_mask, int* err_dev, const halo::EpiReduce* red = nullptr,
-                                 int* ctas_out = nullptr, int sub = 1) {
+                                 int* ctas_out = nullptr) {
   int sms = cached_sm_count(cache) / (cache->share > 0 ? cache->share : 1);
   if (sms < 16) sms = 16;
-  halo::FwdParams p = halo::fwd_params(N, H, W, Ck, Cn, sms);
-  p.sub = sub;
+  const halo::FwdParams p = halo::fwd_params(N, H, W, Ck, Cn, sms);
   const CUtensorMap *mx, *mw;
   cudaError_t e = cached_tile_map(cache, act, N, H, W, Ck, p.G, &mx);
   if (e == cudaSuccess) e = cached_weight_map(cache, wgt, Ck, Cn, &mw);
@@ -325,11 +340,12 @@ inline cudaError_t run_wgrad_wide(cudaStream_t st, TensorMapCache* cache, int N,
 
 // Does the data gradient of this convolution read the flipped/transposed weight copy?
 inline bool dgrad_uses_flipped(const ConvGeom& g) {
-  return rows_eligible(g) || halo_dgrad_eligible(g) || halo_s2_dgrad_eligible(g) || tc_eligible(g) || tc_s2_dgrad_eligible(g) || tc_1x1_dgrad_eligible(g);
+  return rows_eligible(g) || halo_dgrad_eligible(g) || tc_eligible(g) || tc_s2_dgrad_eligible(g) || tc_1x1_dgrad_eligible(g);
 }
-// Do the stride-2 gradients of this convolution run on the tensor cores, given a spread-out copy of dy?
+// Does the stride-2 weight gradient of this convolution run on the tensor cores, given a spread-out copy of dy?  (Also true
+// where only the data gradient does: the workspace of a module has had room for the copy then.)
 inline bool s2_uses_spread_dy(const ConvGeom& g) {
-  return (halo_s2_dgrad_eligible(g) || halo_s2_wgrad_eligible(g) || tc_s2_dgrad_eligible(g) || wide_s2_wgrad_eligible(g)) && g.Co % 8 == 0;
+  return (halo_s2_wgrad_eligible(g) || tc_s2_dgrad_eligible(g) || wide_s2_wgrad_eligible(g)) && g.Co % 8 == 0;
 }
 
 // fp32 scratch elements a weight-gradient call may need (bf16 storage: whichever kernel is chosen).
@@ -404,7 +420,7 @@ inline cudaError_t finish_wide_stats(cudaStream_t st, const ConvGeom& g, const W
 // Can the kernel this forward convolution takes apply a batch norm in its epilogue (`affine`)?
 inline bool bf16_fprop_affine_ok(const ConvGeom& g) {
   if (rows_eligible(g)) return true;
-  if (halo_fprop_eligible(g) || halo_s2_fprop_eligible(g)) return false;
+  if (halo_fprop_eligible(g)) return false;
   if (tc_eligible(g) || tc_s2_fprop_eligible(g) || tc_1x1_fprop_eligible(g)) return 3 * g.Co <= tc::kStatFloats;
   return direct::conv_supported(g, false);
 }
@@ -420,23 +436,29 @@ inline cudaError_t bf16_conv_fprop(cudaStream_t st, TensorMapCache* cache, const
     if (fuse && nparts) *nparts = ctas;
     return e;
   }
-  const bool s1 = halo_fprop_eligible(g), s2 = !s1 && halo_s2_fprop_eligible(g);
-  if (s1 || s2) {
+  if (halo_fprop_eligible(g)) {
     ++*launches;
     const bool fuse = red && red->mode == 1 && halo_reduce_ok(g.Co);
     int ctas = 0;
-    cudaError_t e = run_conv_halo(st, cache, g.N, g.H, g.W, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, fuse ? red : nullptr, &ctas, s2 ? 2 : 1);
+    cudaError_t e = run_conv_halo(st, cache, g.N, g.H, g.W, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, fuse ? red : nullptr, &ctas);
     if (fuse && nparts) *nparts = ctas;
     return e;
   }
   if (tc_eligible(g) || tc_s2_fprop_eligible(g)) {
     ++*launches;
+    const int s2 = g.stride == 2 ? 1 : 0;
+    if (s2 && red && red->mode == 1 && 2 * g.Co <= kEwThreads && (!ws || ws->stats)) {      // narrow: the batch norm behind it adds the rows up
+      int ctas = 0;
+      const cudaError_t e = run_conv_tc(st, cache, g.N, g.P, g.Q, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, 1, 9, 1, red->partial, &ctas, nullptr, s2);
+      if (nparts) *nparts = ctas;
+      return e;
+    }
     if (wide_stats_ok(cache, g, ws)) {
       int ctas = 0;
-      const cudaError_t e = run_conv_tc(st, cache, g.N, g.H, g.W, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, g.stride, 9, 1, ws->partial, &ctas);
+      const cudaError_t e = run_conv_tc(st, cache, g.N, g.P, g.Q, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, 1, 9, 1, ws->partial, &ctas, nullptr, s2);
       return e != cudaSuccess ? e : finish_wide_stats(st, g, ws, ctas, nparts, launches);
     }
-    return run_conv_tc(st, cache, g.N, g.H, g.W, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, g.stride, 9, 1, nullptr, nullptr, affine);
+    return run_conv_tc(st, cache, g.N, g.P, g.Q, g.Ci, g.Co, x, w, y, res, nullptr, err_dev, 1, 9, 1, nullptr, nullptr, affine, s2);
   }
   if (tc_1x1_fprop_eligible(g)) {
     ++*launches;
@@ -452,8 +474,8 @@ inline cudaError_t bf16_conv_fprop(cudaStream_t st, TensorMapCache* cache, const
 }
 
 // dx = conv^T(dy, w) [+ res * [mask > 0]].  `wflip` is the flipped/transposed weight copy (null: CUDA cores);
-// `dy_up` the spread-out dy of a stride-2 layer (null: its gradient stays on the CUDA cores).  `red` (mode 2)
-// asks for the sums of the batch-norm backward that dx feeds.
+// `red` (mode 2) asks for the sums of the batch-norm backward that dx feeds; a stride-2 layer forms them given `dy_up`, the
+// spread-out dy (nullable).
 inline cudaError_t bf16_conv_dgrad(cudaStream_t st, TensorMapCache* cache, const ConvGeom& g, const bf16_t* dy,
                                    const bf16_t* w, const bf16_t* wflip, const bf16_t* dy_up, bf16_t* dx, const bf16_t* res,
                                    const bf16_t* mask, const halo::EpiReduce* red, int* nparts, int* err_dev,
@@ -467,12 +489,12 @@ inline cudaError_t bf16_conv_dgrad(cudaStream_t st, TensorMapCache* cache, const
     if (fuse && nparts) *nparts = ctas;
     return e;
   }
-  const bool h1 = wflip && halo_dgrad_eligible(g), h2 = !h1 && wflip && dy_up && halo_s2_dgrad_eligible(g);
-  if (h1 || h2) {
+  const bool s2_sums = wflip && dy_up && red && red->mode == 2 && halo_s2_dgrad_sums_eligible(g);
+  if ((wflip && halo_dgrad_eligible(g)) || s2_sums) {
     ++*launches;
     const bool fuse = red && red->mode == 2 && halo_reduce_ok(g.Ci);
     int ctas = 0;
-    cudaError_t e = run_conv_halo(st, cache, g.N, g.H, g.W, g.Co, g.Ci, h1 ? dy : dy_up, wflip, dx, res, mask, err_dev, fuse ? red : nullptr, &ctas);
+    cudaError_t e = run_conv_halo(st, cache, g.N, g.H, g.W, g.Co, g.Ci, s2_sums ? dy_up : dy, wflip, dx, res, mask, err_dev, fuse ? red : nullptr, &ctas);
     if (fuse && nparts) *nparts = ctas;
     return e;
   }
@@ -480,9 +502,9 @@ inline cudaError_t bf16_conv_dgrad(cudaStream_t st, TensorMapCache* cache, const
     ++*launches;
     return run_conv_tc(st, cache, g.N, g.H, g.W, g.Co, g.Ci, dy, wflip, dx, res, mask, err_dev);
   }
-  if (wflip && dy_up && tc_s2_dgrad_eligible(g)) {
+  if (wflip && tc_s2_dgrad_eligible(g)) {
     ++*launches;
-    return run_conv_tc(st, cache, g.N, g.H, g.W, g.Co, g.Ci, dy_up, wflip, dx, res, mask, err_dev);
+    return run_conv_tc(st, cache, g.N, g.P, g.Q, g.Co, g.Ci, dy, wflip, dx, res, mask, err_dev, 1, 9, 1, nullptr, nullptr, nullptr, 2);
   }
   if (wflip && tc_1x1_dgrad_eligible(g) && (g.stride == 1 || (!res && !mask))) {
     // stride 2: only the even pixels of dx receive a gradient; the rest of dx is cleared first

@@ -48,8 +48,6 @@ struct FwdParams {
   uint32_t w_tx_bytes;        // bytes one weight-tap load writes
   int nacc;                   // accumulator slots in tensor memory
   uint32_t tmem_cols;
-  int sub;                    // 1, or 2: keep only the pixels with even h and w and store them as an
-                              // [N][H/2][W/2][Cn] tensor (a stride-2 convolution is the stride-1 one subsampled)
 };
 
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -192,7 +190,7 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
       auto prefetch_operands = [&](int tile) {
         int n0 = tile * p.G, n1 = n0 + p.G;
         if (n1 > p.N) n1 = p.N;
-        const size_t img = (size_t)(p.sub == 1 ? p.H * p.W : (p.H >> 1) * (p.W >> 1)) * p.Cn;   // elements per image
+        const size_t img = (size_t)(p.H * p.W) * p.Cn;   // elements per image
         const size_t off = (size_t)n0 * img;
         const uint32_t bytes = (uint32_t)((size_t)(n1 - n0) * img * 2);
         if (res) prefetch_l2_bulk(res + off, bytes);
@@ -306,8 +304,8 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     };
     auto fetch = [&](const Cursor& c, Operands& o) {
       const int n = c.tile * p.G + c.g;
-      o.valid = c.h < p.H && c.w < p.W && c.g < p.G && n < p.N && (p.sub == 1 || ((c.h | c.w) & 1) == 0);
-      const int pix = p.sub == 1 ? (n * p.H + c.h) * p.W + c.w : (n * (p.H >> 1) + (c.h >> 1)) * (p.W >> 1) + (c.w >> 1);
+      o.valid = c.h < p.H && c.w < p.W && c.g < p.G && n < p.N;
+      const int pix = (n * p.H + c.h) * p.W + c.w;
       o.base = (size_t)pix * p.Cn + c.chunk * 16;
       if (red.mode == 2) o.k0 = o.k1 = o.x0 = o.x1 = make_uint4(0, 0, 0, 0);   // read below whether or not the row is valid
       if (!o.valid) return;
@@ -421,8 +419,8 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
       Cursor nxt = cur;
       const bool have_next = advance(nxt);
       const int n = cur.tile * p.G + cur.g;
-      const bool valid = cur.h < p.H && cur.w < p.W && cur.g < p.G && n < p.N && (p.sub == 1 || ((cur.h | cur.w) & 1) == 0);
-      const int pix = p.sub == 1 ? (n * p.H + cur.h) * p.W + cur.w : (n * (p.H >> 1) + (cur.h >> 1)) * (p.W >> 1) + (cur.w >> 1);
+      const bool valid = cur.h < p.H && cur.w < p.W && cur.g < p.G && n < p.N;
+      const int pix = (n * p.H + cur.h) * p.W + cur.w;
       const int slot = cur.slot;
       if (!mbar_wait(&acc_full[slot], cur.aph, abort_flag)) return false;
       tc_fence_after();
@@ -461,8 +459,8 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     struct Operands2 { bool valid; int pix; uint4 k0, k1, x0, x1; };
     auto fetch2 = [&](const Cursor& c, Operands2& o) {
       const int n = c.tile * p.G + c.g;
-      o.valid = c.h < p.H && c.w < p.W && c.g < p.G && n < p.N && (p.sub == 1 || ((c.h | c.w) & 1) == 0);
-      o.pix = p.sub == 1 ? (n * p.H + c.h) * p.W + c.w : (n * (p.H >> 1) + (c.h >> 1)) * (p.W >> 1) + (c.w >> 1);
+      o.valid = c.h < p.H && c.w < p.W && c.g < p.G && n < p.N;
+      o.pix = (n * p.H + c.h) * p.W + c.w;
       o.k0 = o.k1 = o.x0 = o.x1 = make_uint4(0, 0, 0, 0);
       if (!o.valid) return;
       const size_t base = (size_t)o.pix * p.Cn;
@@ -781,7 +779,6 @@ inline bool chan_ok(int c) { return c == 16 || c == 32 || c == 64; }
 inline FwdParams fwd_params(int N, int H, int W, int Ck, int Cn, int sm_count) {
   FwdParams p{};
   p.W = W; p.H = H; p.N = N; p.Wp = W + 2; p.Hp = H + 2; p.Ck = Ck; p.Cn = Cn;
-  p.sub = 1;
   p.img_rows = p.Hp * p.Wp;
   p.pitch = (uint32_t)Ck * 2;
   p.w_tx_bytes = (uint32_t)Cn * p.pitch;

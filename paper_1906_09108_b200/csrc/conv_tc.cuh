@@ -52,9 +52,9 @@ struct ConvTcParams {
   int mpair;                // 128-row tiles a CTA works on at once with one weight tile: 1 (two accumulator sets, the
                             // epilogue of a tile overlaps the next tile's instructions) or 2 (one set of two accumulators:
                             // every weight tile fetched from L2 serves 256 rows)
-  int sub;                  // 1, or 2: store only the pixels with even h and w, as an [N][H/2][W/2][Co] tensor,
-                            // or 3: store pixel (h, w) at (2h, 2w) of an [N][2H][2W][Co] tensor (the data gradient of a
+  int sub;                  // 1, or 3: store pixel (h, w) at (2h, 2w) of an [N][2H][2W][Co] tensor (the data gradient of a
                             // stride-2 1x1 convolution; the other pixels of that tensor are not touched)
+  int s2;                   // 3x3 convolutions of stride 2 on the output grid H x W: 1 forward, 2 data gradient (below), 0 none
   int taps;                 // 9 (3x3, pad 1) or 1 (1x1, pad 0)
   int act_sub;              // 1, or 2: the activation operand is the even pixels of an [N][2H][2W][Ci] tensor
   int patch;                // 1: conv3x3_patch_kernel (16x16-pixel patches with their halo), 0: conv3x3_tc_kernel
@@ -63,6 +63,20 @@ struct ConvTcParams {
   int acc_slots;            // patch mode: accumulators of n_tile columns the 128-row tiles rotate over (3 where tensor
                             // memory holds them: the write-out of a tile then runs beside the next tiles' instructions)
 };
+// A 3x3 convolution of stride 2 and padding 1 on an even image, exactly (the same convolution at stride 1 and every second pixel of
+// it kept is four times the arithmetic):
+//   forward: output (p, q) and tap (r, s) meet pixel (2p + r - 1, 2q + s - 1).  The pixels of one parity are a regular strided
+//     tensor, so a tap reads the map of its parity -- odd for r = 0 and 2, one row up for r = 0; the same for columns;
+//   data gradient: the pixels (2p + a, 2q + b) of dx are a convolution of dy with the taps of one parity: row taps r = 1 (a = 0),
+//     or r = 0 one row further down and r = 2 (a = 1).  One launch takes the four classes one after the other, most taps first.
+// Measured against full resolution, 128 images, forward / data gradient (its dy spread out first): 64 -> 128 channels on 32x32
+// 24.8 / 44.6 -> 13.8 / 27.3 us, 128 -> 256 on 16x16 21.6 / 25.4 -> 16.2 / 20.5, 160 -> 320 on 32x32 90.7 / 119 -> 51.3 / 60.7.
+struct ActMaps { CUtensorMap m[4]; };             // the parities (row, column) of a forward of stride 2; else m[0]
+struct S2Class { int a, b, taps; };
+__host__ __device__ inline S2Class s2_class(const ConvTcParams& p, int cls) {
+  const int a = p.s2 == 2 ? 1 - (cls >> 1) : 0, b = p.s2 == 2 ? 1 - (cls & 1) : 0;
+  return S2Class{a, b, p.s2 == 2 ? (a + 1) * (b + 1) : p.taps};
+}
 constexpr int kPatch = 16;                         // patch side in pixels
 constexpr int kPatchHalo = kPatch + 2;             // with the one-pixel border
 
@@ -253,7 +267,7 @@ __device__ __forceinline__ void affine_apply(const float* area, int Co, int c, f
 // ------------------------------------------------------------------- kernel ----
 // out[m][n] (bf16, row stride Co) = conv + (res ? res[m][n] * [mask ? mask[m][n] > 0 : 1] : 0)
 __global__ void __launch_bounds__(kThreads, 1)
-conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+conv3x3_tc_kernel(const __grid_constant__ ActMaps map_a, const __grid_constant__ CUtensorMap map_b,
                   ConvTcParams p, __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ res,
                   const __nv_bfloat16* __restrict__ res_mask, float* __restrict__ stat_partial, EpiAffine aff, int* __restrict__ error_word) {
   __shared__ __align__(16) float stat_run[kStatFloats];
@@ -288,13 +302,16 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   }
 
   const int chunks = (p.Ci + p.kc - 1) / p.kc;
-  const int k_iters = p.taps * chunks;
-  const int total_tiles = ((p.m_tiles + p.mpair - 1) / p.mpair) * p.n_tiles;     // tiles of mpair * 128 rows
+  const int class_tiles = ((p.m_tiles + p.mpair - 1) / p.mpair) * p.n_tiles;     // tiles of mpair * 128 rows
+  const int total_tiles = p.s2 == 2 ? 4 * class_tiles : class_tiles;
 
   if (warp == 0) {
     if (lane == 0) {
       uint32_t it = 0;
-      for (int tile = blockIdx.x; tile < total_tiles && !*abort_flag; tile += gridDim.x) {
+      for (int tile_id = blockIdx.x; tile_id < total_tiles && !*abort_flag; tile_id += gridDim.x) {
+        const int cls = tile_id / class_tiles, tile = tile_id - cls * class_tiles;
+        const S2Class c2 = s2_class(p, cls);
+        const int k_iters = c2.taps * chunks;
         const int mg = tile / p.n_tiles, nt = tile - mg * p.n_tiles;
         int n0[2], h0[2];
         const int halves = (mg * p.mpair + 1 < p.m_tiles) ? p.mpair : 1;
@@ -308,14 +325,23 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
           const uint32_t ph = (it / p.stages) & 1;
           if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) break;
           const int tap = ki / chunks, cc = ki - tap * chunks;
-          const int r = tap / 3, sx = tap - r * 3;
-          const int dw = p.taps == 1 ? 0 : sx - 1, dh = p.taps == 1 ? 0 : r - 1;
+          int r = tap / 3, sx = tap - r * 3, wtap = tap, parity = 0;
+          int dw = p.taps == 1 ? 0 : sx - 1, dh = p.taps == 1 ? 0 : r - 1;
+          if (p.s2 == 1) {
+            parity = (r != 1 ? 2 : 0) + (sx != 1 ? 1 : 0);
+            dh = r == 0 ? -1 : 0; dw = sx == 0 ? -1 : 0;
+          } else if (p.s2 == 2) {
+            const int i = tap / (c2.b + 1), j = tap - i * (c2.b + 1);
+            r = c2.a ? 2 * i : 1; sx = c2.b ? 2 * j : 1;
+            dh = r == 0 ? 1 : 0; dw = sx == 0 ? 1 : 0;
+            wtap = (2 - r) * 3 + (2 - sx);             // the weights are the flipped copy
+          }
           uint8_t* a_dst = smem + (size_t)s * p.stage_bytes;
           uint8_t* b_dst = a_dst + (size_t)p.mpair * p.a_bytes;
           mbar_expect_tx(&full[s], (uint32_t)halves * p.a_tx_bytes + p.b_tx_bytes);
           for (int hf = 0; hf < halves; ++hf)
-            tma_load_4d(a_dst + (size_t)hf * p.a_bytes, &map_a, &full[s], cc * p.kc, dw, h0[hf] + dh, n0[hf]);
-          tma_load_2d(b_dst, &map_b, &full[s], tap * p.Ci + cc * p.kc, nt * p.n_tile);
+            tma_load_4d(a_dst + (size_t)hf * p.a_bytes, &map_a.m[parity], &full[s], cc * p.kc, dw, h0[hf] + dh, n0[hf]);
+          tma_load_2d(b_dst, &map_b, &full[s], wtap * p.Ci + cc * p.kc, nt * p.n_tile);
         }
       }
     }
@@ -338,7 +364,9 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       const int ksub_full = p.kc / 16, ksub_last = (p.Ci - (chunks - 1) * p.kc + 15) / 16;
       int s = 0;
       uint32_t ph = 0;                                         // it % stages and that stage's phase, kept incrementally
-      for (int tile = blockIdx.x; tile < total_tiles && !*abort_flag; tile += gridDim.x, ++tcount) {
+      for (int tile_id = blockIdx.x; tile_id < total_tiles && !*abort_flag; tile_id += gridDim.x, ++tcount) {
+        const int cls = tile_id / class_tiles, tile = tile_id - cls * class_tiles;
+        const int k_iters = s2_class(p, cls).taps * chunks;
         const int acc = (int)(tcount % nsets);
         const uint32_t acc_ph = (tcount / nsets) & 1;
         if (!mbar_wait(&acc_empty[acc], acc_ph ^ 1, abort_flag)) break;
@@ -382,7 +410,9 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     const int acc_row = lane_grp * 32 + lane;
     const int img_px = p.rows_per_tile * p.W;
     const int di = acc_row / img_px, dh = (acc_row - di * img_px) / p.W, dw = acc_row - di * img_px - dh * p.W;
-    for (int tile = blockIdx.x; tile < total_tiles && !*abort_flag; tile += gridDim.x, ++tcount) {
+    for (int tile_id = blockIdx.x; tile_id < total_tiles && !*abort_flag; tile_id += gridDim.x, ++tcount) {
+      const int cls = tile_id / class_tiles, tile = tile_id - cls * class_tiles;
+      const S2Class c2 = s2_class(p, cls);
       const int mg = tile / p.n_tiles, nt = tile - mg * p.n_tiles;
       const int acc = (int)(tcount % nsets);
       const uint32_t acc_ph = (tcount / nsets) & 1;
@@ -393,14 +423,9 @@ conv3x3_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       const int mt = mg * p.mpair + hf;
       const int grp = mt / p.tiles_per_img;
       const int n = grp * p.imgs_per_tile + di, h = (mt - grp * p.tiles_per_img) * p.rows_per_tile + dh, w = dw;
-      bool keep = di < p.imgs_per_tile && n < p.N && h < p.H;
+      const bool keep = di < p.imgs_per_tile && n < p.N && h < p.H;
       size_t base = ((size_t)n * p.H + h) * p.W + w;
-      if (p.sub == 2) {
-        keep = keep && ((h | w) & 1) == 0;
-        base = ((size_t)n * (p.H >> 1) + (h >> 1)) * (p.W >> 1) + (w >> 1);
-      } else if (p.sub == 3) {
-        base = ((size_t)n * (2 * p.H) + 2 * h) * (2 * p.W) + 2 * w;
-      }
+      if (p.sub == 3 || p.s2 == 2) base = ((size_t)n * (2 * p.H) + 2 * h + c2.a) * (2 * p.W) + 2 * w + c2.b;
       base = base * p.Co + (size_t)nt * p.n_tile;
       const int cols = p.Co - nt * p.n_tile < p.n_tile ? p.Co - nt * p.n_tile : p.n_tile;   // a multiple of 8
       const uint32_t taddr = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(acc + hf) * p.n_tile;
@@ -643,27 +668,19 @@ conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         if (!mbar_wait(&acc_full[slot], use & 1, abort_flag)) { live = false; break; }
         tc_fence_after();
         const int h = ph * kPatch + (i >> 3), w = pw * kPatch + 8 * g + (i & 7);
-        size_t base;
-        bool keep = true;
-        if (p.sub == 1) {
-          base = (((size_t)n * p.H + h) * p.W + w) * p.Co + (size_t)nt * p.n_tile;
-        } else {
-          keep = ((h | w) & 1) == 0;
-          base = (((size_t)n * (p.H >> 1) + (h >> 1)) * (p.W >> 1) + (w >> 1)) * p.Co + (size_t)nt * p.n_tile;
-        }
+        const size_t base = (((size_t)n * p.H + h) * p.W + w) * p.Co + (size_t)nt * p.n_tile;
         const uint32_t taddr = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + slot * (uint32_t)p.n_tile;
         const int cols = p.Co - nt * p.n_tile < p.n_tile ? p.Co - nt * p.n_tile : p.n_tile;
         for (int c0 = 0; c0 < cols; c0 += 16) {
           uint32_t v[16];
           tmem_ld16(taddr + c0, v);
           tmem_ld_wait();
-          if (!keep && !stat_partial) continue;
           const bool both = c0 + 8 < cols;
           float f[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e) f[e] = __uint_as_float(v[e]);
           if (aff.stats) affine_apply(stat_run, p.Co, nt * p.n_tile + c0, f);
-          if (res && keep) {
+          if (res) {
             uint4 r0 = *reinterpret_cast<const uint4*>(res + base + c0);
             uint4 r1 = both ? *reinterpret_cast<const uint4*>(res + base + c0 + 8) : make_uint4(0, 0, 0, 0);
             const __nv_bfloat16* rb0 = reinterpret_cast<const __nv_bfloat16*>(&r0);
@@ -697,12 +714,8 @@ conv3x3_patch_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
             ob0[e] = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
             ob1[e] = __floats2bfloat162_rn(f[8 + 2 * e], f[8 + 2 * e + 1]);
           }
-          if (keep) {
-            *reinterpret_cast<uint4*>(out + base + c0) = o0;
-            if (both) *reinterpret_cast<uint4*>(out + base + c0 + 8) = o1;
-          } else {
-            o0 = o1 = make_uint4(0, 0, 0, 0);
-          }
+          *reinterpret_cast<uint4*>(out + base + c0) = o0;
+          if (both) *reinterpret_cast<uint4*>(out + base + c0 + 8) = o1;
           if (stat_partial) stat_add(stat_run, warp - 2, (nt * p.n_tile + c0) >> 4, o0, o1, lane);
         }
         tc_fence_before();
@@ -766,9 +779,9 @@ inline bool conv_tc_supported(int N, int H, int W, int Ci, int Co, size_t pixels
   return W >= 1 && H >= 1 && W <= kTileM && H <= 256;
 }
 
-inline ConvTcParams conv_tc_params(int N, int H, int W, int Ci, int Co, int taps = 9, int share = 1) {
+inline ConvTcParams conv_tc_params(int N, int H, int W, int Ci, int Co, int taps = 9, int share = 1, int s2 = 0) {
   ConvTcParams p{};
-  p.W = W; p.H = H; p.N = N; p.Ci = Ci; p.Co = Co; p.sub = 1; p.taps = taps; p.act_sub = 1;
+  p.W = W; p.H = H; p.N = N; p.Ci = Ci; p.Co = Co; p.sub = 1; p.taps = taps; p.act_sub = s2 == 1 ? 2 : 1; p.s2 = s2;
   const int rows = kTileM / W;
   if (rows < H) {
     p.tiles_per_img = (H + rows - 1) / rows;
@@ -791,7 +804,7 @@ inline ConvTcParams conv_tc_params(int N, int H, int W, int Ci, int Co, int taps
   }
   p.m_tiles = ((N + p.imgs_per_tile - 1) / p.imgs_per_tile) * p.tiles_per_img;
   // 16x16-pixel patches with their halo wherever the image allows it and the chunks are full swizzle spans
-  p.patch = (taps == 9 && H % kPatch == 0 && W % kPatch == 0 && p.kc == 64) ? 1 : 0;
+  p.patch = (taps == 9 && s2 == 0 && H % kPatch == 0 && W % kPatch == 0 && p.kc == 64) ? 1 : 0;
   // The kernel is bound by the rate at which operand tiles arrive from L2, so a weight tile is shared by two
   // 128-row tiles -- unless the layer has so few pixels (small images, many channels) that the tiles would leave
   // most SMs idle: then single 128-row tiles and narrower column tiles, down to 64, until there are about 96, or, with
@@ -800,7 +813,7 @@ inline ConvTcParams conv_tc_params(int N, int H, int W, int Ci, int Co, int taps
   // 1.76 / 1.55, K = 4 1.74 / 1.51; WRN-16-4 on 24x24 1.11 / 1.03, 0.99 / 0.91, 1.06 / 0.96; WRN-28-10 within 1 % at any K).
   p.mpair = p.m_tiles >= 2 ? 2 : 1;
   if (!p.patch) {
-    auto tiles = [&]() { return ((p.m_tiles + p.mpair - 1) / p.mpair) * ((Co + nt - 1) / nt); };
+    auto tiles = [&]() { return ((p.m_tiles + p.mpair - 1) / p.mpair) * ((Co + nt - 1) / nt) * (s2 == 2 ? 4 : 1); };
     const int fill = 96 / (share > 0 ? share : 1);
     if (tiles() < fill) p.mpair = 1;
     while (tiles() < fill && nt % 32 == 0 && nt / 2 >= 64 && Co % (nt / 2) == 0) nt /= 2;
@@ -873,7 +886,7 @@ inline cudaError_t conv_tc_set_attrs(int dev) {
 }
 
 // `stat_partial` (nullable): room for one row of 2 * Co floats per CTA (at most sm_count rows); *ctas_out = rows written.
-inline cudaError_t conv_tc_launch(cudaStream_t st, const ConvTcParams& p, const CUtensorMap& map_a,
+inline cudaError_t conv_tc_launch(cudaStream_t st, const ConvTcParams& p, const ActMaps& map_a,
                                   const CUtensorMap& map_b, __nv_bfloat16* out, const __nv_bfloat16* res,
                                   const __nv_bfloat16* res_mask, int* error_word, int sm_count,
                                   float* stat_partial = nullptr, int* ctas_out = nullptr, const EpiAffine* affine = nullptr) {
@@ -883,9 +896,9 @@ inline cudaError_t conv_tc_launch(cudaStream_t st, const ConvTcParams& p, const 
     const int tiles = p.N * (p.H / kPatch) * (p.W / kPatch) * p.n_tiles;
     const int grid = tiles < sm_count ? tiles : sm_count;
     if (ctas_out) *ctas_out = grid;
-    return launch_chained(conv3x3_patch_kernel, grid, kPatchThreads, smem, st, map_a, map_b, p, out, res, res_mask, stat_partial, aff, error_word);
+    return launch_chained(conv3x3_patch_kernel, grid, kPatchThreads, smem, st, map_a.m[0], map_b, p, out, res, res_mask, stat_partial, aff, error_word);
   }
-  const int tiles = ((p.m_tiles + p.mpair - 1) / p.mpair) * p.n_tiles;
+  const int tiles = ((p.m_tiles + p.mpair - 1) / p.mpair) * p.n_tiles * (p.s2 == 2 ? 4 : 1);
   const int grid = tiles < sm_count ? tiles : sm_count;
   if (ctas_out) *ctas_out = grid;
   return launch_chained(conv3x3_tc_kernel, grid, kThreads, smem, st, map_a, map_b, p, out, res, res_mask, stat_partial, aff, error_word);

@@ -143,7 +143,7 @@ struct Module {
   int last_out_slot = -1, last_grad_slot = -1;
   cudaStream_t stream = nullptr;
   cudaStream_t stream2 = nullptr;          // side stream: weight gradients run beside the data-gradient chain
-  cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr, ev_buf[4] = {nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr, ev_buf[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t ev_act[kEventRing], ev_grad[kEventRing];
   // running batch-norm statistics (inference): flat vector, and the table the inference pass reads them through
   float* running = nullptr;
@@ -754,13 +754,13 @@ template <typename T> struct NextBnBwd { GateOf<T> mask; const T* x; const float
 
 template <typename T>
 static int conv_dgrad(Launch& L, Module& m, const ConvGeom& g, const T* dy, const T* w, const T* wflip, T* dx,
-                       const T* res, const GateOf<T> mask, const NextBnBwd<T>* next = nullptr, const T* dy_up = nullptr) {
+                       const T* res, const GateOf<T> mask, const NextBnBwd<T>* next = nullptr) {
   L.begin(KC_CONV_DGRAD, (out_elems(g) + w_elems(g) + in_elems(g) * (1 + (res ? 1 : 0) + (mask.tensor ? 1 : 0) + (next ? 2 : 0))) * sizeof(T), conv_flops(g));
   int nparts = 0;
   if constexpr (std::is_same<T, bf16>::value) {
     halo::EpiReduce r{};
     if (next) { r.mode = 2; r.mask = next->mask.tensor; r.mask_bits = next->mask.bits; r.xprev = next->x; r.pstats = next->stats; r.partial = m.red_partial; }
-    L.note(bf16_conv_dgrad(L.st, &L.c->tmaps, g, dy, w, wflip, dy_up, dx, res, mask.tensor, next ? &r : nullptr, &nparts, L.c->tc_error, &L.c->launches, mask.bits));
+    L.note(bf16_conv_dgrad(L.st, &L.c->tmaps, g, dy, w, wflip, nullptr, dx, res, mask.tensor, next ? &r : nullptr, &nparts, L.c->tc_error, &L.c->launches, mask.bits));
   } else {
     direct::Reduce<T> r{};
     if (next) r = direct::Reduce<T>{2, next->mask.tensor, next->x, next->stats, m.red_partial};
@@ -785,13 +785,13 @@ template <> const bf16* flipped_of<bf16>(const Module& m, int vslot, long long o
 }
 
 // dy [N][P][Q][Co] of a stride-2 convolution, spread onto the even pixels of a zero [N][H][W][Co] tensor
-// (module scratch); null when the stride-2 gradients of this shape stay on the CUDA cores.
+// (module scratch), for its weight gradient; null when that stays on the CUDA cores.
 template <typename T>
 static const T* upsample_dy(Launch& L, Module& m, const ConvGeom& g, const T* dy) {
   if constexpr (std::is_same<T, bf16>::value) {
     if (!m.up || !s2_uses_spread_dy(g)) return nullptr;
     T* up = reinterpret_cast<T*>(m.up);
-    L.begin(KC_CONV_DGRAD, (double)g.N * g.H * g.W * g.Co * 2 * 1.25, 0.0);
+    L.begin(KC_CONV_WGRAD, (double)g.N * g.H * g.W * g.Co * 2 * 1.25, 0.0);
     L.note(bf16_spread_dy(L.st, g, dy, up, &L.c->launches));
     return up;
   }
@@ -1035,7 +1035,7 @@ static void head_forward_backward(fdg_ctx* c, Module& m, Launch& L, int64_t tau,
 //   gfirst where the gradient of the module input goes (mailbox slot; unused for module 1)
 // `LS` issues on the module's side stream (the same stream as L when `forked` is false): the weight
 // gradients run there, beside the chain batch-norm backward -> data gradient -> next layer.  Buffers
-// a weight gradient reads (0: T1, 1: T4, 2: T2, 3: the spread-out dy) are not rewritten on the main
+// a weight gradient reads (0: T1, 1: T4, 2: T2) are not rewritten on the main
 // stream before the event recorded behind their last reader.
 template <typename T>
 static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool forked, int64_t tau, int slot, int vslot,
@@ -1052,7 +1052,7 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
   T* T4 = reinterpret_cast<T*>(m.temps[5]);
   auto gate = [&](size_t t, size_t q) { return GateOf<T>{S + t, sizeof(T) == 2 ? reinterpret_cast<const unsigned char*>(S + q) : nullptr}; };
   const GateOf<T> open{};
-  bool buf_read[4] = {false, false, false, false};
+  bool buf_read[3] = {false, false, false};
   bool side_used = false;
   auto fork = [&]() {
     if (!forked) return;
@@ -1193,12 +1193,10 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
         bn_backward<T>(L, m, T3, gate(u.t_b, u.q_b), S + u.t_a, F + u.st1, wf + u.g1, m.grad + u.g1, m.grad + u.b1, nullptr,
                        nullptr, nullptr, nullptr, nullptr, nullptr, T4, nullptr, rows_out, u.co, bn1_parts);      // dc1
         keep(i, 3, T4);
-        const T* up = nullptr;
-        if (u.stride == 2) { wait_buf(3); up = upsample_dy<T>(L, m, g1, T4); }
         fork();
+        const T* up = u.stride == 2 ? upsample_dy<T>(LS, m, g1, T4) : nullptr;
         conv_wgrad<T>(LS, m, g1, x, T4, m.grad + u.w1, up);                                              // side
         side_done(1);
-        if (up) side_done(3);
         const bool need_dx = !(m.k == 1 && i == 0);
         if (u.proj) {
           ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
@@ -1206,14 +1204,14 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
           side_done(2);
           if (need_dx) {
             conv_dgrad<T>(L, m, gs, T2, wt + u.ws, flipped_of<T>(m, vslot, u.fs), T3, nullptr, open);
-            out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, open, next, up);
+            out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, open, next);
           }
         } else if (need_dx && u.zpad) {
           // the shortcut's share: the gated upstream gradient's middle channels, put back at every stride-th pixel
           L.begin(KC_BN_BWD_APPLY, (double)(rows_out * u.co * 2 + rows_in * u.ci) * sizeof(T), 0.0);
           L.note(launch_chained(pad_shortcut_bwd_kernel<T>, ew_blocks(rows_in * u.ci), 256, 0, L.st, dy, S + u.t_y, T3, rows_in, u.P, u.Q, u.H, u.W, u.ci, u.co, u.stride));
           ++c->launches;
-          out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, open, next, up);
+          out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, open, next);
         } else if (need_dx) {
           out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, dy, gate(u.t_y, u.q_y), next);
         }
@@ -1237,7 +1235,7 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
           conv_wgrad<T>(L, m, gs, S + u.t_a, dy, m.grad + u.ws);
           conv_dgrad<T>(L, m, gs, dy, wt + u.ws, flipped_of<T>(m, vslot, u.fs), T3, nullptr, open);
           keep(i, 5, T3);
-          conv_dgrad<T>(L, m, g1, T2, wt + u.w1, flipped_of<T>(m, vslot, u.f1), T1, T3, open, nullptr, up);   // do
+          conv_dgrad<T>(L, m, g1, T2, wt + u.w1, flipped_of<T>(m, vslot, u.f1), T1, T3, open);   // do
         } else {
           conv_dgrad<T>(L, m, g1, T2, wt + u.w1, flipped_of<T>(m, vslot, u.f1), T1, nullptr, open);
         }
@@ -1502,7 +1500,7 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&m.stream2, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.ev_fork2, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.ev_join2, cudaEventDisableTiming);
-    for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&m.ev_buf[i], cudaEventDisableTiming);
+    for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&m.ev_buf[i], cudaEventDisableTiming);
     for (int i = 0; i < kEventRing && e == cudaSuccess; ++i) {
       e = cudaEventCreateWithFlags(&m.ev_act[i], cudaEventDisableTiming);
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.ev_grad[i], cudaEventDisableTiming);
@@ -1550,7 +1548,7 @@ fdg_status fdg_destroy(fdg_ctx* c) {
     if (m.stream2) cudaStreamDestroy(m.stream2);
     if (m.ev_fork2) cudaEventDestroy(m.ev_fork2);
     if (m.ev_join2) cudaEventDestroy(m.ev_join2);
-    for (int i = 0; i < 4; ++i) if (m.ev_buf[i]) cudaEventDestroy(m.ev_buf[i]);
+    for (int i = 0; i < 3; ++i) if (m.ev_buf[i]) cudaEventDestroy(m.ev_buf[i]);
   }
   for (int i = 0; i < kEventRing; ++i) cudaEventDestroy(c->ev_in[i]);
   cudaEventDestroy(c->ev_join);
