@@ -10,7 +10,7 @@
 //   - a convolution's output (rounded to bf16) goes from tensor memory into the operand's place, whose instructions are done
 //     by then: the apply reads it there;
 //   - what the CTAs must know of one another is 2 * C sums per layer: every CTA publishes its own as (value, tag) words and
-//     reads all of them (exchange() below).  The launch is cooperative: its CTAs are resident together, and several such launches
+//     reads all of them (publish and collect below).  The launch is cooperative: its CTAs are resident together, and several such launches
 //     on different streams run side by side (measured: 4 launches of 32 CTAs take the time of one; an exchange costs 1.1 us).
 // Measured, 128 images of 32x32x16 on 64 CTAs: a layer's forward pass 8 us, its backward pass up to the weight gradient 11 us
 // (convolution and apply by themselves: 13 us, and 20 to 25); ResNet-56 with K = 2 1.09 -> 0.84 ms per iteration, an inference
@@ -402,8 +402,8 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
     };
 
     // Sums: `run` holds this thread's, 8 channels each of two statistics.  warp_sums leaves the warp's in shared memory, cta_sum
-    // adds the warps in order, exchange publishes this CTA's and adds everybody's: afterwards s0, s1 are the totals of channel
-    // etid for etid < C.  Barriers of the epilogue warps: one in warp_sums, one in exchange, one behind the use of the totals.
+    // adds the warps in order, publish makes this CTA's known, collect adds everybody's.  What else a layer needs meanwhile is
+    // issued between the two.  Barriers of the epilogue warps: one in warp_sums, one in collect, one behind the use of the totals.
     auto warp_sums = [&](const f32x2 (&run2)[8]) {
       float run[16];
 #pragma unroll
@@ -423,21 +423,28 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
       for (int w = 0; w < kEpiWarps; ++w) a += d[w * 2 * C];
       return a;
     };
-    auto exchange = [&](int number, float own, double& s0, double& s1) { // `own`: this CTA's sum etid (etid < 2 * C)
-      unsigned long long* words = ex.words + (size_t)(number & 1) * kMaxCtas * 2 * C;
+    auto words_of = [&](int number) { return ex.words + (size_t)(number & 1) * kMaxCtas * 2 * C; };
+    auto publish = [&](int number, float own) {     // `own`: this CTA's sum etid, for etid < 2 * C
+      if (etid < 2 * C) st_word(words_of(number) + (size_t)blockIdx.x * 2 * C + etid, epoch + 1u + (uint32_t)number, own);
+    };
+    // First thread (sum etid % (2 * C), segment etid / (2 * C)) adds every kSegs-th CTA's word; then a warp has C / 16 channels:
+    // lane (channel, statistic, segment).  A channel's leader ends up with its totals.  (A CTA's words lie in a row of their own:
+    // with all CTAs' words of a sum side by side an exchange took twice as long.)
+    constexpr int kSegs = kEpiThreads / (2 * C);
+    const int chan = ewarp * (C / 16) + lane / (2 * kSegs);
+    const bool leader = lane % (2 * kSegs) == 0;
+    auto collect = [&](int number, double& s0, double& s1) {
       const uint32_t tag = epoch + 1u + (uint32_t)number;
-      if (etid < 2 * C) st_word(words + (size_t)blockIdx.x * 2 * C + etid, tag, own);
-      constexpr int nseg = kEpiThreads / (2 * C);
-      const int pr = etid % (2 * C), seg = etid / (2 * C);
+      const unsigned long long* mine = words_of(number) + etid % (2 * C);
       double a = 0.0;
-      for (int b0 = seg; b0 < step; b0 += 8 * nseg) {
+      for (int b0 = etid / (2 * C); b0 < step; b0 += 8 * kSegs) {
         unsigned long long v[8];
         for (uint32_t i = 0; ; ++i) {
           bool all = true;
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
-            const int b = b0 + u * nseg;
-            v[u] = b < step ? ld_word(words + (size_t)b * 2 * C + pr) : (unsigned long long)tag << 32;
+            const int b = b0 + u * kSegs;
+            v[u] = b < step ? ld_word(mine + (size_t)b * 2 * C) : (unsigned long long)tag << 32;
             all = all && (uint32_t)(v[u] >> 32) == tag;
           }
           if (all) break;
@@ -449,9 +456,11 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
       }
       part[etid] = a;
       epi_sync();
-      s0 = s1 = 0.0;
-      if (etid < C)
-        for (int q = 0; q < nseg; ++q) { s0 += part[q * 2 * C + etid]; s1 += part[q * 2 * C + C + etid]; }
+      a = part[lane % kSegs * (2 * C) + lane / kSegs % 2 * C + chan];
+#pragma unroll
+      for (int o = kSegs / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      s0 = a;
+      s1 = __shfl_down_sync(0xffffffffu, a, kSegs);
     };
 
     if constexpr (PASS != BACKWARD) {
@@ -542,22 +551,23 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
             }
           }
           warp_sums(run);
+          publish(l, etid < 2 * C ? cta_sum(etid) : 0.f);
           if (!last) fetch_weights(l + 1, 0);       // every instruction of this layer is done
-          const float ga = etid < C ? gamma[etid] : 0.f, be = etid < C ? gamma[C + etid] : 0.f;
-          float* run_at = fa.running + (size_t)l * 2 * C + etid;
-          const bool keeper = blockIdx.x == 0 && etid < C;
-          const float rmean = keeper ? run_at[0] : 0.f, rvar = keeper ? run_at[C] : 0.f;      // ahead of the exchange: see update_running
+          const float ga = gamma[chan], be = gamma[C + chan];
+          float* run_at = fa.running + (size_t)l * 2 * C + chan;
+          const bool keeper = blockIdx.x == 0 && leader;
+          const float rmean = keeper ? run_at[0] : 0.f, rvar = keeper ? run_at[C] : 0.f;      // see update_running
           double s0, s1;
-          exchange(l, etid < 2 * C ? cta_sum(etid) : 0.f, s0, s1);
+          collect(l, s0, s1);
           if (!last) weights_done(0);
-          if (etid < C) {
+          if (leader) {
             const double mean = s0 * fa.inv_count;
             double var = s1 * fa.inv_count - mean * mean;
             if (var < 0.0) var = 0.0;
             const float mu = (float)mean, inv = inverse_sqrt(var + (double)fa.eps);
-            k[etid] = -mu; k[C + etid] = ga * inv; k[2 * C + etid] = be;
-            if (blockIdx.x == 0) {
-              stats[etid] = mu; stats[C + etid] = inv;
+            k[chan] = -mu; k[C + chan] = ga * inv; k[2 * C + chan] = be;
+            if (keeper) {
+              stats[chan] = mu; stats[C + chan] = inv;
               run_at[0] = (1.f - fa.momentum) * rmean + fa.momentum * mu;
               run_at[C] = (1.f - fa.momentum) * rvar + fa.momentum * ((float)var * fa.unbias);
             }
@@ -734,32 +744,32 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
         const uint32_t ph = (uint32_t)s & 1u;
         // -- totals of batch norm l; constants of the next one (l - 1, or the one in front of the run)
         warp_sums(run);
-        if (s > 0) fetch_weights(l, 0);             // every instruction of the layer before is done
-        ask(l - 2);
-        Px v;                                       // the apply's first operand, ahead of the exchange
-        load(conv_out_of(l), place(tab[stream < tiles ? stream : 0], 0), v);
-        float ga = 0.f, nmean = 0.f, ninv = 0.f, own = 0.f;
-        const float* nst = l > 0 ? ts.stats + (size_t)(l - 1) * ts.st_step : ba.out_stats;
-        if (etid < C) {
-          ga = ts.gamma[(size_t)l * ts.p_step + etid];
-          if (nst) { nmean = nst[etid]; ninv = nst[C + etid]; }
-        }
+        float own = 0.f;
         if (etid < 2 * C) {
           own = cta_sum(etid);
           if (etid >= C) own *= k[etid];            // invstd of channel etid - C
         }
+        publish(s, own);
+        if (s > 0) fetch_weights(l, 0);             // every instruction of the layer before is done
+        ask(l - 2);
+        Px v;                                       // the apply's first operand
+        load(conv_out_of(l), place(tab[stream < tiles ? stream : 0], 0), v);
+        float nmean = 0.f, ninv = 0.f;
+        const float ga = ts.gamma[(size_t)l * ts.p_step + chan];
+        const float* nst = l > 0 ? ts.stats + (size_t)(l - 1) * ts.st_step : ba.out_stats;
+        if (nst) { nmean = nst[chan]; ninv = nst[C + chan]; }
         double s0, s1;
-        exchange(s, own, s0, s1);
+        collect(s, s0, s1);
         weights_done(0);
         float* kn = cst + ((l + 1) & 1) * 5 * C;
-        if (etid < C) {
-          const float inv = k[C + etid], gi = ga * inv;
+        if (leader) {
+          const float inv = k[C + chan], gi = ga * inv;
           const float t0 = (float)s0, t1 = (float)s1;
-          k[2 * C + etid] = gi; k[3 * C + etid] = -(t0 * ba.inv_m * gi); k[4 * C + etid] = -(t1 * ba.inv_m * (gi * inv));
-          kn[etid] = -nmean; kn[C + etid] = ninv;
+          k[2 * C + chan] = gi; k[3 * C + chan] = -(t0 * ba.inv_m * gi); k[4 * C + chan] = -(t1 * ba.inv_m * (gi * inv));
+          kn[chan] = -nmean; kn[C + chan] = ninv;
           if (blockIdx.x == 0) {
             float* dg = ba.dgamma + (size_t)l * ts.p_step;
-            dg[etid] = t1; dg[C + etid] = t0;
+            dg[chan] = t1; dg[C + chan] = t0;
           }
         }
         epi_sync();
