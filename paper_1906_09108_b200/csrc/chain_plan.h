@@ -36,7 +36,7 @@ constexpr size_t kSmemLimit = 226 * 1024;
 // launch waits for a CTA elsewhere.  Their registers forbid it already (640 threads of 96); their shared memory does too.
 constexpr size_t kSmemLeast = 120 * 1024;
 inline size_t fixed_smem(int C) {
-  return (size_t)kEpiThreads * 8 + (size_t)kEpiWarps * 2 * C * 4 + (size_t)2 * 5 * C * 4 + (3 * kAccSlots + 2) * 8 + 16 + kAccSlots * sizeof(Tile) + 1024;
+  return (size_t)kEpiThreads * 8 + (size_t)kEpiWarps * 2 * C * 4 + (size_t)2 * 5 * C * 4 + (3 * kAccSlots + 4) * 8 + 16 + kAccSlots * sizeof(Tile) + 1024;
 }
 // Launch shape: about `sms` CTAs; images = 0 where the shape is not covered.  A CTA holds its images' operands and accumulators.
 inline Geom chain_geom(int N, int H, int W, int C, int layers, int sms, int pass) {

@@ -20,10 +20,10 @@
 // bytes), a tile 16 image rows x 8 groups.  Pixel i of a group has the columns from (G - 1 - i) * C on: in this order the
 // filter taps a window position needs are neighbours in memory, and the nine taps are kept once (9 * C * C values).
 //
-// Roles by warp: 0..1 issue instructions (alternate tiles), 4..19 epilogue: a thread has 8 channels of a pixel in two
-// neighbouring groups of every tile.  They also bring the next layer's weights while the sums travel, and, in the backward
-// pass, ask for the saved tensors two layers ahead into L2.  Every wait is bounded; after one that ran out the roles run to their ends without
-// waiting any more (barriers among them stay matched) and the CTA raises an error word.
+// Roles by warp: 0..1 issue instructions (alternate tiles), 2..3 bring the weights of the next layer (and, in the backward pass,
+// ask for the saved tensors two layers ahead into L2), 4..19 epilogue: a thread has 8 channels of two pixels of every part of
+// a tile.  Every wait is bounded; after one that ran out the roles run to their ends without waiting any more (barriers among
+// them stay matched) and the CTA raises an error word.
 #pragma once
 #include <type_traits>
 
@@ -36,7 +36,7 @@ namespace chain {
 using namespace fdg::tc;
 using rows::Window;
 
-constexpr int kIssuers = 2;
+constexpr int kIssuers = 2, kLoaders = 2;
 constexpr int kFirstEpi = 4;                      // a warpgroup of its own for the issuers: it gives its registers to the others
 constexpr int kIssuerRegs = 56, kEpiRegs = 104;  // of 96 each at launch: 128 * 56 + 512 * 104 <= 640 * 96
 constexpr int kThreads = 32 * kFirstEpi + kEpiThreads;
@@ -211,7 +211,8 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
   uint64_t* a_ready = a_full + kAccSlots;           // [images]  rewritten by the epilogue
   uint64_t* acc_full = a_ready + kAccSlots;         // [tiles]   accumulator complete
   uint64_t* w_full = acc_full + kAccSlots;          // [w_stages]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 2);
+  uint64_t* w_empty = w_full + 2;                   // [w_stages]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint32_t* epoch_smem = tmem_slot + 2;
   Tile* tab = reinterpret_cast<Tile*>(tmem_slot + 4);                                     // [kAccSlots]
@@ -220,9 +221,9 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
   const int step = (int)gridDim.x;
   const int images = (p.N - 1 - (int)blockIdx.x) / step + 1;           // the grid has at most N CTAs
   const int tiles = images * p.tpi;
-  if (threadIdx.x < (unsigned)(3 * kAccSlots + 2)) {
+  if (threadIdx.x < (unsigned)(3 * kAccSlots + 4)) {
     const int i = threadIdx.x;
-    const uint32_t count = i < kAccSlots ? 1 : (i < 2 * kAccSlots ? p.tpi * kEpiWarps / S : (i < 3 * kAccSlots ? 1 : kEpiWarps));
+    const uint32_t count = i < kAccSlots ? 1 : (i < 2 * kAccSlots ? p.tpi * kEpiWarps / S : (i < 3 * kAccSlots ? 1 : (i < 3 * kAccSlots + 2 ? kLoaders : kIssuers)));
     mbar_init(bars + i, count);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -274,8 +275,42 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
             rows::commit_by(leader, &acc_full[t]);
           }
       }
+      if (ok) rows::commit_by(leader, &w_empty[ws]);
       if (++ws == p.w_stages) { ws = 0; wph ^= 1u; }
     }
+    } else {
+      // shared memory: [tap][c_out] rows of C channels, swizzled; global memory: [c_out][tap][C]
+      constexpr uint32_t mask = C == 64 ? 7u : (C == 32 ? 3u : 1u);
+      constexpr int kPieces = C / 8;                // 16-byte pieces of a row
+      const int lt = (warp - kIssuers) * 32 + lane;
+      const uint32_t img_elems = (uint32_t)(p.H * p.W) * C;
+      auto ask = [&](int l) {                       // the saved tensors of batch norm l, into L2
+        if (l < 0 || lt >= images) return;
+        const size_t n = (size_t)((int)blockIdx.x + lt * step);
+        halo::prefetch_l2_bulk(ts.t0 + (size_t)(l >> 1) * ts.b_step + ((l & 1) ? 2 * ts.t_step : 0) + n * img_elems, img_elems * 2);
+        if (img_elems % 128 == 0)
+          halo::prefetch_l2_bulk(ts.q0 + (size_t)(l >> 1) * ts.b_step * 2 + ((l & 1) ? ts.q_step : 0) + n * (img_elems / 8), img_elems / 8);
+      };
+      if (PASS == BACKWARD) ask(p.layers - 2);
+      int ws = 0;
+      uint32_t wph = 0;
+      for (int s = 0; s < p.layers; ++s) {
+        const int l = PASS == BACKWARD ? p.layers - 1 - s : s;
+        if (s >= p.w_stages) chain_wait(&w_empty[ws], wph ^ 1u, abort_flag);
+        const uint32_t dst = smem_u32(w_smem + (size_t)ws * p.w_bytes);
+        const __nv_bfloat16* src = ts.w + (size_t)l * ts.w_step;
+        for (int i = lt; i < 9 * C * kPieces; i += 32 * kLoaders) {
+          const int r = i / kPieces, pc = i - r * kPieces, tap = r / C, co = r - tap * C;
+          const uint32_t o = (uint32_t)i * 16;
+          cp_async16(dst + (o ^ (((o >> 7) & mask) << 4)), src + (co * 9 + tap) * C + pc * 8);
+        }
+        if (PASS == BACKWARD) ask(l - 2);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        halo::fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&w_full[ws]);
+        if (++ws == p.w_stages) { ws = 0; wph ^= 1u; }
+      }
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpiRegs));
@@ -297,25 +332,6 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
         mbar_expect_tx(&a_full[j], p.a_tx);
         tma_load_4d(smem + (size_t)j * p.a_bytes, &map_x, &a_full[j], 0, -1, -1, (int)blockIdx.x + j * step);
       }
-    // The weights of convolution l: requested into stage `ws`, and handed to the issuers once they have landed.  Shared memory:
-    // [tap][c_out] rows of C channels, swizzled; global memory: [c_out][tap][C].
-    auto fetch_weights = [&](int l, int ws) {
-      constexpr uint32_t mask = C == 64 ? 7u : (C == 32 ? 3u : 1u);
-      constexpr int kPieces = C / 8;                // 16-byte pieces of a row
-      const uint32_t dst = smem_u32(w_smem + (size_t)ws * p.w_bytes);
-      const __nv_bfloat16* src = ts.w + (size_t)l * ts.w_step;
-      for (int i = etid; i < 9 * C * kPieces; i += kEpiThreads) {
-        const int r = i / kPieces, pc = i - r * kPieces, tap = r / C, co = r - tap * C;
-        const uint32_t o = (uint32_t)i * 16;
-        cp_async16(dst + (o ^ (((o >> 7) & mask) << 4)), src + (co * 9 + tap) * C + pc * 8);
-      }
-    };
-    auto weights_done = [&](int ws) {
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      halo::fence_proxy_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&w_full[ws]);
-    };
     // Relative to a tile: elements of a tensor, bytes of the operands (a tile and an image start at a multiple of 8 lines, so the
     // swizzle of a line does not depend on them).
     const uint32_t row_elems = (uint32_t)p.WG * 64u, pitch = (uint32_t)(kTileGroups * p.cb + 2);
@@ -464,9 +480,6 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
     };
 
     if constexpr (PASS != BACKWARD) {
-      fetch_weights(0, 0);
-      weights_done(0);
-      if (PASS == INFER && p.w_stages == 2) fetch_weights(1, 1);
       if (PASS == INFER && etid < C) {
         cst[etid] = -ts.stats[etid]; cst[C + etid] = ts.gamma[etid] * ts.stats[C + etid]; cst[2 * C + etid] = ts.gamma[C + etid];
       }
@@ -552,14 +565,12 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
           }
           warp_sums(run);
           publish(l, etid < 2 * C ? cta_sum(etid) : 0.f);
-          if (!last) fetch_weights(l + 1, 0);       // every instruction of this layer is done
           const float ga = gamma[chan], be = gamma[C + chan];
           float* run_at = fa.running + (size_t)l * 2 * C + chan;
           const bool keeper = blockIdx.x == 0 && leader;
           const float rmean = keeper ? run_at[0] : 0.f, rvar = keeper ? run_at[C] : 0.f;      // see update_running
           double s0, s1;
           collect(l, s0, s1);
-          if (!last) weights_done(0);
           if (leader) {
             const double mean = s0 * fa.inv_count;
             double var = s1 * fa.inv_count - mean * mean;
@@ -574,22 +585,23 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
           }
           epi_sync();
         } else {
-          epi_sync();                               // every warp is done with the layer before: its constants' place is free
-          if (p.w_stages == 2 && !last) weights_done((l + 1) & 1);
+          // The next layer's constants: requested now, put down when this layer's first convolution is done (every warp is done
+          // with the layer before then, and with its constants).
+          float n0 = 0.f, n1 = 0.f, n2 = 0.f;
           if (!last && etid < C) {
-            float* kn = cst + ((l + 1) & 1) * 5 * C;
             const float* sn = stats + ts.st_step;
             const float* gn = gamma + ts.p_step;
-            kn[etid] = -sn[etid]; kn[C + etid] = gn[etid] * sn[C + etid]; kn[2 * C + etid] = gn[C + etid];
+            n0 = -sn[etid]; n1 = gn[etid] * sn[C + etid]; n2 = gn[C + etid];
+          }
+          epi_sync();
+          wait_image(tab[0], ph);
+          if (!last && etid < C) {
+            float* kn = cst + ((l + 1) & 1) * 5 * C;
+            kn[etid] = n0; kn[C + etid] = n1; kn[2 * C + etid] = n2;
           }
         }
         if (second) apply(std::true_type{}, k, ph, last, res, act_out, bits);
         else apply(std::false_type{}, k, ph, last, nullptr, act_out, bits);
-        if (PASS == INFER && l + p.w_stages < p.layers) {                // once every instruction of this layer is done
-          for (int t = 0; t < tiles; ++t) chain_wait(&acc_full[t], ph, abort_flag);
-          fetch_weights(l + p.w_stages, p.w_stages == 2 ? l & 1 : 0);
-          if (p.w_stages == 1) weights_done(0);
-        }
       }
       if (PASS == TRAIN && blockIdx.x == 0 && etid == 0) *ex.epoch = epoch + (uint32_t)p.layers;
     } else {
@@ -619,16 +631,6 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
         float* k = cst + (top & 1) * 5 * C;
         k[etid] = -st[etid]; k[C + etid] = st[C + etid];
       }
-      fetch_weights(top, 0);
-      // the saved tensors of batch norm l, asked into L2
-      const uint32_t img_bytes = (uint32_t)((size_t)p.H * p.W * C * 2);
-      auto ask = [&](int l) {
-        if (l < 0 || etid >= images) return;
-        const size_t n = (size_t)((int)blockIdx.x + etid * step);
-        halo::prefetch_l2_bulk(conv_out_of(l) + n * (img_bytes / 2), img_bytes);
-        if (img_bytes % 256 == 0) halo::prefetch_l2_bulk(bits_of(l) + n * (img_bytes / 16), img_bytes / 16);
-      };
-      ask(top - 1);
       epi_sync();
       // The gradient of the last block's output: gated (the operand's place has it, and `dy` in place of itself for the shortcut),
       // with the sums of that block's second batch norm.
@@ -750,8 +752,6 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
           if (etid >= C) own *= k[etid];            // invstd of channel etid - C
         }
         publish(s, own);
-        if (s > 0) fetch_weights(l, 0);             // every instruction of the layer before is done
-        ask(l - 2);
         Px v;                                       // the apply's first operand
         load(conv_out_of(l), place(tab[stream < tiles ? stream : 0], 0), v);
         float nmean = 0.f, ninv = 0.f;
@@ -760,7 +760,6 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
         if (nst) { nmean = nst[chan]; ninv = nst[C + chan]; }
         double s0, s1;
         collect(s, s0, s1);
-        weights_done(0);
         float* kn = cst + ((l + 1) & 1) * 5 * C;
         if (leader) {
           const float inv = k[C + chan], gi = ga * inv;
