@@ -267,7 +267,7 @@ inline cudaError_t run_wgrad_halo(cudaStream_t st, TensorMapCache* cache, int N,
   if (n >= ((size_t)1 << 17) && ctas <= 8)        // large filters, few partials: four outputs per thread, partials in turn
     return launch_chained(wide::wgrad_wide_sum_kernel, dim3((unsigned)((n / 4 + 255) / 256)), dim3(256), 0, st,
                           reinterpret_cast<const float4*>(scratch), reinterpret_cast<float4*>(dw), n / 4, ctas);
-  return launch_chained(halo::wgrad_halo_reduce_kernel, dim3((unsigned)((n + 31) / 32)), dim3(256), 0, st, (const float*)scratch, dw, n, ctas, n);
+  return launch_chained(halo::wgrad_halo_reduce_kernel, dim3((unsigned)((n + 31) / 32)), dim3(256), 0, st, (const float*)scratch, dw, n, ctas);
 }
 // The weight gradients of `layers` layers of one shape (c_in = c_out = C) in two launches: x[i], dy[i] -> dw + i * dw_step.
 // `scratch`: wgrad_group_scratch_elems floats.
@@ -277,9 +277,10 @@ inline size_t wgrad_group_scratch_elems(int N, int H, int W, int C, int layers, 
 }
 inline cudaError_t run_wgrad_group(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int C, int layers, const bf16_t* const* x,
                                    const bf16_t* const* dy, float* dw, size_t dw_step, float* scratch, int* err_dev, int cap, uint64_t* launches) {
-  const halo::WgradParams p = halo::wgrad_params(N, H, W, C, C);
+  halo::WgradParams p = halo::wgrad_params(N, H, W, C, C);
   cudaError_t e = halo::set_smem_attrs(cached_device(cache));
   const int ctas = halo::wgrad_ctas(p, cap);
+  p.stages = 1;                                   // two CTAs per SM instead
   const size_t n = (size_t)C * 9 * C;
   for (int l0 = 0; l0 < layers && e == cudaSuccess; l0 += halo::kWgradLayers) {
     const int nl = std::min(halo::kWgradLayers, layers - l0);
@@ -295,8 +296,8 @@ inline cudaError_t run_wgrad_group(cudaStream_t st, TensorMapCache* cache, int N
     e = launch_chained(halo::wgrad_halo_kernel<halo::kWgradLayers>, dim3(ctas, halo::wgrad_pairs(p), nl), dim3(halo::kFwdThreads),
                        halo::wgrad_smem_bytes(p), st, maps, p, scratch, err_dev);
     if (e == cudaSuccess)
-      e = launch_chained(halo::wgrad_halo_reduce_kernel, dim3((unsigned)((n + 31) / 32), nl), dim3(256), 0, st, (const float*)scratch,
-                         dw + (size_t)l0 * dw_step, n, ctas, dw_step);
+      e = launch_chained(halo::wgrad_group_sum_kernel, dim3((unsigned)((n / 2 + 127) / 128), nl), dim3(128), 0, st,
+                         reinterpret_cast<const float2*>(scratch), dw + (size_t)l0 * dw_step, (int)(n / 2), ctas, dw_step);
     *launches += 2;
   }
   return e;

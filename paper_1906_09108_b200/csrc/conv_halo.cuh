@@ -596,11 +596,13 @@ struct WgradParams {
 };
 
 // One launch takes up to NL layers of the same shape (blockIdx.z): a layer's split is bounded by what the sums cost, so one
-// layer alone leaves most SMs idle, and every launch costs its start and its end.
+// layer alone leaves most SMs idle, and every launch costs its start and its end.  With several layers two CTAs share an SM, each
+// with one stage of tiles: the start, the loads and the write-out of one run beside the instructions of the other (ResNet-110
+// K = 4 10.31 -> 9.96 ms a logging interval, ResNet-1202 29.99 -> 29.31, ResNet-56 K = 2 6.45 -> 6.40).
 constexpr int kWgradLayers = 32;
 template <int NL> struct WgradMaps { CUtensorMap x[NL], y[NL]; };
 template <int NL>
-__global__ void __launch_bounds__(kFwdThreads, 1)
+__global__ void __launch_bounds__(kFwdThreads, NL == 1 ? 1 : 2)
 wgrad_halo_kernel(const __grid_constant__ WgradMaps<NL> maps, WgradParams p, float* __restrict__ partial, int* __restrict__ error_word) {
   const CUtensorMap& map_x = maps.x[NL == 1 ? 0 : blockIdx.z];
   const CUtensorMap& map_y = maps.y[NL == 1 ? 0 : blockIdx.z];
@@ -745,11 +747,8 @@ wgrad_halo_kernel(const __grid_constant__ WgradMaps<NL> maps, WgradParams p, flo
 }
 
 // dw[i] = sum over the pixel-split CTAs of partial[cta][i], in CTA order.  A block owns 32
-// consecutive outputs; its 8 warps take interleaved CTAs and are added in warp order.  blockIdx.y: layers, `dw_step` apart.
-__global__ void __launch_bounds__(256) wgrad_halo_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, size_t n, int ctas,
-                                                                size_t dw_step) {
-  partial += (size_t)blockIdx.y * ctas * n;
-  dw += (size_t)blockIdx.y * dw_step;
+// consecutive outputs; its 8 warps take interleaved CTAs and are added in warp order.
+__global__ void __launch_bounds__(256) wgrad_halo_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dw, size_t n, int ctas) {
   __shared__ float part[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const size_t i = (size_t)blockIdx.x * 32 + lane;
@@ -767,6 +766,26 @@ __global__ void __launch_bounds__(256) wgrad_halo_reduce_kernel(const float* __r
     for (int w = 0; w < 8; ++w) t += part[w][lane];
     dw[i] = t;
   }
+}
+// The same for several layers (blockIdx.y, `dw_step` floats apart; n even, dw 8-byte aligned): a thread adds two outputs, every
+// eighth CTA into one of eight sums, those in order.  128 threads of 32 registers: such a block still finds room beside a CTA of
+// conv_chain.cuh (640 threads of 96), which the kernel above, at one block of 256 per 32 outputs, does not (ResNet-1202 K = 4: 45 us
+// a launch of up to 24 layers, now 15; 29.3 -> 27.2 ms a logging interval).
+__global__ void __launch_bounds__(128, 16) wgrad_group_sum_kernel(const float2* __restrict__ partial, float* __restrict__ dw, int n2, int ctas, size_t dw_step) {
+  const int i = blockIdx.x * 128 + threadIdx.x;
+  grid_dependency_wait();
+  if (i >= n2) return;
+  const float2* src = partial + (size_t)blockIdx.y * ctas * n2 + i;
+  float2 a[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) a[u] = u < ctas ? src[(size_t)u * n2] : make_float2(0.f, 0.f);
+  for (int z = 8; z < ctas; z += 8)
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (z + u < ctas) { const float2 v = src[(size_t)(z + u) * n2]; a[u].x += v.x; a[u].y += v.y; }
+#pragma unroll
+  for (int u = 1; u < 8; ++u) { a[0].x += a[u].x; a[0].y += a[u].y; }
+  *reinterpret_cast<float2*>(dw + (size_t)blockIdx.y * dw_step + 2 * (size_t)i) = a[0];
 }
 
 // ----------------------------------------------------------------- host side ---
