@@ -131,6 +131,10 @@ struct Module {
   size_t dc_elems = 0;
   float* stem_scratch = nullptr;           // partial sums of the stem's weight gradient, which runs beside the side stream's last ones
   size_t stem_scratch_floats = 0;
+  char* side_tmp = nullptr;                // gradient of a block's input through its projection, formed beside the main chain
+  float* side_partial = nullptr;           // as red_partial and scratch, for a projection's forward beside the main chain
+  float* side_scratch = nullptr;
+  bool has_proj = false;
   float* group_scratch = nullptr;          // partial sums of the grouped weight gradients
   size_t group_scratch_floats = 0;
   unsigned long long* exchange = nullptr;  // words of chain::Exchange, the epoch behind them
@@ -143,7 +147,7 @@ struct Module {
   int last_out_slot = -1, last_grad_slot = -1;
   cudaStream_t stream = nullptr;
   cudaStream_t stream2 = nullptr;          // side stream: weight gradients run beside the data-gradient chain
-  cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr, ev_buf[3] = {nullptr, nullptr, nullptr};
+  cudaEvent_t ev_fork2 = nullptr, ev_join2 = nullptr, ev_proj = nullptr, ev_buf[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t ev_act[kEventRing], ev_grad[kEventRing];
   // running batch-norm statistics (inference): flat vector, and the table the inference pass reads them through
   float* running = nullptr;
@@ -463,6 +467,7 @@ static void plan_modules(fdg_ctx* c) {
           m.stem_scratch_floats = conv_wgrad_scratch_elems(c->bf16_mode, ConvGeom{a.batch, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, 3, 1, 1});
           break;
         case U_BASIC:
+          m.has_proj = m.has_proj || u.proj;
           u.t_a = tens(out_e); u.t_b = tens(out_e); u.t_c = tens(out_e); u.t_y = tens(out_e);
           u.q_b = bits(out_e); u.q_y = bits(out_e);
           u.st1 = stat(u.co); u.st2 = stat(u.co);
@@ -617,6 +622,11 @@ static size_t carve(fdg_ctx* c, char* base, size_t* saved) {
   *saved = align_up(cv.off, 256);
   for (Module& m : c->mods) {
     if (m.stem_scratch_floats) m.stem_scratch = cv.take<float>(m.stem_scratch_floats * 4);
+    if (m.has_proj && c->use_graphs) {
+      m.side_tmp = cv.take<char>(align_up(m.max_act, 128) * es);
+      m.side_partial = cv.take<float>(m.red_partial_floats * 4);
+      m.side_scratch = cv.take<float>(std::max<size_t>(m.scratch_floats, 64) * 4);
+    }
     if (m.chains.empty()) continue;
     m.dc = cv.take<bf16>(m.dc_elems * 2);
     m.group_scratch = cv.take<float>(m.group_scratch_floats * 4);
@@ -659,9 +669,9 @@ struct Launch {
 // `run`: offset of this batch norm's running statistics in the module's vector (the kernel that forms the
 // batch statistics also folds them into the running ones).
 template <typename T>
-static void bn_stats(Launch& L, Module& m, const T* x, size_t rows, int C, float eps, float* stats, long long run) {
+static void bn_stats(Launch& L, Module& m, const T* x, size_t rows, int C, float eps, float* stats, long long run, float* scratch = nullptr) {
   L.begin(KC_BN_STATS, (double)rows * C * sizeof(T), 3.0 * rows * C);
-  L.note(launch_bn_stats<T>(L.st, x, rows, C, eps, stats, m.scratch, run >= 0 ? m.running + run : nullptr, kBnMomentum));
+  L.note(launch_bn_stats<T>(L.st, x, rows, C, eps, stats, scratch ? scratch : m.scratch, run >= 0 ? m.running + run : nullptr, kBnMomentum));
   L.c->launches += 2;
 }
 
@@ -730,18 +740,20 @@ template <typename T>
 // a narrow layer), 0 when it formed none, or -1 when the statistics are already in `stats` (a wide layer, whose
 // totals are finalised right behind the convolution; needs `stats`, with `run` the running statistics' offset or -1).
 static int conv_fprop(Launch& L, Module& m, const ConvGeom& g, const T* x, const T* w, T* y, const T* res,
-                      bool want_stats = false, float* stats = nullptr, long long run = -1, const EpiAffine* affine = nullptr) {
+                      bool want_stats = false, float* stats = nullptr, long long run = -1, const EpiAffine* affine = nullptr,
+                      float* partial = nullptr) {
+  if (!partial) partial = m.red_partial;
   L.begin(KC_CONV_FPROP, (in_elems(g) + w_elems(g) + out_elems(g) * (res ? 2 : 1)) * sizeof(T), conv_flops(g));
   int nparts = 0;
   if constexpr (std::is_same<T, bf16>::value) {
     halo::EpiReduce r{};
-    r.mode = 1; r.partial = m.red_partial;
-    const WideStats ws{m.red_partial, m.red_partial_floats, stats, (size_t)g.N * g.P * g.Q, L.c->arch.bn_eps,
+    r.mode = 1; r.partial = partial;
+    const WideStats ws{partial, m.red_partial_floats, stats, (size_t)g.N * g.P * g.Q, L.c->arch.bn_eps,
                        run >= 0 ? m.running + run : nullptr, kBnMomentum};
     L.note(bf16_conv_fprop(L.st, &L.c->tmaps, g, x, w, y, res, want_stats ? &r : nullptr, &nparts, L.c->tc_error, &L.c->launches,
                            (want_stats && stats) ? &ws : nullptr, affine));
   } else {
-    const direct::Reduce<T> r{1, nullptr, nullptr, nullptr, m.red_partial};
+    const direct::Reduce<T> r{1, nullptr, nullptr, nullptr, partial};
     L.note(cuda_core_conv<T>(L.st, g, false, x, w, y, res, nullptr, want_stats ? &r : nullptr, &nparts, &L.c->launches, affine));
   }
   return nparts;
@@ -853,9 +865,10 @@ static void chain_forward(fdg_ctx* c, Module& m, Launch& L, const Chain& ch, con
 // Forward of the module's units into FIFO slot `slot` with weight version `vslot`.  Training (`eval` false):
 // batch statistics, formed in the convolution epilogues where the kernel can, saved for the backward and
 // folded into the running statistics.  Inference (`eval` true): the statistics of every batch norm were put
-// into the slot beforehand from the running ones (bn_eval_stats_kernel), nothing is reduced.
+// into the slot beforehand from the running ones (bn_eval_stats_kernel), nothing is reduced.  `LS` (nullable): a side stream for
+// the projections, which need nothing of the block's own convolutions.
 template <typename T>
-static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int slot, int vslot, bool eval = false) {
+static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int slot, int vslot, bool eval = false, Launch* LS = nullptr) {
   const int B = c->arch.batch;
   const float eps = c->arch.bn_eps;
   const T* wt = weights_of<T>(m, vslot);
@@ -914,12 +927,21 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
       case U_BASIC: {
         ConvGeom g1 = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, u.stride, 1);
         ConvGeom g2 = geom(B, u.P, u.Q, u.co, u.P, u.Q, u.co, 3, 1, 1);
+        const bool beside = u.proj && LS;
+        if (beside) {
+          ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
+          L.note(cudaEventRecord(m.ev_fork2, L.st));
+          LS->note(cudaStreamWaitEvent(LS->st, m.ev_fork2, 0));
+          const int nps = conv_fprop<T>(*LS, m, gs, x, wt + u.ws, S + u.t_s, nullptr, true, F + u.sts, u.rs, nullptr, m.side_partial);   // cs
+          if (nps >= 0) bn_stats<T>(*LS, m, S + u.t_s, rows_out, u.co, eps, F + u.sts, u.rs, m.side_scratch);
+          LS->note(cudaEventRecord(m.ev_join2, LS->st));
+        }
         if (!conv_bn_eval(g1, x, wt + u.w1, F + u.st1, wf + u.g1, wf + u.b1, nullptr, S + u.t_b)) {
           const int np1 = conv_fprop<T>(L, m, g1, x, wt + u.w1, S + u.t_a, nullptr, !eval, F + u.st1, u.r1);   // c1
           stats_of(np1, S + u.t_a, rows_out, u.co, F + u.st1, u.r1);
           bn_apply<T>(L, m, S + u.t_a, F + u.st1, wf + u.g1, wf + u.b1, nullptr, nullptr, nullptr, nullptr, true, S + u.t_b, rows_out, u.co, np1, u.r1, gate_bits(u.q_b));  // a1
         }
-        if (u.proj) {          // shortcut first: its statistics must not disturb the partial sums conv2 leaves for BN2
+        if (u.proj && !beside) {          // shortcut first: its statistics must not disturb the partial sums conv2 leaves for BN2
           ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
           const int nps = conv_fprop<T>(L, m, gs, x, wt + u.ws, S + u.t_s, nullptr, !eval, F + u.sts, u.rs);   // cs
           stats_of(nps < 0 ? nps : 0, S + u.t_s, rows_out, u.co, F + u.sts, u.rs);
@@ -934,6 +956,7 @@ static void forward_module(fdg_ctx* c, Module& m, Launch& L, int64_t tau, int sl
         if (!u.proj && conv_bn_eval(g2, S + u.t_b, wt + u.w2, F + u.st2, wf + u.g2, wf + u.b2, shortcut, S + u.t_y)) break;
         const int np2 = conv_fprop<T>(L, m, g2, S + u.t_b, wt + u.w2, S + u.t_c, nullptr, !eval, F + u.st2, u.r2);   // c2
         stats_of(np2, S + u.t_c, rows_out, u.co, F + u.st2, u.r2);
+        if (beside) L.note(cudaStreamWaitEvent(L.st, m.ev_join2, 0));
         if (u.proj) {
           bn_apply<T>(L, m, S + u.t_c, F + u.st2, wf + u.g2, wf + u.b2, S + u.t_s, F + u.sts, wf + u.gs, wf + u.bs, true, S + u.t_y, rows_out, u.co, np2, u.r2, gate_bits(u.q_y));
         } else {
@@ -1184,6 +1207,15 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
         keep(i, 1, T1);
         if (u.proj) keep(i, 5, T2);
         fork();
+        const bool need_dx = !(m.k == 1 && i == 0);
+        // the gradient through the projection, beside the main chain where there is room for it (a recorded iteration)
+        const bool beside = forked && u.proj && need_dx && m.side_tmp && c->graph_mode_entered;
+        T* through = beside ? reinterpret_cast<T*>(m.side_tmp) : T3;
+        if (beside) {
+          ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
+          conv_dgrad<T>(LS, m, gs, T2, wt + u.ws, flipped_of<T>(m, vslot, u.fs), through, nullptr, open);
+          LS.note(cudaEventRecord(m.ev_proj, LS.st));
+        }
         conv_wgrad<T>(LS, m, g2, S + u.t_b, T1, m.grad + u.w2);                                          // side
         side_done(0);
         const NextBnBwd<T> bn1{gate(u.t_b, u.q_b), S + u.t_a, F + u.st1};
@@ -1197,14 +1229,14 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
         const T* up = u.stride == 2 ? upsample_dy<T>(LS, m, g1, T4) : nullptr;
         conv_wgrad<T>(LS, m, g1, x, T4, m.grad + u.w1, up);                                              // side
         side_done(1);
-        const bool need_dx = !(m.k == 1 && i == 0);
         if (u.proj) {
           ConvGeom gs = geom(B, u.H, u.W, u.ci, u.P, u.Q, u.co, 1, u.stride, 0);
           conv_wgrad<T>(LS, m, gs, x, T2, m.grad + u.ws);                                                // side
           side_done(2);
           if (need_dx) {
-            conv_dgrad<T>(L, m, gs, T2, wt + u.ws, flipped_of<T>(m, vslot, u.fs), T3, nullptr, open);
-            out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, T3, open, next);
+            if (beside) L.note(cudaStreamWaitEvent(L.st, m.ev_proj, 0));
+            else conv_dgrad<T>(L, m, gs, T2, wt + u.ws, flipped_of<T>(m, vslot, u.fs), through, nullptr, open);
+            out_sum_parts = conv_dgrad<T>(L, m, g1, T4, wt + u.w1, flipped_of<T>(m, vslot, u.f1), gout, through, open, next);
           }
         } else if (need_dx && u.zpad) {
           // the shortcut's share: the gated upstream gradient's middle channels, put back at every stride-th pixel
@@ -1307,7 +1339,12 @@ static cudaError_t module_step(fdg_ctx* c, Module& m, cudaStream_t st, StepMode 
   auto do_forward = [&]() {
     if (tau_f < 1 || tau_f > c->last_batch) return;
     const int slot = (int)(tau_f % m.D), vslot = (int)(m.updates % m.Dw);
-    if (enqueue) forward_module<T>(c, m, L, tau_f, slot, vslot);
+    if (enqueue) {
+      // the projections beside the main chain in a recorded iteration only: issued one by one, their events cost the host more
+      Launch LS{c, m.stream2};
+      forward_module<T>(c, m, L, tau_f, slot, vslot, false, mode == RUN_CAPTURE && c->cfg.serial == 0 && m.side_tmp ? &LS : nullptr);
+      if (L.err == cudaSuccess) L.err = LS.err;
+    }
     m.slot_version[slot] = m.updates; m.slot_batch[slot] = tau_f;
     row.tau_f = tau_f; row.ver_f = m.updates; row.slot_f = slot;
     sig(slot); sig(vslot); sig(k == 1 ? tau_f % m.Din : 0);
@@ -1500,6 +1537,7 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&m.stream2, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.ev_fork2, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.ev_join2, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.ev_proj, cudaEventDisableTiming);
     for (int i = 0; i < 3 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&m.ev_buf[i], cudaEventDisableTiming);
     for (int i = 0; i < kEventRing && e == cudaSuccess; ++i) {
       e = cudaEventCreateWithFlags(&m.ev_act[i], cudaEventDisableTiming);
@@ -1548,6 +1586,7 @@ fdg_status fdg_destroy(fdg_ctx* c) {
     if (m.stream2) cudaStreamDestroy(m.stream2);
     if (m.ev_fork2) cudaEventDestroy(m.ev_fork2);
     if (m.ev_join2) cudaEventDestroy(m.ev_join2);
+    if (m.ev_proj) cudaEventDestroy(m.ev_proj);
     for (int i = 0; i < 3; ++i) if (m.ev_buf[i]) cudaEventDestroy(m.ev_buf[i]);
   }
   for (int i = 0; i < kEventRing; ++i) cudaEventDestroy(c->ev_in[i]);
