@@ -565,7 +565,7 @@ def run_gpu(args):
 
     line = None
     if rank == 0:
-        # dominant kernel class, timed alone on a serial context of the same workload
+        # kernel classes, timed alone on a serial context of the same workload (a run of blocks counts as a convolution)
         peaks = measured_peaks()
         gs = make_fdg(B, precision, serial=True)
         for i in range(2 * K_MODULES + 3):
@@ -582,9 +582,10 @@ def run_gpu(args):
         sec = top["total_ms"] * 1e-3
         hbm_frac = top["bytes"] / sec / 1e9 / peaks["hbm_gbs"]
         if args.precision == "bf16":
-            # Dominant kernel (largest share of device time in an ncu launch list of this workload): the halo-tile
-            # convolution.  Timed alone on its most frequent shape; a 16-channel 3x3 layer has 72 flop per byte,
-            # far below the machine balance, so HBM is the roofline that bounds it.
+            # The narrow layers' convolution as an operator of its own: the instructions that chain_kernel, which has the
+            # largest share of this workload's device time, issues for whole runs of blocks.  Timed alone on its most
+            # frequent shape; a 16-channel 3x3 layer has 72 flop per byte, far below the machine balance, so HBM is the
+            # roofline that bounds it.
             us, nbytes, flops = kernel_bench(B, "fprop", "stage1")
             roof = dict(bound="hbm", achieved=nbytes / us / 1e3, peak=peaks["hbm_gbs"], unit="GB/s",
                         kernel="conv_rows_kernel, 3x3 stride-1 forward, [128,32,32,16] -> 16 channels",

@@ -275,7 +275,8 @@ fdg_status fdg_debug_raise_flag(fdg_ctx* ctx, int which);
  * a kernel that ran past the end of its buffer is then named by the buffer it overran.  fdg_debug_guard_count and
  * fdg_debug_guard_offset give the number of regions and the byte offset of region `index` from the workspace
  * base the caller passed to fdg_create (for a report, or for a test that damages one on purpose from the host).
- * The regions are part of fdg_workspace_bytes and of a saved state.  No counterpart in the paper: a debugging aid. */
+ * The regions are part of fdg_workspace_bytes; those of scratch that no call leaves anything in are not part of a saved
+ * state.  No counterpart in the paper: a debugging aid. */
 fdg_status fdg_debug_guard_count(const fdg_ctx* ctx, size_t* out_count);
 fdg_status fdg_debug_guard_offset(const fdg_ctx* ctx, size_t index, size_t* out_byte_offset);
 fdg_status fdg_debug_check_guards(fdg_ctx* ctx, long long* first_bad);
