@@ -961,10 +961,20 @@ __global__ void cast_kernel(const float* __restrict__ in, T* __restrict__ out, s
 // Inference-mode statistics of all batch norms of a module in one launch: for table entry e,
 // out[soff .. soff+C) = running mean, out[soff+C .. soff+2C) = 1/sqrt(running variance + eps).
 struct EvalStatEntry { size_t roff, soff; int C; };
-__global__ void bn_eval_stats_kernel(const float* __restrict__ running, float* __restrict__ out,
-                                     const EvalStatEntry* __restrict__ table, float eps) {
+// All modules in one launch (blockIdx.y: the module; one per module stood between their passes: ResNet-110, K = 4, 1.6 % of a batch).
+constexpr int kMaxModules = 64;
+struct EvalStatModules {
+  const float* running[kMaxModules];
+  float* out[kMaxModules];
+  const EvalStatEntry* table[kMaxModules];
+  int entries[kMaxModules];
+};
+__global__ void bn_eval_stats_kernel(const __grid_constant__ EvalStatModules mods, float eps) {
   grid_dependency_wait();
-  const EvalStatEntry e = table[blockIdx.x];
+  if ((int)blockIdx.x >= mods.entries[blockIdx.y]) return;
+  const float* __restrict__ running = mods.running[blockIdx.y];
+  float* __restrict__ out = mods.out[blockIdx.y];
+  const EvalStatEntry e = mods.table[blockIdx.y][blockIdx.x];
   for (int c = threadIdx.x; c < e.C; c += blockDim.x) {
     out[e.soff + c] = running[e.roff + c];
     out[e.soff + e.C + c] = 1.f / sqrtf(running[e.roff + e.C + c] + eps);

@@ -289,7 +289,7 @@ static fdg_status validate(const fdg_arch* a, const fdg_config* c, std::string* 
       prev = a->widths[i];
     }
   }
-  if (c->K < 1 || c->K > 64) { *why = "K out of range"; return FDG_ERR_INVALID_ARG; }
+  if (c->K < 1 || c->K > kMaxModules) { *why = "K out of range"; return FDG_ERR_INVALID_ARG; }
   if (c->K > 1 && !c->split_after_block) { *why = "split_after_block is null"; return FDG_ERR_INVALID_ARG; }
   int nblocks = 0;
   for (int i = 0; i < a->n_stages; ++i) nblocks += a->blocks[i];
@@ -1993,12 +1993,20 @@ static cudaError_t eval_all(fdg_ctx* c, cudaStream_t cs, const float* images_dev
   L.note(launch_ingest<T>(cs, images_dev, reinterpret_cast<T*>(m1.in_ring) + (size_t)m1.Din * align_up(m1.in_elems, 128), rows,
                           c->arch.in_c, m1.in_c, nullptr, nullptr, 0));
   ++c->launches;
+  EvalStatModules em{};
+  size_t most = 0;
+  for (size_t k = 0; k < c->mods.size(); ++k) {
+    const Module& m = c->mods[k];
+    em.running[k] = m.running; em.out[k] = slot_F(m, m.D); em.table[k] = m.eval_table_dev;
+    em.entries[k] = m.eval_table_dev ? (int)m.eval_table.size() : 0;
+    most = std::max(most, (size_t)em.entries[k]);
+  }
+  if (most) {
+    L.note(launch_chained(bn_eval_stats_kernel, dim3((unsigned)most, (unsigned)c->K), dim3(128), 0, cs, em, c->arch.bn_eps));
+    ++c->launches;
+  }
   for (Module& m : c->mods) {
     const int vslot = (int)(m.updates % m.Dw);
-    if (m.eval_table_dev) {
-      L.note(launch_chained(bn_eval_stats_kernel, dim3((unsigned)m.eval_table.size()), dim3(128), 0, cs, m.running, slot_F(m, m.D), m.eval_table_dev, c->arch.bn_eps));
-      ++c->launches;
-    }
     forward_module<T>(c, m, L, 0, m.D, vslot, true);
     if (m.k == c->K) head_eval<T>(c, m, L, m.D, vslot, labels_dev, logits_dev, correct_dev);
   }
