@@ -219,6 +219,9 @@ struct fdg_ctx {
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t ev_staged = nullptr, ev_ingested = nullptr;
   bool record_ingested = false;
+  // an inference pass that the next iteration has to wait for: it runs on the caller's stream, which module streams do not follow
+  cudaEvent_t ev_eval = nullptr;
+  bool eval_pending = false;
   std::vector<cudaEvent_t> ev_cjoin;
   float* lr_dev = nullptr;
   float lr_on_device = -1.f;
@@ -1550,6 +1553,7 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_staged, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_ingested, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_eval, cudaEventDisableTiming);
   if (e == cudaSuccess && c->use_graphs) e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
   c->ev_cjoin.assign(c->K, nullptr);
   for (int k = 0; k < c->K && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&c->ev_cjoin[k], cudaEventDisableTiming);
@@ -1594,6 +1598,7 @@ fdg_status fdg_destroy(fdg_ctx* c) {
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_staged) cudaEventDestroy(c->ev_staged);
   if (c->ev_ingested) cudaEventDestroy(c->ev_ingested);
+  if (c->ev_eval) cudaEventDestroy(c->ev_eval);
   if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   for (cudaEvent_t ev : c->ev_cjoin) if (ev) cudaEventDestroy(ev);
@@ -1793,6 +1798,13 @@ fdg_status fdg_step(fdg_ctx* c, fdg_stream stream, const float* images_dev, cons
   if (c->has_schedule) fdg_lr_at(&c->schedule, t, &c->lr);
   Module& m1 = c->mods[0];
   cudaError_t e = cudaSuccess;
+  // An inference pass still reads weights and running statistics that this iteration writes.
+  if (c->eval_pending) {
+    e = cudaStreamWaitEvent(cs, c->ev_eval, 0);
+    for (Module& m : c->mods) if (e == cudaSuccess && !serial) e = cudaStreamWaitEvent(m.stream, c->ev_eval, 0);
+    if (e != cudaSuccess) return cuda_fail(c, e, "waiting for the inference pass");
+    c->eval_pending = false;
+  }
   // Graphs take over once every module has run each of its passes at least once (all kernels
   // have been launched the ordinary way, their attributes are set, the pipeline is full).
   if (c->use_graphs && !c->graph_mode_entered && t > 2 * (int64_t)c->K + 1) {
@@ -2029,6 +2041,8 @@ fdg_status fdg_eval(fdg_ctx* c, fdg_stream stream, const float* images_dev, cons
                    : eval_all<float>(c, cs, images_dev, labels_dev, logits_dev, correct_dev);
   c->tmaps.share = share;
   c->last_stream = cs; c->stepped = true;
+  if (e == cudaSuccess) e = cudaEventRecord(c->ev_eval, cs);
+  c->eval_pending = true;
   return e == cudaSuccess ? FDG_OK : cuda_fail(c, e, "inference pass");
 }
 

@@ -212,3 +212,36 @@ def test_saved_state_continues_bit_for_bit(precision, graphs):
         other.load_state(blob)
     other.close()
     h.close()
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_an_iteration_issued_behind_an_inference_pass_leaves_it_its_weights(precision, graphs):
+    """The inference pass waits on its stream (held for some milliseconds) while two iterations are issued behind it, on the
+    same stream or (with graphs) another one: logits and parameters are those of a run that waits for every call."""
+    from paper_1906_09108_b200 import binding as B
+    a = ARCHS["tc"]
+    res = []
+    for held in (False, True):
+        _, g = _pair(B, a, 2, (2,), precision, graphs)
+        batches = [tuple(torch.from_numpy(v).cuda() for v in _batch(a, t)) for t in range(1, 13)]
+        for x, y in batches[:10]:
+            g.step(x, y)
+        g.sync()
+        logits = torch.empty((a["batch"], a["num_classes"]), device="cuda")
+        one, other = torch.cuda.Stream(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        if held:
+            with torch.cuda.stream(one):
+                torch.cuda._sleep(20_000_000)
+        g.eval(*batches[0], logits_dev=logits, stream=one.cuda_stream)
+        if not held:
+            torch.cuda.synchronize()
+        for x, y in batches[10:]:
+            g.step(x, y, stream=(other if graphs else one).cuda_stream)
+        g.sync(stream=(other if graphs else one).cuda_stream)
+        torch.cuda.synchronize()
+        res.append([logits.cpu().numpy()] + [np.asarray(g.get_params(k)) for k in (1, 2)])
+        g.close()
+    for u, v in zip(*res):
+        assert np.array_equal(u, v)
