@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <vector>
 
 namespace fdg {
 namespace chain {
@@ -67,6 +68,56 @@ inline bool chain_supported(int N, int H, int W, int C) {
   if (W % G || H + 2 > 256 || W / G + 2 > 256 || kTileGroups * ((W / G + kTileGroups - 1) / kTileGroups) + 2 > 256) return false;
   const Geom p = chain_geom(N, H, W, C, 2, kMaxCtas, TRAIN);
   return p.images >= 1 && p.a_tx < (1u << 20) && chain_ctas(p) <= kMaxCtas;
+}
+
+// Runs of all modules, and whether each trains as one launch per pass.  A module has one such launch on the device at a time, but
+// the modules' launches go side by side, and CTAs that wait for one another must all be resident: a launch takes the device's SMs
+// as if every other module had its largest one there.
+struct Run { int module, blocks, N, H, W, C; bool launch; };
+constexpr int kLeastShare = 16;                  // a module's share of the SMs is not taken to be smaller
+inline int module_share(int sms, int modules) { return std::max(kLeastShare, sms / std::max(1, modules)); }
+inline int run_ctas(const Run& r, int share) {
+  int most = 0;
+  for (int pass : {TRAIN, BACKWARD}) {
+    const Geom p = chain_geom(r.N, r.H, r.W, r.C, 2, share, pass);
+    if (p.images < 1) return kMaxCtas + 1;
+    most = std::max(most, chain_ctas(p));
+  }
+  return most;
+}
+inline bool within_share(int ctas, int share) { return 5 * ctas <= 8 * share; }
+// `modules`: how many have streams of their own (1: all on one stream, each launch has the device to itself).
+// A launch's CTAs exceed its module's share where shared memory or the accumulators cap its images per CTA (128 images of 40x40x16:
+// 128 CTAs at any share).  Beyond 8/5 of the share a run goes layer by layer: the other modules then wait for SMs, and one image per
+// CTA gains little.  (ms per iteration, by runs / layer by layer.  K = 4, 18 blocks a stage: 150 images of 32x32x16, 1.03 shares,
+// 1.24 / 1.62; 40x40x16, 48 images, 1.3 shares, 1.02 / 1.36, 56 images, 1.5 shares, 1.30 / 1.44, 72 images, 1.9 shares, 1.82 / 1.65;
+// K = 4, 128 images, 1.7 shares: 20x20x32 1.40 / 1.34, 32x32x32 1.064 / 1.045; K = 2, 24x24x64, 1.7 shares, 1.64 / 1.53.)
+// Where the modules' largest launches together still want more than `sms`, those runs go as launches that hold the most blocks within
+// it (what a block gains hardly depends on its shape): the best sum over the modules of the blocks in runs of at most so many CTAs.
+inline void fit_device(std::vector<Run>& runs, int modules, int sms) {
+  const int share = module_share(sms, modules);
+  std::vector<int> ctas;
+  for (Run& r : runs) {
+    ctas.push_back(run_ctas(r, share));
+    r.launch = ctas.back() <= std::min(sms, kMaxCtas) && (modules <= 1 || within_share(ctas.back(), share));
+  }
+  if (modules <= 1) return;
+  std::vector<std::vector<int>> best(modules + 1, std::vector<int>(sms + 1, 0)), limit = best;
+  for (int k = 0; k < modules; ++k)
+    for (int have = 0; have <= sms; ++have) {
+      best[k + 1][have] = best[k][have];
+      for (size_t i = 0; i < runs.size(); ++i) {
+        if (runs[i].module != k || !runs[i].launch || ctas[i] > have) continue;
+        int blocks = best[k][have - ctas[i]];
+        for (size_t j = 0; j < runs.size(); ++j) blocks += runs[j].module == k && runs[j].launch && ctas[j] <= ctas[i] ? runs[j].blocks : 0;
+        if (blocks > best[k + 1][have]) { best[k + 1][have] = blocks; limit[k + 1][have] = ctas[i]; }
+      }
+    }
+  for (int k = modules - 1, have = sms; k >= 0; --k) {
+    const int most = limit[k + 1][have];
+    for (size_t i = 0; i < runs.size(); ++i) if (runs[i].module == k && ctas[i] > most) runs[i].launch = false;
+    have -= most;
+  }
 }
 
 // Tiles at once: as many as share the CTA's tiles evenly (inference, few tiles: at most 2; the others at least 2).

@@ -11,7 +11,9 @@
 //     by then: the apply reads it there;
 //   - what the CTAs must know of one another is 2 * C sums per layer: every CTA publishes its own as (value, tag) words and
 //     reads all of them (publish and collect below).  The launch is cooperative: its CTAs are resident together, and several such launches
-//     on different streams run side by side (measured: 4 launches of 32 CTAs take the time of one; an exchange costs 1.1 us).
+//     on different streams run side by side (measured: 4 launches of 32 CTAs take the time of one; an exchange costs 1.1 us).  Those
+//     of one context always fit the device together (chain_plan.h: fit_device); those of two contexts at work on one device at the
+//     same time may not, and then a launch waits until all of its CTAs find room, which is what a cooperative launch promises.
 // Measured, 128 images of 32x32x16 on 64 CTAs: a layer's forward pass 8 us, its backward pass up to the weight gradient 11 us
 // (convolution and apply by themselves: 13 us, and 20 to 25); ResNet-56 with K = 2 1.09 -> 0.84 ms per iteration, an inference
 // batch of ResNet-110 0.79 -> 0.46 ms.  What bounds a layer now: the exchange (2.5 us with the CTAs' skew) and the latencies of

@@ -77,7 +77,11 @@ struct Unit {
 
 // Consecutive identity blocks that run as one launch per pass (conv_chain.cuh): units first .. last, 2 * (last - first + 1)
 // convolutions of C channels.  Offsets of a unit's tensors, parameters and statistics grow evenly inside a run.
-struct Chain { int first, last, C; size_t dc; };   // dc: where its gradients of convolution outputs start in Module::dc
+struct Chain {
+  int first, last, C;
+  size_t dc;                                        // where its gradients of convolution outputs start in Module::dc
+  bool train;                                       // trains as one launch per pass (chain::fit_device); inference always does
+};
 // The backward pass takes a run in pieces, from its end: the weight gradients of a piece run beside the next one.  The last
 // piece is short, because nothing runs beside its weight gradients.
 // (ResNet-56 K = 2 / ResNet-110 K = 4 / ResNet-1202 K = 4, ms a logging interval: pieces of 12 and 4 blocks 6.86 / 10.78 / 31.2, 8 and 3
@@ -357,10 +361,25 @@ static void plan_chains(const fdg_arch& a, Module& m, bool bf16_mode) {
              u.w1 == v.w2 + cc + 2 * u.co && u.r1 == v.r2 + 2 * u.co && (size_t)(u.f1 - v.f2) == align_up(cc, 64);
     }
     if (join) m.chains.back().last = i;
-    else m.chains.push_back(Chain{i, i, u.co, m.dc_elems});
+    else m.chains.push_back(Chain{i, i, u.co, m.dc_elems, true});
     m.chain_of[i] = (int)m.chains.size() - 1;
     m.dc_elems += 2 * E;
   }
+}
+
+// Which runs train as one launch on a device of `sms` SMs; those that a smaller device gave up stay given up.
+static void fit_chains(fdg_ctx* c, int sms) {
+  std::vector<chain::Run> runs;
+  std::vector<Chain*> of;
+  for (Module& m : c->mods)
+    for (Chain& ch : m.chains) {
+      const Unit& u = m.units[ch.first];
+      if (!ch.train) continue;
+      runs.push_back(chain::Run{m.k - 1, ch.last - ch.first + 1, c->arch.batch, u.P, u.Q, ch.C, true});
+      of.push_back(&ch);
+    }
+  chain::fit_device(runs, c->cfg.serial ? 1 : c->K, sms);
+  for (size_t i = 0; i < runs.size(); ++i) of[i]->train = runs[i].launch;
 }
 
 static long long add_running(Module& m, int C) {
@@ -562,6 +581,7 @@ static void plan_modules(fdg_ctx* c) {
     m.slot_version.assign(m.D, -1);
     m.slot_batch.assign(m.D, -1);
   }
+  fit_chains(c, chain::kMaxCtas);
 }
 
 // Assigns every device pointer; with base == nullptr only measures.  Returns the whole size, `*saved` the part that a saved
@@ -842,11 +862,13 @@ static chain::Tensors chain_tensors(const Module& m, const Chain& ch, int first,
   t.p_step = cc + 2 * ch.C;
   return t;
 }
-// How a run is launched now (images = 0: layer by layer): its CTAs wait for one another, so they must all fit the device.
+// How a run is launched now (images = 0: layer by layer): in training its CTAs wait for one another, so they must all fit the
+// device, together with those of the other modules' runs.
 static chain::Geom chain_shape(fdg_ctx* c, const Module& m, const Chain& ch, int blocks, int pass) {
   const Unit& u = m.units[ch.first];
-  const int sms = cached_sm_count(&c->tmaps), share = c->tmaps.share > 0 ? c->tmaps.share : 1;
-  chain::Geom p = chain::chain_geom(c->arch.batch, u.P, u.Q, ch.C, 2 * blocks, std::max(16, sms / share), pass);
+  const int sms = cached_sm_count(&c->tmaps);
+  if (pass != chain::INFER && !ch.train) return chain::Geom{};
+  chain::Geom p = chain::chain_geom(c->arch.batch, u.P, u.Q, ch.C, 2 * blocks, chain::module_share(sms, c->tmaps.share), pass);
   if (p.images > 0 && chain::chain_ctas(p) > std::min(sms, chain::kMaxCtas)) p.images = 0;
   return p;
 }
@@ -1562,6 +1584,7 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
   // 8 tiles per CTA: the four chains' convolutions then fit the SMs together and a CTA's start-up is paid once
   // per four tiles).
   c->tmaps.share = c->cfg.serial ? 1 : c->K;
+  if (e == cudaSuccess && cached_sm_count(&c->tmaps) < chain::kMaxCtas) fit_chains(c, c->tmaps.sm_count);
   // A weight gradient on a side stream takes as many CTAs as give each four images (measured with the present data
   // gradients: 16 / 24 / 32 / 48 CTAs at batch 128: K = 2 1228 / 1148 / 1091 / 1085 us per ResNet-56 iteration, K = 4
   // 1580 / 1505 / 1484 / 1498 us per ResNet-110 iteration; at batch 64 16 CTAs are the best by 1 %).

@@ -117,3 +117,58 @@ def test_runs_of_blocks_fit_an_sm_and_the_device(tmp_path):
       if (pass == chain::INFER ? st > 2 : st < 2) report("streams", g, (size_t)st);
     }
   }""")
+
+
+def test_runs_of_all_modules_fit_the_device_together(tmp_path):
+    """CTAs of a run wait for one another: whatever the modules' runs are, the launches that may meet want no more SMs than there
+    are, none is given up where all fit, and the shape each is launched with is the one that was counted."""
+    _run(tmp_path, r"""
+  unsigned seed = 1;
+  auto pick = [&](int n) { seed = seed * 1664525u + 1013904223u; return (int)((seed >> 8) % (unsigned)n); };
+  for (int it = 0; it < 40000; ++it) {
+    const int modules = 1 + pick(16), sms = pick(4) ? 148 : 16 + pick(133), N = 1 + pick(pick(2) ? 160 : 600), side = 4 * (1 + pick(16)), share = chain::module_share(sms, modules);
+    std::vector<chain::Run> runs;
+    for (int k = 0; k < modules; ++k)
+      for (int j = pick(4); j > 0; --j) {
+        const int down = pick(3), C = 16 << pick(3), H = side >> down;
+        if (H >= 1 && chain::chain_supported(N, H, H, C)) runs.push_back(chain::Run{k, 1 + pick(20), N, H, H, C, false});
+      }
+    std::vector<int> all(modules, 0), on(modules, 0);
+    bool alone = true;
+    chain::fit_device(runs, modules, sms);
+    for (const chain::Run& r : runs) {
+      const int n = chain::run_ctas(r, share);
+      for (int pass : {chain::TRAIN, chain::BACKWARD}) {
+        const chain::Geom p = chain::chain_geom(r.N, r.H, r.W, r.C, 2, share, pass);
+        if (p.images < 1 || chain::chain_ctas(p) > n) report("counted", ConvGeom{r.N, r.H, r.W, r.C, r.H, r.W, r.C, 3, 3, 1, 1}, (size_t)n);
+      }
+      all[r.module] = std::max(all[r.module], n);
+      if (r.launch) on[r.module] = std::max(on[r.module], n);
+      alone = alone && n <= sms && (modules == 1 || chain::within_share(n, share));
+    }
+    int want = 0, have = 0;
+    for (int k = 0; k < modules; ++k) { want += all[k]; have += on[k]; }
+    const ConvGeom g{N, side, side, modules, side, side, sms, 3, 3, 1, 1};
+    if (have > sms) report("together", g, (size_t)have);
+    for (const chain::Run& r : runs) {
+      const int n = chain::run_ctas(r, share);
+      if (r.launch && modules > 1 && !chain::within_share(n, share)) report("beyond its share", g, (size_t)n);
+      if (r.launch) continue;
+      if (alone && (want <= sms || modules == 1)) report("given up", g, (size_t)want);
+      if (modules > 1 && chain::within_share(n, share) && have - on[r.module] + std::max(on[r.module], n) <= sms) report("left out", g, (size_t)have);
+    }
+  }
+  // 128 images: two modules of 40x40x16 (128 CTAs each), four or three of 32x32x32 (64 each), four of 16x16x64 (43 each) and of 32x32x16 (32 each)
+  struct { int n, side, C, kept; } known[] = {{2, 40, 16, 0}, {4, 32, 32, 0}, {3, 32, 32, 2}, {4, 16, 64, 3}, {4, 32, 16, 4}};
+  for (auto& q : known) {
+    std::vector<chain::Run> runs;
+    for (int k = 0; k < q.n; ++k) runs.push_back(chain::Run{k, 4, 128, q.side, q.side, q.C, false});
+    chain::fit_device(runs, q.n, 148);
+    int kept = 0;
+    for (const chain::Run& r : runs) kept += r.launch;
+    if (kept != q.kept) report("kept", ConvGeom{128, q.side, q.side, q.C, q.side, q.side, q.C, 3, 3, 1, 1}, (size_t)kept);
+  }
+  // the most blocks, not the most modules: 64 + 64 CTAs hold 4 + 2 + 2 of them, 43 + 43 and 64 + 43 at most 7
+  std::vector<chain::Run> runs = {{0, 4, 128, 32, 32, 32, false}, {1, 2, 128, 32, 32, 32, false}, {1, 2, 128, 16, 16, 64, false}, {2, 3, 128, 16, 16, 64, false}};
+  chain::fit_device(runs, 3, 148);
+  if (!runs[0].launch || !runs[1].launch || !runs[2].launch || runs[3].launch) report("most blocks", ConvGeom{128, 32, 32, 32, 32, 32, 32, 3, 3, 1, 1}, 0);""")

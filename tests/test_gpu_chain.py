@@ -17,7 +17,9 @@ EPS = 1e-5
 # several column blocks (40) and tiles per image; more images than CTAs (149, 161) and the most that a CTA holds; one-pixel maps;
 # runs of one block, of several pieces in the backward pass
 CASES = [(1, 12, 2, 1, ()), (5, 28, 3, 1, ()), (3, 40, 2, 2, (3,)), (149, 16, 2, 1, ()), (161, 32, 2, 4, (1, 2, 4)), (7, 4, 3, 1, ()),
-         (9, 20, 5, 1, ()), (2, 8, 13, 1, ())]
+         (9, 20, 5, 1, ()), (2, 8, 13, 1, ()),
+         # two modules whose runs do not fit the device together (76 + 76 CTAs of one image): one of them goes layer by layer
+         (76, 40, 2, 2, (1,))]
 
 
 def _context(case, lr=0.0, **kw):
