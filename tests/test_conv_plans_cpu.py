@@ -9,6 +9,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 PROLOGUE = r"""
 #include <cstdio>
+#include <cstring>
 #include <cuda.h>
 #include "fdg_ops.h"
 #include "chain_plan.h"
@@ -172,3 +173,30 @@ def test_runs_of_all_modules_fit_the_device_together(tmp_path):
   std::vector<chain::Run> runs = {{0, 4, 128, 32, 32, 32, false}, {1, 2, 128, 32, 32, 32, false}, {1, 2, 128, 16, 16, 64, false}, {2, 3, 128, 16, 16, 64, false}};
   chain::fit_device(runs, 3, 148);
   if (!runs[0].launch || !runs[1].launch || !runs[2].launch || runs[3].launch) report("most blocks", ConvGeom{128, 32, 32, 32, 32, 32, 32, 3, 3, 1, 1}, 0);""")
+
+
+def test_a_run_s_inverse_square_root_is_the_64_bit_one_rounded(tmp_path):
+    """1 / sqrt(v) of a run's batch norms: what the short way returns is (float)(1.0 / sqrt(v)) to the last bit, with a seed as far
+    off as an fp32 approximation may be (4 units; rsqrtf promises 2), for ordinary arguments and for those whose result lies
+    next to the middle of two fp32 values; and nearly every ordinary argument takes it."""
+    _run(tmp_path, r"""
+  unsigned long long seed = 1;
+  auto next = [&]() { seed = seed * 6364136223846793005ull + 1442695040888963407ull; return (double)(seed >> 11) / 9007199254740992.0; };
+  auto units = [](float x, int n) { unsigned u; memcpy(&u, &x, 4); u += n; memcpy(&x, &u, 4); return x; };
+  const ConvGeom none{};
+  long taken = 0, all = 0;
+  for (int it = 0; it < 2000000; ++it) {
+    const bool tie = it & 1;
+    double v = exp2(next() * 120.0 - 60.0);
+    if (tie) {
+      const float f = (float)(1.0 / sqrt(v));
+      const double middle = 0.5 * ((double)f + (double)units(f, 1));
+      v = 1.0 / (middle * middle) * (1.0 + (next() - 0.5) * exp2(-36.0 - 16.0 * next()));
+    }
+    const float want = (float)(1.0 / sqrt(v)), s = units((float)(1.0 / sqrt((double)(float)v)), (int)(next() * 9.0) - 4);
+    float r;
+    const bool ok = chain::inverse_sqrt_from(v, s, r);
+    if (ok && r != want) report("last bit", none, (size_t)it);
+    if (!tie) { ++all; taken += ok; }
+  }
+  if (all - taken > all / 10000) report("taken", none, (size_t)(all - taken));""")
