@@ -281,9 +281,10 @@ fdg_status fdg_debug_guard_count(const fdg_ctx* ctx, size_t* out_count);
 fdg_status fdg_debug_guard_offset(const fdg_ctx* ctx, size_t index, size_t* out_byte_offset);
 fdg_status fdg_debug_check_guards(fdg_ctx* ctx, long long* first_bad);
 
-/* A wait that really runs out, without a kernel that misbehaves: enqueues on `stream` a one-warp kernel that
- * waits, with the bounded wait of the tensor-core kernels, on a barrier nothing ever arrives at.  After
- * `poll_limit` polls (1..2^20; a poll is well under a microsecond) the wait gives up, the kernel raises the
+/* Waits that really run out, without a kernel that misbehaves: enqueues on `stream` a kernel of two warps, of
+ * which one waits, with the bounded wait of the tensor-core kernels, on a barrier nothing ever arrives at, and
+ * the other, with the bounded poll by which CTAs exchange sums, for a word nothing writes.  After `poll_limit`
+ * polls (1..2^20; a poll is a microsecond at most) a wait gives up; when both have, the kernel raises the
  * time-out status word as a convolution kernel would, and returns: no copy is in flight and no tensor memory
  * is held.  The next fdg_sync returns FDG_ERR_TIMEOUT (latched); the CUDA context stays usable.  Does not block. */
 fdg_status fdg_debug_wait_probe(fdg_ctx* ctx, fdg_stream stream, unsigned poll_limit);

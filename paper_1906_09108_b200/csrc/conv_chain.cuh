@@ -98,6 +98,44 @@ __device__ __forceinline__ unsigned long long ld_word(const unsigned long long* 
   asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
   return w;
 }
+// Waits until the words of CTAs b0, b0 + stride, .. (eight of them, those below n; `pitch` words apart) carry `tag`: false when
+// the limit is hit or another role has raised *abort_flag.
+__device__ __forceinline__ bool poll_words(unsigned long long (&v)[8], const unsigned long long* words, size_t pitch, int b0, int stride, int n,
+                                           uint32_t tag, volatile int* abort_flag, uint32_t limit = kPollLimit) {
+  for (uint32_t i = 0; ; ++i) {
+    bool all = true;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int b = b0 + u * stride;
+      v[u] = b < n ? ld_word(words + (size_t)b * pitch) : (unsigned long long)tag << 32;
+      all = all && (uint32_t)(v[u] >> 32) == tag;
+    }
+    if (all) return true;
+    if ((i & 63u) == 63u && *abort_flag) return false;
+    if (i == limit) { *abort_flag = 1; return false; }
+  }
+}
+// Two warps wait as the kernels do: one, with their bounded wait, on a barrier that nothing ever arrives at, the other, with the
+// bounded poll of an exchange, for a word that carries no tag.  After `limit` polls each gives up, and when both have, that is
+// reported the way the kernels report it.  Nothing is in flight and no tensor memory is held when the kernel leaves.  Lets the
+// host-side handling of a wait that ran out be exercised without making a real kernel misbehave.
+__global__ void wait_probe_kernel(uint32_t limit, const unsigned long long* untagged, int* error_word) {
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ int flags[2];
+  if (threadIdx.x == 0) {
+    flags[0] = flags[1] = 0;
+    mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) mbar_wait(&bar, 0, &flags[0], limit);
+  if (threadIdx.x >= 32) {
+    unsigned long long v[8];
+    poll_words(v, untagged, 0, 0, 1, 8, 1u, &flags[1], limit);
+  }
+  __syncthreads();
+  if (*(volatile int*)&flags[0] && *(volatile int*)&flags[1] && threadIdx.x == 0 && error_word) atomicExch(error_word, 1);
+}
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -201,6 +239,7 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
   using Wd = Window<C>;
   constexpr int G = Wd::G;
   extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t issued[kIssuers];      // nothing of the issuer's is in flight
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* w_smem = smem + (size_t)p.images * p.a_bytes;
   double* part = reinterpret_cast<double*>(w_smem + (size_t)p.w_stages * p.w_bytes);      // [kEpiThreads]
@@ -238,6 +277,8 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
   }
   if (threadIdx.x == 64) {
     *abort_flag = 0;
+    for (int i = 0; i < kIssuers; ++i) mbar_init(&issued[i], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_x)) : "memory");
     if (PASS != INFER) *epoch_smem = *ex.epoch;
   }
@@ -258,8 +299,9 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
     const uint32_t row_units = p.row_bytes >> 4;
     int ws = 0;
     uint32_t wph = 0;
+    bool ok = true;                                 // after a wait that ran out nothing more is issued
     for (int s = 0; s < p.layers; ++s) {
-      bool ok = chain_wait(&w_full[ws], wph, abort_flag);
+      ok = chain_wait(&w_full[ws], wph, abort_flag) && ok;
       const uint64_t b_desc = smem_desc_kmajor(smem_u32(w_smem + (size_t)ws * p.w_bytes), C * 2);
       int t = 0;
       for (int j = 0; j < images; ++j) {
@@ -278,6 +320,7 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
       if (ok) rows::commit_by(leader, &w_empty[ws]);
       if (++ws == p.w_stages) { ws = 0; wph ^= 1u; }
     }
+    rows::commit_by(leader, &issued[warp]);
     } else {
       // shared memory: [tap][c_out] rows of C channels, swizzled; global memory: [c_out][tap][C]
       constexpr uint32_t mask = C == 64 ? 7u : (C == 32 ? 3u : 1u);
@@ -455,18 +498,7 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
       double a = 0.0;
       for (int b0 = etid / (2 * C); b0 < step; b0 += 8 * kSegs) {
         unsigned long long v[8];
-        for (uint32_t i = 0; ; ++i) {
-          bool all = true;
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int b = b0 + u * kSegs;
-            v[u] = b < step ? ld_word(mine + (size_t)b * 2 * C) : (unsigned long long)tag << 32;
-            all = all && (uint32_t)(v[u] >> 32) == tag;
-          }
-          if (all) break;
-          if ((i & 63u) == 63u && *abort_flag) break;
-          if (i == kPollLimit) { *abort_flag = 1; break; }
-        }
+        poll_words(v, mine, 2 * C, b0, kSegs, step, tag, abort_flag);
 #pragma unroll
         for (int u = 0; u < 8; ++u) a += (double)__uint_as_float((uint32_t)v[u]);
       }
@@ -793,17 +825,17 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
     }
   }
 
-  // Teardown.  After an abort copies may still be in flight towards this CTA's shared memory: give their barriers a bounded
-  // chance to complete before leaving.
+  // Teardown.  After an abort copies towards this CTA's shared memory may still be in flight, and instructions that read it and
+  // write tensor memory: give their barriers a bounded chance to complete before that memory is given back.
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
     if (threadIdx.x == 0) {
       if (error_word) atomicExch(error_word, 1);
+      auto settle = [](uint64_t* bar) { for (uint32_t i = 0; i < (1u << 16) && !mbar_try_wait(bar, 0); ++i) {} };
       if (PASS != BACKWARD)
-        for (int j = 0; j < images; ++j)
-          for (uint32_t i = 0; i < (1u << 16); ++i)
-            if (mbar_try_wait(&a_full[j], 0)) break;
+        for (int j = 0; j < images; ++j) settle(&a_full[j]);
+      for (int i = 0; i < kIssuers; ++i) settle(&issued[i]);
     }
     __syncthreads();
   }

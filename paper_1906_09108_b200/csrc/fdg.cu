@@ -1958,7 +1958,8 @@ fdg_status fdg_debug_check_guards(fdg_ctx* c, long long* out_first_bad) {
 fdg_status fdg_debug_wait_probe(fdg_ctx* c, fdg_stream stream, unsigned poll_limit) {
   if (!c) return FDG_ERR_INVALID_ARG;
   if (poll_limit < 1 || poll_limit > (1u << 20)) return fail(c, FDG_ERR_INVALID_ARG, "poll limit outside 1..2^20");
-  tc::wait_probe_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(poll_limit, c->flags + 2);
+  // (the words behind the status words stay zero: no tag)
+  chain::wait_probe_kernel<<<1, 64, 0, static_cast<cudaStream_t>(stream)>>>(poll_limit, reinterpret_cast<const unsigned long long*>(c->flags + 8), c->flags + 2);
   ++c->launches;
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? FDG_OK : cuda_fail(c, e, "wait probe");
