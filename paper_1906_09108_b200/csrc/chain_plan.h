@@ -60,6 +60,7 @@ inline Geom chain_geom(int N, int H, int W, int C, int layers, int sms, int pass
   return p;
 }
 inline int chain_ctas(const Geom& p) { return (p.N + p.images - 1) / p.images; }
+inline size_t exchange_words(int N, int C) { return (size_t)2 * std::min(N, kMaxCtas) * 2 * C; }      // for any launch of a run
 inline size_t chain_smem_bytes(const Geom& p, int C) {
   return std::max(kSmemLeast, (size_t)p.images * p.a_bytes + (size_t)p.w_stages * p.w_bytes + fixed_smem(C));
 }

@@ -82,12 +82,12 @@ struct BackwardArgs {
   __nv_bfloat16* keep_x;
   size_t keep_step;
 };
-// Published sums: [2][148][2 * 64] words of (tag << 32 | value); `epoch` counts the exchanges of this module.
+// Published sums: [CTAs][2][2 * C] words of (tag << 32 | value); `epoch` counts the exchanges of this module, so that no tag occurs
+// twice.
 struct Exchange {
   unsigned long long* words;
   unsigned int* epoch;
 };
-constexpr size_t kExchangeWords = (size_t)2 * kMaxCtas * 2 * 64;
 
 __device__ __forceinline__ void st_word(unsigned long long* p, uint32_t tag, float v) {
   const unsigned long long w = ((unsigned long long)tag << 32) | __float_as_uint(v);
@@ -482,9 +482,9 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
       for (int w = 0; w < kEpiWarps; ++w) a += d[w * 2 * C];
       return a;
     };
-    auto words_of = [&](int number) { return ex.words + (size_t)(number & 1) * kMaxCtas * 2 * C; };
+    auto words_of = [&](int number) { return ex.words + (size_t)(number & 1) * 2 * C; };
     auto publish = [&](int number, float own) {     // `own`: this CTA's sum etid, for etid < 2 * C
-      if (etid < 2 * C) st_word(words_of(number) + (size_t)blockIdx.x * 2 * C + etid, epoch + 1u + (uint32_t)number, own);
+      if (etid < 2 * C) st_word(words_of(number) + (size_t)blockIdx.x * 4 * C + etid, epoch + 1u + (uint32_t)number, own);
     };
     // First thread (sum etid % (2 * C), segment etid / (2 * C)) adds every kSegs-th CTA's word; then a warp has C / 16 channels:
     // lane (channel, statistic, segment).  A channel's leader ends up with its totals.  (A CTA's words lie in a row of their own:
@@ -498,7 +498,7 @@ chain_kernel(const __grid_constant__ CUtensorMap map_x, const Geom p, const Tens
       double a = 0.0;
       for (int b0 = etid / (2 * C); b0 < step; b0 += 8 * kSegs) {
         unsigned long long v[8];
-        poll_words(v, mine, 2 * C, b0, kSegs, step, tag, abort_flag);
+        poll_words(v, mine, 4 * C, b0, kSegs, step, tag, abort_flag);
 #pragma unroll
         for (int u = 0; u < 8; ++u) a += (double)__uint_as_float((uint32_t)v[u]);
       }

@@ -261,7 +261,7 @@ inline cudaError_t run_wgrad_halo(cudaStream_t st, TensorMapCache* cache, int N,
   halo::WgradMaps<1> maps;
   maps.x[0] = *mx; maps.y[0] = *my;
   e = launch_chained(halo::wgrad_halo_kernel<1>, dim3(ctas, halo::wgrad_pairs(p)), dim3(halo::kFwdThreads), halo::wgrad_smem_bytes(p), st,
-                     maps, p, scratch, err_dev);
+                     maps, p, halo::GroupScratch{scratch, 1, nullptr}, err_dev);
   if (e != cudaSuccess) return e;
   const size_t n = (size_t)Co * 9 * Ci;
   if (n >= ((size_t)1 << 17) && ctas <= 8)        // large filters, few partials: four outputs per thread, partials in turn
@@ -269,21 +269,26 @@ inline cudaError_t run_wgrad_halo(cudaStream_t st, TensorMapCache* cache, int N,
                           reinterpret_cast<const float4*>(scratch), reinterpret_cast<float4*>(dw), n / 4, ctas);
   return launch_chained(halo::wgrad_halo_reduce_kernel, dim3((unsigned)((n + 31) / 32)), dim3(256), 0, st, (const float*)scratch, dw, n, ctas);
 }
-// The weight gradients of `layers` layers of one shape (c_in = c_out = C) in two launches: x[i], dy[i] -> dw + i * dw_step.
-// `scratch`: wgrad_group_scratch_elems floats.
+// The weight gradients of `layers` layers of one shape (c_in = c_out = C), two launches for as many of them as the two pieces of scratch
+// (floats in each) hold partial sums of (at least one): x[i], dy[i] -> dw + i * dw_step.
 inline size_t wgrad_group_scratch_elems(int N, int H, int W, int C, int layers, int cap) {
-  const int group = layers < halo::kWgradLayers ? layers : halo::kWgradLayers;
-  return (size_t)group * halo::wgrad_ctas(halo::wgrad_params(N, H, W, C, C), cap) * C * 9 * C;
+  return (size_t)std::min(layers, halo::kWgradLayers) * halo::wgrad_ctas(halo::wgrad_params(N, H, W, C, C), cap) * C * 9 * C;
 }
 inline cudaError_t run_wgrad_group(cudaStream_t st, TensorMapCache* cache, int N, int H, int W, int C, int layers, const bf16_t* const* x,
-                                   const bf16_t* const* dy, float* dw, size_t dw_step, float* scratch, int* err_dev, int cap, uint64_t* launches) {
+                                   const bf16_t* const* dy, float* dw, size_t dw_step, float* const (&scratch)[2], const size_t (&scratch_floats)[2], int* err_dev, int cap,
+                                   uint64_t* launches) {
   halo::WgradParams p = halo::wgrad_params(N, H, W, C, C);
   cudaError_t e = halo::set_smem_attrs(cached_device(cache));
   const int ctas = halo::wgrad_ctas(p, cap);
   p.stages = 1;                                   // two CTAs per SM instead
   const size_t n = (size_t)C * 9 * C;
-  for (int l0 = 0; l0 < layers && e == cudaSuccess; l0 += halo::kWgradLayers) {
-    const int nl = std::min(halo::kWgradLayers, layers - l0);
+  const size_t hold0 = scratch_floats[0] / (n * ctas), hold1 = scratch_floats[1] / (n * ctas);
+  const int most = (int)std::min<size_t>(halo::kWgradLayers, hold0 + hold1);
+  if (most < 1) return cudaErrorInvalidValue;
+  const halo::GroupScratch parts_at{scratch[0], (int)std::min<size_t>(hold0, halo::kWgradLayers), scratch[1]};
+  const int parts = (layers + most - 1) / most, group = (layers + parts - 1) / parts;
+  for (int l0 = 0; l0 < layers && e == cudaSuccess; l0 += group) {
+    const int nl = std::min(group, layers - l0);
     halo::WgradMaps<halo::kWgradLayers> maps;
     for (int i = 0; i < halo::kWgradLayers && e == cudaSuccess; ++i) {
       const CUtensorMap *mx, *my;
@@ -294,10 +299,10 @@ inline cudaError_t run_wgrad_group(cudaStream_t st, TensorMapCache* cache, int N
     }
     if (e != cudaSuccess) return e;
     e = launch_chained(halo::wgrad_halo_kernel<halo::kWgradLayers>, dim3(ctas, halo::wgrad_pairs(p), nl), dim3(halo::kFwdThreads),
-                       halo::wgrad_smem_bytes(p), st, maps, p, scratch, err_dev);
+                       halo::wgrad_smem_bytes(p), st, maps, p, parts_at, err_dev);
     if (e == cudaSuccess)
       e = launch_chained(halo::wgrad_group_sum_kernel, dim3((unsigned)((n / 2 + 127) / 128), nl), dim3(128), 0, st,
-                         reinterpret_cast<const float2*>(scratch), dw + (size_t)l0 * dw_step, (int)(n / 2), ctas, dw_step);
+                         parts_at, dw + (size_t)l0 * dw_step, (int)(n / 2), ctas, dw_step);
     *launches += 2;
   }
   return e;

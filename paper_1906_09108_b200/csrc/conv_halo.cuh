@@ -599,11 +599,19 @@ struct WgradParams {
 // layer alone leaves most SMs idle, and every launch costs its start and its end.  With several layers two CTAs share an SM, each
 // with one stage of tiles: the start, the loads and the write-out of one run beside the instructions of the other (ResNet-110
 // K = 4 10.31 -> 9.96 ms a logging interval, ResNet-1202 29.99 -> 29.31, ResNet-56 K = 2 6.45 -> 6.40).
+// As many layers a launch as a piece of a run has, up to 24, of which each is a split of 16 to 32 CTAs: at most 32 / 24 / 16 / 12 / 8 / 6 / 4
+// of them ResNet-56 K = 2 6.22 / 6.22 / 6.22 / 6.22 / 6.46 / 6.48 / 6.72, ResNet-110 K = 4 9.82 / 9.81 / 9.98 / 9.99 / 10.04 / 10.14 / 10.14,
+// ResNet-1202 27.23 / 27.24 / 27.32 / 27.31 / 27.27 / 27.26 / 27.44 ms a logging interval.
 constexpr int kWgradLayers = 32;
 template <int NL> struct WgradMaps { CUtensorMap x[NL], y[NL]; };
+// Partial sums of several layers: those of the first `first_layers` in one place, of the others in another.
+struct GroupScratch {
+  float* first; int first_layers; float* other;
+  __device__ __forceinline__ float* layer(int z, size_t floats) const { return z < first_layers ? first + (size_t)z * floats : other + (size_t)(z - first_layers) * floats; }
+};
 template <int NL>
 __global__ void __launch_bounds__(kFwdThreads, NL == 1 ? 1 : 2)
-wgrad_halo_kernel(const __grid_constant__ WgradMaps<NL> maps, WgradParams p, float* __restrict__ partial, int* __restrict__ error_word) {
+wgrad_halo_kernel(const __grid_constant__ WgradMaps<NL> maps, WgradParams p, GroupScratch scratch, int* __restrict__ error_word) {
   const CUtensorMap& map_x = maps.x[NL == 1 ? 0 : blockIdx.z];
   const CUtensorMap& map_y = maps.y[NL == 1 ? 0 : blockIdx.z];
   extern __shared__ uint8_t smem_raw[];
@@ -703,7 +711,8 @@ wgrad_halo_kernel(const __grid_constant__ WgradMaps<NL> maps, WgradParams p, flo
       tc_fence_after();
       const int row = lane_grp * 32 + lane;
       const int sblk = row / p.kcx, ci = chunk_a * p.kcx + (row - sblk * p.kcx);
-      float* dst = partial + ((size_t)blockIdx.z * gridDim.x + blockIdx.x) * ((size_t)p.Co * 9 * p.Ci);
+      const size_t n = (size_t)p.Co * 9 * p.Ci;
+      float* dst = (NL == 1 ? scratch.first : scratch.layer(blockIdx.z, gridDim.x * n)) + blockIdx.x * n;
       const int nchunks = ncols >> 4;
       const size_t co_stride = (size_t)9 * p.Ci;
       for (int item = group; item < p.sgroups * nchunks; item += kEpiGroups) {
@@ -771,11 +780,11 @@ __global__ void __launch_bounds__(256) wgrad_halo_reduce_kernel(const float* __r
 // eighth CTA into one of eight sums, those in order.  128 threads of 32 registers: such a block still finds room beside a CTA of
 // conv_chain.cuh (640 threads of 96), which the kernel above, at one block of 256 per 32 outputs, does not (ResNet-1202 K = 4: 45 us
 // a launch of up to 24 layers, now 15; 29.3 -> 27.2 ms a logging interval).
-__global__ void __launch_bounds__(128, 16) wgrad_group_sum_kernel(const float2* __restrict__ partial, float* __restrict__ dw, int n2, int ctas, size_t dw_step) {
+__global__ void __launch_bounds__(128, 16) wgrad_group_sum_kernel(GroupScratch scratch, float* __restrict__ dw, int n2, int ctas, size_t dw_step) {
   const int i = blockIdx.x * 128 + threadIdx.x;
   grid_dependency_wait();
   if (i >= n2) return;
-  const float2* src = partial + (size_t)blockIdx.y * ctas * n2 + i;
+  const float2* src = reinterpret_cast<const float2*>(scratch.layer(blockIdx.y, (size_t)ctas * n2 * 2)) + i;
   float2 a[8];
 #pragma unroll
   for (int u = 0; u < 8; ++u) a[u] = u < ctas ? src[(size_t)u * n2] : make_float2(0.f, 0.f);

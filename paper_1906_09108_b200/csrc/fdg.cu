@@ -90,11 +90,16 @@ constexpr int kChainBlocks = 12, kLastBlocks = 4;
 inline int chain_piece(int blocks_left) {
   return blocks_left <= kLastBlocks ? blocks_left : std::min(kChainBlocks, blocks_left - kLastBlocks);
 }
+
 inline int largest_piece(int blocks) {
   int most = 0;
   for (int left = blocks; left > 0; left -= chain_piece(left)) most = std::max(most, chain_piece(left));
   return most;
 }
+// A weight gradient on a side stream takes as many CTAs as give each four images (measured with the present data
+// gradients: 16 / 24 / 32 / 48 CTAs at batch 128: K = 2 1228 / 1148 / 1091 / 1085 us per ResNet-56 iteration, K = 4
+// 1580 / 1505 / 1484 / 1498 us per ResNet-110 iteration; at batch 64 16 CTAs are the best by 1 %).
+inline int side_wgrad_cap(int batch) { return std::max(16, (batch + 3) / 4); }
 
 struct Module {
   int k;                                   // 1-based
@@ -131,17 +136,19 @@ struct Module {
   size_t red_partial_floats = 0;
   std::vector<Chain> chains;
   std::vector<int> chain_of;               // per unit: index into chains, or -1
+  // Scratch of a training iteration, in the FIFO slot of the inference pass (carve)
   bf16* dc = nullptr;                      // gradients of the chains' convolution outputs
   size_t dc_elems = 0;
-  float* stem_scratch = nullptr;           // partial sums of the stem's weight gradient, which runs beside the side stream's last ones
+  float* stem_scratch = nullptr;           // partial sums of the stem's weight gradient, which runs beside the side stream's last ones (null: behind them)
   size_t stem_scratch_floats = 0;
   char* side_tmp = nullptr;                // gradient of a block's input through its projection, formed beside the main chain
   float* side_partial = nullptr;           // as red_partial and scratch, for a projection's forward beside the main chain
   float* side_scratch = nullptr;
-  bool has_proj = false;
-  float* group_scratch = nullptr;          // partial sums of the grouped weight gradients
-  size_t group_scratch_floats = 0;
+  size_t side_elems = 0, side_partial_floats = 0, side_scratch_floats = 0;
+  float* group_scratch = nullptr;          // partial sums of the grouped weight gradients, beside wscratch (same stream, one behind the other)
+  size_t group_scratch_floats = 0, group_want_floats = 0;
   unsigned long long* exchange = nullptr;  // words of chain::Exchange, the epoch behind them
+  size_t exchange_words = 0;
   float *pooled = nullptr, *dlogits = nullptr, *loss_n = nullptr, *loss = nullptr;   // head
   // host state
   int64_t updates = 0;
@@ -226,6 +233,7 @@ struct fdg_ctx {
   // an inference pass that the next iteration has to wait for: it runs on the caller's stream, which module streams do not follow
   cudaEvent_t ev_eval = nullptr;
   bool eval_pending = false;
+  bool exchange_stale = false;             // the words of the modules' exchanges are another's (an inference pass, a loaded state)
   std::vector<cudaEvent_t> ev_cjoin;
   float* lr_dev = nullptr;
   float lr_on_device = -1.f;
@@ -489,11 +497,16 @@ static void plan_modules(fdg_ctx* c) {
           m.stem_scratch_floats = conv_wgrad_scratch_elems(c->bf16_mode, ConvGeom{a.batch, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, 3, 1, 1});
           break;
         case U_BASIC:
-          m.has_proj = m.has_proj || u.proj;
           u.t_a = tens(out_e); u.t_b = tens(out_e); u.t_c = tens(out_e); u.t_y = tens(out_e);
           u.q_b = bits(out_e); u.q_y = bits(out_e);
           u.st1 = stat(u.co); u.st2 = stat(u.co);
-          if (u.proj) { u.t_s = tens(out_e); u.sts = stat(u.co); }
+          if (u.proj) {
+            u.t_s = tens(out_e); u.sts = stat(u.co);
+            const int V = c->bf16_mode ? full_vec<bf16>() : full_vec<float>();
+            m.side_elems = std::max(m.side_elems, in_e);
+            m.side_partial_floats = std::max(m.side_partial_floats, (size_t)kRedPartialCtas * 2 * std::min(u.co, tc::kStatChunks * 16));
+            m.side_scratch_floats = std::max(m.side_scratch_floats, (size_t)red_geom((int)(out_e / u.co), u.co, u.co % V == 0 ? V : 1, c->esize).blocks * 2 * u.co);
+          }
           red_scratch(B * u.P * u.Q, u.co);
           wg_scratch(a.batch, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, u.stride, 1);
           wg_scratch(a.batch, u.P, u.Q, u.co, u.P, u.Q, u.co, 3, 1, 1);
@@ -546,10 +559,12 @@ static void plan_modules(fdg_ctx* c) {
       m.flip_blocks = (unsigned)std::min<size_t>(std::max<size_t>(largest / 8192, 8), 128);
     }
     plan_chains(a, m, c->bf16_mode);
-    m.group_scratch_floats = 0;
+    m.exchange_words = 0;
+    m.group_want_floats = 0;
     for (const Chain& ch : m.chains) {
       const Unit& u = m.units[ch.first];
-      m.group_scratch_floats = std::max(m.group_scratch_floats, wgrad_group_scratch_elems(a.batch, u.P, u.Q, ch.C, 2 * largest_piece(ch.last - ch.first + 1), 0));
+      m.exchange_words = std::max(m.exchange_words, chain::exchange_words(a.batch, ch.C) + 32);
+      m.group_want_floats = std::max(m.group_want_floats, wgrad_group_scratch_elems(a.batch, u.P, u.Q, ch.C, 2 * largest_piece(ch.last - ch.first + 1), c->cfg.serial ? 0 : side_wgrad_cap(a.batch)));
     }
     m.slot_elems = te; m.slot_floats = tf; m.max_act = maxa; m.scratch_floats = scr; m.wscratch_floats = wscr;
     for (const Unit& u : m.units) {     // where the inference pass finds each batch norm's statistics
@@ -643,17 +658,49 @@ static size_t carve(fdg_ctx* c, char* base, size_t* saved) {
   c->guard_table = cv.take<unsigned long long>((cv.count + 1) * sizeof(unsigned long long));   // one entry per buffer, itself included
   c->guards_saved = c->guard_offsets.size();
   *saved = align_up(cv.off, 256);
+  // Scratch of a training iteration takes the FIFO slots of the inference pass, so that a workspace is no larger for it: an iteration
+  // waits for the inference pass before it, and a pass for every iteration.  What finds no room there is done without.
+  struct Rest { char* at; size_t bytes; };
+  std::vector<Rest> rest;
+  for (const Module& m : c->mods) rest.push_back(Rest{m.fifo ? m.fifo + (size_t)m.D * m.slot_elems * es : nullptr, m.slot_elems * es});
+  auto take = [](Rest& r, size_t bytes) {
+    bytes = align_up(bytes, 256);
+    char* p = r.at;
+    if (p) r.at += bytes;
+    r.bytes -= bytes;
+    return p;
+  };
+  auto with_room = [&](size_t bytes) -> Rest* {                         // the smallest that has it, whosever slot it is
+    Rest* best = nullptr;
+    for (Rest& r : rest) if (bytes > 0 && r.bytes >= align_up(bytes, 256) && (!best || r.bytes < best->bytes)) best = &r;
+    return best;
+  };
+  for (Module& m : c->mods)
+    if (!m.chains.empty()) m.dc = reinterpret_cast<bf16*>(take(rest[m.k - 1], m.dc_elems * 2));      // half of what the slot has for these blocks
   for (Module& m : c->mods) {
-    if (m.stem_scratch_floats) m.stem_scratch = cv.take<float>(m.stem_scratch_floats * 4);
-    if (m.has_proj && c->use_graphs) {
-      m.side_tmp = cv.take<char>(align_up(m.max_act, 128) * es);
-      m.side_partial = cv.take<float>(m.red_partial_floats * 4);
-      m.side_scratch = cv.take<float>(std::max<size_t>(m.scratch_floats, 64) * 4);
-    }
     if (m.chains.empty()) continue;
-    m.dc = cv.take<bf16>(m.dc_elems * 2);
-    m.group_scratch = cv.take<float>(m.group_scratch_floats * 4);
-    m.exchange = cv.take<unsigned long long>((chain::kExchangeWords + 32) * 8);
+    Rest* r = with_room(m.exchange_words * 8);
+    m.exchange = r ? reinterpret_cast<unsigned long long*>(take(*r, m.exchange_words * 8)) : cv.take<unsigned long long>(m.exchange_words * 8);
+  }
+  for (Module& m : c->mods) {
+    Rest* r = with_room(m.stem_scratch_floats * 4);
+    m.stem_scratch = r ? reinterpret_cast<float*>(take(*r, m.stem_scratch_floats * 4)) : nullptr;
+    const size_t tmp = align_up(m.side_elems * es, 256), sums = align_up(m.side_partial_floats * 4, 256), scr = m.side_scratch_floats * 4;
+    r = c->use_graphs ? with_room(tmp + sums + scr) : nullptr;
+    if (r) {
+      m.side_tmp = take(*r, tmp);
+      m.side_partial = reinterpret_cast<float*>(take(*r, sums));
+      m.side_scratch = reinterpret_cast<float*>(take(*r, scr));
+    }
+  }
+  // The grouped weight gradients want most where the images are smallest: the module that wants most picks the largest rest.
+  std::vector<Module*> order;
+  for (Module& m : c->mods) if (m.group_want_floats > m.wscratch_floats) order.push_back(&m);
+  std::stable_sort(order.begin(), order.end(), [](const Module* x, const Module* y) { return x->group_want_floats > y->group_want_floats; });
+  for (Module* m : order) {
+    Rest& r = *std::max_element(rest.begin(), rest.end(), [](const Rest& x, const Rest& y) { return x.bytes < y.bytes; });
+    m->group_scratch_floats = std::min(m->group_want_floats, r.bytes / 4);
+    m->group_scratch = reinterpret_cast<float*>(take(r, m->group_scratch_floats * 4));
   }
   const size_t behind = c->guard_offsets.size() - c->guards_saved;
   c->guard_table2 = behind ? cv.take<unsigned long long>((behind + 1) * sizeof(unsigned long long)) : nullptr;
@@ -765,13 +812,14 @@ template <typename T>
 static int conv_fprop(Launch& L, Module& m, const ConvGeom& g, const T* x, const T* w, T* y, const T* res,
                       bool want_stats = false, float* stats = nullptr, long long run = -1, const EpiAffine* affine = nullptr,
                       float* partial = nullptr) {
+  const size_t partial_floats = partial ? m.side_partial_floats : m.red_partial_floats;
   if (!partial) partial = m.red_partial;
   L.begin(KC_CONV_FPROP, (in_elems(g) + w_elems(g) + out_elems(g) * (res ? 2 : 1)) * sizeof(T), conv_flops(g));
   int nparts = 0;
   if constexpr (std::is_same<T, bf16>::value) {
     halo::EpiReduce r{};
     r.mode = 1; r.partial = partial;
-    const WideStats ws{partial, m.red_partial_floats, stats, (size_t)g.N * g.P * g.Q, L.c->arch.bn_eps,
+    const WideStats ws{partial, partial_floats, stats, (size_t)g.N * g.P * g.Q, L.c->arch.bn_eps,
                        run >= 0 ? m.running + run : nullptr, kBnMomentum};
     L.note(bf16_conv_fprop(L.st, &L.c->tmaps, g, x, w, y, res, want_stats ? &r : nullptr, &nparts, L.c->tc_error, &L.c->launches,
                            (want_stats && stats) ? &ws : nullptr, affine));
@@ -878,7 +926,7 @@ static void chain_forward(fdg_ctx* c, Module& m, Launch& L, const Chain& ch, con
   chain::Tensors t = chain_tensors(m, ch, ch.first, slot, vslot, false);
   chain::TrainArgs fa{x, m.running + u.r1, kBnMomentum, rows > 1 ? (float)((double)rows / (double)(rows - 1)) : 1.f, c->arch.bn_eps, 1.0 / (double)rows};
   if (eval) { t.q0 = nullptr; fa.running = nullptr; }
-  const chain::Exchange ex{m.exchange, reinterpret_cast<unsigned int*>(m.exchange + chain::kExchangeWords)};
+  const chain::Exchange ex{m.exchange, reinterpret_cast<unsigned int*>(m.exchange + m.exchange_words - 32)};
   L.begin(KC_CONV_FPROP, (double)rows * ch.C * 2 * (2 * p.layers + 1), 18.0 * rows * ch.C * ch.C * p.layers);
   const CUtensorMap* mx;
   cudaError_t e = cached_group_map(&c->tmaps, x, p.N, p.H, p.W, ch.C, rows::kTileGroups * p.cb + 2, p.H + 2, &mx);
@@ -1162,7 +1210,7 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
           keep(i, 0, dy);
         }
         const chain::Tensors t = chain_tensors(m, ch, first, slot, vslot, true);
-        const chain::Exchange ex{m.exchange, reinterpret_cast<unsigned int*>(m.exchange + chain::kExchangeWords)};
+        const chain::Exchange ex{m.exchange, reinterpret_cast<unsigned int*>(m.exchange + m.exchange_words - 32)};
         L.begin(KC_CONV_DGRAD, (double)rows * ch.C * 2 * (3 * p.layers + 2), 18.0 * rows * ch.C * ch.C * p.layers);
         L.note(chain::launch(L.st, ch.C, chain::BACKWARD, CUtensorMap{}, p, t, chain::TrainArgs{}, ba, ex, c->tc_error));
         ++c->launches;
@@ -1180,8 +1228,9 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
           wy[l] = ba.dc + (size_t)l * E;
         }
         LS.begin(KC_CONV_WGRAD, (double)rows * ch.C * 4 * p.layers, 18.0 * rows * ch.C * ch.C * p.layers);
-        LS.note(run_wgrad_group(LS.st, &c->tmaps, p.N, p.H, p.W, ch.C, p.layers, wx.data(), wy.data(), m.grad + f.w1, t.p_step, m.group_scratch,
-                                c->tc_error, LS.st == m.stream2 ? c->tmaps.wgrad_side_cap : 0, &c->launches));
+        float* const scratch[2] = {m.group_scratch, m.wscratch};
+        const size_t scratch_floats[2] = {m.group_scratch_floats, m.wscratch_floats};
+        LS.note(run_wgrad_group(LS.st, &c->tmaps, p.N, p.H, p.W, ch.C, p.layers, wx.data(), wy.data(), m.grad + f.w1, t.p_step, scratch, scratch_floats, c->tc_error, LS.st == m.stream2 ? c->tmaps.wgrad_side_cap : 0, &c->launches));
         dy = ba.dx;
         i = first;
         continue;
@@ -1213,7 +1262,9 @@ static void backward_module(fdg_ctx* c, Module& m, Launch& L, Launch& LS, bool f
           keep(i, 3, T1);
         }
         // nothing follows on this stream: beside the side stream's last weight gradients, with partial sums of its own
-        conv_wgrad<T>(L, m, g, x, dc, m.grad + u.w1, nullptr, m.stem_scratch);
+        if (m.stem_scratch) { conv_wgrad<T>(L, m, g, x, dc, m.grad + u.w1, nullptr, m.stem_scratch); break; }
+        fork();
+        conv_wgrad<T>(LS, m, g, x, dc, m.grad + u.w1);
         break;
       }
       case U_BASIC: {
@@ -1585,10 +1636,7 @@ fdg_status fdg_create(const fdg_arch* arch, const fdg_config* cfg, void* dev_wor
   // per four tiles).
   c->tmaps.share = c->cfg.serial ? 1 : c->K;
   if (e == cudaSuccess && cached_sm_count(&c->tmaps) < chain::kMaxCtas) fit_chains(c, c->tmaps.sm_count);
-  // A weight gradient on a side stream takes as many CTAs as give each four images (measured with the present data
-  // gradients: 16 / 24 / 32 / 48 CTAs at batch 128: K = 2 1228 / 1148 / 1091 / 1085 us per ResNet-56 iteration, K = 4
-  // 1580 / 1505 / 1484 / 1498 us per ResNet-110 iteration; at batch 64 16 CTAs are the best by 1 %).
-  c->tmaps.wgrad_side_cap = std::max(16, (c->arch.batch + 3) / 4);
+  c->tmaps.wgrad_side_cap = side_wgrad_cap(c->arch.batch);
   // Blocks of a batch-norm apply kernel that first re-adds a convolution's partial sums: 4 per SM shared
   // between the module streams, not fewer than 222 (measured: 222 blocks at K = 4 against 74 / 111 / 148 / 185 /
   // 259 / 296; K = 2 is flat between 222 and 592).
@@ -1809,6 +1857,21 @@ static cudaError_t graph_step(fdg_ctx* c, cudaStream_t cs, float* loss_dev) {
   return e;
 }
 
+// Before an iteration: an inference pass still reads weights and running statistics that the iteration writes, and has worked where
+// the words of the exchanges are (their tags may be anything now: both start again at zero).
+static cudaError_t follow_eval(fdg_ctx* c, cudaStream_t cs) {
+  cudaError_t e = cudaSuccess;
+  if (c->eval_pending) {
+    e = cudaStreamWaitEvent(cs, c->ev_eval, 0);
+    for (Module& m : c->mods) if (e == cudaSuccess && !c->cfg.serial) e = cudaStreamWaitEvent(m.stream, c->ev_eval, 0);
+  }
+  if (c->exchange_stale)
+    for (Module& m : c->mods)
+      if (e == cudaSuccess && m.exchange) e = cudaMemsetAsync(m.exchange, 0, m.exchange_words * 8, (c->cfg.serial || c->graph_mode_entered) ? cs : m.stream);
+  if (e == cudaSuccess) c->eval_pending = c->exchange_stale = false;
+  return e;
+}
+
 fdg_status fdg_step(fdg_ctx* c, fdg_stream stream, const float* images_dev, const int32_t* labels_dev, float* loss_dev) {
   if (!c) return FDG_ERR_INVALID_ARG;
   if (!images_dev || !labels_dev) return fail(c, FDG_ERR_INVALID_ARG, "images and labels must not be null");
@@ -1821,13 +1884,8 @@ fdg_status fdg_step(fdg_ctx* c, fdg_stream stream, const float* images_dev, cons
   if (c->has_schedule) fdg_lr_at(&c->schedule, t, &c->lr);
   Module& m1 = c->mods[0];
   cudaError_t e = cudaSuccess;
-  // An inference pass still reads weights and running statistics that this iteration writes.
-  if (c->eval_pending) {
-    e = cudaStreamWaitEvent(cs, c->ev_eval, 0);
-    for (Module& m : c->mods) if (e == cudaSuccess && !serial) e = cudaStreamWaitEvent(m.stream, c->ev_eval, 0);
-    if (e != cudaSuccess) return cuda_fail(c, e, "waiting for the inference pass");
-    c->eval_pending = false;
-  }
+  e = follow_eval(c, cs);
+  if (e != cudaSuccess) return cuda_fail(c, e, "waiting for the inference pass");
   // Graphs take over once every module has run each of its passes at least once (all kernels
   // have been launched the ordinary way, their attributes are set, the pipeline is full).
   if (c->use_graphs && !c->graph_mode_entered && t > 2 * (int64_t)c->K + 1) {
@@ -2066,7 +2124,7 @@ fdg_status fdg_eval(fdg_ctx* c, fdg_stream stream, const float* images_dev, cons
   c->tmaps.share = share;
   c->last_stream = cs; c->stepped = true;
   if (e == cudaSuccess) e = cudaEventRecord(c->ev_eval, cs);
-  c->eval_pending = true;
+  c->eval_pending = c->exchange_stale = true;
   return e == cudaSuccess ? FDG_OK : cuda_fail(c, e, "inference pass");
 }
 
@@ -2082,6 +2140,7 @@ fdg_status fdg_drain(fdg_ctx* c, fdg_stream stream, float* losses_dev) {
     c->graph_mode_entered = false;
     c->last_batch = c->t;
     c->last_stream = cs; c->stepped = true;
+    e = follow_eval(c, cs);
     for (int i = 0; i < 2 * c->K - 2 && e == cudaSuccess; ++i) {
       c->t += 1;
       if (c->has_schedule) fdg_lr_at(&c->schedule, c->t, &c->lr);
@@ -2158,6 +2217,7 @@ fdg_status fdg_load_state(fdg_ctx* c, const void* src, size_t bytes) {
   e = cudaMemcpy(c->ws_base, static_cast<const char*>(src) + hb, c->ws_bytes, cudaMemcpyDefault);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) { c->latched = FDG_ERR_CUDA; return cuda_fail(c, e, "loading the state"); }
+  c->exchange_stale = true;
   c->t = h.t; c->lr = h.lr; c->lr_on_device = -1.f;
   c->graph_mode_entered = c->use_graphs && h.graph_mode_entered != 0;
   const int64_t* p = reinterpret_cast<const int64_t*>(host.data() + sizeof(StateHeader));

@@ -128,3 +128,33 @@ def test_inference(case):
     # half a bfloat16 unit (2^-9) for each tensor rounded differently, 6 n + 2 of them in a row at worst, adding up like noise
     assert np.linalg.norm(got - want) <= 2.0 ** -9 * (6 * case[2] + 2) ** 0.5 * np.linalg.norm(want)
     g.close()
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+@pytest.mark.parametrize("case", [(9, 20, 5, 1, ()), (76, 16, 3, 2, (4,)), (8, 12, 2, 3, (1, 3))])
+def test_inference_and_a_loaded_state_leave_a_run_s_training_as_it_is(case, graphs):
+    """Training keeps its scratch, the words of the exchanges among it, where an inference pass works: with passes in between and
+    a saved state loaded, parameters, momentum and running statistics are those of a run without, bit for bit."""
+    batch, hw, K = case[0], case[1], case[3]
+    feeds = [(torch.from_numpy(S.images(0, t, batch, hw, hw, 3)).cuda(), torch.from_numpy(S.labels(0, t, batch, 10)).cuda()) for t in range(1, 31)]
+    res = []
+    for between in (False, True):
+        g, _, _ = _context(case, lr=0.05, graphs=graphs)
+        blob = None
+        for t, (x, y) in enumerate(feeds):
+            g.step(x, y)
+            if between and t in (3, 14, 15, 24):
+                g.eval(x, y)
+            if between and t == 20:
+                blob = g.save_state()
+            if between and t == 22:                       # two iterations again, from the state of before
+                g.eval(x, y)
+                g.load_state(blob)
+                for again in feeds[21:23]:
+                    g.step(*again)
+        g.sync()
+        assert g.check_guards() == -1
+        res.append([np.asarray(get(k)) for get in (g.get_params, g.get_momentum, g.get_running) for k in range(1, K + 1)])
+        g.close()
+    for u, v in zip(*res):
+        assert np.isfinite(u).all() and np.array_equal(u, v)

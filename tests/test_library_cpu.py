@@ -92,3 +92,17 @@ def test_workspace_bytes_and_argument_checks(lib):
     assert lib.fdg_bn_scratch_bytes(64, C.byref(n)) == 0 and n.value >= 74 * 3 * 64 * 4
     assert lib.fdg_bn_scratch_bytes(0, C.byref(n)) == 1
     assert lib.fdg_bn_stats(0, C.c_void_p(256), 16, 64, 1e-5, C.c_void_p(256), C.c_void_p(256), 16, None) == 2
+
+
+@pytest.mark.parametrize("graphs, most", [(0, (363662, 866692, 3038155, 15990877, 1403272)), (1, (365934, 869761, 3543583, 18635078, 1416732))])
+def test_runs_of_blocks_take_no_workspace_of_their_own(lib, graphs, most):
+    """Scratch of the runs of blocks and of what goes beside the main chain lives in the slot of the inference pass: a
+    workspace is no larger (KiB) than what the layer-by-layer path alone was given."""
+    nets = [dict(n_per_stage=3), dict(n_per_stage=9), dict(n_per_stage=18), dict(n_per_stage=200, batch=64),
+            dict(blocks=(2, 2, 2, 2), widths=(64, 128, 256, 512), stem_width=64)]
+    for net, K, limit in zip(nets, (2, 2, 4, 4, 2), most):
+        blocks = sum(net["blocks"]) if "blocks" in net else 3 * net["n_per_stage"]
+        arch, cfg = B.make_arch(**net), _cfg(K, tuple(round(blocks * (i + 1) / K) for i in range(K - 1)), precision=B.FDG_BF16_TC, graphs=graphs)
+        n = C.c_size_t()
+        assert lib.fdg_workspace_bytes(C.byref(arch), C.byref(cfg), C.byref(n)) == 0
+        assert n.value <= limit * 1024, (net, K, n.value)
