@@ -108,10 +108,12 @@ inline bool s2_planned(const ConvGeom& g, int Ck, int Cn) {
   return (tc::conv_tc_supported(g.N, g.H, g.W, Ck, Cn, (size_t)g.N * g.P * g.Q) || halo::fwd_supported(g.N, g.H, g.W, Ck, Cn)) &&
          tc::conv_tc_supported(g.N, g.P, g.Q, Ck, Cn, (size_t)g.N * g.P * g.Q);
 }
-// (H and W, not P and Q: images of more than 128 columns stay with the CUDA cores, as their workspaces were planned)
+// (H and W, not P and Q: images of more than 128 columns, or 254 between layers of 16, 32 and 64 channels, stay with the CUDA cores,
+// as their workspaces were planned)
 inline bool tc_s2_fprop_eligible(const ConvGeom& g) { return halo_s2_shape(g) && s2_planned(g, g.Ci, g.Co); }
 inline bool tc_s2_dgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && s2_planned(g, g.Co, g.Ci); }
 // with the sums of the batch-norm backward that dx feeds: those are formed by the halo kernel, at full resolution from a spread-out dy
+// (an operator-level call may ask for them; the module-step does without)
 inline bool halo_s2_dgrad_sums_eligible(const ConvGeom& g) { return halo_s2_shape(g) && halo::fwd_supported(g.N, g.H, g.W, g.Co, g.Ci) && g.Ci <= 64; }
 inline bool halo_s2_wgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && halo::wgrad_supported(g.N, g.H, g.W, g.Ci, g.Co); }
 // 1x1 convolutions without padding (projection shortcuts), stride 1 or 2: one "tap" of the per-tap kernel on the output
@@ -348,11 +350,10 @@ inline cudaError_t run_wgrad_wide(cudaStream_t st, TensorMapCache* cache, int N,
 inline bool dgrad_uses_flipped(const ConvGeom& g) {
   return rows_eligible(g) || halo_dgrad_eligible(g) || tc_eligible(g) || tc_s2_dgrad_eligible(g) || tc_1x1_dgrad_eligible(g);
 }
-// Does the stride-2 weight gradient of this convolution run on the tensor cores, given a spread-out copy of dy?  (Also true
-// where only the data gradient does: the workspace of a module has had room for the copy then.)
-inline bool s2_uses_spread_dy(const ConvGeom& g) {
-  return (halo_s2_wgrad_eligible(g) || tc_s2_dgrad_eligible(g) || wide_s2_wgrad_eligible(g)) && g.Co % 8 == 0;
-}
+// Does the stride-2 weight gradient of this convolution run on the tensor cores, given a spread-out copy of dy?
+inline bool s2_uses_spread_dy(const ConvGeom& g) { return (halo_s2_wgrad_eligible(g) || wide_s2_wgrad_eligible(g)) && g.Co % 8 == 0; }
+// Has a module's workspace room for that copy?  Also where only the data gradient runs on the tensor cores: a saved state holds it.
+inline bool s2_has_spread_room(const ConvGeom& g) { return s2_uses_spread_dy(g) || (tc_s2_dgrad_eligible(g) && g.Co % 8 == 0); }
 
 // fp32 scratch elements a weight-gradient call may need (bf16 storage: whichever kernel is chosen).
 inline size_t conv_wgrad_scratch_elems(bool bf16_storage, const ConvGeom& g) {

@@ -530,7 +530,7 @@ static void plan_modules(fdg_ctx* c) {
       for (const Unit& u : m.units) {
         if ((u.type != U_BASIC && u.type != U_PREACT) || u.stride != 2) continue;
         ConvGeom g1{a.batch, u.H, u.W, u.ci, u.P, u.Q, u.co, 3, 3, u.stride, 1};
-        if (s2_uses_spread_dy(g1))
+        if (s2_has_spread_room(g1))
           m.up_elems = std::max(m.up_elems, B * u.H * u.W * u.co);
       }
     if (c->bf16_mode) {

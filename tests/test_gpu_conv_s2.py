@@ -41,14 +41,43 @@ def test_stride_2(shape, share):
     _close(ops.forward(s, x, wt, res=resy, share=share), want + resyo)
     y, part = ops.forward(s, x, wt, share=share, reduce=True)
     _close(y, want)
-    if part.shape[0]:
-        ys = y.float().cpu().numpy().astype(np.float64).reshape(-1, co)
-        tot = part.double().sum(dim=0).cpu().numpy()
-        # fp32 sums of at most a few thousand values per thread and row of sums
-        assert np.abs(tot[:co] - ys.sum(0)).max() <= 1e-5 * np.abs(ys).sum(0).max()
-        assert np.abs(tot[co:] - (ys ** 2).sum(0)).max() <= 1e-5 * (ys ** 2).sum(0).max()
+    assert part.shape[0] > 0
+    ys = y.float().cpu().numpy().astype(np.float64).reshape(-1, co)
+    tot = part.double().sum(dim=0).cpu().numpy()
+    # fp32 sums of at most a few thousand values per thread and row of sums
+    assert np.abs(tot[:co] - ys.sum(0)).max() <= 1e-5 * np.abs(ys).sum(0).max()
+    assert np.abs(tot[co:] - (ys ** 2).sum(0)).max() <= 1e-5 * (ys ** 2).sum(0).max()
     wf = ops.flip_weights(s, wt)
     dxo, _ = L.conv2d_backward(dyo, xo, wo, 2, 1)
     _close(ops.dgrad(s, dy, wt, wf, share=share), dxo)
     _close(ops.dgrad(s, dy, wt, wf, res=res, res_mask=gate, share=share), dxo + reso * (gateo > 0))
+    assert not ops.timed_out()
+
+
+@pytest.mark.parametrize("shape, spread", [((4, 2, 66, 8, 16), False), ((4, 4, 66, 48, 24), False), ((8, 8, 8, 16, 32), True), ((8, 8, 12, 24, 40), True)])
+def test_dy_is_spread_only_for_a_weight_gradient_that_reads_it(shape, spread):
+    """Rows of more than 64 pixels outside the halo-tile kernel's channels: the weight gradient runs on the CUDA cores, from dy
+    itself, and the scratch for the spread-out copy is left alone; elsewhere it holds dy at the even pixels of zeros."""
+    import ctypes as C
+    from paper_1906_09108_b200 import binding as B
+    ops = B.ConvOps(B.FDG_BF16_TC)
+    n, h, w, ci, co = shape
+    s = B.fdg_conv_shape(n, h, w, ci, co, 3, 2, 1)
+    assert ops.path(s, 1) and bool(ops.path(s, 2)) == spread
+    (x, xo), (dy, dyo) = _mk((n, h, w, ci), 1), _mk((n, h // 2, w // 2, co), 2)
+    room = C.c_size_t()
+    assert ops.lib.fdg_conv_wgrad_scratch_bytes(B.FDG_BF16_TC, C.byref(s), C.byref(room)) == B.FDG_OK
+    scratch, dw = torch.empty(room.value, dtype=torch.uint8, device="cuda"), torch.empty((co, 3, 3, ci), device="cuda")
+    ex = B.fdg_conv_extra()
+    up = torch.full((n, h, w, co), 7.0, dtype=torch.bfloat16, device="cuda")
+    ex.dy_spread = up.data_ptr()
+    assert ops.lib.fdg_conv_wgrad(B.FDG_BF16_TC, C.byref(s), x.data_ptr(), dy.data_ptr(), dw.data_ptr(), scratch.data_ptr(), room.value,
+                                  C.byref(ex), ops.status.data_ptr(), torch.cuda.current_stream().cuda_stream) == B.FDG_OK
+    want = torch.full_like(up, 7.0)
+    if spread:
+        want.zero_()
+        want[:, ::2, ::2] = dy
+    assert torch.equal(up, want)
+    dwo = L.conv2d_backward(dyo, xo, np.zeros((co, 3, 3, ci)), 2, 1)[1]
+    _close(dw, dwo, 1e-3)
     assert not ops.timed_out()
