@@ -583,20 +583,22 @@ def run_gpu(args):
         hbm_frac = top["bytes"] / sec / 1e9 / peaks["hbm_gbs"]
         if args.precision == "bf16":
             # The narrow layers' convolution as an operator of its own: the instructions that chain_kernel, which has the
-            # largest share of this workload's device time, issues for whole runs of blocks.  Timed alone on its most
-            # frequent shape; a 16-channel 3x3 layer has 72 flop per byte, far below the machine balance, so HBM is the
-            # roofline that bounds it.
+            # largest share of this workload's device time, issues for whole runs of blocks (the step launches this kernel
+            # only where a run does not: for blocks that change the shape).  Timed alone on the first stage's shape; a
+            # 16-channel 3x3 layer has 72 flop per byte, far below the machine balance, so HBM is the roofline that bounds it.
             us, nbytes, flops = kernel_bench(B, "fprop", "stage1")
             roof = dict(bound="hbm", achieved=nbytes / us / 1e3, peak=peaks["hbm_gbs"], unit="GB/s",
                         kernel="conv_rows_kernel, 3x3 stride-1 forward, [128,32,32,16] -> 16 channels",
                         avg_us=us, tflops=flops / us / 1e6,
                         how="64 launches on distinct buffers (pool > 2 x L2) replayed from a CUDA graph, CUDA events "
                             "on the replay stream",
+                        note="an operator-level launch: in the timed step chain_kernel takes these layers, whole runs of "
+                             "blocks at a time (per_class: conv_fprop and conv_dgrad)",
                         # dram__bytes_read.sum + dram__bytes_write.sum of one launch of this kernel on this shape,
                         # from the committed ncu summary; null once the kernel's source has changed since
                         traffic=profiled_traffic())
-            # The same kernels in the launch shape the module-step issues them in (a quarter of the SMs, four image
-            # tiles per CTA, reductions fused into the epilogue), the two batch-norm apply kernels at the stage-1
+            # The same kernels in the launch shape that the module-step gives a single layer (a quarter of the SMs, four
+            # image tiles per CTA, reductions fused into the epilogue), the two batch-norm apply kernels at the stage-1
             # shape, and the wide-layer convolution against the tensor roofline: each timed alone the same way.
             iso = {}
             for kind in STEP_VARIANTS:

@@ -15,9 +15,11 @@
 //     of one context always fit the device together (chain_plan.h: fit_device); those of two contexts at work on one device at the
 //     same time may not, and then a launch waits until all of its CTAs find room, which is what a cooperative launch promises.
 // Measured, 128 images of 32x32x16 on 64 CTAs: a layer's forward pass 8 us, its backward pass up to the weight gradient 11 us
-// (convolution and apply by themselves: 13 us, and 20 to 25); ResNet-56 with K = 2 1.09 -> 0.84 ms per iteration, an inference
-// batch of ResNet-110 0.79 -> 0.46 ms.  What bounds a layer now: the exchange (2.5 us with the CTAs' skew) and the latencies of
-// an epilogue of 16 warps (42 % of the issue slots), then the tensor instructions (1 us per image).
+// (convolution and apply by themselves: 13 us, and 20 to 25); ResNet-56 with K = 2 1.09 -> 0.78 ms per iteration, an inference
+// batch of ResNet-110 0.79 -> 0.41 ms.  What bounds a layer now: the exchange (2.5 us with the CTAs' skew) and the latencies of
+// an epilogue of 16 warps (42 % of the issue slots), then the tensor instructions (1 us per image).  640 threads leave the epilogue
+// 104 registers: 13 of the 18 variants spill, the backward ones of 12 to 16 bytes with 88 to 108 bytes of loads (16 channels in
+// four streams: none), the others 4 to 8 with 20 to 28 (64 channels: none).
 // The tensor instructions are those of conv_rows.cuh: an accumulator row is a group of G = 64 / C neighbouring pixels (128
 // bytes), a tile 16 image rows x 8 groups.  Pixel i of a group has the columns from (G - 1 - i) * C on: in this order the
 // filter taps a window position needs are neighbours in memory, and the nine taps are kept once (9 * C * C values).

@@ -34,6 +34,43 @@ def _context(case, lr=0.0, **kw):
     return g, params, arch
 
 
+def _runs(g, K):
+    """[(blocks of a run, runs)] of every module, and the blocks with a projection: what a context's layouts say."""
+    runs, proj = [], 0
+    for k in range(1, K + 1):
+        last = None
+        for name, ent in units_of(g.param_layout(k)):
+            if not name.startswith("block"):
+                last = None
+            elif len(ent) > 6:
+                proj, last = proj + 1, None
+            elif last is None:
+                runs.append(1)
+                last = True
+            else:
+                runs[-1] += 1
+    return runs, proj
+
+
+@pytest.mark.parametrize("case", CASES[:-1])
+def test_every_run_is_one_launch_forward_and_one_a_piece_backward(case):
+    """Convolution launches of one iteration in flight: stem, three a projection block, one a run; backward one for each
+    piece of a run (the last of up to 4 blocks, the others of up to 12)."""
+    g, _, arch = _context(case)
+    b, hw, K = arch["batch"], arch["in_h"], case[3]
+    runs, proj = _runs(g, K)
+    for t in range(1, 2 * K + 4):
+        if t == 2 * K + 3:
+            g.sync()
+            g.profile_enable()
+        g.step(torch.from_numpy(S.images(0, t, b, hw, hw, 3)).cuda(), torch.from_numpy(S.labels(0, t, b, 10)).cuda())
+    g.sync()
+    rows = {r["name"]: r["launches"] for r in g.profile_read()}
+    assert rows["conv_fprop"] == 1 + 3 * proj + len(runs)
+    assert rows["conv_dgrad"] == 3 * proj + sum(1 if n <= 4 else 1 + -(-(n - 4) // 12) for n in runs)
+    g.close()
+
+
 def _relmax(a, b):
     return float(np.abs(a - b).max() / max(np.abs(b).max(), 1e-30))
 
@@ -75,6 +112,40 @@ def test_forward(case, graphs):
             assert _relmax(y, L.round_bf16(L.relu_forward(L.batchnorm_forward(c2, *bn2, EPS)[0] + x))) <= 1e-2, (k, name)
             checked += 1
     assert checked > 0 and g.check_guards() == -1
+    g.close()
+
+
+@pytest.mark.parametrize("case", [(5, 28, 3, 1, ()), (149, 16, 2, 1, ()), (161, 32, 2, 4, (1, 2, 4)), (9, 20, 5, 1, ()), (2, 8, 13, 1, ())])
+def test_running_statistics_of_every_layer_of_a_run(case):
+    """One iteration moves the running mean and (unbiased) variance of each batch norm by a tenth towards those of the
+    convolution output that the iteration saved."""
+    g, _, arch = _context(case)
+    b, hw, K = arch["batch"], arch["in_h"], case[3]
+    for t in range(1, 2 * K + 4):
+        if t == 2 * K + 3:
+            before = [np.asarray(g.get_running(k), dtype=np.float64) for k in range(1, K + 1)]
+        g.step(torch.from_numpy(S.images(0, t, b, hw, hw, 3)).cuda(), torch.from_numpy(S.labels(0, t, b, 10)).cuda())
+    g.sync()
+    checked = 0
+    for k in range(1, K + 1):
+        after, at = np.asarray(g.get_running(k), dtype=np.float64), 0
+        for u, (name, ent) in enumerate(units_of(g.param_layout(k))):
+            if name == "head":
+                continue
+            co = ent[0][1][0]
+            for which in ((0,) if name == "stem" else (0, 2)):
+                if name != "stem" and len(ent) <= 6:
+                    c = g.saved_tensor(k, u, which)[1].reshape(-1, co).astype(np.float64)
+                    sq = (c ** 2).mean(0)
+                    for stat, got, old in ((c.mean(0), after[at:at + co], before[k - 1][at:at + co]),
+                                           (c.var(0) * len(c) / (len(c) - 1), after[at + co:at + 2 * co], before[k - 1][at + co:at + 2 * co])):
+                        # fp32 sums of a few hundred values a thread, fp32 results
+                        assert (np.abs(got - (0.9 * old + 0.1 * stat)) <= 1e-5 * (np.abs(old) + np.sqrt(sq) + sq)).all(), (k, name, which)
+                    checked += 1
+                at += 2 * co
+            at += 2 * co if len(ent) > 6 else 0
+        assert at == after.size
+    assert checked == 2 * (3 * case[2] - 2)
     g.close()
 
 

@@ -104,8 +104,8 @@ def _run(prec_name, shape, expect_tc):
     if expect_tc:
         # the launch shapes of a module-step: a quarter of the SMs per kernel (four modules side by side),
         # the weight gradient's pixel split capped as on the side stream (four images per CTA, at least 16 CTAs: 16 for
-        # these batches up to 64, 32 for 128), and, for stride 2, both gradients on the tensor cores through the
-        # spread-out dy
+        # these batches up to 64, 32 for 128), and, for stride 2, the weight gradient on the tensor cores through the
+        # spread-out dy (the data gradient runs on the output grid and leaves that scratch alone)
         sp = st == 2
         if sp:
             assert ops.path(s, 1)

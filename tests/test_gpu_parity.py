@@ -377,7 +377,7 @@ def test_resnet18_form_bf16():
 def test_wrn_widths_bf16_layer_by_layer():
     """Pre-activation blocks at the channel widths of WRN-28-10 (160 / 320 / 640, two blocks per stage, batch 4, K = 2):
     every layer of one backward pass of both modules -- the patch-tile and per-tap tensor-core convolutions, the
-    exact-tile weight gradient, the strided 3x3 layers through the spread-out dy, the 1x1 shortcuts (stride 1 from 16
+    exact-tile weight gradient (of the strided 3x3 layers through the spread-out dy), the 1x1 shortcuts (stride 1 from 16
     channels, stride 2 through the strided tensor map), the head with its batch norm -- recomputed by the oracle's
     layer functions from the library's own inputs to that layer, at 1e-2."""
     import fdg_synth as S
