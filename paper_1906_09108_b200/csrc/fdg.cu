@@ -84,8 +84,10 @@ struct Chain {
 };
 // The backward pass takes a run in pieces, from its end: the weight gradients of a piece run beside the next one.  The last
 // piece is short, because nothing runs beside its weight gradients.
-// (ResNet-56 K = 2 / ResNet-110 K = 4 / ResNet-1202 K = 4, ms a logging interval: pieces of 12 and 4 blocks 6.86 / 10.78 / 31.2, 8 and 3
-// 6.95 / 10.73 / 31.2, 5 and 2 7.08 / 10.85 / 31.4, up to 20 in one 7.00 / 11.09 / 30.5.)
+// (ResNet-56 K = 2 / its K = 3 on 28x28 / ResNet-110 K = 4 / ResNet-1202 K = 4, ms a logging interval: pieces of 12 and 4 blocks
+// 6.28 / 4.27 / 9.82 / 27.26, 16 and 4 6.27 / 4.28 / 9.81 / 27.13, 20 and 4 6.27 / 4.27 / 9.79 / 26.95, 16 and 8 6.37 / 4.28 / 9.81 / 26.93, 8 and 3
+// 6.38 / 4.28 / 9.82 / 27.68, 6 and 3 6.38 / 4.28 / 9.77 / 28.08, 12 and 2 6.48 / 4.26 / 9.89 / 27.18: the short last piece counts for the short
+// runs; longer ones before it gain 1 % where a run has 100 blocks.)
 constexpr int kChainBlocks = 12, kLastBlocks = 4;
 inline int chain_piece(int blocks_left) {
   return blocks_left <= kLastBlocks ? blocks_left : std::min(kChainBlocks, blocks_left - kLastBlocks);
