@@ -108,8 +108,8 @@ inline bool s2_planned(const ConvGeom& g, int Ck, int Cn) {
   return (tc::conv_tc_supported(g.N, g.H, g.W, Ck, Cn, (size_t)g.N * g.P * g.Q) || halo::fwd_supported(g.N, g.H, g.W, Ck, Cn)) &&
          tc::conv_tc_supported(g.N, g.P, g.Q, Ck, Cn, (size_t)g.N * g.P * g.Q);
 }
-// (H and W, not P and Q: images of more than 128 columns, or 254 between layers of 16, 32 and 64 channels, stay with the CUDA cores,
-// as their workspaces were planned)
+// (H and W, not P and Q: images of more than 128 columns, or 254 where the halo kernel covers the channels, stay with the CUDA
+// cores, as their workspaces were planned)
 inline bool tc_s2_fprop_eligible(const ConvGeom& g) { return halo_s2_shape(g) && s2_planned(g, g.Ci, g.Co); }
 inline bool tc_s2_dgrad_eligible(const ConvGeom& g) { return halo_s2_shape(g) && s2_planned(g, g.Co, g.Ci); }
 // with the sums of the batch-norm backward that dx feeds: those are formed by the halo kernel, at full resolution from a spread-out dy

@@ -10,9 +10,10 @@ from oracle import layers as L
 pytestmark = pytest.mark.gpu
 
 # (N, H, W, Ci, Co): one output pixel, rows that fill no tile, several images or row groups per tile, channel counts of less than
-# a chunk or of no whole number of chunks, several column tiles, the longest rows
+# a chunk or of no whole number of chunks, several column tiles, the longest rows (128; 254 for the channels of the halo kernel)
 SHAPES = [(1, 2, 2, 16, 32), (5, 6, 10, 16, 32), (5, 12, 12, 24, 40), (130, 14, 14, 32, 64), (2, 34, 20, 64, 128), (7, 8, 8, 256, 512),
-          (2, 32, 32, 160, 320), (1, 4, 128, 64, 64), (33, 4, 4, 48, 96)]
+          (2, 32, 32, 160, 320), (1, 4, 128, 64, 64), (33, 4, 4, 48, 96), (2, 6, 200, 16, 32),
+          (1, 4, 254, 16, 32)]
 
 
 def _mk(shape, seed, scale=1.0):
